@@ -131,13 +131,13 @@ struct MmaArgs {
     const long long* a1p_off;
     float* partial;             // k_dftgemm_ws3: 2 slots per block of 4 x 128 x 64 partial sums
     int* counters;              // k_dftgemm_ws3: per item, blocks that stored a part (reset by the last)
-    int sub;                    // k_dftgemm_ws3<2>: samples per image set
-    int iv0;                    // k_dftgemm_ws3<2>: image set of the chunk's first sample
+    int sub;                    // k_dftgemm_ws3: samples per image set
+    int iv0;                    // k_dftgemm_ws3: image set of the chunk's first sample
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
     int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..4)
-    const long long* wcum;      // k_dftgemm_ws3<1>: [C + 1] prefix sums of the channels' item costs per frame
-    const int* item_order;      // k_dftgemm_ws3<0>: per channel group (from c0 ipc), items in the order dealt to blocks
+    const long long* wcum;      // k_dftgemm_ws3<true>: [C + 1] prefix sums of the channels' item costs per frame
+    const int* item_order;      // k_dftgemm_ws3<false>: per channel group (from c0 ipc), items in the order dealt to blocks
 };
 
 __device__ __forceinline__ uint32_t pack_h2(float a, float b)
@@ -173,32 +173,6 @@ __device__ __forceinline__ void store_pixels16(float* op, int nk, int accumulate
 #pragma unroll
         for (int i = 0; i < 16; ++i)
             if (i < nk) op[i] = (accumulate ? op[i] : 0.f) + v[i];
-    }
-}
-
-// store_pixels16 for the sub-integration flush of k_dftgemm_ws3<2>: the same stores, the tail
-// of a tile cut by an 8-column grid in a rolled loop.  Indexing the sums at run time there
-// makes the compiler keep them in memory rather than spill the frame loop around an unrolled
-// flush inside it: measured 10.1 against 17-20 ms for the LWA block with an image set every 4
-// samples.  (The other schedules store once per work item and keep the unrolled form: for them
-// sums in memory cost 2x.)
-__device__ __forceinline__ void store_pixels16_flush(float* op, int nk, int accumulate, const float (&v)[16])
-{
-    if (nk == 16) {
-#pragma unroll
-        for (int i = 0; i < 16; i += 4) {
-            float4 w = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            if (accumulate) {
-                const float4 u = *reinterpret_cast<const float4*>(op + i);
-                w.x += u.x;
-                w.y += u.y;
-                w.z += u.z;
-                w.w += u.w;
-            }
-            *reinterpret_cast<float4*>(op + i) = w;
-        }
-    } else {
-        for (int i = 0; i < nk; ++i) op[i] = (accumulate ? op[i] : 0.f) + v[i];
     }
 }
 
@@ -2207,486 +2181,726 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 }
 
 // ---------------------------------------------------------------------------------
-// Third warp-specialised kernel: 16 epilogue warps and a control warpgroup in
-// separate register budgets (setmaxnreg), so that the threads issuing the MMAs and
-// tile copies -- blocking while the tensor pipe is busy -- hold up no epilogue warp.
+// Third warp-specialised kernel: the two epilogues run on warps of their own, so that
+// epilogue 1 of the next (sub-)frame, epilogue 2 of the last frame and the tensor core all
+// work at once, and the threads that issue MMAs and copies (which block while the tensor
+// pipe is busy) hold up none of them.  What bounds it is the tensor pipe with its
+// shared-memory operand reads: a frame of an LWA-station item (48 x 48 box, two pols) is
+// 1056 cycles of MMAs at the math rate.  With both epilogues on the same 16 warps, one
+// after the other (the form before this one), a frame took about 2.9 k cycles.
 // Work item, operands and TMEM layout as k_dftgemm_ws2, except that a channel's box rows
 // may come in H row parts (tall boxes): stage 2 sums over the box rows, so part h of frame t
 // is a step of its own -- its tile part through stage 1 (D1 of P nyh columns), epilogue 1 and
 // a stage-2 chain over its K range that adds to D2 (h > 0) -- and D2 holds the frame once
-// its last part is in.  Sub-frame u = t H + h; NB (2..4) tile-part buffers:
-//   copy thread (warp 18, lane 0), per sub-frame u:
-//     wait d1_full(u) -> copy tile part u+NB into the buffer S1(u) read (frames ahead -> L2)
-//   stage-1 issuer (warp 17, lane 0), per sub-frame u:
-//     wait b2_full(u) and tile part u+2 -> S1(u+2) -> d1_full[u&1]
-//   stage-2 issuer (warp 16, lane 0), per sub-frame u:
-//     wait b2_full(u) [and, at h = 0, d2_empty(t-1)] -> S2(u) -> b2_free[u&1] (H > 1),
-//     and at h = H-1 -> d2_full
-//   epilogue warps 0-15, per sub-frame u:
-//     wait d1_full(u) [and b2_free(u-2)] -> epilogue 1 (u) -> arrive b2_full[u&1];
-//     at h = 0: wait d2_full(t-1) -> epilogue 2 (t-1) -> arrive d2_empty
-// Epilogue 2 of frame t-1 runs after epilogue 1 of part 0 of frame t, before the later parts,
-// so the stage-2 chain of part 0 (which waits for it) never waits on a later epilogue 1.
-// Items are separated by two block-wide named barriers (operands loaded; item done).
-constexpr int kWs3Threads = 640;
-// Grid tiles requested into L2 this many frames before the shared-memory copy that
-// needs them: with two tile buffers a tile is copied only one frame ahead of its
-// stage-1 MMAs, which is less than the HBM latency; from L2 it arrives in time.
-constexpr int kTilePrefetch = 8;
+// its last part is in.  Stage 2 and D2 come in two halves of 32 kx, so that the chain of one
+// half runs while epilogue 2 reads the other.  Sub-frames u = t H + h are counted through all
+// the items of a block: no barrier separates items, only the operand tables wait (A1 for the
+// last S1 of the item before, A2 for its last S2).  NB (2..4) tile-part buffers:
+//   copy thread (warp 2, lane 0), per sub-frame u:
+//     wait tile_free(u-NB) -> copy tile part u -> tile_full
+//   stage-1 issuer (warp 1, lane 0), per sub-frame u:
+//     wait d1_free(u-2) and tile_full(u) -> S1(u) -> d1_full[u&1], tile_free
+//   epilogue-1 warps 4-7 (one per SM sub-partition: all 128 rows of D1), per sub-frame u:
+//     wait d1_full(u) and b2_free(u-2) -> D1 to registers -> arrive d1_free[u&1]
+//     -> FP16 operand B2[u&1] -> arrive b2_full[u&1]
+//   stage-2 issuer (warp 0, lane 0), per sub-frame u and half f:
+//     wait b2_full(u) [and, at h = 0, d2_empty[f](t-1)] -> S2(u, f)
+//     -> at h = H-1 d2_full[f]; after both halves b2_free[u&1]
+//   epilogue-2 warps 8-11 (half 0) and 12-15 (half 1), per frame t:
+//     wait d2_full[f](t) -> D2 to registers -> arrive d2_empty[f] -> products
+// Registers: 512 threads x 128 at launch = 128 control x 40 + 128 epilogue-1 x 88 + 256
+// epilogue-2 x 192: an epilogue-2 thread holds 32 pixels (128 sums) and 48 registers of
+// TMEM loads in flight.
+constexpr int kWs3Threads = 512;
+constexpr int kWs3CtlRegs = 72, kWs3E1Regs = 88, kWs3E2Regs = 176;
+static_assert(kWs3CtlRegs + kWs3E1Regs + 2 * kWs3E2Regs == 4 * 128, "setmaxnreg shares are the launch's registers");
 constexpr int kWs3MaxBlocks = 256;  // blocks per launch (one per SM) the split bookkeeping holds
 constexpr int kWs3MaxTileBufs = 4;  // tile-part buffers of k_dftgemm_ws3 (short row parts need more in flight)
 
-__device__ __forceinline__ void bar_all(int id)
+// x of lane 0: the same for the warp (a value every lane holds alike, but read from memory)
+__device__ __forceinline__ int ws3_uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// A whole warp's bounded wait for a barrier phase: the same answer for every lane.
+__device__ __forceinline__ bool ws3_wait(uint64_t* bar, uint32_t parity)
 {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(kWs3Threads) : "memory");
+    if (__all_sync(0xffffffffu, tc::mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+        if (__all_sync(0xffffffffu, tc::mbar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, clock64() - t0 > kWaitBudget)) return false;
+    }
 }
 
-// A split work item (k_dftgemm_ws3, equal shares) after this block stored its part
-// to its slot: the block that stores the item's last part -- counted on the item's
-// counter -- adds all parts in block order and writes (or adds) the images.  Kept
-// out of line so that the frame loop's register allocation does not carry it.
-__device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, int c, int ky, int kx0, size_t px,
-                                              long long U, int tid, int* split_slot, int* split_n)
+// The same with the phase's parity in bit `slot` of ph, which flips when the phase is over.
+__device__ __forceinline__ bool ws3_wait(uint64_t* bar, uint32_t& ph, int slot)
 {
+    if (!ws3_wait(bar, (ph >> slot) & 1u)) return false;
+    ph ^= 1u << slot;
+    return true;
+}
+
+// One warp's share of epilogue 1: lanes = 32 kx of one (half, re | im) quarter of D1, NYC chunks
+// of 8 columns per pol -> the 16-byte chunks of B2 rows row (real part of E) and row + 32
+// (imaginary part).  B2's K order interleaves the parts: chunk 2 j holds rows 8 j .. 8 j + 7 of
+// the first part of [Hr | -Hi] or [Hi | Hr], chunk 2 j + 1 those of the second, so that the four
+// chunks of a batch sit at fixed offsets of one 64-wide K panel.  With one warp per SM
+// sub-partition the step is bound by its instructions, and a taken branch costs about 20 cycles
+// against 1.5 for straight-line code, so it is unrolled for each NYC.  The next batch is loaded
+// while the last one is stored; d1_free is signalled as soon as the last load is in registers.
+template <int NYC>
+__device__ __forceinline__ void ws3_epilogue1(uint32_t taddr, int P, bool imw, int lane, uint32_t b2, int row, int R2,
+                                              uint64_t* d1_free)
+{
+    constexpr int NB = (NYC + 3) / 4;  // batches of up to 4 chunks (one K panel) per pol
+    const uint32_t panel = (uint32_t)R2 * 128, sg = imw ? 0x80008000u : 0u;
+    const uint32_t x7 = (uint32_t)(lane & 7) << 4;
+    const uint32_t d0 = b2 + (uint32_t)(row + lane) * 128, e0 = imw ? 16u : 0u;
+    uint32_t r[32];
+    auto load = [&](uint32_t ta, int n) {
+        if (n == 4) tc::tmem_ld32(ta, r);
+        else if (n == 2) tc::tmem_ld16(ta, r);
+        else if (n == 1) tmem_ld8(ta, r);
+        else {
+            tc::tmem_ld16(ta, r);
+            tmem_ld8(ta + 16, r + 16);
+        }
+    };
+    constexpr int first = NYC < 4 ? NYC : 4;
+    load(taddr, first);
+#pragma unroll 1
+    for (int p = 0; p < P; ++p) {
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            const int n = NYC - 4 * j < 4 ? NYC - 4 * j : 4;
+            tc::tmem_wait_ld(r);
+            uint32_t h[16];
+#pragma unroll
+            for (int i = 0; i < 4 * n; ++i) h[i] = pack_h2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+            if (j + 1 < NB) {
+                load(taddr + 8 * (NYC * p + 4 * (j + 1)), NYC - 4 * (j + 1) < 4 ? NYC - 4 * (j + 1) : 4);
+            } else if (p + 1 < P) {
+                load(taddr + 8 * NYC, first);
+            } else {  // D1 is read
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(d1_free);
+            }
+            const uint32_t q = d0 + p * (64 * 128) + j * panel;
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                const uint32_t lo = q + ((uint32_t)(32 * i) ^ x7 ^ e0), hi = q + ((uint32_t)(32 * i + 16) ^ x7 ^ e0);
+                tc::st_shared_v4(lo, h[4 * i] ^ sg, h[4 * i + 1] ^ sg, h[4 * i + 2] ^ sg, h[4 * i + 3] ^ sg);
+                tc::st_shared_v4(hi + 32 * 128, h[4 * i], h[4 * i + 1], h[4 * i + 2], h[4 * i + 3]);
+            }
+        }
+    }
+}
+
+// |X|^2 of 8 pixels (x: 8 real, 8 imaginary parts) added to xx[o..o+7]
+__device__ __forceinline__ void ws3_xx(const uint32_t (&x)[16], int o, float (&xx)[32])
+{
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+        const float r0 = __uint_as_float(x[i]), r1 = __uint_as_float(x[i + 1]);
+        const float i0 = __uint_as_float(x[8 + i]), i1 = __uint_as_float(x[9 + i]);
+        fma2x2(xx[o + i], xx[o + i + 1], i0, i1, i0, i1);
+        fma2x2(xx[o + i], xx[o + i + 1], r0, r1, r0, r1);
+    }
+}
+
+// X Y* of 8 pixels added to rx, ix [o..o+7]
+__device__ __forceinline__ void ws3_xy(const uint32_t (&x)[16], const uint32_t (&y)[16], int o, float (&rx)[32],
+                                       float (&ix)[32])
+{
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+        const float xr0 = __uint_as_float(x[i]), xr1 = __uint_as_float(x[i + 1]);
+        const float xi0 = __uint_as_float(x[8 + i]), xi1 = __uint_as_float(x[9 + i]);
+        const float yr0 = __uint_as_float(y[i]), yr1 = __uint_as_float(y[i + 1]);
+        const float yi0 = __uint_as_float(y[8 + i]), yi1 = __uint_as_float(y[9 + i]);
+        fma2x2(rx[o + i], rx[o + i + 1], xi0, xi1, yi0, yi1);
+        fma2x2(rx[o + i], rx[o + i + 1], xr0, xr1, yr0, yr1);
+        fma2x2(ix[o + i], ix[o + i + 1], -xr0, -xr1, yi0, yi1);
+        fma2x2(ix[o + i], ix[o + i + 1], xi0, xi1, yr0, yr1);
+    }
+}
+
+// One warp's share of epilogue 2: its 32 ky rows x 32 kx, 8 kx per batch; the loads of Y run
+// under the products of X and the next X under those of Y.
+template <int P>
+__device__ __forceinline__ void ws3_epilogue2(uint32_t taddr, float (&xx)[32], float (&yy)[32], float (&rx)[32],
+                                              float (&ix)[32], int lane, uint64_t* d2_empty)
+{
+    uint32_t x[2][16], y[16];
+    auto load_x = [&](int b) {
+        tmem_ld8(taddr + 8 * b, x[b & 1]);
+        tmem_ld8(taddr + 32 + 8 * b, x[b & 1] + 8);
+    };
+    auto done = [&]() {  // this warp's part of D2 is in registers
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(d2_empty);
+    };
+    load_x(0);
+    tc::tmem_wait_ld(x[0]);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        if (P == 2) {
+            tmem_ld8(taddr + 64 + 8 * b, y);
+            tmem_ld8(taddr + 96 + 8 * b, y + 8);
+        } else if (b < 3) {
+            load_x(b + 1);
+        }
+        ws3_xx(x[b & 1], 8 * b, xx);
+        if (P == 2) {
+            tc::tmem_wait_ld(y);
+            if (b < 3) load_x(b + 1);
+            else done();
+            ws3_xx(y, 8 * b, yy);
+            ws3_xy(x[b & 1], y, 8 * b, rx, ix);
+        } else if (b == 3) {
+            done();
+        }
+        if (b < 3) tc::tmem_wait_ld(x[(b + 1) & 1]);
+    }
+}
+
+// 32 consecutive image pixels of one product (nk of them inside the image, a multiple of 8):
+// written, or added to what is there
+__device__ __forceinline__ void ws3_store32(float* o, int nk, int accumulate, const float (&v)[32])
+{
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+        if (i < nk) {
+            float4 w = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            if (accumulate) {
+                const float4 u = *reinterpret_cast<const float4*>(o + i);
+                w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
+            }
+            *reinterpret_cast<float4*>(o + i) = w;
+        }
+    }
+}
+
+// Partial sums of a split item, as epilogue-2 thread `tid2` of 256 holds them: float4 k of
+// product pr at ((8 pr + k) 256 + tid2) 4 (consecutive threads, consecutive 16 bytes).
+__device__ __forceinline__ void ws3_store_partial(float* slot, int pr, int tid2, const float (&v)[32])
+{
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        *reinterpret_cast<float4*>(slot + ((size_t)(8 * pr + k) * 256 + tid2) * 4) =
+            make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+}
+
+// A split work item (equal shares) after this block stored its part to its slot: the block
+// that stores the item's last part -- counted on the item's counter -- adds all parts in block
+// order and writes (or adds) the images.  start: first unit of every block (shared memory,
+// filled once per launch: searching the plan's weights here, on one thread, cost 40 us an
+// item).  Kept out of line so that the frame loop's register allocation does not carry it.
+__device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float* o, int nk, int tid2,
+                                              const uint32_t* start, int* split_b)
+{
+    const uint32_t s0 = (uint32_t)item * (uint32_t)a.nt, s1 = s0 + (uint32_t)a.nt - 1;
     __threadfence();
-    asm volatile("bar.sync 3, 512;" ::: "memory");
-    if (tid == 0) {
-        const long long s0 = (long long)item * a.nt, s1 = s0 + a.nt - 1;
-        const int G = gridDim.x, ipc = a.n_kb * a.n_g;
-        auto start = [&](int b) { return split_start(a.wcum, a.c0, a.n_ch, ipc, a.nt, b, G); };
-        auto owner = [&](long long f) {  // the block whose range [start(b), start(b + 1)) holds f
+    asm volatile("bar.sync 3, 256;" ::: "memory");
+    if (tid2 == 0) {
+        const int G = gridDim.x;
+        auto owner = [&](uint32_t f) {  // the block whose range [start[b], start[b + 1]) holds f
             int lo = 0, hi = G;
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (start(mid) <= f) lo = mid;
+                if (start[mid] <= f) lo = mid;
                 else hi = mid;
             }
             return lo;
         };
-        (void)U;
-        int n = 0;
-        const int b1 = owner(s1);
-        for (int b = owner(s0); b <= b1; ++b) {
-            const long long bw0 = start(b);
-            if (bw0 == start(b + 1)) continue;  // no frames: no part
-            split_slot[n++] = 2 * b + (s0 <= bw0 ? 0 : 1);
-        }
+        const int b0 = owner(s0), b1 = owner(s1);
+        int n = 0;  // parts: blocks with any frames
+        for (int b = b0; b <= b1; ++b) n += start[b] != start[b + 1];
         const bool last = atomicAdd(&a.counters[item], 1) == n - 1;
         if (last) a.counters[item] = 0;  // ready for the next launch
-        *split_n = last ? n : 0;
+        split_b[0] = b0;
+        split_b[1] = last ? b1 : -1;
     }
-    asm volatile("bar.sync 3, 512;" ::: "memory");
-    const int n = *split_n;
-    if (n > 0 && ky < a.N && kx0 < a.N) {
+    asm volatile("bar.sync 3, 256;" ::: "memory");
+    const int b0 = split_b[0], b1 = split_b[1];
+    if (b1 >= 0 && nk > 0) {
         __threadfence();
         const size_t NN = (size_t)a.N * a.N;
-        const int nk = min(16, a.N - kx0);
-        for (int pr = 0; pr < a.nprod; ++pr) {  // one product at a time: 16 live sums
-            float sum[16];
+        for (int pr = 0; pr < a.nprod; ++pr) {  // one product at a time: 32 live sums
+            float sum[32];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) sum[i] = 0.f;
-            for (int k = 0; k < n; ++k) {
-                const float* q = a.partial + ((size_t)split_slot[k] * 4 + pr) * 8192 + px;
+            for (int i = 0; i < 32; ++i) sum[i] = 0.f;
+            for (int b = b0; b <= b1; ++b) {
+                if (start[b] == start[b + 1]) continue;
+                const float4* q =
+                    reinterpret_cast<const float4*>(a.partial + (size_t)(2 * b + (s0 <= start[b] ? 0 : 1)) * 4 * 8192) +
+                    (size_t)8 * pr * 256 + tid2;
 #pragma unroll
-                for (int i = 0; i < 16; i += 4) {
-                    const float4 u = __ldcg(reinterpret_cast<const float4*>(q + i));
-                    sum[i] += u.x;
-                    sum[i + 1] += u.y;
-                    sum[i + 2] += u.z;
-                    sum[i + 3] += u.w;
+                for (int i = 0; i < 8; ++i) {
+                    const float4 u = __ldcg(q + (size_t)i * 256);
+                    sum[4 * i] += u.x;
+                    sum[4 * i + 1] += u.y;
+                    sum[4 * i + 2] += u.z;
+                    sum[4 * i + 3] += u.w;
                 }
             }
-            store_pixels16(a.out + ((size_t)c * a.nprod + pr) * NN + (size_t)ky * a.N + kx0, nk, a.accumulate, sum);
+            ws3_store32(o + (size_t)pr * NN, nk, a.accumulate, sum);
         }
     }
+    asm volatile("bar.sync 3, 256;" ::: "memory");  // split_b is free again
 }
 
-// MODE 0: whole items, 1: equal shares (split items), 2: whole items, sub-integrations.
-// PARTS: some channel of the plan has more than one row part (else every H is 1 at compile time).
-template <int MODE, bool PARTS>
+// The segments (work item, first frame, frames) of a block: every role walks them alike.
+// SPLIT: the (item, frame) units [w, w1) in item-major order; else whole items.
+struct Ws3Seg {
+    int item, fs, nt;
+};
+
+template <bool SPLIT>
+__device__ __forceinline__ bool ws3_next(const MmaArgs& a, int items, int it, long long& w, long long w1, Ws3Seg& s)
+{
+    if (SPLIT) {
+        if (w >= w1) return false;
+        s.item = (int)(w / a.nt);
+        s.fs = (int)(w % a.nt);
+        s.nt = (int)min((long long)(a.nt - s.fs), w1 - w);
+        w += s.nt;
+        return true;
+    }
+    s.item = blockIdx.x + it * gridDim.x;
+    if (s.item >= items) return false;
+    if (a.item_order) s.item = a.item_order[(size_t)a.c0 * a.n_kb * a.n_g + s.item];
+    s.fs = 0;
+    s.nt = a.nt;
+    return true;
+}
+
+// Whether any of the 256 epilogue-2 threads says so, the same answer for all of them.
+__device__ __forceinline__ bool ws3_e2_any(bool mine)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "bar.red.or.pred p, 3, 256, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)mine)
+        : "memory");
+    return r != 0;
+}
+
+// The epilogue-2 warps' walk through the block's segments.  Returns false when a wait ran out.
+template <bool SPLIT, int P>
+__device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int items, long long w0, long long w1,
+                                            int warp, int lane, uint64_t* d2_full, uint64_t* d2_empty,
+                                            const uint32_t* start, int* split_b)
+{
+    const int q4 = warp & 3, hf = (warp >> 2) & 1, tid2 = 32 * (warp - 8) + lane;
+    const uint32_t taddr = tmem + ((uint32_t)(32 * q4) << 16) + 256 + 64 * P * hf;
+    const size_t NN = (size_t)a.N * a.N;
+    uint32_t ph = 0;
+    long long w = w0;
+    Ws3Seg s;
+    for (int it = 0; ws3_next<SPLIT>(a, items, it, w, w1, s); ++it) {
+        const int g = s.item % a.n_g, kb = (s.item / a.n_g) % a.n_kb, c = a.c0 + s.item / (a.n_g * a.n_kb);
+        // this thread's pixels: row ky, kx0 .. kx0 + nk - 1 (none outside the image)
+        const int ky = 128 * kb + 32 * q4 + lane, kx0 = 64 * g + 32 * hf;
+        const int nk = ky < a.N ? min(32, max(0, a.N - kx0)) : 0;
+        const size_t px = (size_t)c * a.nprod * NN + (size_t)ky * a.N + kx0;
+        float xx[32], yy[32], rx[32], ix[32];
+        auto clear = [&]() {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) xx[i] = yy[i] = rx[i] = ix[i] = 0.f;
+        };
+        auto store = [&](float* o) {
+            ws3_store32(o, nk, a.accumulate, xx);
+            if (P == 2) {
+                ws3_store32(o + NN, nk, a.accumulate, yy);
+                ws3_store32(o + 2 * NN, nk, a.accumulate, rx);
+                ws3_store32(o + 3 * NN, nk, a.accumulate, ix);
+            }
+        };
+        clear();
+        int iv = a.iv0, left = a.sub;  // sub-integrations: image set of this frame and frames left in it
+        bool good = true;
+        for (int t = 0; t < s.nt; ++t) {
+            good = ws3_wait(&d2_full[hf], ph);
+            if (!good) break;
+            ph ^= 1u;
+            tc::fence_after_sync();
+            ws3_epilogue2<P>(taddr, xx, yy, rx, ix, lane, &d2_empty[hf]);
+            if (!SPLIT && --left == 0) {  // write (or add) this interval's sums (without sub-integrations: never)
+                store(a.out + (size_t)iv * a.C * a.nprod * NN + px);
+                clear();
+                ++iv;
+                left = a.sub;
+            }
+        }
+        // the epilogue-2 warps leave together when one of them gave up (ws3_split_finish has barriers)
+        if (SPLIT) good = !ws3_e2_any(!good);
+        if (!good) return false;
+        if (SPLIT && s.nt != a.nt) {  // part of an item: to this block's slot
+            float* slot = a.partial + (2 * (size_t)blockIdx.x + (it == 0 ? 0 : 1)) * 4 * 8192;
+            ws3_store_partial(slot, 0, tid2, xx);
+            if (P == 2) {
+                ws3_store_partial(slot, 1, tid2, yy);
+                ws3_store_partial(slot, 2, tid2, rx);
+                ws3_store_partial(slot, 3, tid2, ix);
+            }
+            ws3_split_finish(a, s.item, a.out + px, nk, tid2, start, split_b);
+        } else if (a.sub == 0) {
+            store(a.out + px);
+        }
+    }
+    return true;
+}
+
+// What the stage issuers and epilogue 1 share: operand addresses and barriers of the block.
+struct Ws3Bars {
+    uint64_t bar_a, a2_full, d1_full[2], d1_free[2], b2_full[2], b2_free[2], d2_full[2], d2_empty[2],
+        tile_full[kWs3MaxTileBufs], tile_free[kWs3MaxTileBufs], drain[2];
+};
+
+// The issuers' and epilogue 1's steps through NU sub-frames of one item, each unrolled for the
+// item's K steps (KS = 0: any number): a step is bound by its own instructions -- about 90 cycles
+// a wait, 20 a taken branch -- beside MMAs of 48 to 64 cycles.
+
+// Stage 1: KS K steps of 16 from A1 and tile buffer b into D1[u & 1].
+template <int KS>
+__device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, int& b, int NB, uint32_t& ph_free,
+                                       uint32_t& ph_tile, uint32_t tmem, uint32_t d1_cols, uint32_t da, uint32_t b1,
+                                       uint32_t b1_bytes, int N1, uint32_t lead)
+{
+    const uint32_t id1 = tc::idesc_f16_f32(128, N1), pb = (uint32_t)N1 * 8;
+#pragma unroll 1
+    for (const unsigned end = u + NU; u != end; ++u) {
+        const int sl = u & 1;
+        if (u >= 2 && !ws3_wait(&m.d1_free[sl], ph_free, sl)) return false;  // E1(u-2) has read D1[sl]
+        if (!ws3_wait(&m.tile_full[b], ph_tile, b)) return false;
+        tc::fence_after_sync();
+        const uint32_t db = tc::desc_sw128_lo(b1 + b * b1_bytes);
+        const uint32_t d = tmem + sl * d1_cols;
+        if (KS) {
+#pragma unroll
+            for (int k = 0; k < KS; ++k)
+                tc::mma_f16_lead(d, da + (k >> 2) * (128 * 8) + (k & 3) * 2, db + (k >> 2) * pb + (k & 3) * 2, id1, k > 0,
+                                 lead);
+        } else {
+            for (int k = 0; k < ks; ++k)
+                tc::mma_f16_lead(d, da + (k >> 2) * (128 * 8) + (k & 3) * 2, db + (k >> 2) * pb + (k & 3) * 2, id1, k > 0,
+                                 lead);
+        }
+        tc::mma_commit_lead(&m.d1_full[sl], lead);
+        tc::mma_commit_lead(&m.tile_free[b], lead);
+        if (++b == NB) b = 0;
+    }
+    return true;
+}
+
+// Stage 2: KS = nyh / 8 K steps from A2 (TMEM, part h at nyh words) and B2[u & 1] into both halves of D2.
+template <int KS>
+__device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsigned& u, bool& any, uint32_t& ph_b2,
+                                       uint32_t& ph_e, uint32_t d2, uint32_t a2, int P, uint32_t b2, uint32_t b2_bytes,
+                                       uint32_t lead)
+{
+    const uint32_t id2 = tc::idesc_f16_f32(128, 64 * P), pb = (uint32_t)(128 * P) * 8;
+#pragma unroll 1
+    for (int t = 0; t < nt; ++t) {
+#pragma unroll 1
+        for (int h = 0; h < H; ++h, ++u) {
+            const int sl = u & 1;
+            if (!ws3_wait(&m.b2_full[sl], ph_b2, sl)) return false;
+            const uint32_t at = a2 + h * 8 * ks;
+#pragma unroll
+            for (int f = 0; f < 2; ++f) {
+                if (h == 0 && any && !ws3_wait(&m.d2_empty[f], ph_e, f)) return false;
+                tc::fence_after_sync();
+                const uint32_t db = tc::desc_sw128_lo(b2 + sl * b2_bytes + 64 * P * 128 * f);
+                const uint32_t d = d2 + 64 * P * f;
+                if (KS) {
+#pragma unroll
+                    for (int k = 0; k < KS; ++k)
+                        tc::mma_f16_ta_lead(d, at + 8 * k, db + (k >> 2) * pb + (k & 3) * 2, id2, k > 0 || h > 0, lead);
+                } else {
+                    for (int k = 0; k < ks; ++k)
+                        tc::mma_f16_ta_lead(d, at + 8 * k, db + (k >> 2) * pb + (k & 3) * 2, id2, k > 0 || h > 0, lead);
+                }
+                if (h == H - 1) tc::mma_commit_lead(&m.d2_full[f], lead);
+            }
+            tc::mma_commit_lead(&m.b2_free[sl], lead);  // S2(u) has read B2[sl]
+        }
+        any = true;
+    }
+    return true;
+}
+
+// Epilogue 1 of NU sub-frames.  held: B2 slots whose S2 was not waited for yet.
+template <int NYC>
+__device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t& ph_d1, uint32_t& ph_bf, uint32_t& held,
+                                       uint32_t taddr, uint32_t d1_cols, int P, bool imw, int lane, uint32_t b2,
+                                       uint32_t b2_bytes, int row)
+{
+#pragma unroll 1
+    for (const unsigned end = u + NU; u != end; ++u) {
+        const int sl = u & 1;
+        if (!ws3_wait(&m.d1_full[sl], ph_d1, sl)) return false;
+        if (((held >> sl) & 1u) && !ws3_wait(&m.b2_free[sl], ph_bf, sl)) return false;
+        held |= 1u << sl;
+        tc::fence_after_sync();
+        ws3_epilogue1<NYC>(taddr + sl * d1_cols, P, imw, lane, b2 + sl * b2_bytes, row, 128 * P, &m.d1_free[sl]);
+        tc::fence_proxy_async();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&m.b2_full[sl]);
+    }
+    return true;
+}
+
+// SPLIT: equal shares of the launch's (item, frame) units (items may be split between blocks),
+// else whole items, with sub-integrations when a.sub > 0.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ uint64_t bar_a, d1_full[2], b2_full[2], b2_free[2], d2_full, d2_empty, tile_full[kWs3MaxTileBufs],
-        tile_free[kWs3MaxTileBufs], drain[2];
+    __shared__ Ws3Bars m;
     __shared__ uint32_t tmem_sh;
     __shared__ int err_sh;
-    __shared__ int split_slot[kWs3MaxBlocks];  // partial slots of a split item, in block order
-    __shared__ int split_n;                    // > 0: this block completes the item; sum split_n slots
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ uint32_t start[SPLIT ? kWs3MaxBlocks + 1 : 1];  // first unit of every block
+    __shared__ int split_b[2];  // blocks of a split item; the second is -1 unless this block completes it
+    const int tid = threadIdx.x, warp = ws3_uni(tid >> 5), lane = tid & 31;
     if (warp == 0) {
         tc::tmem_alloc(&tmem_sh, 512);
         tc::tmem_relinquish();
     }
-    if (tid == 0) {
-        tc::mbar_init(&bar_a, 1);
+    if (tid == 32) {
+        tc::mbar_init(&m.bar_a, 1);
+        tc::mbar_init(&m.a2_full, 4);
         for (int i = 0; i < 2; ++i) {
-            tc::mbar_init(&d1_full[i], 1);
-            tc::mbar_init(&b2_full[i], 16);
-            tc::mbar_init(&b2_free[i], 1);
-            tc::mbar_init(&drain[i], 1);
+            tc::mbar_init(&m.d1_full[i], 1);
+            tc::mbar_init(&m.d1_free[i], 4);
+            tc::mbar_init(&m.b2_full[i], 4);
+            tc::mbar_init(&m.b2_free[i], 1);
+            tc::mbar_init(&m.d2_full[i], 1);
+            tc::mbar_init(&m.d2_empty[i], 4);
+            tc::mbar_init(&m.drain[i], 1);
         }
         for (int i = 0; i < kWs3MaxTileBufs; ++i) {
-            tc::mbar_init(&tile_full[i], 1);
-            tc::mbar_init(&tile_free[i], 1);
+            tc::mbar_init(&m.tile_full[i], 1);
+            tc::mbar_init(&m.tile_free[i], 1);
         }
-        tc::mbar_init(&d2_full, 1);
-        tc::mbar_init(&d2_empty, 16);
         err_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    const int ipc = a.n_kb * a.n_g, items = a.n_ch * ipc;  // items per channel, of the launch
+    if (SPLIT)
+        for (int b = tid; b <= (int)gridDim.x; b += kWs3Threads)
+            start[b] = (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc, a.nt, b, gridDim.x);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = tmem_sh;
+    const uint32_t tmem = ws3_uni(tmem_sh);
     uint8_t* sbase = smem + ((1024u - (tc::smem_u32(smem) & 1023u)) & 1023u);
     uint8_t* sA1 = sbase + a.sA1;
     const int P = a.P;
-    const int R2 = 2 * 64 * P;
     const uint32_t a2col = 2u * a.d1_cols;
-    const int items = a.n_ch * a.n_kb * a.n_g;
-    // this block's share of the launch.  split: the (item, frame) pairs [wb0, wb1) in
-    // item-major order (equal shares; items cut at share boundaries are summed by the
-    // block that stores their last part); else whole items blockIdx.x, + gridDim.x, ...
-    const long long U = (long long)items * a.nt;
-    const int ipc = a.n_kb * a.n_g;  // items per channel
-    const long long wb0 = split_start(a.wcum, a.c0, a.n_ch, ipc, a.nt, blockIdx.x, gridDim.x);
-    const long long wb1 = split_start(a.wcum, a.c0, a.n_ch, ipc, a.nt, blockIdx.x + 1, gridDim.x);
+    const uint32_t b2a = tc::smem_u32(sbase + a.sB2);
+    // this block's share of the launch.  SPLIT: the (item, frame) units [wb0, wb1) in item-major
+    // order (items cut at share boundaries are summed by the block that stores their last part);
+    // else whole items blockIdx.x, + gridDim.x, ...
+    const long long wb0 = SPLIT ? start[blockIdx.x] : 0, wb1 = SPLIT ? start[blockIdx.x + 1] : 0;
+    Ws3Seg s;
+    long long w = wb0;
+    bool good = true;
 
-    if (warp >= 16) {
+    if (warp < 4) {
         // ------------------------------------------------------------ control warpgroup
-        // 4 control warps x 32 lanes x 32 registers + 16 epilogue warps x 32 lanes x 112 =
-        // 61,440: exactly the 640 threads x 96 registers the block is launched with
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;" ::: "memory");
-        uint32_t ph_d1 = 0, ph_b2 = 0, ph_tile = 0, ph_free = 0, ph_a = 0, ph_e2 = 0;
-        uint32_t pend = 0;  // copy thread: bulk copies in flight (bit j tile buffer j, bit 7 A1)
-        uint32_t cph = 0;   // copy thread: parity of the phase the next copy into buffer j (bit j)
-                            // or of A1 (bit 7) completes
-        const bool iss1 = warp == 17 && lane == 0;  // stage 1: S1 chains
-        const bool iss2 = warp == 16 && lane == 0;  // stage 2 chains
-        const bool cpy = warp == 18 && lane == 0;   // A1 and tile-part copies, L2 prefetches
-        const int NB = a.nbt;                       // tile-part buffers in shared memory (2..4)
-        long long w = wb0;
-        for (int it = 0;; ++it) {
-            int item, fs, nt;  // work item, its first frame and the frames of this segment
-            if (MODE == 1) {
-                if (w >= wb1) break;
-                item = (int)(w / a.nt);
-                fs = (int)(w % a.nt);
-                nt = (int)min((long long)(a.nt - fs), wb1 - w);
-                w += nt;
-            } else {
-                item = blockIdx.x + it * gridDim.x;
-                if (item >= items) break;
-                if (a.item_order) item = a.item_order[(size_t)a.c0 * ipc + item];
-                fs = 0;
-                nt = a.nt;
-            }
-            const int g = item % a.n_g, cl = item / (a.n_g * a.n_kb);
-            const int c = a.c0 + cl;
-            const int4 bx = a.box[c];
-            const int4 tp = a.tbox[c];
-            const int nxp = bx.z, nyh = tp.x, H = PARTS ? tp.y : 1;
-            const int K1 = 2 * nxp, K2h = 2 * nyh, N1 = P * nyh;
-            const int NU = nt * H;  // sub-frames u = t H + h: frame t, row part h
-            const uint32_t part_bytes = (uint32_t)N1 * pad64(K1) * 2;
-            auto buf = [&](int b) { return sbase + a.sB1 + (size_t)b * a.b1_bytes; };
-            auto wait_bit = [&](uint64_t* bar, uint32_t& ph, int slot) -> bool {
-                const bool r = tc::mbar_wait(bar, (ph >> slot) & 1u, kWaitBudget);
-                if (r) ph ^= 1u << slot;
-                return r;
-            };
-            // copy thread: A1 and the first NB tile parts now, then part u+NB once S1(u) has read
-            // its buffer (after the barrier: S1 is issued only past it)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWs3CtlRegs) : "memory");
+        const int NB = a.nbt;
+        if (warp == 2 && lane == 0) {  // A1 and tile-part copies
             const size_t frame_step = (size_t)a.n_ch * a.tile_stride;
-            const uint8_t* tiles_c = a.tiles + (size_t)cl * a.tile_stride + (size_t)fs * frame_step;
-            const uint8_t* nxt = tiles_c;  // next part to copy, advanced without division
-            int nxt_h = 0;
-            auto copy_next = [&](int b) {
-                tc::mbar_expect_tx(&tile_full[b], part_bytes);
-                tc::bulk_g2s(buf(b), nxt, part_bytes, &tile_full[b]);
-                pend |= 1u << b;
-                cph ^= 1u << b;
-                if (++nxt_h == H) {
-                    nxt_h = 0;
-                    nxt += frame_step - (size_t)(H - 1) * part_bytes;
-                } else {
-                    nxt += part_bytes;
-                }
+            uint32_t used = 0, ph_free = 0, cph = 0, aph = 0;  // used: copied, its S1 not yet waited for
+            int b = 0;
+            auto free_buf = [&](int j) -> bool {
+                if (!((used >> j) & 1u)) return true;
+                // S1 of the part copied there is done.  tile_free[j] cannot complete again before
+                // this thread refills buffer j
+                if (!tc::mbar_wait(&m.tile_free[j], (ph_free >> j) & 1u, kWaitBudget)) return false;
+                ph_free ^= 1u << j;
+                used &= ~(1u << j);
+                return true;
             };
-            if (cpy) {
-                const uint32_t a1_bytes = 256u * pad64(K1);
-                tc::mbar_expect_tx(&bar_a, a1_bytes);
-                tc::bulk_g2s(sA1, a.a1p + a.a1p_off[(size_t)c * a.n_g + g], a1_bytes, &bar_a);
-                pend |= 0x80u;
-                cph ^= 0x80u;
-                for (int j = 0; j < NB && j < NU; ++j) copy_next(j);
-                for (int j = 1; j <= kTilePrefetch && j < nt; ++j)  // later frames: HBM -> L2 ahead of use
-                    tc::bulk_prefetch_l2(tiles_c + (size_t)j * frame_step, part_bytes * H);
-            }
-            bar_all(1);  // A2 is in TMEM
-            if (iss1) {  // per sub-frame u: E1(u) has read D1[u&1] and tile part u+2 is in -> S1(u+2)
-                const uint32_t id1 = tc::idesc_f16_f32(128, N1);
-                auto issue_s1 = [&](int slot, int b) {
-                    issue_ss(K1 / 16, tmem + slot * a.d1_cols, tc::smem_u32(sA1), tc::smem_u32(buf(b)), 128 * 128,
-                             N1 * 128, id1);
-                    tc::mma_commit(&d1_full[slot]);
-                    tc::mma_commit(&tile_free[b]);  // the copy thread's signal that buffer b was read
-                };
-                bool good = wait_bit(&bar_a, ph_a, 0);
-                for (int j = 0; j < 2 && j < NU && good; ++j) {
-                    good = wait_bit(&tile_full[j], ph_tile, j);
-                    if (good) {
-                        tc::fence_after_sync();
-                        issue_s1(j, j);
+            for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+                const int g = s.item % a.n_g, cl = s.item / ipc, c = a.c0 + cl;
+                const int4 tp = a.tbox[c];
+                const int H = tp.y, NU = s.nt * H;
+                const int K1p = pad64(2 * a.box[c].z);
+                const uint32_t part_bytes = (uint32_t)(P * tp.x) * K1p * 2;
+                // next part to copy, advanced without division
+                const uint8_t* nxt = a.tiles + (size_t)cl * a.tile_stride + (size_t)s.fs * frame_step;
+                const uint32_t a1_bytes = 256u * K1p;
+                const uint16_t* a1src = a.a1p + a.a1p_off[(size_t)c * a.n_g + g];
+                if (it > 0) tc::bulk_prefetch_l2(a1src, a1_bytes);
+                int nh = 0;
+                for (int k = 0; k < NU && good; ++k) {
+                    good = free_buf(b);
+                    if (!good) break;
+                    tc::mbar_expect_tx(&m.tile_full[b], part_bytes);
+                    tc::bulk_g2s(sbase + a.sB1 + (size_t)b * a.b1_bytes, nxt, part_bytes, &m.tile_full[b]);
+                    used |= 1u << b;
+                    cph ^= 1u << b;
+                    if (++b == NB) b = 0;
+                    if (++nh == H) {
+                        nh = 0;
+                        nxt += frame_step - (size_t)(H - 1) * part_bytes;
+                    } else {
+                        nxt += part_bytes;
                     }
-                }
-                int bu2 = 2 % NB;  // buffer of sub-frame u + 2
-                for (int u = 0; u < NU - 2 && good; ++u) {
-                    const int sl = u & 1;
-                    good = wait_bit(&b2_full[sl], ph_b2, sl);  // E1(u) has read D1[sl]
-                    if (good) good = wait_bit(&tile_full[bu2], ph_tile, bu2);
-                    if (good) {
-                        tc::fence_after_sync();
-                        issue_s1(sl, bu2);
-                    }
-                    if (++bu2 == NB) bu2 = 0;
-                }
-                for (int u = max(0, NU - 2); u < NU && good; ++u)  // the last two E1s, so parities stay paired
-                    good = wait_bit(&b2_full[u & 1], ph_b2, u & 1);
-                if (!good) err_sh = 1;
-            } else if (iss2) {  // per sub-frame u: E1(u) wrote B2[u&1] (and E2(t-1) read D2) -> S2(u)
-                const uint32_t id2 = tc::idesc_f16_f32(128, 128 * P);
-                bool good = true;
-                for (int t = 0; t < nt && good; ++t)
-                    for (int h = 0; h < H && good; ++h) {
-                        const int sl = (t * H + h) & 1;
-                        good = wait_bit(&b2_full[sl], ph_b2, sl);
-                        if (good && h == 0 && t >= 1) good = wait_bit(&d2_empty, ph_e2, 0);
+                    if (k == min(NB, NU) - 1) {
+                        // A1 once every S1 of the item before is done: its parts are in the buffers
+                        // refilled above, or in those this short segment left alone
+                        for (int j = 0; j < NB - NU && good; ++j) good = free_buf((b + j) % NB);
                         if (!good) break;
-                        tc::fence_after_sync();
-                        issue_ts(K2h / 16, tmem + 256, tmem + a2col + h * nyh,
-                                 tc::smem_u32(sbase + a.sB2 + (size_t)sl * a.b2_bytes), R2 * 128, id2, h > 0);
-                        if (H > 1) tc::mma_commit(&b2_free[sl]);  // S2(u) has read B2[sl]
-                        if (h == H - 1) tc::mma_commit(&d2_full);
-                    }
-                if (!good) err_sh = 1;
-            } else if (cpy) {
-                bool good = true;
-                int bu = 0, hu = 0, tu = 0;  // buffer, row part and frame of u
-                for (int u = 0; u < NU && good; ++u) {
-                    // S1(u) done: buffer bu is free.  Its own barrier, not d1_full[u & 1]: with
-                    // more than two buffers S1(u + 2) needs no refill from this thread, so
-                    // d1_full[u & 1] could complete twice before this wait and its parity alias;
-                    // tile_free[bu] cannot complete again before this thread refills bu
-                    good = wait_bit(&tile_free[bu], ph_free, bu);
-                    if (good) pend &= ~((1u << bu) | 0x80u);  // its copy (and A1) had landed: S1(u) read them
-                    if (good && u + NB < NU) copy_next(bu);
-                    if (good && hu == 0 && tu + 1 + kTilePrefetch < nt)
-                        tc::bulk_prefetch_l2(tiles_c + (size_t)(tu + 1 + kTilePrefetch) * frame_step, part_bytes * H);
-                    if (++bu == NB) bu = 0;
-                    if (++hu == H) {
-                        hu = 0;
-                        ++tu;
+                        tc::mbar_expect_tx(&m.bar_a, a1_bytes);
+                        tc::bulk_g2s(sA1, a1src, a1_bytes, &m.bar_a);
+                        aph ^= 1u;
+                        cph |= 0x80u;
                     }
                 }
-                if (!good) err_sh = 1;
             }
-            __syncwarp();
-            bar_all(2);  // item done
-            if (err_sh) break;
+            for (int j = 0; j < NB && good; ++j) good = free_buf(j);
+            if (!good) {  // a wait ran out: no bulk copy may be in flight when the block releases its memory
+                err_sh = 1;
+                for (int j = 0; j < NB; ++j)  // a copy completes the phase before cph's
+                    if ((used >> j) & 1u) tc::mbar_wait(&m.tile_full[j], ((cph >> j) & 1u) ^ 1u, kWaitBudget);
+                if (cph & 0x80u) tc::mbar_wait(&m.bar_a, aph ^ 1u, kWaitBudget);
+            }
+        } else if (warp == 1) {  // stage 1: the whole warp in step, its leader issues
+            const uint32_t lead = tc::elect_one();
+            const uint32_t da = tc::desc_sw128_lo(tc::smem_u32(sA1));
+            uint32_t ph_free = 0, ph_tile = 0, ph_a = 0;
+            int b = 0;
+            unsigned u = 0;  // sub-frames of all segments
+            for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+                const int c = a.c0 + s.item / ipc;
+                const int4 tp = a.tbox[c];
+                const int ks = ws3_uni(a.box[c].z / 8), N1 = ws3_uni(P * tp.x), NU = ws3_uni(s.nt * tp.y);
+                good = ws3_wait(&m.bar_a, ph_a, 0);
+                if (!good) break;
+                switch (ks) {
+#define EPIC_S1(n)                                                                                                   case n:                                                                                                              good = ws3_s1<n>(m, n, NU, u, b, NB, ph_free, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1),                          a.b1_bytes, N1, lead);                                                                          break;
+                    EPIC_KS_CASES(EPIC_S1)
+#undef EPIC_S1
+                    default:
+                        good = ws3_s1<0>(m, ks, NU, u, b, NB, ph_free, ph_tile, tmem, a.d1_cols, da,
+                                         tc::smem_u32(sbase + a.sB1), a.b1_bytes, N1, lead);
+                }
+            }
+            if (!good) {  // a wait ran out: let this warp's MMAs finish (bounded)
+                err_sh = 1;
+                tc::mma_commit_lead(&m.drain[0], lead);
+                tc::mbar_wait(&m.drain[0], 0, kWaitBudget);
+            }
+        } else if (warp == 0) {  // stage 2, likewise
+            const uint32_t lead = tc::elect_one();
+            uint32_t ph_b2 = 0, ph_e = 0, ph_a2 = 0;
+            unsigned u = 0;
+            bool any = false;  // a frame was issued before
+            for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+                const int4 tp = a.tbox[a.c0 + s.item / ipc];
+                const int ks = ws3_uni(tp.x / 8), H = ws3_uni(tp.y), nt = ws3_uni(s.nt);
+                good = ws3_wait(&m.a2_full, ph_a2, 0);
+                if (!good) break;
+                switch (ks) {
+#define EPIC_S2(n)                                                                                                      case n:                                                                                                                 good = ws3_s2<n>(m, n, nt, H, u, any, ph_b2, ph_e, tmem + 256, tmem + a2col, P, b2a, a.b2_bytes, lead);              break;
+                    EPIC_KS_CASES(EPIC_S2)
+#undef EPIC_S2
+                    default:
+                        good = ws3_s2<0>(m, ks, nt, H, u, any, ph_b2, ph_e, tmem + 256, tmem + a2col, P, b2a,
+                                         a.b2_bytes, lead);
+                }
+            }
+            if (!good) {
+                err_sh = 1;
+                tc::mma_commit_lead(&m.drain[1], lead);
+                tc::mbar_wait(&m.drain[1], 0, kWaitBudget);
+            }
         }
-        if (err_sh && (iss1 || iss2)) {  // a wait ran out: let this thread's MMAs finish (bounded)
-            tc::mma_commit(&drain[iss2 ? 1 : 0]);
-            tc::mbar_wait(&drain[iss2 ? 1 : 0], 0, kWaitBudget);
-        }
-        if (err_sh && cpy) {  // and the bulk copies in flight, before the block releases its memory
-            for (int j = 0; j < kWs3MaxTileBufs; ++j)  // a pending copy completes the phase before cph's
-                if ((pend >> j) & 1u) tc::mbar_wait(&tile_full[j], ((cph >> j) & 1u) ^ 1u, kWaitBudget);
-            if (pend & 0x80u) tc::mbar_wait(&bar_a, ((cph >> 7) & 1u) ^ 1u, kWaitBudget);
-        }
-    } else {
-        // ------------------------------------------------------------ epilogue warps
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 112;" ::: "memory");
-        uint32_t ph_d1 = 0, ph_d2 = 0, ph_bf = 0;
-        const int q4 = warp & 3, j4 = warp >> 2;
+        __syncwarp();
+    } else if (warp < 8) {
+        // ------------------------------------------------------------ epilogue 1
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWs3E1Regs) : "memory");
+        uint32_t ph_d1 = 0, ph_bf = 0, held = 0;
+        const int q4 = warp & 3;
         const uint32_t lane_base = (uint32_t)(32 * q4) << 16;
-        const int h2 = j4 >> 1;
-        long long w = wb0;
-        for (int it = 0;; ++it) {
-            int item, fs, nt;  // work item, its first frame and the frames of this segment
-            if (MODE == 1) {
-                if (w >= wb1) break;
-                item = (int)(w / a.nt);
-                fs = (int)(w % a.nt);
-                nt = (int)min((long long)(a.nt - fs), wb1 - w);
-                w += nt;
-            } else {
-                item = blockIdx.x + it * gridDim.x;
-                if (item >= items) break;
-                if (a.item_order) item = a.item_order[(size_t)a.c0 * ipc + item];
-                fs = 0;
-                nt = a.nt;
-            }
-            const bool first_seg = it == 0;
-            const int g = item % a.n_g, kb = (item / a.n_g) % a.n_kb, cl = item / (a.n_g * a.n_kb);
-            const int c = a.c0 + cl;
+        unsigned u = 0;
+        auto free_b2 = [&](int sl) -> bool {
+            if (!((held >> sl) & 1u)) return true;
+            held &= ~(1u << sl);
+            return ws3_wait(&m.b2_free[sl], ph_bf, sl);
+        };
+        for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+            const int kb = (s.item / a.n_g) % a.n_kb, c = a.c0 + s.item / ipc;
             const int4 tp = a.tbox[c];
-            const int nyh = tp.x, H = PARTS ? tp.y : 1, nyt = tp.z;
-            if (warp < 4) {  // stage-2 DFT operand (every row part) -> TMEM (lane = ky row)
-                // rows of nyt words (a multiple of 8) from a 32-byte aligned table: 32 words per
-                // round of 16-byte loads, so an item waits for nyt / 32 load latencies, not nyt / 8
+            const int nyt = tp.z, nyc = ws3_uni(tp.x >> 3), H = tp.y, NU = ws3_uni(s.nt * H);
+            good = free_b2(0) && free_b2(1);  // every S2 of the item before has read A2
+            if (!good) break;
+            tc::fence_after_sync();
+            {   // stage-2 DFT operand (every row part) -> TMEM (lane = ky row).  A row's part is
+                // nyh words in the table, real pairs then imaginary pairs; here 4 words of each in
+                // turn, the K order of B2.  Four such groups per round of 16-byte loads.
+                const int ng = H * nyc;
                 const uint4* src = reinterpret_cast<const uint4*>(a.a2w + a.a2w_off[(size_t)c * a.n_kb + kb] +
-                                                                  (size_t)(32 * warp + lane) * nyt);
-                for (int jj = 0; jj < nyt; jj += 32) {
+                                                                  (size_t)(32 * q4 + lane) * nyt);
+                int j = 0;  // group within its part
+                for (int g0 = 0; g0 < ng; g0 += 4) {
                     uint4 q[8];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        q[i] = jj + 4 * i < nyt ? __ldg(src + (jj >> 2) + i) : make_uint4(0u, 0u, 0u, 0u);
+                    for (int i = 0; i < 4; ++i) {
+                        if (g0 + i < ng) {
+                            q[2 * i] = __ldg(src + j);
+                            q[2 * i + 1] = __ldg(src + nyc + j);
+                        }
+                        if (++j == nyc) {
+                            j = 0;
+                            src += 2 * nyc;
+                        }
+                    }
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        if (jj + 8 * g >= nyt) break;
-                        const uint32_t r[8] = {q[2 * g].x,     q[2 * g].y,     q[2 * g].z,     q[2 * g].w,
-                                               q[2 * g + 1].x, q[2 * g + 1].y, q[2 * g + 1].z, q[2 * g + 1].w};
-                        tc::tmem_st8(tmem + lane_base + a2col + jj + 8 * g, r);
+                    for (int i = 0; i < 4; ++i) {
+                        if (g0 + i >= ng) break;
+                        const uint32_t r[8] = {q[2 * i].x,     q[2 * i].y,     q[2 * i].z,     q[2 * i].w,
+                                               q[2 * i + 1].x, q[2 * i + 1].y, q[2 * i + 1].z, q[2 * i + 1].w};
+                        tc::tmem_st8(tmem + lane_base + a2col + 8 * (g0 + i), r);
                     }
                 }
                 tc::tmem_wait_st();
-            }
-            tc::fence_before_sync();
-            bar_all(1);
-            tc::fence_after_sync();
-            float axx[16], ayy[16], arx[16], aix[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) axx[i] = ayy[i] = arx[i] = aix[i] = 0.f;
-            const int hh = q4 & 1;
-            const bool imw = (q4 >> 1) != 0;
-            const int nyc = nyh >> 3;
-            int p1, yc0, yc1;
-            if (P == 2) {
-                p1 = j4 >> 1;
-                const int mid = (nyc + 1) >> 1;
-                yc0 = (j4 & 1) ? mid : 0;
-                yc1 = (j4 & 1) ? nyc : mid;
-            } else {
-                p1 = 0;
-                yc0 = (nyc * j4) >> 2;
-                yc1 = (nyc * (j4 + 1)) >> 2;
-            }
-            const uint32_t e2addr = tmem + lane_base + 256 + 64 * P * h2 + 16 * (j4 & 1);
-            // sub-integrations: after frame f (chunk-local) ends an interval, write (or add)
-            // the sums to image set iv0 + f / sub and restart them
-            auto flush_interval = [&](int f) {
-                const int ky = 128 * kb + 32 * q4 + lane;
-                const int kx0 = 64 * g + 32 * h2 + 16 * (j4 & 1);
-                if (ky < a.N && kx0 < a.N) {
-                    const size_t NN = (size_t)a.N * a.N;
-                    float* o = a.out + ((size_t)(a.iv0 + f / a.sub) * a.C + c) * a.nprod * NN + (size_t)ky * a.N + kx0;
-                    const int nk = min(16, a.N - kx0);
-                    store_pixels16_flush(o, nk, a.accumulate, axx);
-                    if (a.nprod == 4) {
-                        store_pixels16_flush(o + NN, nk, a.accumulate, ayy);
-                        store_pixels16_flush(o + 2 * NN, nk, a.accumulate, arx);
-                        store_pixels16_flush(o + 3 * NN, nk, a.accumulate, aix);
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) axx[i] = ayy[i] = arx[i] = aix[i] = 0.f;
-            };
-            const int NU = nt * H;
-            bool live = true;
-            for (int u = 0, t = 0, h = 0; u < NU && live; ++u) {
-                const int sl = u & 1;
-                bool w = tc::mbar_wait(&d1_full[sl], (ph_d1 >> sl) & 1u, kWaitBudget);
-                ph_d1 ^= 1u << sl;
-                if (w && H > 1 && u >= 2) {  // S2(u-2) has read B2[sl]
-                    w = tc::mbar_wait(&b2_free[sl], (ph_bf >> sl) & 1u, kWaitBudget);
-                    ph_bf ^= 1u << sl;
-                }
-                __syncwarp();
-                tc::fence_after_sync();
-                if (w)
-                    // one TMEM load per round without row parts (fewer spills), two with them (a
-                    // short part's stores cannot hide a second round's load latency)
-                    ws2_epilogue1<PARTS ? 2 : 1>(tmem + lane_base + sl * a.d1_cols + p1 * nyh, nyh, yc0, yc1, imw, lane,
-                                  sbase + a.sB2 + (size_t)sl * a.b2_bytes, 64 * P * hh + 64 * p1, R2);
-                tc::fence_proxy_async();
                 tc::fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&b2_full[sl]);
-                bool w2 = true;
-                if (h == 0 && t >= 1) {
-                    w2 = tc::mbar_wait(&d2_full, ph_d2 & 1u, kWaitBudget);
-                    ph_d2 ^= 1u;
-                    __syncwarp();
-                    tc::fence_after_sync();
-                    if (w2) ws_epilogue2(e2addr, P, axx, ayy, arx, aix);
-                    tc::fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&d2_empty);
-                    if (MODE == 2 && w2 && t % a.sub == 0) flush_interval(t - 1);  // frame t-1 ends one
-                }
-                if (!w || !w2) err_sh = 1;
-                live = !__any_sync(0xffffffffu, err_sh != 0);
-                if (++h == H) {
-                    h = 0;
-                    ++t;
-                }
+                if (lane == 0) mbar_arrive(&m.a2_full);
             }
-            if (nt > 0 && live) {
-                bool w2 = tc::mbar_wait(&d2_full, ph_d2 & 1u, kWaitBudget);
-                ph_d2 ^= 1u;
-                // the last two stage-2 steps' B2 releases, waited on by no later epilogue 1
-                for (int u = max(0, NU - 2); w2 && H > 1 && u < NU; ++u) {
-                    w2 = tc::mbar_wait(&b2_free[u & 1], (ph_bf >> (u & 1)) & 1u, kWaitBudget);
-                    ph_bf ^= 1u << (u & 1);
-                }
-                if (!w2) err_sh = 1;
-                __syncwarp();
-                tc::fence_after_sync();
-                if (w2) ws_epilogue2(e2addr, P, axx, ayy, arx, aix);
-                if (MODE == 2 && w2) flush_interval(nt - 1);
-            }
-            tc::fence_before_sync();
-            bar_all(2);
-            tc::fence_after_sync();
-            if (err_sh) break;
-            // images: row ky = 128 kb + 32 q4 + lane, 16 kx from 64 g + 32 h2 + 16 (j4 & 1); a
-            // segment that is only part of its item goes to this block's partial slot
-            const int ky = 128 * kb + 32 * q4 + lane;
-            const int kx0 = 64 * g + 32 * h2 + 16 * (j4 & 1);
-            if (MODE == 1 && (fs != 0 || nt != a.nt)) {
-                const size_t px = (size_t)(32 * q4 + lane) * 64 + 32 * h2 + 16 * (j4 & 1);
-                float* o = a.partial + (2 * (size_t)blockIdx.x + (first_seg ? 0 : 1)) * 4 * 8192 + px;
-                store_pixels16(o, 16, 0, axx);
-                if (a.nprod == 4) {
-                    store_pixels16(o + 8192, 16, 0, ayy);
-                    store_pixels16(o + 2 * 8192, 16, 0, arx);
-                    store_pixels16(o + 3 * 8192, 16, 0, aix);
-                }
-                ws3_split_finish(a, item, c, ky, kx0, px, U, tid, split_slot, &split_n);
-            } else if (MODE != 2 && ky < a.N && kx0 < a.N) {
-                const size_t NN = (size_t)a.N * a.N;
-                float* o = a.out + (size_t)c * a.nprod * NN + (size_t)ky * a.N + kx0;
-                const int nk = min(16, a.N - kx0);
-                store_pixels16(o, nk, a.accumulate, axx);
-                if (a.nprod == 4) {
-                    store_pixels16(o + NN, nk, a.accumulate, ayy);
-                    store_pixels16(o + 2 * NN, nk, a.accumulate, arx);
-                    store_pixels16(o + 3 * NN, nk, a.accumulate, aix);
-                }
+            switch (nyc) {  // P nyh <= 256 columns and two slots of D1 beside A2: nyc <= 15
+#define EPIC_E1(n)                                                                                                    case n:                                                                                                               good = ws3_e1<n>(m, NU, u, ph_d1, ph_bf, held, tmem + lane_base, a.d1_cols, P, (q4 >> 1) != 0, lane, b2a,                          a.b2_bytes, 64 * P * (q4 & 1));                                                                  break;
+                EPIC_KS_CASES(EPIC_E1)
+#undef EPIC_E1
+                default: good = false;
             }
         }
+        if (good) good = free_b2(0) && free_b2(1);
+        if (!good) err_sh = 1;
+    } else {
+        // ------------------------------------------------------------ epilogue 2
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWs3E2Regs) : "memory");
+        good = P == 2 ? ws3_role_e2<SPLIT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b)
+                      : ws3_role_e2<SPLIT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b);
+        if (!good) err_sh = 1;
     }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem, 512);
     if (err_sh && tid == 0) atomicExch(a.status, 1);
 }
-
-
-
-
 
 }  // namespace
 
@@ -2702,6 +2916,11 @@ epic_status dftgemm_set_kernel(epic_plan_s* p, int variant)
 }
 
 static epic_status upload_item_order(epic_plan_s* p);
+
+// SM cycles of one frame of a work item with row parts r = (nyh, H, H nyh), as measured with 152
+// channels of one frequency: 24 x 24 box 1444, 48 x 48 1882, 64 x 64 (H = 2) 2851, 72 x 72
+// (H = 3) 3607, 96 x 96 (H = 3) 4264.
+static long long ws3_item_cost(int4 r) { return 300 + 700LL * r.y + 18LL * r.z; }
 
 // Channels per launch of the warp-specialised kernels: 0 = groups of about two work items
 // per SM (whole items per block balance), 1 = every channel in one group (the fewest
@@ -2749,7 +2968,7 @@ static epic_status upload_item_order(epic_plan_s* p)
         const int ng = std::min(p->tc.cg, C - c0), L = ng * ipc, G = std::min(L, p->sm_count);
         auto w = [&](int i) {
             const int4 r = p->tc.tbox_h[c0 + i / ipc];
-            return 1000LL + 1200LL * r.y + 10LL * r.z;
+            return ws3_item_cost(r);
         };
         std::vector<int> idx(L);
         for (int i = 0; i < L; ++i) idx[i] = i;
@@ -3163,14 +3382,12 @@ epic_status dftgemm_setup(epic_plan_s* p)
     p->dt.dft_bytes = (n1 + n2 + n1p) * 2 + nw * 4 +
                       (a1_off.size() + a2_off.size() + a1p_off.size() + a2w_off.size()) * sizeof(long long);
 
-    // Work split weights of k_dftgemm_ws3's equal shares, per frame of a channel's work item:
-    // a fixed epilogue 2, an epilogue 1 per row part and stage-2 work in proportion to the rows
-    // (about 1000 + 1200 H + 10 H nyh SM cycles, from clock64 timelines of the kernel).
+    // work split weights of k_dftgemm_ws3's equal shares, per frame of a channel's work item
     {
         std::vector<long long> wc(C + 1, 0);
         for (int c = 0; c < C; ++c) {
             const int4 r = p->tc.tbox_h[c];
-            wc[c + 1] = wc[c] + 1000 + 1200LL * r.y + 10LL * r.z;
+            wc[c + 1] = wc[c] + ws3_item_cost(r);
         }
         cudaError_t ew = cudaMalloc(&p->tc.wcum, (C + 1) * sizeof(long long));
         if (ew == cudaSuccess) ew = cudaMemcpy(p->tc.wcum, wc.data(), (C + 1) * sizeof(long long), cudaMemcpyHostToDevice);
@@ -3455,12 +3672,8 @@ epic_status dftgemm_setup(epic_plan_s* p)
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_dftgemm_grid)");
     e = allow_max_smem((const void*)k_dftgemm_ws<0>, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws2<0>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<0, false>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<1, false>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<2, false>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<0, true>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<1, true>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<2, true>, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<false>, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<true>, p->smem_optin);
     p->tc.ws_variant = p->tc.ws ? 3 : 0;
     if (p->tc.ws && p->sm_count > kWs3MaxBlocks) p->tc.ws_variant = 1;
     if (p->tc.parts && p->tc.ws_variant != 3) {
@@ -3667,15 +3880,11 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                 if (p->tc.ws_variant == 3) {
                     a.partial = p->tc.partial;
                     a.counters = p->tc.counters;
-                    if (p->sub > 0)
-                        p->tc.parts ? k_dftgemm_ws3<2, true><<<grid, kWs3Threads, p->tc.smem, s>>>(a)
-                                    : k_dftgemm_ws3<2, false><<<grid, kWs3Threads, p->tc.smem, s>>>(a);
-                    else if (p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0))
-                        p->tc.parts ? k_dftgemm_ws3<1, true><<<p->sm_count, kWs3Threads, p->tc.smem, s>>>(a)
-                                    : k_dftgemm_ws3<1, false><<<p->sm_count, kWs3Threads, p->tc.smem, s>>>(a);
+                    if (p->sub == 0 && (p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
+                        (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
+                        k_dftgemm_ws3<true><<<p->sm_count, kWs3Threads, p->tc.smem, s>>>(a);
                     else
-                        p->tc.parts ? k_dftgemm_ws3<0, true><<<grid, kWs3Threads, p->tc.smem, s>>>(a)
-                                    : k_dftgemm_ws3<0, false><<<grid, kWs3Threads, p->tc.smem, s>>>(a);
+                        k_dftgemm_ws3<false><<<grid, kWs3Threads, p->tc.smem, s>>>(a);
                 }
                 else if (p->tc.ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);
                 else k_dftgemm_ws<0><<<grid, kWsThreads, p->tc.smem, s>>>(a);

@@ -11,6 +11,12 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// 16 bytes to a shared-memory address
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+
 // ---------------------------------------------------------------- packed FP32
 // (a.x b.x + c.x, a.y b.y + c.y), each rounded once as by fmaf: one sm_100-family
 // packed FP32 FMA instead of two.
@@ -181,6 +187,56 @@ __device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uin
         : "memory");
 }
 
+// The forms for a whole warp in step: every lane runs the instruction's set-up (so operands stay
+// in the warp's uniform registers) and the one lane with lead != 0 issues it.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r));
+    return r;
+}
+// Operand descriptors by their low words: the high word of smem_desc_sw128 is a constant.
+__device__ __forceinline__ uint32_t desc_sw128_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
+constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                             uint32_t accumulate, uint32_t lead)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 x, y;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "mov.b64 x, {%1, %6};\n\t"
+        "mov.b64 y, {%2, %6};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(kDescSw128Hi)
+        : "memory");
+}
+__device__ __forceinline__ void mma_f16_ta_lead(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t idesc,
+                                                uint32_t accumulate, uint32_t lead)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 y;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "mov.b64 y, {%2, %6};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], y, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(kDescSw128Hi)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_lead(uint64_t* bar, uint32_t lead)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+        "r"(lead)
+        : "memory");
+}
+
 // 8 consecutive 32-bit TMEM columns of this thread's lane <- r[0..7]
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r)
 {
@@ -206,6 +262,21 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r)
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+
+// The same for 32 columns.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr)
         : "memory");
 }
