@@ -478,6 +478,8 @@ epic_status call_scratch_fit(epic_plan_s* p, CallScratch& c)
         *have = 0;
         cudaError_t e = cudaMalloc(ptr, need);
         if (e == cudaSuccess) e = cudaMemset(*ptr, 0, need);
+        // the slot's stream does not wait for the default stream: the zeros must be in before its kernels
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
         if (e != cudaSuccess) return cuda_fail(p, e, what);
         *have = need;
         return EPIC_OK;

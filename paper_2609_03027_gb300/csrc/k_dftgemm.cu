@@ -3004,6 +3004,7 @@ epic_status dftgemm_set_chunk(epic_plan_s* p, size_t budget)
     // zero once: tile bytes no gridding kernel writes (K padding past 2 nx) then hold zeros or
     // FP16 values of other tiles, never stale non-finite bits, and meet zero DFT operands
     e = cudaMemset(p->scratch, 0, bytes);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // a later call's stream may not wait for the default one
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaMemset(tensor path tile buffer)");
     p->scratch_bytes = bytes;
     return EPIC_OK;
