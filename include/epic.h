@@ -236,8 +236,11 @@ epic_status epic_plan_get_info(epic_plan_t plan, epic_plan_info* info);
  *                              the items divide evenly), 0 whole work items per SM, 1 equal
  *                              (item, time sample) shares per SM;
  *                 grid_kernel  gridding kernel: 1 row-major cell walk, 2 cells in lists sorted
- *                              by length (Gaussian GCF, when its tiles fit in shared memory);
- *                 grid_frames  frames per pass of the gridding kernel;
+ *                              by length (Gaussian GCF, when its tiles fit in shared memory),
+ *                              3 row-major lists of cell pairs (Gaussian GCF), 4 tensor cores
+ *                              (max_time >= 16);
+ *                 grid_frames  frames per pass of the gridding kernel (4: groups of 64 / n_pol
+ *                              frames staged at once);
  *                 chunk_mb     tile-buffer budget of one (channel group, time chunk), 96 MiB to
  *                              24 GiB (the block's samples at most)
  * Images after tuning equal those before up to FP32 rounding order.  reps calls

@@ -90,6 +90,12 @@ void free_path_state(epic_plan_s* p)
     cudaFree(p->tc.pl_off);
     cudaFree(p->tc.pl_e);
     cudaFree(p->tc.pl_w);
+    cudaFree(p->tc.gt_tile0);
+    cudaFree(p->tc.gt_unit0);
+    cudaFree(p->tc.gt_ent0);
+    cudaFree(p->tc.gt_ent);
+    cudaFree(p->tc.gt_el);
+    cudaFree(p->tc.gt_wcum);
     cudaFree(p->scratch);
     int* status = p->tc.status;
     p->tc = epic::TcState{};

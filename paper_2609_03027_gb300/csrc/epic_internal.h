@@ -55,7 +55,8 @@ struct TcState {
     int grid_blocks = 0;           // blocks of the persistent gridding kernel
     int grid_max_cells = 0;        // largest occupied box (cells)
     int grid_max_list = 0;         // (cell, element) entries per channel
-    int grid_variant = 1;          // 1: persistent row-major gather, 2: balanced task lists, 3: pair lists
+    int grid_variant = 1;          // 1: persistent row-major gather, 2: balanced task lists, 3: pair lists,
+                                   //   4: tensor cores
     long long* wcum = nullptr;     // [C + 1] prefix sums of k_dftgemm_ws3 item costs per frame (work split)
     int* item_order = nullptr;     // k_dftgemm_ws3 whole items: per channel group, the order items are dealt to blocks
     int* pl_ptr = nullptr;         // pair-list gridding: per channel entry offsets of the box's cell
@@ -65,6 +66,14 @@ struct TcState {
     int pl_max_ptr = 0;            //   most offsets / entries of one channel
     int pl_max_ent = 0;
     bool pl_stage = false;         //   the kernel stages a channel's lists in shared memory
+    bool lists_built = false;      // the pair lists and task lists below exist (or do not fit the plan)
+    int* gt_tile0 = nullptr;       // tensor-core gridding (k_grid_tc.cu): first cell-pair tile of each channel,
+    int* gt_unit0 = nullptr;       //   first K step of each tile, first weight and the elements
+    int* gt_ent0 = nullptr;        //   of each step, the weights (offset in the operand, value),
+    int2* gt_ent = nullptr;        //   prefix sums of the channels' costs and the power of two
+    int* gt_el = nullptr;          //   the weights are scaled by
+    long long* gt_wcum = nullptr;
+    int gt_scale = 0;
     int4* gtask = nullptr;         // balanced gridding: per-channel task lists (device)
     int* gtask_off = nullptr;      // [C + 1]
     int gtask_max = 0;             // largest task list
@@ -236,5 +245,10 @@ epic_status dftgemm_set_kernel(epic_plan_s* p, int variant);
 epic_status dftgemm_set_grid_kernel(epic_plan_s* p, int variant);
 epic_status dftgemm_set_split(epic_plan_s* p, int mode);
 epic_status dftgemm_set_group(epic_plan_s* p, int v);
+
+// k_grid_tc.cu
+epic_status grid_tc_setup(epic_plan_s* p);
+epic_status grid_tc_config(epic_plan_s* p, int gc);
+void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0, int n_ch, cudaStream_t s);
 
 }  // namespace epic

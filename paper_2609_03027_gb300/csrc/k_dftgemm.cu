@@ -11,6 +11,7 @@
 //   stage 1: D1[(q, kx)][(p, y)] = A1[(q, kx)][(q', x)] . B1[(p, y)][(q', x)]
 //            A1 rows (re, kx) = [ Fr | -Fi ], rows (im, kx) = [ Fi | Fr ]   (128 = 2 x 64 kx)
 //            B1 row (p, y)   = [ Gr_p[y][:] | Gi_p[y][:] ]                  (the grid tile)
+//            K in the order of the cell pairs: (re x, re x+1, im x, im x+1) for x = 0, 2, ...
 //   stage 2: D2_p[ky][n]     = A2[ky][(q', y)] . B2_p[n][(q', y)]
 //            A2 row ky       = [ Fr[:][ky] | Fi[:][ky] ]
 //            B2_p row kx     = [ Hr[:][kx] | -Hi[:][kx] ],  row 32+kx = [ Hi | Hr ]
@@ -35,6 +36,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "dftgemm_common.cuh"
 #include "epic_internal.h"
 #include "kcommon.cuh"
 #include "tc_ptx.cuh"
@@ -45,7 +47,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr size_t kScratchBudget = 3072ull << 20;  // grid tiles of one (channel group, time chunk)
-constexpr long long kWaitBudget = 4000000000LL;  // clock cycles before a wait gives up (~2 s)
+constexpr int kGridTcMinTime = 16;                // shortest max_time that takes the tensor-core gridding kernel
 constexpr int kGridFramesPerBlock = 8;            // frames gridded per block (cell lists read once)
 
 // ------------------------------------------------------------------ host helpers
@@ -80,10 +82,6 @@ inline size_t sw_off(int r, int k, int R)
 {
     return (size_t)(k >> 6) * ((size_t)R * 64) + (size_t)r * 64 + ((((k >> 3) & 7) ^ (r & 7)) << 3) + (k & 7);
 }
-
-__host__ __device__ inline int pad64(int k) { return (k + 63) & ~63; }
-
-inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Row parts of a box of `rows` rows (a multiple of 8 for two pols, 16 for one) for
 // k_dftgemm_ws3 with D1 slots of D TMEM columns: the fewest parts H whose equal height
@@ -140,12 +138,6 @@ struct MmaArgs {
     const int* item_order;      // k_dftgemm_ws3<false>: per channel group (from c0 ipc), items in the order dealt to blocks
 };
 
-__device__ __forceinline__ uint32_t pack_h2(float a, float b)
-{
-    __half2 h = __floats2half2_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&h);
-}
-
 // byte offset of 16-byte chunk c (8 halves of K) of row r in an R-row operand in the
 // 128-byte swizzled K-major layout
 __device__ __forceinline__ size_t sw_chunk(int r, int c, int R)
@@ -174,28 +166,6 @@ __device__ __forceinline__ void store_pixels16(float* op, int nk, int accumulate
         for (int i = 0; i < 16; ++i)
             if (i < nk) op[i] = (accumulate ? op[i] : 0.f) + v[i];
     }
-}
-
-// First unit of block b of G when a launch's units -- ipc items of each of n_ch channels from
-// c0 in channel order, nt frames per item, item-major -- are cut into G ranges of equal cost,
-// a unit costing its channel's weight (wcum: prefix sums of the weights over the plan's
-// channels).  Without weights, G ranges of equal numbers of units.  Non-decreasing in b,
-// 0 at b = 0 and every unit at b = G.
-__device__ __forceinline__ long long split_start(const long long* wcum, int c0, int n_ch, int ipc, int nt, int b, int G)
-{
-    const long long per = (long long)ipc * nt;  // units of one channel
-    if (!wcum) return (long long)n_ch * per * b / G;
-    const long long base = wcum[c0];
-    const long long s = per * (wcum[c0 + n_ch] - base) * b / G;  // cost position of the block's start
-    int lo = 0, hi = n_ch;                                        // last channel whose units start at or before s
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (per * (wcum[c0 + mid] - base) <= s) lo = mid;
-        else hi = mid;
-    }
-    const long long w = wcum[c0 + lo + 1] - wcum[c0 + lo];
-    const long long u = min(per, (s - per * (wcum[c0 + lo] - base)) / w);
-    return (long long)lo * per + u;
 }
 
 // Unpack and gather-grid frames of one chunk into FP16 UMMA tiles.  A block
@@ -289,20 +259,20 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __rest
                     }
                 }
             }
-            // cells (y, x) and (y, x+1): K index x (re) and nxp + x (im), in row part y / nyh at
+            // cells (y, x) and (y, x+1): K index 2 x (re) and 2 x + 2 (im), in row part y / nyh at
             // rows p*nyh + y % nyh
-            const int kc_re = x >> 3, kc_im = (nxp + x) >> 3, within = (x & 7) * 2;
+            const int kc = x >> 2, within = (x & 2) * 4;  // K index 2 x (re pair) and 2 x + 2 (im pair)
             const int hpart = y / nyh, R0 = y - hpart * nyh;
 #pragma unroll
             for (int f = 0; f < F; ++f) {
                 if (f >= nf) break;
                 uint8_t* tile = tiles + ((size_t)(tb + f) * n_ch + cl) * tile_stride + (size_t)hpart * part_bytes;
-                *reinterpret_cast<uint32_t*>(tile + sw_chunk(R0, kc_re, N1h) + within) = pack_h2(g[0][f].x, g[1][f].x);
-                *reinterpret_cast<uint32_t*>(tile + sw_chunk(R0, kc_im, N1h) + within) = pack_h2(g[0][f].y, g[1][f].y);
+                *reinterpret_cast<uint2*>(tile + sw_chunk(R0, kc, N1h) + within) =
+                    make_uint2(pack_h2(g[0][f].x, g[1][f].x), pack_h2(g[0][f].y, g[1][f].y));
                 if (P == 2) {
                     const int R1 = nyh + R0;
-                    *reinterpret_cast<uint32_t*>(tile + sw_chunk(R1, kc_re, N1h) + within) = pack_h2(g[0][f].z, g[1][f].z);
-                    *reinterpret_cast<uint32_t*>(tile + sw_chunk(R1, kc_im, N1h) + within) = pack_h2(g[0][f].w, g[1][f].w);
+                    *reinterpret_cast<uint2*>(tile + sw_chunk(R1, kc, N1h) + within) =
+                        make_uint2(pack_h2(g[0][f].z, g[1][f].z), pack_h2(g[0][f].w, g[1][f].w));
                 }
             }
         }
@@ -484,21 +454,19 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid_ps(GridArgs a)
                     }
                 }
             }
-            const int kc_re = x >> 3, kc_im = (nxp + x) >> 3, within = (x & 7) * 2;
+            const int kc = x >> 2, within = (x & 2) * 4;  // K index 2 x (re pair) and 2 x + 2 (im pair)
             const int hpart = y / nyh, R0 = y - hpart * nyh;
 #pragma unroll
             for (int fi = 0; fi < F; ++fi) {
                 if (fi >= nf) break;
                 uint8_t* tile =
                     a.tiles + ((size_t)(f + fi) * a.n_ch + cl) * a.tile_stride + (size_t)hpart * part_bytes;
-                *reinterpret_cast<uint32_t*>(tile + sw_chunk(R0, kc_re, N1h) + within) = pack_h2(g[0][fi].x, g[1][fi].x);
-                *reinterpret_cast<uint32_t*>(tile + sw_chunk(R0, kc_im, N1h) + within) = pack_h2(g[0][fi].y, g[1][fi].y);
+                *reinterpret_cast<uint2*>(tile + sw_chunk(R0, kc, N1h) + within) =
+                    make_uint2(pack_h2(g[0][fi].x, g[1][fi].x), pack_h2(g[0][fi].y, g[1][fi].y));
                 if (P == 2) {
                     const int R1 = nyh + R0;
-                    *reinterpret_cast<uint32_t*>(tile + sw_chunk(R1, kc_re, N1h) + within) =
-                        pack_h2(g[0][fi].z, g[1][fi].z);
-                    *reinterpret_cast<uint32_t*>(tile + sw_chunk(R1, kc_im, N1h) + within) =
-                        pack_h2(g[0][fi].w, g[1][fi].w);
+                    *reinterpret_cast<uint2*>(tile + sw_chunk(R1, kc, N1h) + within) =
+                        make_uint2(pack_h2(g[0][fi].z, g[1][fi].z), pack_h2(g[0][fi].w, g[1][fi].w));
                 }
             }
         }
@@ -573,21 +541,6 @@ __host__ __device__ inline size_t grid_bal_smem(int F, int A, int frame_bytes, i
     b += 2ull * F * tile_max;                  // tile buffers
     b += 16ull * max_tasks + (4ull + sizeof(TaskW)) * max_list;  // task list, entries (weights, elements)
     return b;
-}
-
-__host__ __device__ __forceinline__ uint32_t tile_half_off(int R, int k, int N1)
-{
-    return (uint32_t)((k >> 6) * (N1 * 128) + R * 128 + ((((k >> 3) & 7) ^ (R & 7)) << 4) + ((k & 7) << 1));
-}
-
-// Byte offset of the FP16 at (pol-X row y, K index k) of a grid tile cut into row parts of
-// nyh rows: part h = y / nyh is an operand of its own (P nyh rows: pol X rows 0..nyh-1, pol
-// Y rows nyh..2 nyh-1, so a pol-Y value sits nyh * 128 bytes after its pol-X value),
-// part_bytes apart.  One part (nyh = box rows) is the plain layout.
-__host__ __device__ __forceinline__ uint32_t tile_part_off(int y, int k, int nyh, int P, uint32_t part_bytes)
-{
-    const int h = y / nyh;
-    return (uint32_t)h * part_bytes + tile_half_off(y - h * nyh, k, P * nyh);
 }
 
 template <int F, bool H>
@@ -1028,21 +981,19 @@ __global__ void __launch_bounds__(kGridPlThreads) k_dftgemm_grid_pl(GridPlArgs p
                 load(ent_e[k], v0);
                 apply(ent_w[k], v0);
             }
-            const int kc_re = x >> 3, kc_im = (nxp + x) >> 3, within = (x & 7) * 2;
+            const int kc = x >> 2, within = (x & 2) * 4;  // K index 2 x (re pair) and 2 x + 2 (im pair)
             const int hpart = y / nyh, R0 = y - hpart * nyh;
 #pragma unroll
             for (int fi = 0; fi < F; ++fi) {
                 if (fi >= nf) break;
                 uint8_t* tile =
                     a.tiles + ((size_t)(f + fi) * a.n_ch + cl) * a.tile_stride + (size_t)hpart * part_bytes;
-                *reinterpret_cast<uint32_t*>(tile + sw_chunk(R0, kc_re, N1h) + within) = pack_h2(g[0][fi].x, g[1][fi].x);
-                *reinterpret_cast<uint32_t*>(tile + sw_chunk(R0, kc_im, N1h) + within) = pack_h2(g[0][fi].y, g[1][fi].y);
+                *reinterpret_cast<uint2*>(tile + sw_chunk(R0, kc, N1h) + within) =
+                    make_uint2(pack_h2(g[0][fi].x, g[1][fi].x), pack_h2(g[0][fi].y, g[1][fi].y));
                 if (P == 2) {
                     const int R1 = nyh + R0;
-                    *reinterpret_cast<uint32_t*>(tile + sw_chunk(R1, kc_re, N1h) + within) =
-                        pack_h2(g[0][fi].z, g[1][fi].z);
-                    *reinterpret_cast<uint32_t*>(tile + sw_chunk(R1, kc_im, N1h) + within) =
-                        pack_h2(g[0][fi].w, g[1][fi].w);
+                    *reinterpret_cast<uint2*>(tile + sw_chunk(R1, kc, N1h) + within) =
+                        make_uint2(pack_h2(g[0][fi].z, g[1][fi].z), pack_h2(g[0][fi].w, g[1][fi].w));
                 }
             }
         }
@@ -1056,14 +1007,6 @@ __global__ void __launch_bounds__(kGridPlThreads) k_dftgemm_grid_pl(GridPlArgs p
             if ((pending >> b2) & 1u) tc::mbar_wait(&bar_raw[b2], (ph >> b2) & 1u, kWaitBudget);
         atomicExch(a.status, 1);
     }
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r)
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
 }
 
 __device__ __forceinline__ bool wait_flag_uniform(uint64_t* bar, uint32_t parity, const volatile int* err)
@@ -1590,11 +1533,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_dftgemm_mma_fast(MmaArgs a)
 // and S1(t+2) (after b2_full(t) frees D1[t&1] and tile t+2 has landed).
 // TMEM: D1[0..1] at 0 and d1_cols, A2 at 2 d1_cols, D2 half h at 256 + 128 h.
 constexpr int kWsThreads = 512;
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
-}
 
 // Epilogue 1 of one warp: the stage-1 result in this warp's lane quarter (lanes =
 // 32 kx of half h; part 0 = Hr, part 1 = Hi), columns [c0, c1) of pol p, written to
@@ -3051,6 +2989,7 @@ epic_status dftgemm_grid_config(epic_plan_s* p, int F)
 {
     if (p->tc.grid_variant == 2) return grid_bal_config(p, F);
     if (p->tc.grid_variant == 3) return grid_pl_config(p, F);
+    if (p->tc.grid_variant == 4) return grid_tc_config(p, F);
     if (F != 1 && F != 2 && F != 4 && F != 8) return EPIC_ERR_UNSUPPORTED;
     const size_t bytes =
         grid_ps_smem(F, p->A, p->A * p->P * (p->bits / 4), p->tc.grid_max_cells, p->tc.grid_max_list, p->tc.grid_cplx);
@@ -3107,16 +3046,27 @@ static epic_status grid_bal_config(epic_plan_s* p, int F)
     return EPIC_OK;
 }
 
+static epic_status grid_lists_setup(epic_plan_s* p);
+
 // Gridding kernel variant: 1 = persistent row-major gather, 2 = balanced task lists,
-// 3 = row-major pair lists.  Keeps the frames per pass if the variant allows them, else
-// the largest it allows.
+// 3 = row-major pair lists, 4 = tensor cores.  Keeps the frames per pass if the variant
+// allows them, else the largest it allows.  The lists of 2 and 3 are built when first asked for.
 epic_status dftgemm_set_grid_kernel(epic_plan_s* p, int variant)
 {
-    if (variant < 1 || variant > 3) return EPIC_ERR_UNSUPPORTED;
+    if (variant < 1 || variant > 4) return EPIC_ERR_UNSUPPORTED;
+    const int old_variant = p->tc.grid_variant, old_f = p->tc.grid_frames;
+    if ((variant == 2 || variant == 3) && !p->tc.lists_built) {
+        const epic_status ls = grid_lists_setup(p);
+        p->tc.grid_variant = old_variant;
+        if (ls != EPIC_OK) {
+            dftgemm_grid_config(p, old_f);
+            return ls;
+        }
+    }
+    if (variant == 4 && !p->tc.gt_tile0) return EPIC_ERR_UNSUPPORTED;
     if (variant == 2 && !p->tc.gtask) return EPIC_ERR_UNSUPPORTED;
     if (variant == 3 && !p->tc.pl_ptr) return EPIC_ERR_UNSUPPORTED;
     if (variant == 1 && !p->tc.grid_ps) return EPIC_ERR_UNSUPPORTED;
-    const int old_variant = p->tc.grid_variant, old_f = p->tc.grid_frames;
     p->tc.grid_variant = variant;
     epic_status st = EPIC_ERR_UNSUPPORTED;
     for (int F = old_f; F >= 1 && st == EPIC_ERR_UNSUPPORTED; F >>= 1) st = dftgemm_grid_config(p, F);
@@ -3125,6 +3075,224 @@ epic_status dftgemm_set_grid_kernel(epic_plan_s* p, int variant)
         dftgemm_grid_config(p, old_f);
     }
     return st;
+}
+
+// Lists of the gather kernels (real GCF weights): per channel the cell pairs' entries row-major
+// (pair-list kernel) and as task lists of non-empty pairs, longest first (balanced kernel).
+// Chooses between the two kernels as the plan's default; leaves both out for a complex GCF.
+static epic_status grid_lists_setup(epic_plan_s* p)
+{
+    const int C = p->C;
+    p->tc.lists_built = true;
+    if (p->tc.grid_cplx) return EPIC_OK;
+    cudaError_t e = cudaSuccess;
+    std::vector<int> coff, cptr, ce;
+    std::vector<float2> cw;
+    build_csr(p, coff, cptr, ce, cw);
+    // A task is the run of kTaskCells cells (x, x + 1, ...), x a multiple of kTaskCells,
+    // of one row of a channel's box; its entries are the elements that reach any of them
+    // (the union of the cells' element-ordered lists) with one weight per cell.  Runs of
+    // a channel are sorted by entry count (equal counts in Morton order, so that a warp's
+    // runs are near one another and share elements); groups of 32 consecutive runs (the
+    // lanes of one warp) store their entries interleaved, entry k of lane l at 32 k + l,
+    // padded with zero weights to the group's longest list, in the order
+    // order_warp_entries picks.
+    std::vector<int4> tasks;
+    std::vector<int> ell_e;
+    std::vector<TaskW> ell_w;
+    std::vector<int> toff(C + 1, 0), eoff(C + 1, 0);
+    std::vector<TaskW> pw;  // weights of the channel's run lists
+    std::vector<int2> ord;
+    std::vector<int> pl_ptr, pl_off(C), pl_e;  // the same lists row-major (pair-list kernel)
+    std::vector<TaskW> pl_w;
+    bool fits = true;
+    int tmax = 0, emax = 0;
+    for (int c = 0; c < C && fits; ++c) {
+        toff[c] = (int)tasks.size();
+        eoff[c] = (int)ell_e.size();
+        const int* ptr = &cptr[coff[c]];
+        const Box bx = p->box[c];
+        const int hp = bx.nx / kTaskCells;  // runs per row (nx is a multiple of 8)
+        std::vector<std::vector<int2>> plist((size_t)hp * bx.ny);  // (element, 1 + index into pw)
+        pw.clear();
+        for (int y = 0; y < bx.ny; ++y)
+            for (int j = 0; j < hp; ++j) {
+                const int r0 = y * bx.nx + kTaskCells * j;
+                int at[kTaskCells];
+                for (int q = 0; q < kTaskCells; ++q) at[q] = ptr[r0 + q];
+                std::vector<int2>& L = plist[(size_t)y * hp + j];
+                for (;;) {  // merge of the cells' element-ordered lists
+                    int el = INT32_MAX;
+                    for (int q = 0; q < kTaskCells; ++q)
+                        if (at[q] < ptr[r0 + q + 1]) el = std::min(el, ce[at[q]]);
+                    if (el == INT32_MAX) break;
+                    float wq[4] = {0.f, 0.f, 0.f, 0.f};
+                    for (int q = 0; q < kTaskCells; ++q)
+                        if (at[q] < ptr[r0 + q + 1] && ce[at[q]] == el) wq[q] = cw[at[q]++].x;
+                    TaskW w;
+                    task_w_set(w, wq);
+                    pw.push_back(w);
+                    L.push_back(make_int2(el, (int)pw.size()));
+                }
+            }
+        pl_off[c] = (int)pl_ptr.size();
+        for (const std::vector<int2>& L : plist) {
+            pl_ptr.push_back((int)pl_e.size());
+            for (const int2& en : L) {
+                pl_e.push_back(en.x);
+                pl_w.push_back(pw[en.y - 1]);
+            }
+        }
+        pl_ptr.push_back((int)pl_e.size());
+        std::vector<int> idx;
+        for (int q = 0; q < hp * bx.ny; ++q)
+            if (!plist[q].empty()) idx.push_back(q);
+        auto morton = [hp](int q) {
+            const unsigned x = (unsigned)(kTaskCells * (q % hp)), y = (unsigned)(q / hp);
+            unsigned m = 0;
+            for (int bit = 0; bit < 12; ++bit) m |= ((x >> bit) & 1u) << (2 * bit) | ((y >> bit) & 1u) << (2 * bit + 1);
+            return m;
+        };
+        std::stable_sort(idx.begin(), idx.end(), [&](int u, int v) {
+            const size_t nu = plist[u].size(), nv = plist[v].size();
+            return nu != nv ? nu > nv : morton(u) < morton(v);
+        });
+        const int nyh = p->tc.tbox_h[c].x;
+        const uint32_t part_bytes = (uint32_t)(p->P * nyh) * pad64(2 * bx.nx) * 2;
+        std::vector<std::vector<int4>> gtasks;  // the 32 tasks of each group (padding tasks: no store)
+        std::vector<int> gcost;
+        for (size_t g0 = 0; g0 < idx.size(); g0 += 32) {
+            const int members = (int)std::min<size_t>(32, idx.size() - g0);
+            const int nmax = (int)plist[idx[g0]].size();
+            const int base = (int)ell_e.size() - eoff[c];
+            if (nmax > 255) fits = false;
+            std::vector<std::vector<int2>> lists(members);
+            for (int l = 0; l < members; ++l) lists[l] = plist[idx[g0 + l]];
+            ord.assign(32ull * nmax, make_int2(0, 0));
+            order_warp_entries(lists, nmax, ord.data());
+            for (const int2& en : ord) {
+                ell_e.push_back(en.x);
+                ell_w.push_back(en.y > 0 ? pw[en.y - 1] : TaskW{});
+            }
+            std::vector<int4> gt(32, make_int4(nmax << 24, base, -1, -1));
+            for (int l = 0; l < members; ++l) {
+                const int q = idx[g0 + l];
+                if (q >= (1 << 24)) fits = false;
+                const int y = q / hp, x = kTaskCells * (q % hp);
+                gt[l] = make_int4(q | (nmax << 24), base, (int)tile_part_off(y, 2 * x, nyh, p->P, part_bytes),
+                                  (int)tile_part_off(y, 2 * x + 2, nyh, p->P, part_bytes));
+            }
+            gtasks.push_back(gt);
+            gcost.push_back(nmax + 1);  // list steps + the tile stores
+        }
+        // Warp w of the kernel takes groups w, w + W, w + 2 W, ... of the task list (W
+        // gridding warps) and a pass ends when its slowest warp does, so the groups are
+        // dealt out longest first to the least-loaded warp and laid out in that order;
+        // positions a warp does not use hold groups of padding tasks (no entries, no store).
+        const int W = kGridBalThreads / 32;
+        std::vector<std::vector<int>> wl(W);
+        std::vector<long long> load(W, 0);
+        for (int g = 0; g < (int)gtasks.size(); ++g) {  // groups are in decreasing cost order
+            int w = 0;
+            for (int v = 1; v < W; ++v)
+                if (load[v] < load[w]) w = v;
+            wl[w].push_back(g);
+            load[w] += gcost[g];
+        }
+        size_t rounds = 0;
+        for (const auto& l : wl) rounds = std::max(rounds, l.size());
+        const std::vector<int4> pad(32, make_int4(0, 0, -1, -1));
+        for (size_t j = 0; j < rounds; ++j)
+            for (int w = 0; w < W; ++w) {
+                const std::vector<int4>& gt = j < wl[w].size() ? gtasks[wl[w][j]] : pad;
+                tasks.insert(tasks.end(), gt.begin(), gt.end());
+            }
+        tmax = std::max(tmax, (int)(tasks.size() - toff[c]));
+        emax = std::max(emax, (int)ell_e.size() - eoff[c]);
+    }
+    toff[C] = (int)tasks.size();
+    eoff[C] = (int)ell_e.size();
+    for (int c = 0; c < C; ++c) {  // largest offsets / entries of a channel (staged lists)
+        const int np = p->box[c].ny * (p->box[c].nx / kTaskCells) + 1;
+        p->tc.pl_max_ptr = std::max(p->tc.pl_max_ptr, np);
+        p->tc.pl_max_ent = std::max(p->tc.pl_max_ent, pl_ptr[pl_off[c] + np - 1] - pl_ptr[pl_off[c]]);
+    }
+    if (kTaskCells == 2 && !pl_e.empty() && pl_e.size() < (1u << 31)) {  // pair lists for k_dftgemm_grid_pl
+        e = cudaMalloc(&p->tc.pl_ptr, pl_ptr.size() * sizeof(int));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(p->tc.pl_ptr, pl_ptr.data(), pl_ptr.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_off, pl_off.size() * sizeof(int));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(p->tc.pl_off, pl_off.data(), pl_off.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_e, pl_e.size() * sizeof(int));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(p->tc.pl_e, pl_e.data(), pl_e.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_w, pl_w.size() * sizeof(float2));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(p->tc.pl_w, pl_w.data(), pl_w.size() * sizeof(float2), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_fail(p, e, "pair-list upload");
+        p->dt.dft_bytes += (pl_ptr.size() + pl_off.size() + pl_e.size()) * sizeof(int) + pl_w.size() * sizeof(float2);
+    }
+    if (fits && !tasks.empty()) {
+        e = cudaMalloc(&p->tc.gtask, tasks.size() * sizeof(int4));
+        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gtask, tasks.data(), tasks.size() * sizeof(int4),
+                                             cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gtask_off, toff.size() * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gtask_off, toff.data(), toff.size() * sizeof(int),
+                                             cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_e, ell_e.size() * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_e, ell_e.data(), ell_e.size() * sizeof(int),
+                                             cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_w, ell_w.size() * sizeof(TaskW));
+        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_w, ell_w.data(), ell_w.size() * sizeof(TaskW),
+                                             cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_off, eoff.size() * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_off, eoff.data(), eoff.size() * sizeof(int),
+                                             cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_fail(p, e, "gridding task lists upload");
+        p->tc.gtask_max = tmax;
+        p->tc.gell_max = emax;
+        const int keep_f = p->tc.grid_frames;
+        p->tc.grid_variant = 2;
+        epic_status bst = EPIC_ERR_UNSUPPORTED;
+        for (int gf = 2; gf >= 1 && bst == EPIC_ERR_UNSUPPORTED; gf >>= 1) bst = grid_bal_config(p, gf);
+        if (bst != EPIC_OK) {  // the balanced kernel does not fit: the pair-list one, else row-major
+            if (bst != EPIC_ERR_UNSUPPORTED) return bst;
+            p->tc.grid_variant = 1;
+            cudaFree(p->tc.gtask);
+            cudaFree(p->tc.gtask_off);
+            cudaFree(p->tc.gell_e);
+            cudaFree(p->tc.gell_w);
+            cudaFree(p->tc.gell_off);
+            p->tc.gtask = nullptr;
+            p->tc.gtask_off = nullptr;
+            p->tc.gell_e = nullptr;
+            p->tc.gell_w = nullptr;
+            p->tc.gell_off = nullptr;
+            p->tc.gtask_max = 0;
+            if (p->tc.grid_ps) {
+                const epic_status kst = dftgemm_grid_config(p, keep_f);
+                if (kst != EPIC_OK) return kst;
+            }
+            if (p->tc.pl_ptr) {
+                p->tc.grid_variant = 3;
+                epic_status pst = EPIC_ERR_UNSUPPORTED;
+                for (int gf = 4; gf >= 1 && pst == EPIC_ERR_UNSUPPORTED; gf >>= 1) pst = grid_pl_config(p, gf);
+                if (pst != EPIC_OK) {
+                    if (pst != EPIC_ERR_UNSUPPORTED) return pst;
+                    p->tc.grid_variant = 1;
+                    if (p->tc.grid_ps) {
+                        const epic_status kst = dftgemm_grid_config(p, keep_f);
+                        if (kst != EPIC_OK) return kst;
+                    }
+                }
+            }
+        } else {
+            p->dt.dft_bytes += tasks.size() * sizeof(int4) + ell_e.size() * (sizeof(int) + sizeof(TaskW)) +
+                               (toff.size() + eoff.size()) * sizeof(int);
+        }
+    }
+    return EPIC_OK;
 }
 
 epic_status dftgemm_setup(epic_plan_s* p)
@@ -3267,12 +3435,11 @@ epic_status dftgemm_setup(epic_plan_s* p)
                 const int q = r / 32, kx = 32 * sl + r % 32;
                 if (kx >= N) continue;
                 for (int k = 0; k < K1; ++k) {
-                    const int x = b.x0 + (k % b.nx);
                     double fr, fi;
-                    F(x, kx, &fr, &fi);
+                    F(b.x0 + tile_k_x(k), kx, &fr, &fi);
                     double v;
-                    if (q == 0) v = k < b.nx ? fr : -fi;
-                    else v = k < b.nx ? fi : fr;
+                    if (q == 0) v = tile_k_im(k) ? -fi : fr;
+                    else v = tile_k_im(k) ? fr : fi;
                     t[sw_off(r, k, 128)] = f16_bits(v);
                 }
             }
@@ -3310,10 +3477,9 @@ epic_status dftgemm_setup(epic_plan_s* p)
                 const int q = r / 64, kx = 64 * g + r % 64;
                 if (kx >= N) continue;
                 for (int k = 0; k < K1; ++k) {
-                    const int x = b.x0 + (k % b.nx);
                     double fr, fi;
-                    F(x, kx, &fr, &fi);
-                    const double v = q == 0 ? (k < b.nx ? fr : -fi) : (k < b.nx ? fi : fr);
+                    F(b.x0 + tile_k_x(k), kx, &fr, &fi);
+                    const double v = q == 0 ? (tile_k_im(k) ? -fi : fr) : (tile_k_im(k) ? fr : fi);
                     t[sw_off(r, k, 128)] = f16_bits(v);
                 }
             }
@@ -3432,214 +3598,21 @@ epic_status dftgemm_setup(epic_plan_s* p)
         if (gst == EPIC_OK) p->tc.grid_ps = true;
         else if (gst != EPIC_ERR_UNSUPPORTED) return gst;
     }
-    if (!cplx) {  // per-channel task lists of non-empty cell pairs, longest list first
-        std::vector<int> coff, cptr, ce;
-        std::vector<float2> cw;
-        build_csr(p, coff, cptr, ce, cw);
-        // A task is the run of kTaskCells cells (x, x + 1, ...), x a multiple of kTaskCells,
-        // of one row of a channel's box; its entries are the elements that reach any of them
-        // (the union of the cells' element-ordered lists) with one weight per cell.  Runs of
-        // a channel are sorted by entry count (equal counts in Morton order, so that a warp's
-        // runs are near one another and share elements); groups of 32 consecutive runs (the
-        // lanes of one warp) store their entries interleaved, entry k of lane l at 32 k + l,
-        // padded with zero weights to the group's longest list, in the order
-        // order_warp_entries picks.
-        std::vector<int4> tasks;
-        std::vector<int> ell_e;
-        std::vector<TaskW> ell_w;
-        std::vector<int> toff(C + 1, 0), eoff(C + 1, 0);
-        std::vector<TaskW> pw;  // weights of the channel's run lists
-        std::vector<int2> ord;
-        std::vector<int> pl_ptr, pl_off(C), pl_e;  // the same lists row-major (pair-list kernel)
-        std::vector<TaskW> pl_w;
-        bool fits = true;
-        int tmax = 0, emax = 0;
-        for (int c = 0; c < C && fits; ++c) {
-            toff[c] = (int)tasks.size();
-            eoff[c] = (int)ell_e.size();
-            const int* ptr = &cptr[coff[c]];
-            const Box bx = p->box[c];
-            const int hp = bx.nx / kTaskCells;  // runs per row (nx is a multiple of 8)
-            std::vector<std::vector<int2>> plist((size_t)hp * bx.ny);  // (element, 1 + index into pw)
-            pw.clear();
-            for (int y = 0; y < bx.ny; ++y)
-                for (int j = 0; j < hp; ++j) {
-                    const int r0 = y * bx.nx + kTaskCells * j;
-                    int at[kTaskCells];
-                    for (int q = 0; q < kTaskCells; ++q) at[q] = ptr[r0 + q];
-                    std::vector<int2>& L = plist[(size_t)y * hp + j];
-                    for (;;) {  // merge of the cells' element-ordered lists
-                        int el = INT32_MAX;
-                        for (int q = 0; q < kTaskCells; ++q)
-                            if (at[q] < ptr[r0 + q + 1]) el = std::min(el, ce[at[q]]);
-                        if (el == INT32_MAX) break;
-                        float wq[4] = {0.f, 0.f, 0.f, 0.f};
-                        for (int q = 0; q < kTaskCells; ++q)
-                            if (at[q] < ptr[r0 + q + 1] && ce[at[q]] == el) wq[q] = cw[at[q]++].x;
-                        TaskW w;
-                        task_w_set(w, wq);
-                        pw.push_back(w);
-                        L.push_back(make_int2(el, (int)pw.size()));
-                    }
-                }
-            pl_off[c] = (int)pl_ptr.size();
-            for (const std::vector<int2>& L : plist) {
-                pl_ptr.push_back((int)pl_e.size());
-                for (const int2& en : L) {
-                    pl_e.push_back(en.x);
-                    pl_w.push_back(pw[en.y - 1]);
-                }
-            }
-            pl_ptr.push_back((int)pl_e.size());
-            std::vector<int> idx;
-            for (int q = 0; q < hp * bx.ny; ++q)
-                if (!plist[q].empty()) idx.push_back(q);
-            auto morton = [hp](int q) {
-                const unsigned x = (unsigned)(kTaskCells * (q % hp)), y = (unsigned)(q / hp);
-                unsigned m = 0;
-                for (int bit = 0; bit < 12; ++bit) m |= ((x >> bit) & 1u) << (2 * bit) | ((y >> bit) & 1u) << (2 * bit + 1);
-                return m;
-            };
-            std::stable_sort(idx.begin(), idx.end(), [&](int u, int v) {
-                const size_t nu = plist[u].size(), nv = plist[v].size();
-                return nu != nv ? nu > nv : morton(u) < morton(v);
-            });
-            const int nyh = p->tc.tbox_h[c].x;
-            const uint32_t part_bytes = (uint32_t)(p->P * nyh) * pad64(2 * bx.nx) * 2;
-            std::vector<std::vector<int4>> gtasks;  // the 32 tasks of each group (padding tasks: no store)
-            std::vector<int> gcost;
-            for (size_t g0 = 0; g0 < idx.size(); g0 += 32) {
-                const int members = (int)std::min<size_t>(32, idx.size() - g0);
-                const int nmax = (int)plist[idx[g0]].size();
-                const int base = (int)ell_e.size() - eoff[c];
-                if (nmax > 255) fits = false;
-                std::vector<std::vector<int2>> lists(members);
-                for (int l = 0; l < members; ++l) lists[l] = plist[idx[g0 + l]];
-                ord.assign(32ull * nmax, make_int2(0, 0));
-                order_warp_entries(lists, nmax, ord.data());
-                for (const int2& en : ord) {
-                    ell_e.push_back(en.x);
-                    ell_w.push_back(en.y > 0 ? pw[en.y - 1] : TaskW{});
-                }
-                std::vector<int4> gt(32, make_int4(nmax << 24, base, -1, -1));
-                for (int l = 0; l < members; ++l) {
-                    const int q = idx[g0 + l];
-                    if (q >= (1 << 24)) fits = false;
-                    const int y = q / hp, x = kTaskCells * (q % hp);
-                    gt[l] = make_int4(q | (nmax << 24), base, (int)tile_part_off(y, x, nyh, p->P, part_bytes),
-                                      (int)tile_part_off(y, bx.nx + x, nyh, p->P, part_bytes));
-                }
-                gtasks.push_back(gt);
-                gcost.push_back(nmax + 1);  // list steps + the tile stores
-            }
-            // Warp w of the kernel takes groups w, w + W, w + 2 W, ... of the task list (W
-            // gridding warps) and a pass ends when its slowest warp does, so the groups are
-            // dealt out longest first to the least-loaded warp and laid out in that order;
-            // positions a warp does not use hold groups of padding tasks (no entries, no store).
-            const int W = kGridBalThreads / 32;
-            std::vector<std::vector<int>> wl(W);
-            std::vector<long long> load(W, 0);
-            for (int g = 0; g < (int)gtasks.size(); ++g) {  // groups are in decreasing cost order
-                int w = 0;
-                for (int v = 1; v < W; ++v)
-                    if (load[v] < load[w]) w = v;
-                wl[w].push_back(g);
-                load[w] += gcost[g];
-            }
-            size_t rounds = 0;
-            for (const auto& l : wl) rounds = std::max(rounds, l.size());
-            const std::vector<int4> pad(32, make_int4(0, 0, -1, -1));
-            for (size_t j = 0; j < rounds; ++j)
-                for (int w = 0; w < W; ++w) {
-                    const std::vector<int4>& gt = j < wl[w].size() ? gtasks[wl[w][j]] : pad;
-                    tasks.insert(tasks.end(), gt.begin(), gt.end());
-                }
-            tmax = std::max(tmax, (int)(tasks.size() - toff[c]));
-            emax = std::max(emax, (int)ell_e.size() - eoff[c]);
-        }
-        toff[C] = (int)tasks.size();
-        eoff[C] = (int)ell_e.size();
-        for (int c = 0; c < C; ++c) {  // largest offsets / entries of a channel (staged lists)
-            const int np = p->box[c].ny * (p->box[c].nx / kTaskCells) + 1;
-            p->tc.pl_max_ptr = std::max(p->tc.pl_max_ptr, np);
-            p->tc.pl_max_ent = std::max(p->tc.pl_max_ent, pl_ptr[pl_off[c] + np - 1] - pl_ptr[pl_off[c]]);
-        }
-        if (kTaskCells == 2 && !pl_e.empty() && pl_e.size() < (1u << 31)) {  // pair lists for k_dftgemm_grid_pl
-            e = cudaMalloc(&p->tc.pl_ptr, pl_ptr.size() * sizeof(int));
-            if (e == cudaSuccess)
-                e = cudaMemcpy(p->tc.pl_ptr, pl_ptr.data(), pl_ptr.size() * sizeof(int), cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_off, pl_off.size() * sizeof(int));
-            if (e == cudaSuccess)
-                e = cudaMemcpy(p->tc.pl_off, pl_off.data(), pl_off.size() * sizeof(int), cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_e, pl_e.size() * sizeof(int));
-            if (e == cudaSuccess)
-                e = cudaMemcpy(p->tc.pl_e, pl_e.data(), pl_e.size() * sizeof(int), cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_w, pl_w.size() * sizeof(float2));
-            if (e == cudaSuccess)
-                e = cudaMemcpy(p->tc.pl_w, pl_w.data(), pl_w.size() * sizeof(float2), cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) return cuda_fail(p, e, "pair-list upload");
-            p->dt.dft_bytes += (pl_ptr.size() + pl_off.size() + pl_e.size()) * sizeof(int) + pl_w.size() * sizeof(float2);
-        }
-        if (fits && !tasks.empty()) {
-            e = cudaMalloc(&p->tc.gtask, tasks.size() * sizeof(int4));
-            if (e == cudaSuccess) e = cudaMemcpy(p->tc.gtask, tasks.data(), tasks.size() * sizeof(int4),
-                                                 cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.gtask_off, toff.size() * sizeof(int));
-            if (e == cudaSuccess) e = cudaMemcpy(p->tc.gtask_off, toff.data(), toff.size() * sizeof(int),
-                                                 cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_e, ell_e.size() * sizeof(int));
-            if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_e, ell_e.data(), ell_e.size() * sizeof(int),
-                                                 cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_w, ell_w.size() * sizeof(TaskW));
-            if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_w, ell_w.data(), ell_w.size() * sizeof(TaskW),
-                                                 cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_off, eoff.size() * sizeof(int));
-            if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_off, eoff.data(), eoff.size() * sizeof(int),
-                                                 cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) return cuda_fail(p, e, "gridding task lists upload");
-            p->tc.gtask_max = tmax;
-            p->tc.gell_max = emax;
-            const int keep_f = p->tc.grid_frames;
-            p->tc.grid_variant = 2;
-            epic_status bst = EPIC_ERR_UNSUPPORTED;
-            for (int gf = 2; gf >= 1 && bst == EPIC_ERR_UNSUPPORTED; gf >>= 1) bst = grid_bal_config(p, gf);
-            if (bst != EPIC_OK) {  // the balanced kernel does not fit: the pair-list one, else row-major
-                if (bst != EPIC_ERR_UNSUPPORTED) return bst;
-                p->tc.grid_variant = 1;
-                cudaFree(p->tc.gtask);
-                cudaFree(p->tc.gtask_off);
-                cudaFree(p->tc.gell_e);
-                cudaFree(p->tc.gell_w);
-                cudaFree(p->tc.gell_off);
-                p->tc.gtask = nullptr;
-                p->tc.gtask_off = nullptr;
-                p->tc.gell_e = nullptr;
-                p->tc.gell_w = nullptr;
-                p->tc.gell_off = nullptr;
-                p->tc.gtask_max = 0;
-                if (p->tc.grid_ps) {
-                    const epic_status kst = dftgemm_grid_config(p, keep_f);
-                    if (kst != EPIC_OK) return kst;
-                }
-                if (p->tc.pl_ptr) {
-                    p->tc.grid_variant = 3;
-                    epic_status pst = EPIC_ERR_UNSUPPORTED;
-                    for (int gf = 4; gf >= 1 && pst == EPIC_ERR_UNSUPPORTED; gf >>= 1) pst = grid_pl_config(p, gf);
-                    if (pst != EPIC_OK) {
-                        if (pst != EPIC_ERR_UNSUPPORTED) return pst;
-                        p->tc.grid_variant = 1;
-                        if (p->tc.grid_ps) {
-                            const epic_status kst = dftgemm_grid_config(p, keep_f);
-                            if (kst != EPIC_OK) return kst;
-                        }
-                    }
-                }
-            } else {
-                p->dt.dft_bytes += tasks.size() * sizeof(int4) + ell_e.size() * (sizeof(int) + sizeof(TaskW)) +
-                                   (toff.size() + eoff.size()) * sizeof(int);
-            }
+    // a group of frames fills the tensor-core gridding kernel's columns; shorter blocks, and
+    // plans it does not take, go through the gather kernels' lists
+    epic_status gst = p->max_time >= kGridTcMinTime ? grid_tc_setup(p) : EPIC_ERR_UNSUPPORTED;
+    if (gst == EPIC_OK) {
+        const int keep_v = p->tc.grid_variant, keep_f = p->tc.grid_frames;
+        p->tc.grid_variant = 4;
+        gst = EPIC_ERR_UNSUPPORTED;
+        for (int gc = 4; gc >= 1 && gst == EPIC_ERR_UNSUPPORTED; gc >>= 1) gst = grid_tc_config(p, gc);
+        if (gst != EPIC_OK) {
+            p->tc.grid_variant = keep_v;
+            p->tc.grid_frames = keep_f;
         }
     }
+    if (gst == EPIC_ERR_UNSUPPORTED) gst = grid_lists_setup(p);
+    if (gst != EPIC_OK) return gst;
     const size_t max_list_l = (size_t)max_list;
     const size_t csr_bytes = sizeof(int) * (size_t)((max_cells + 2) & ~1) + sizeof(int2) * max_list_l;
     const size_t gl = (size_t)p->smem_optin;
@@ -3747,7 +3720,11 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
         for (int t0 = 0; t0 < T; t0 += p->tc.tc) {
             const int nt = std::min(p->tc.tc, T - t0);
             const dim3 gg((nt + fpc - 1) / fpc, ng);
-            if (p->tc.grid_ps || p->tc.grid_variant >= 2) {
+            if (p->tc.grid_variant == 4) {
+                ev_begin(p, "k_dftgemm_grid", s);
+                grid_tc_launch(p, volt, t0, nt, c0, ng, s);
+                ev_end(p, s);
+            } else if (p->tc.grid_ps || p->tc.grid_variant >= 2) {
                 // the launch's shared memory must be the chosen kernel's layout for F frames
                 const int fb = A * P * (p->bits / 4);
                 const size_t need = p->tc.grid_variant == 3 ? grid_pl_smem(F, A, fb, p->jones.empty(), p->tc.pl_stage,

@@ -123,19 +123,6 @@ __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---------------------------------------------------------------- descriptors
-// Shared-memory matrix descriptor, no swizzle, K-major "core matrix" layout:
-// 8 rows x 16 bytes per core matrix; lbo = byte step between core matrices along
-// K, sbo = byte step between 8-row groups along M/N.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version of the tcgen05 family
-    return d;                // base offset 0, absolute LBO mode off, swizzle none
-}
-
 // Shared-memory matrix descriptor for the 128-byte swizzled K-major layout:
 // rows of 128 bytes (64 halves of K), 8-row atoms of 1024 bytes (sbo), the
 // 16-byte chunk c of row r stored at chunk position c ^ (r & 7).  The operand
@@ -202,6 +189,11 @@ __device__ __forceinline__ uint32_t elect_one()
 // Operand descriptors by their low words: the high word of smem_desc_sw128 is a constant.
 __device__ __forceinline__ uint32_t desc_sw128_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
 constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+// The same for an operand of 128 rows x 16 halves without swizzle: two K-major columns of 16-byte
+// row chunks, 2048 bytes apart (8 rows x 16 bytes a core matrix, 128 bytes to the next 8 rows).
+__device__ __forceinline__ uint32_t desc_step128_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | ((2048u >> 4) << 16); }
+constexpr uint32_t kDescStep128Hi = (128u >> 4) | (1u << 14);
+template <uint32_t HI = kDescSw128Hi>
 __device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
                                              uint32_t accumulate, uint32_t lead)
 {
@@ -212,7 +204,7 @@ __device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint
         "mov.b64 x, {%1, %6};\n\t"
         "mov.b64 y, {%2, %6};\n\t"
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(kDescSw128Hi)
+        "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(HI)
         : "memory");
 }
 __device__ __forceinline__ void mma_f16_ta_lead(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t idesc,

@@ -46,9 +46,12 @@ std::vector<Knob> knobs_for(const epic_plan_s* p)
             knobs.push_back({"mma_kernel", {1, 2, 3}, p->tc.ws_variant, set_dft_kernel});
             knobs.push_back({"split", {-1, 0, 1}, p->tc.split, set_dft_split});
         }
-        if ((p->tc.grid_ps ? 1 : 0) + (p->tc.gtask ? 1 : 0) + (p->tc.pl_ptr ? 1 : 0) >= 2)
-            knobs.push_back({"grid_kernel", {1, 2, 3}, p->tc.grid_variant, set_dft_grid_kernel});
-        if (p->tc.grid_ps || p->tc.gtask || p->tc.pl_ptr)
+        // the gather kernels' lists may still be unbuilt: setting the parameter builds them
+        const bool lists = p->tc.gtask || p->tc.pl_ptr || !p->tc.lists_built;
+        if ((p->tc.grid_ps ? 1 : 0) + (p->tc.gtask ? 1 : 0) + (p->tc.pl_ptr || !p->tc.lists_built ? 1 : 0) +
+                (p->tc.gt_tile0 ? 1 : 0) >= 2)
+            knobs.push_back({"grid_kernel", {1, 2, 3, 4}, p->tc.grid_variant, set_dft_grid_kernel});
+        if (p->tc.grid_ps || lists || p->tc.gt_tile0)
             knobs.push_back({"grid_frames", {1, 2, 4, 8}, p->tc.grid_frames, set_dft_frames});
         knobs.push_back({"chunk_mb", {96, 192, 384, 768, 1536, 3072, 6144, 12288, 24576}, budget_mb, set_dft_chunk});
     }
@@ -124,6 +127,8 @@ extern "C" epic_status epic_plan_tune(epic_plan_t p, const uint8_t* volt, int T,
     ++timed;
     for (size_t k = 0; k < knobs.size() && st == EPIC_OK; ++k) {
         Knob& kb = knobs[k];
+        for (const Knob& now : knobs_for(p))  // an earlier parameter may have changed this one's value
+            if (std::string(now.name) == kb.name) kb.current = now.current;
         int best_v = kb.current;
         for (int v : kb.values) {
             if (v == kb.current) continue;
