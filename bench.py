@@ -78,6 +78,11 @@ def kernel_model(name, cfg, T, info):
     tc = max(1, info.get("time_chunk") or T)
     nt = min(tc, T)
     grid_bytes = nt * C * P * N * N * 8
+    row_bytes = nt * C * P * min(N, info.get("box_max_y", N)) * N * 8
+    if name == "k_plain_rows":
+        return "hbm", nt * C * A * P + row_bytes, "B"
+    if name == "k_plain_cols":
+        return "hbm", row_bytes + 2 * C * nprod * N * N * 4, "B"
     if name == "k_plain_grid":
         return "hbm", nt * C * A * P + grid_bytes, "B"
     if name in ("k_plain_fft_rows", "k_plain_fft_cols"):

@@ -62,8 +62,8 @@ typedef enum {
 
 /* Which implementation of the hot path a plan uses. */
 typedef enum {
-    EPIC_PATH_PLAIN_FP32 = 0,   /* unfused FP32: grid kernel -> HBM -> row FFT -> HBM -> column FFT
-                                   -> HBM -> square/accumulate kernel (the plain comparator)      */
+    EPIC_PATH_PLAIN_FP32 = 0,   /* FP32 FFT: gridding and row FFT kernel -> box rows in HBM -> column
+                                   FFT, products and accumulation kernel (the plain comparator)   */
     EPIC_PATH_FUSED_FP32 = 1,   /* one fused kernel per block: grid -> FP32 FFT -> products ->
                                    on-chip accumulation, images written once                      */
     EPIC_PATH_DFTGEMM_FP16 = 2, /* a gridding kernel writes FP16 grid tiles, then one tensor-core
@@ -223,8 +223,9 @@ epic_status epic_plan_get_info(epic_plan_t plan, epic_plan_info* info);
  * the plan configured with them.  Parameters by path:
  *   AUTO plans    path         0 plain FP32, 1 fused FP32, 2 DFT-as-GEMM (timed first; the chosen
  *                              path's own parameters follow)
- *   PLAIN_FP32    fft          FFT kernels: 0 register-resident two-pass transforms (one
- *                              shared-memory exchange), 1 radix-4/2 Stockham in shared memory
+ *   PLAIN_FP32    fft          0 two kernels with register-resident two-pass transforms (one
+ *                              shared-memory exchange), 1 four kernels (grid, rows, columns,
+ *                              products) with radix-4/2 Stockham transforms in shared memory
  *                 chunk_mb     grid-buffer budget of one time chunk (MiB)
  *   FUSED_FP32    slab         image columns per work item
  *   DFTGEMM_FP16  group        channels per launch: 0 groups of about two work items per SM,

@@ -164,7 +164,8 @@ struct epic_plan_s {
     int fused_variant = 0;                // kernel variant chosen for fused paths
     bool auto_path = false;               // created with EPIC_PATH_AUTO: the tuner may change path
     int slab = 0;                         // output columns per work item (fused paths)
-    int plain_fft = 0;                    // plain path FFT kernels: 0 register two-pass, 1 shared-memory Stockham
+    int plain_fft = 0;                    // plain path: 0 register two-pass FFTs, 1 shared-memory Stockham
+    int plain_slices = 1;                 // plain path: slices of a chunk's frames in k_plain_cols
 
     size_t chunk_budget = 0;              // scratch budget of one time chunk (chunked paths)
 

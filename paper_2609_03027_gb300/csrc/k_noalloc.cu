@@ -143,7 +143,15 @@ __global__ void __launch_bounds__(kNaThreads) k_na_sqacc(const float2* __restric
     const int c = blockIdx.y;
     if (pix >= NN) return;
     float xx = 0.f, yy = 0.f, rxy = 0.f, ixy = 0.f;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;  // of whole runs of 64 samples: the rounding of long sums stays small
     for (int tl = 0; tl < nt; ++tl) {
+        if ((tl & 63) == 0) {
+            s0 += xx;
+            s1 += yy;
+            s2 += rxy;
+            s3 += ixy;
+            xx = yy = rxy = ixy = 0.f;
+        }
         const float2* g = grid + ((size_t)tl * C + c) * P * NN;
         const float2 X = g[pix];
         xx = fmaf(X.x, X.x, fmaf(X.y, X.y, xx));
@@ -154,6 +162,10 @@ __global__ void __launch_bounds__(kNaThreads) k_na_sqacc(const float2* __restric
             ixy = fmaf(X.y, Y.x, fmaf(-X.x, Y.y, ixy));
         }
     }
+    xx += s0;
+    yy += s1;
+    rxy += s2;
+    ixy += s3;
     const int nprod = P == 2 ? 4 : 1;
     float* o = out + (size_t)c * nprod * NN + pix;
     o[0] = (accumulate ? o[0] : 0.f) + xx;

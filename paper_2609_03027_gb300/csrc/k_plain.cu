@@ -1,17 +1,20 @@
-// Plain, unfused FP32 path of the EPIC hot loop (paper Sec. 2, Eq. 1-2): the
-// comparator for the fused paths.  Per chunk of time samples, four kernels with
-// HBM round trips between them:
-//   k_plain_grid     unpack the voltages (and mix polarisations, when the plan
-//                    has a mixing kernel) and gather-grid every (t, c, p)
-//                    frame onto a full N x N complex grid (Eq. 1 bracket)
-//   k_plain_fft_rows FFT along x of every grid row (Eq. 1 sum)
-//   k_plain_fft_cols the same along y, on tiles of adjacent columns
-// Two forms of the FFT kernels: register-resident two-pass transforms (the
-// default, one shared-memory exchange per transform) and radix-4/2 Stockham
-// transforms in shared memory (a pass over shared memory per radix-4 stage).
-//   k_plain_sqacc    XX, YY, XY products summed over the chunk's frames and
-//                    added to the images (Eq. 2)
+// Plain FP32 path of the EPIC hot loop (paper Sec. 2, Eq. 1-2).  Per chunk of time samples, two
+// kernels with one HBM round trip of the occupied rows between them:
+//   k_plain_rows     unpack the voltages (and mix polarisations, when the plan has a mixing
+//                    kernel), gather-grid the occupied box of every (t, c) frame (Eq. 1 bracket)
+//                    row by row into shared memory and FFT each row along x
+//   k_plain_cols     the FFT along y on tiles of adjacent columns (rows outside the box are
+//                    zero), the XX, YY, XY products, summed over the chunk's frames in registers
+//                    and added to the images (Eq. 2)
+//   k_plain_sum      adds the partial sums up where a chunk's frames were cut into slices
+// The transforms are register-resident two-pass FFTs.  With full N x N grids going through HBM
+// between four kernels (grid, rows, columns, products) the LWA-station block took 34.0 ms, six
+// passes over 33.5 GB at 0.97 of the copy rate; the box rows are 48 of 128 there and go through
+// once each way.  The tuner's second form (fft = 1) keeps the four kernels with radix-4/2 Stockham
+// transforms in shared memory:
+//   k_plain_grid, k_plain_fft_rows_smem, k_plain_fft_cols_smem, k_plain_sqacc
 #include <algorithm>
+#include <cmath>
 
 #include "epic_internal.h"
 #include "kcommon.cuh"
@@ -92,119 +95,436 @@ __device__ __forceinline__ void load_step_twiddles(float2* tw, const float2* __r
     }
 }
 
-constexpr int kRegThreads = 256;
+// Samples of element e (0 .. P-1 pols) of a frame: staged FP32 pairs, or decoded from its bytes.
+template <int P, bool STAGED>
+__device__ __forceinline__ void frame_sample(const float2* sv, const uint8_t* fr, int e, int bits, const float4* jm,
+                                             float2 (&v)[P])
+{
+    if (STAGED) {
+        if (P == 2) {
+            const float4 q = *reinterpret_cast<const float4*>(sv + 2 * e);
+            v[0] = make_float2(q.x, q.y);
+            v[P - 1] = make_float2(q.z, q.w);
+        } else {
+            v[0] = sv[e];
+        }
+    } else if (P == 2) {
+        const float4 q = load_pair(fr, e, bits, jm);
+        v[0] = make_float2(q.x, q.y);
+        v[P - 1] = make_float2(q.z, q.w);
+    } else {
+        v[0] = load_sample(fr, e, bits);
+    }
+}
 
-// Rows of N = N1 N2 points, 256 / N2 rows per block, N2 threads per row.  Thread j
-// of a row takes n1 = j (and j + N2) in pass 1 and k2 = j in pass 2.  Y of a row is
-// stored [k2][n1] with stride N1 + 1, which no pass-1 store or pass-2 load of a warp
-// meets twice in one bank.
+constexpr int kRowThreads = 256;
+constexpr int kRowFrames = 2;  // frames of a block: each list entry read from L1 serves both
+
+// bytes of k_plain_rows's shared memory: twiddles, Y, the rows' box columns, the frames
+inline int rows_ld(int nx) { return (nx & 15) == 8 ? nx : nx + 8; }  // row stride = 8 mod 16
 template <int N1, int N2>
-__global__ void __launch_bounds__(kRegThreads) k_plain_fft_rows(float2* __restrict__ grid, size_t n_rows,
-                                                                const float2* __restrict__ twg)
+__host__ __device__ constexpr size_t rows_fft_smem()
 {
-    constexpr int N = N1 * N2, RPC = kRegThreads / N2, S = N2 * (N1 + 1), T = N1 / N2;
-    constexpr int L1 = ilog2(N1), L2 = ilog2(N2);
+    return sizeof(float2) * ((size_t)N1 * N2 + (size_t)(kRowThreads / N2) * N2 * (N1 + 1));
+}
+
+// Gridded and row-transformed frames (LWA station: 5.5 ms a block, 2.9 ms of it the 12.9 GB of row
+// stores, the rest the gather's dependent list and voltage reads): block = frames 2 blockIdx.x, + 1 of channel blockIdx.y.
+// Rows go in batches of 256 / N2 (both frames, all pols, a few y): the batch's cells are gathered
+// one per thread and step, both frames and pols at once, then N2 threads a row run the two FFT
+// passes (thread j takes n1 = j, j + N2 in pass 1 and k2 = j in pass 2; Y is stored [k2][n1] with
+// stride N1 + 1, which no pass-1 store or pass-2 load of a warp meets twice in one bank) and
+// store rows[(t C + c) P + p][y - y0][N].
+template <int N1, int N2, int P, bool STAGED, bool CPLX>
+__global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __restrict__ volt, int t0, int nt, int C, int A,
+                                                            int bits, const int4* __restrict__ box,
+                                                            const int* __restrict__ cell_off,
+                                                            const int* __restrict__ cell_ptr,
+                                                            const int* __restrict__ ce, const float2* __restrict__ cw,
+                                                            const float4* __restrict__ jones, int frame_in_smem,
+                                                            int ld, int ny_max, const float2* __restrict__ twg,
+                                                            float2* __restrict__ rows)
+{
+    constexpr int N = N1 * N2, RPC = kRowThreads / N2, S = N2 * (N1 + 1), T = N1 / N2, F = kRowFrames;
+    constexpr int L1 = ilog2(N1), L2 = ilog2(N2), YR = RPC / (F * P);
+    static_assert(YR >= 1, "a batch holds a row of every frame and pol");
     extern __shared__ float2 sm[];
-    float2* tw = sm;      // [N2][N1]
-    float2* y = sm + N;   // [RPC][N2][N1 + 1]
-    load_step_twiddles<N1, N2>(tw, twg);
-    const int rl = threadIdx.x / N2, j = threadIdx.x % N2;
-    const size_t r = (size_t)blockIdx.x * RPC + rl;
-    const bool live = r < n_rows;
-    float2* row = grid + (live ? r : 0) * N;
-    float2 u[T][N2];
+    const int tid = threadIdx.x, c = blockIdx.y, f0 = F * blockIdx.x;
+    const int4 b = box[c];
+    const int nx = min(b.z, N - b.x), ny = min(b.w, N - b.y);  // box padding beyond the grid holds nothing
+    float2* tw = sm;               // [N2][N1]
+    float2* y = tw + N;            // [RPC][N2][N1 + 1]
+    float2* g = y + RPC * S;       // [F][P][YR][ld]
+    uint8_t* fr_s = reinterpret_cast<uint8_t*>(g + F * P * YR * ld);
+    float2* sv = reinterpret_cast<float2*>(fr_s);  // [F][A][P]
+    const int FB = A * P * (bits / 4);
+    const float4* jm = jones ? jones + (size_t)c * A * 2 : nullptr;
+    const uint8_t* fr[F];
 #pragma unroll
-    for (int t = 0; t < T; ++t)
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) u[t][n2] = live ? row[j + N2 * t + N1 * n2] : make_float2(0.f, 0.f);
-    __syncthreads();  // twiddles
-    float2* yr = y + rl * S;
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-        dft_reg<N2>(u[t]);
-        const int n1 = j + N2 * t;
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2)
-            yr[k2 * (N1 + 1) + n1] = cmul(u[t][bit_reverse(k2, L2)], tw[k2 * N1 + n1]);
+    for (int f = 0; f < F; ++f) {
+        fr[f] = volt + ((size_t)(t0 + min(f0 + f, nt - 1)) * C + c) * (size_t)FB;  // an odd last frame twice
+        if (STAGED) {
+            stage_frame(sv + (size_t)f * A * P, fr[f], A, P, bits, jm);
+        } else if (frame_in_smem) {
+            uint8_t* d = fr_s + (size_t)f * ((FB + 15) & ~15);
+            if (((FB | (int)(uintptr_t)fr[f]) & 3) == 0)
+                for (int i = tid; i < FB >> 2; i += kRowThreads)
+                    reinterpret_cast<uint32_t*>(d)[i] = __ldg(reinterpret_cast<const uint32_t*>(fr[f]) + i);
+            else
+                for (int i = tid; i < FB; i += kRowThreads) d[i] = __ldg(fr[f] + i);
+            fr[f] = d;
+        }
     }
-    __syncthreads();
-    float2 z[N1];
+    load_step_twiddles<N1, N2>(tw, twg);
+    const int* ptr = cell_ptr + cell_off[c];
+    const int rl = tid / N2, j = tid % N2;             // this thread's row of a batch and its place in it
+    const int rf = rl / (P * YR), rp = rl / YR % P, ry = rl % YR;
+    for (int yb = 0; yb < ny; yb += YR) {
+        __syncthreads();  // frames staged; the last batch's rows are read
+        for (int i = tid; i < YR * nx; i += kRowThreads) {
+            const int r = i / nx, x = i - r * nx;
+            float2 acc[F][P];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) z[n1] = yr[j * (N1 + 1) + n1];
-    dft_reg<N1>(z);
-    if (live) {
+            for (int f = 0; f < F; ++f)
 #pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) row[j + N2 * k1] = z[bit_reverse(k1, L1)];
+                for (int p = 0; p < P; ++p) acc[f][p] = make_float2(0.f, 0.f);
+            if (yb + r < ny) {
+                const int cell = (yb + r) * b.z + x, q1 = __ldg(ptr + cell + 1);
+                for (int q = __ldg(ptr + cell); q < q1; ++q) {
+                    const int e = __ldg(ce + q);
+                    const float2 w = CPLX ? __ldg(cw + q) : make_float2(__ldg(&cw[q].x), 0.f);
+#pragma unroll
+                    for (int f = 0; f < F; ++f) {
+                        float2 v[P];
+                        frame_sample<P, STAGED>(sv + (size_t)f * A * P, fr[f], e, bits, jm, v);
+#pragma unroll
+                        for (int p = 0; p < P; ++p) {
+                            if (CPLX) acc[f][p] = cfma(w, v[p], acc[f][p]);
+                            else acc[f][p] = make_float2(fmaf(w.x, v[p].x, acc[f][p].x), fmaf(w.x, v[p].y, acc[f][p].y));
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int f = 0; f < F; ++f)
+#pragma unroll
+                for (int p = 0; p < P; ++p) g[((f * P + p) * YR + r) * ld + x] = acc[f][p];
+        }
+        __syncthreads();
+        const float2* gr = g + (size_t)rl * ld;
+        float2 u[T][N2];
+        float2* yr = y + rl * S;
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+#pragma unroll
+            for (int n2 = 0; n2 < N2; ++n2) {
+                const int x = j + N2 * t + N1 * n2 - b.x;
+                u[t][n2] = x >= 0 && x < nx ? gr[x] : make_float2(0.f, 0.f);
+            }
+            dft_reg<N2>(u[t]);
+            const int n1 = j + N2 * t;
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) yr[k2 * (N1 + 1) + n1] = cmul(u[t][bit_reverse(k2, L2)], tw[k2 * N1 + n1]);
+        }
+        __syncthreads();
+        float2 z[N1];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) z[n1] = yr[j * (N1 + 1) + n1];
+        dft_reg<N1>(z);
+        if (f0 + rf < nt && yb + ry < ny) {
+            float2* o = rows + ((((size_t)(f0 + rf) * C + c) * P + rp) * ny_max + yb + ry) * N + j;
+#pragma unroll
+            for (int k1 = 0; k1 < N1; ++k1) o[N2 * k1] = z[bit_reverse(k1, L1)];
+        }
     }
 }
 
-// Columns of one N x N frame (blockIdx.y), TX adjacent columns per block, N2 threads
-// per column; a warp's lanes take adjacent columns, so every global access of a warp
-// is one contiguous run and Y ([n1][k2][column]) is read and written without bank
-// conflicts.
-template <int N1, int N2, int TX>
-__global__ void __launch_bounds__(TX * N2) k_plain_fft_cols(float2* __restrict__ grid, const float2* __restrict__ twg)
+// One pixel's products added to its sums.
+template <int P>
+__device__ __forceinline__ void add_products(float2 X, float2 Y, float& xx, float& yy, float& rxy, float& ixy)
 {
-    constexpr int N = N1 * N2, T = N1 / N2;
-    constexpr int L1 = ilog2(N1), L2 = ilog2(N2);
-    extern __shared__ float2 sm[];
-    float2* tw = sm;      // [N2][N1]
-    float2* y = sm + N;   // [N1][N2][TX]
-    load_step_twiddles<N1, N2>(tw, twg);
-    const int xl = threadIdx.x % TX, j = threadIdx.x / TX;
-    float2* g = grid + (size_t)blockIdx.y * N * N + (size_t)blockIdx.x * TX + xl;
-    float2 u[T][N2];
-#pragma unroll
-    for (int t = 0; t < T; ++t)
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) u[t][n2] = g[(size_t)(j + N2 * t + N1 * n2) * N];
-    __syncthreads();  // twiddles
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-        dft_reg<N2>(u[t]);
-        const int n1 = j + N2 * t;
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2)
-            y[(n1 * N2 + k2) * TX + xl] = cmul(u[t][bit_reverse(k2, L2)], tw[k2 * N1 + n1]);
+    xx = fmaf(X.x, X.x, fmaf(X.y, X.y, xx));
+    if (P == 2) {
+        yy = fmaf(Y.x, Y.x, fmaf(Y.y, Y.y, yy));
+        rxy = fmaf(X.x, Y.x, fmaf(X.y, Y.y, rxy));
+        ixy = fmaf(X.y, Y.x, fmaf(-X.x, Y.y, ixy));
     }
-    __syncthreads();
-    float2 z[N1];
-#pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) z[n1] = y[(n1 * N2 + j) * TX + xl];
-    dft_reg<N1>(z);
-#pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) g[(size_t)(j + N2 * k1) * N] = z[bit_reverse(k1, L1)];
 }
 
-// launch shapes of the register FFT kernels of one N
+__device__ __forceinline__ void cp_async16(void* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int K>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(K) : "memory");
+}
+
+// frames k_plain_cols sums in registers before it adds them to memory: the rounding error of long
+// sums stays that of short ones
+constexpr int kColRun = 64;
+
+// frames of box columns k_plain_cols holds in shared memory (two in flight); none at N = 512, where
+// one would take half an SM
+constexpr int col_stages(int N) { return N <= 256 ? 3 : 0; }
+
+// Column transforms and products: block = TX adjacent columns of channel blockIdx.y and slice
+// blockIdx.z of the chunk's frames (of its intervals, with sub-integrations); N2 threads a column,
+// lanes on adjacent columns (every global access of a warp one contiguous run per row, Y
+// [n1][k2][column] without bank conflicts).  The box rows of the next two frames are on their way
+// into shared memory while a frame is transformed (loaded when needed, the HBM latency of each
+// pol showed: 4.4 k cycles a tile and frame).  A thread ends up with the pixels ky = j + N2 k1 of
+// its column and keeps their sums in registers; at N1 = 32 X's pixels wait in the thread's own
+// slots of the exchange buffer while Y is transformed.  out: the images, or the slice's partial sums.
+template <int N1, int N2, int TX, int P>
+__global__ void __launch_bounds__(TX * N2) k_plain_cols(const float2* __restrict__ rows, int nt, int C, int ny_max,
+                                                        const int4* __restrict__ box, const float2* __restrict__ twg,
+                                                        float* __restrict__ out, float* __restrict__ partial,
+                                                        int accumulate, int sub, int out_iv0)
+{
+    constexpr int N = N1 * N2, T = N1 / N2, L1 = ilog2(N1), L2 = ilog2(N2), NP = P == 2 ? 4 : 1, ST = col_stages(N);
+    constexpr size_t NN = (size_t)N * N;
+    constexpr bool kKeep = N1 <= 16;  // X's pixels stay in registers
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;                          // [N2][N1]
+    float2* y = sm + N;                       // [P][N1][N2][TX]
+    float2* stage = y + (size_t)P * N * TX;   // [ST][P][ny_max][TX]
+    const int xl = threadIdx.x % TX, j = threadIdx.x / TX, c = blockIdx.y, xb = blockIdx.x * TX;
+    const int4 b = box[c];
+    const int y0 = b.y, ny = min(b.w, N - b.y);
+    load_step_twiddles<N1, N2>(tw, twg);
+    const int unit = sub > 0 ? sub : 1, units = nt / unit, S = gridDim.z;
+    const int ta = (int)((long long)units * blockIdx.z / S) * unit, tb = (int)((long long)units * (blockIdx.z + 1) / S) * unit;
+    float xx[N1], yy[P == 2 ? N1 : 1], rxy[P == 2 ? N1 : 1], ixy[P == 2 ? N1 : 1];
+    auto clear = [&]() {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+            xx[i] = 0.f;
+            if (P == 2) yy[i] = rxy[i] = ixy[i] = 0.f;
+        }
+    };
+    auto store = [&](float* o, bool add) {
+        o += (size_t)j * N + xb + xl;
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            float* q = o + (size_t)(N2 * k1) * N;
+            q[0] = (add ? q[0] : 0.f) + xx[k1];
+            if (P == 2) {
+                q[NN] = (add ? q[NN] : 0.f) + yy[k1];
+                q[2 * NN] = (add ? q[2 * NN] : 0.f) + rxy[k1];
+                q[3 * NN] = (add ? q[3 * NN] : 0.f) + ixy[k1];
+            }
+        }
+    };
+    auto frame = [&](int t, int p) { return rows + (((size_t)t * C + c) * P + p) * (size_t)ny_max * N + xb; };
+    auto fetch = [&](int t) {  // frame t's box columns -> its stage (a group is committed either way)
+        if (t < tb) {
+            float2* d = stage + (size_t)(t % (ST ? ST : 1)) * P * ny_max * TX;
+            constexpr int Q = TX / 2;  // 16-byte chunks of a row
+            for (int i = threadIdx.x; i < P * ny * Q; i += TX * N2) {
+                const int row = i / Q, q = i % Q, p = P == 2 && row >= ny ? 1 : 0, r = row - p * ny;
+                cp_async16(d + ((size_t)p * ny_max + r) * TX + 2 * q, frame(t, p) + (size_t)r * N + 2 * q);
+            }
+        }
+        cp_async_commit();
+    };
+    auto image = [&](int t) {  // where frame t's sums go
+        return sub > 0 ? out + ((size_t)(out_iv0 + t / sub) * C + c) * NP * NN
+                       : (partial ? partial + (size_t)blockIdx.z * C * NP * NN : out) + (size_t)c * NP * NN;
+    };
+    clear();
+    bool add = accumulate != 0;
+    if (ST) {
+        fetch(ta);
+        fetch(ta + 1);
+    }
+    for (int t = ta; t < tb;) {
+        // a run: up to kColRun frames of one image set
+        const int te = min(min(t + kColRun, tb), sub > 0 ? t - t % sub + sub : tb);
+        float* const target = image(t);
+        const bool end = te == tb || (sub > 0 && te % sub == 0);
+        for (; t < te; ++t) {
+            if (ST) cp_async_wait<1>();
+            __syncthreads();  // this frame's columns (and the twiddles) are in; the last frame's buffers are read
+            if (ST) fetch(t + 2);
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const float2* r = ST ? stage + ((size_t)(t % (ST ? ST : 1)) * P + p) * ny_max * TX + xl : frame(t, p) + xl;
+                const int ld = ST ? TX : N;
+                float2 u[T][N2];
+#pragma unroll
+                for (int i = 0; i < T; ++i)
+#pragma unroll
+                    for (int n2 = 0; n2 < N2; ++n2) {
+                        const int row = j + N2 * i + N1 * n2 - y0;
+                        u[i][n2] = row >= 0 && row < ny ? r[(size_t)row * ld] : make_float2(0.f, 0.f);
+                    }
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    dft_reg<N2>(u[i]);
+                    const int n1 = j + N2 * i;
+#pragma unroll
+                    for (int k2 = 0; k2 < N2; ++k2)
+                        y[((p * N1 + n1) * N2 + k2) * TX + xl] = cmul(u[i][bit_reverse(k2, L2)], tw[k2 * N1 + n1]);
+                }
+            }
+            __syncthreads();
+            float2* own = y + (size_t)j * TX + xl;  // this thread's k2 = j, stride N2 TX over n1
+            float2 zx[N1];
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) zx[n1] = own[n1 * N2 * TX];
+            dft_reg<N1>(zx);
+            if (P == 1) {
+#pragma unroll
+                for (int k1 = 0; k1 < N1; ++k1) {
+                    const float2 X = zx[bit_reverse(k1, L1)];
+                    add_products<1>(X, X, xx[k1], yy[0], rxy[0], ixy[0]);
+                }
+            } else {
+                if (!kKeep) {
+#pragma unroll
+                    for (int k1 = 0; k1 < N1; ++k1) own[k1 * N2 * TX] = zx[bit_reverse(k1, L1)];
+                }
+                float2 zy[N1];
+#pragma unroll
+                for (int n1 = 0; n1 < N1; ++n1) zy[n1] = own[(N1 + n1) * N2 * TX];
+                dft_reg<N1>(zy);
+#pragma unroll
+                for (int k1 = 0; k1 < N1; ++k1) {
+                    const float2 X = kKeep ? zx[bit_reverse(k1, L1)] : own[k1 * N2 * TX];
+                    constexpr int m = P == 2 ? 1 : 0;
+                    add_products<P>(X, zy[bit_reverse(k1, L1)], xx[k1], yy[m * k1], rxy[m * k1], ixy[m * k1]);
+                }
+            }
+        }
+        store(target, add);
+        clear();
+        add = end ? accumulate != 0 : true;
+    }
+    if (ST) cp_async_wait<0>();
+    if (sub == 0 && ta >= tb) store(image(ta), add);  // no frames: zeros
+}
+
+// out (+)= the slices' partial sums, in slice order
+__global__ void __launch_bounds__(kThreads) k_plain_sum(const float4* __restrict__ partial, size_t n4, int S,
+                                                        float4* __restrict__ out, int accumulate)
+{
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n4; i += (size_t)gridDim.x * kThreads) {
+        float4 a = partial[i];
+        for (int k = 1; k < S; ++k) {
+            const float4 v = partial[k * n4 + i];
+            a = make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w);
+        }
+        if (accumulate) {
+            const float4 o = out[i];
+            a = make_float4(a.x + o.x, a.y + o.y, a.z + o.z, a.w + o.w);
+        }
+        out[i] = a;
+    }
+}
+
+// the register-FFT kernels of one N, number of pols and form of the frames and weights
 struct RegFft {
-    void (*rows)(float2*, size_t, const float2*);
-    void (*cols)(float2*, const float2*);
-    int rows_per_cta, col_tile, col_threads;
-    size_t rows_smem, cols_smem;
+    void (*rows)(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
+                 const float4*, int, int, int, const float2*, float2*);
+    void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int);
+    int col_tile, col_threads;
+    size_t rows_fft, rows_cells;  // rows_cells: per box column, what a block gathers per batch
+    size_t cols_smem, cols_row;   // cols_row: per box row, the staged frames
 };
 
-template <int N1, int N2>
-RegFft reg_fft()
+template <int N1, int N2, int P>
+RegFft reg_fft_p(bool staged, bool cplx)
 {
-    constexpr int N = N1 * N2, TX = (N2 <= 8 ? 32 : 16) < N ? (N2 <= 8 ? 32 : 16) : N;
-    return {k_plain_fft_rows<N1, N2>, k_plain_fft_cols<N1, N2, TX>, kRegThreads / N2, TX, TX * N2,
-            sizeof(float2) * ((size_t)N + (size_t)(kRegThreads / N2) * N2 * (N1 + 1)),
-            sizeof(float2) * ((size_t)N + (size_t)N * TX)};
+    constexpr int N = N1 * N2;
+    // 128 threads a block (fewer for the smallest grids): four to eight blocks an SM hide the barriers
+    constexpr int TX = 128 / N2 < N ? 128 / N2 : N;
+    RegFft f{};
+    f.rows = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true> : k_plain_rows<N1, N2, P, true, false>)
+                    : (cplx ? k_plain_rows<N1, N2, P, false, true> : k_plain_rows<N1, N2, P, false, false>);
+    f.cols = k_plain_cols<N1, N2, TX, P>;
+    f.col_tile = TX;
+    f.col_threads = TX * N2;
+    f.rows_fft = rows_fft_smem<N1, N2>();
+    f.rows_cells = sizeof(float2) * (kRowThreads / N2);  // F P YR rows
+    f.cols_smem = sizeof(float2) * ((size_t)N + (size_t)P * N * TX);
+    f.cols_row = sizeof(float2) * (size_t)col_stages(N) * P * TX;
+    return f;
 }
 
-// N = 2^logN, 8 <= N <= 512
-RegFft reg_fft_for(int logN)
+template <int N1, int N2>
+RegFft reg_fft(int P, bool staged, bool cplx)
 {
-    switch (logN) {
-        case 3: return reg_fft<4, 2>();
-        case 4: return reg_fft<4, 4>();
-        case 5: return reg_fft<8, 4>();
-        case 6: return reg_fft<8, 8>();
-        case 7: return reg_fft<16, 8>();
-        case 8: return reg_fft<16, 16>();
-        default: return reg_fft<32, 16>();
+    return P == 2 ? reg_fft_p<N1, N2, 2>(staged, cplx) : reg_fft_p<N1, N2, 1>(staged, cplx);
+}
+
+// Frames as staged FP32 samples (as many bytes as fit beside the FFT in a third of an SM), else as
+// bytes in shared memory, else read through L1.
+enum FrameForm { kFrameStaged, kFrameBytes, kFrameGlobal };
+
+// N = 2^logN, 8 <= N <= 512
+RegFft reg_fft_for(const epic_plan_s* p, bool staged)
+{
+    const bool cplx = p->gcf.kind != EPIC_GCF_GAUSSIAN;
+    switch (p->logN) {
+        case 3: return reg_fft<4, 2>(p->P, staged, cplx);
+        case 4: return reg_fft<4, 4>(p->P, staged, cplx);
+        case 5: return reg_fft<8, 4>(p->P, staged, cplx);
+        case 6: return reg_fft<8, 8>(p->P, staged, cplx);
+        case 7: return reg_fft<16, 8>(p->P, staged, cplx);
+        case 8: return reg_fft<16, 16>(p->P, staged, cplx);
+        default: return reg_fft<32, 16>(p->P, staged, cplx);
     }
+}
+
+size_t rows_base_smem(const epic_plan_s* p, const RegFft& f)
+{
+    return f.rows_fft + f.rows_cells * rows_ld(std::min(p->box_max_x, p->N));
+}
+
+size_t cols_smem_for(const epic_plan_s* p, const RegFft& f)
+{
+    return f.cols_smem + f.cols_row * std::min(p->box_max_y, p->N);
+}
+
+size_t frame_smem(const epic_plan_s* p, FrameForm form)
+{
+    const size_t fb = (size_t)p->A * p->P * (p->bits / 4);
+    if (form == kFrameStaged) return kRowFrames * sizeof(float2) * (size_t)p->A * p->P;
+    return form == kFrameBytes ? kRowFrames * ((fb + 15) & ~(size_t)15) : 0;
+}
+
+FrameForm frame_form(const epic_plan_s* p)
+{
+    const size_t base = rows_base_smem(p, reg_fft_for(p, true)), lim = (size_t)p->smem_optin;
+    if (base + frame_smem(p, kFrameStaged) <= lim) return kFrameStaged;
+    return base + frame_smem(p, kFrameBytes) <= lim ? kFrameBytes : kFrameGlobal;
+}
+
+// Slices of a chunk's frames for k_plain_cols: the number that loses least to the last wave -- of
+// blocks over the resident ones and over the SMs, a part-filled wave running faster per block, half
+// each -- and to the partial sums' traffic beside the rows'.  One for the LWA station's 1024 tiles
+// (6.1 ms a block; 6.8 in three slices), nine for the 64 tiles of the one-channel 512 x 512 station
+// (1.65 ms; 1.84 in four, 3.4 in two).
+int col_slices(const epic_plan_s* p, const RegFft& f, int nt, int slots)
+{
+    const double B = (double)(p->N / f.col_tile) * p->C;
+    const double img = sizeof(float) * (double)p->C * p->nprod * p->N * p->N;
+    const double rows = sizeof(float2) * (double)nt * p->C * p->P * p->box_max_y * p->N;
+    int best = 1;
+    double cost = 1e30;
+    for (int S = 1; S <= 16 && S <= std::max(1, nt / 4); ++S) {
+        const double w = B * S / slots, m = B * S / p->sm_count;
+        const double k = 0.5 * std::ceil(w) / w + 0.5 * std::ceil(m) / m + (S > 1 && p->sub == 0 ? 2.0 * S * img / rows : 0.0);
+        if (k < cost - 1e-9) {
+            cost = k;
+            best = S;
+        }
+    }
+    return best;
 }
 
 // Zeros of the N x N planes (P of them, NN apart) outside the occupied box b =
@@ -394,11 +714,12 @@ size_t cols_smem(int N) { return sizeof(float2) * ((size_t)N / 2 + 2ull * col_ti
 
 }  // namespace
 
-// Time samples per chunk so that the chunk's grids take at most `budget` bytes
-// (at least one sample), and the grid buffer for them.
+// Time samples per chunk so that the chunk's rows (fft = 1: whole grids) take at most `budget`
+// bytes (at least one sample), and the buffer for them and for the slices' partial sums.
 epic_status plain_set_chunk(epic_plan_s* p, size_t budget)
 {
-    const size_t per_t = (size_t)p->C * p->P * p->N * p->N * sizeof(float2);
+    const int rows = p->plain_fft == 0 ? std::min(p->box_max_y, p->N) : p->N;
+    const size_t per_t = (size_t)p->C * p->P * rows * p->N * sizeof(float2);
     // at most 65,535 (sample, channel, pol) columns: the second grid dimension of the column FFT
     const size_t max_t = 65535 / ((size_t)p->C * p->P);
     int tcn = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>((size_t)p->max_time, max_t), budget / per_t));
@@ -407,37 +728,51 @@ epic_status plain_set_chunk(epic_plan_s* p, size_t budget)
         p->last_error = "plain path: sub_int x n_chan x n_pol exceeds 65,535";
         return EPIC_ERR_UNSUPPORTED;
     }
-    const size_t bytes = per_t * tcn;
-    p->chunk_budget = budget;
-    if (p->scratch && bytes == p->scratch_bytes) {
-        p->time_chunk = tcn;
-        return EPIC_OK;
+    size_t bytes = (per_t * tcn + 255) & ~(size_t)255;
+    int slices = 1;
+    if (p->plain_fft == 0) {
+        const RegFft f = reg_fft_for(p, frame_form(p) == kFrameStaged);
+        int occ = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)f.cols, f.col_threads, cols_smem_for(p, f));
+        if (e != cudaSuccess) return cuda_fail(p, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(k_plain_cols)");
+        slices = col_slices(p, f, tcn, std::max(1, occ) * p->sm_count);
+        if (p->sub == 0 && slices > 1) bytes += sizeof(float) * (size_t)slices * p->C * p->nprod * p->N * p->N;
     }
+    p->chunk_budget = budget;
+    p->plain_slices = slices;
+    p->time_chunk = tcn;
+    if (p->scratch && bytes == p->scratch_bytes) return EPIC_OK;
     cudaFree(p->scratch);
     p->scratch = nullptr;
     p->scratch_bytes = 0;
     cudaError_t e = cudaMalloc(&p->scratch, bytes);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaMalloc(plain grid buffer)");
     p->scratch_bytes = bytes;
-    p->time_chunk = tcn;
     return EPIC_OK;
 }
 
-// FFT kernels of the plain path: 0 register two-pass, 1 shared-memory Stockham
+// Form of the plain path: 0 two kernels with register two-pass transforms, 1 four kernels with
+// shared-memory Stockham transforms
 epic_status plain_set_fft(epic_plan_s* p, int v)
 {
     if (v != 0 && v != 1) {
         p->last_error = "plain path: FFT form must be 0 or 1";
         return EPIC_ERR_INVALID_ARG;
     }
+    if (v == p->plain_fft) return EPIC_OK;
+    const int old = p->plain_fft;
     p->plain_fft = v;
-    return EPIC_OK;
+    epic_status st = plain_set_chunk(p, p->chunk_budget);  // the chunk's buffer holds other rows
+    if (st != EPIC_OK) {
+        p->plain_fft = old;
+        plain_set_chunk(p, p->chunk_budget);
+    }
+    return st;
 }
 
 epic_status plain_setup(epic_plan_s* p)
 {
-    epic_status st = plain_set_chunk(p, kGridBudget);
-    if (st != EPIC_OK) return st;
+    p->plain_fft = 0;
     cudaError_t e = cudaSuccess;
     const size_t sg = sizeof(float2) * (size_t)p->A * p->P;
     if (sg > 48 * 1024 && (int)sg <= p->smem_optin) {  // larger frames use k_plain_grid_g
@@ -448,16 +783,16 @@ epic_status plain_setup(epic_plan_s* p)
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_fft_rows_smem)");
     e = allow_max_smem((const void*)k_plain_fft_cols_smem, p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_fft_cols_smem)");
-    const RegFft rf = reg_fft_for(p->logN);
-    if (rf.rows_smem > (size_t)p->smem_optin || rf.cols_smem > (size_t)p->smem_optin) {
+    const RegFft rf = reg_fft_for(p, frame_form(p) == kFrameStaged);
+    if (rows_base_smem(p, rf) > (size_t)p->smem_optin || cols_smem_for(p, rf) > (size_t)p->smem_optin) {
         p->last_error = "plain path: FFT shared memory exceeds the device limit";
         return EPIC_ERR_UNSUPPORTED;
     }
     e = allow_max_smem((const void*)rf.rows, p->smem_optin);
-    if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_fft_rows)");
+    if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_rows)");
     e = allow_max_smem((const void*)rf.cols, p->smem_optin);
-    if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_fft_cols)");
-    return EPIC_OK;
+    if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_cols)");
+    return plain_set_chunk(p, kGridBudget);
 }
 
 epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s, float* out, bool accumulate)
@@ -468,26 +803,45 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
     const int bits = p->bits;
     for (int t0 = 0; t0 < T; t0 += p->time_chunk) {
         const int nt = std::min(p->time_chunk, T - t0);
-        ev_begin(p, "k_plain_grid", s);
-        if ((int)sg <= p->smem_optin)
-            k_plain_grid<<<dim3(nt, C), kThreads, sg, s>>>(volt, t0, C, A, P, N, bits, p->dt.box, p->dt.cell_off,
-                                                           p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, grid);
-        else
-            k_plain_grid_g<<<dim3(nt, C), kThreads, 0, s>>>(volt, t0, C, A, P, N, bits, p->dt.box, p->dt.cell_off,
-                                                            p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, grid);
-        ev_end(p, s);
-        const size_t n_rows = (size_t)nt * C * P * N;
+        const int acc = (accumulate || (t0 > 0 && p->sub == 0)) ? 1 : 0;
         if (p->plain_fft == 0) {
-            const RegFft rf = reg_fft_for(p->logN);
-            ev_begin(p, "k_plain_fft_rows", s);
-            rf.rows<<<(unsigned)((n_rows + rf.rows_per_cta - 1) / rf.rows_per_cta), kRegThreads, rf.rows_smem, s>>>(
-                grid, n_rows, p->dt.twiddle);
+            const FrameForm form = frame_form(p);
+            const RegFft rf = reg_fft_for(p, form == kFrameStaged);
+            const int ny_max = std::min(p->box_max_y, N);
+            ev_begin(p, "k_plain_rows", s);
+            rf.rows<<<dim3((nt + kRowFrames - 1) / kRowFrames, C), kRowThreads, rows_base_smem(p, rf) + frame_smem(p, form), s>>>(
+                volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off, p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w,
+                p->dt.jones, form == kFrameBytes ? 1 : 0, rows_ld(std::min(p->box_max_x, N)), ny_max, p->dt.twiddle, grid);
             ev_end(p, s);
-            ev_begin(p, "k_plain_fft_cols", s);
-            rf.cols<<<dim3(N / rf.col_tile, (unsigned)((size_t)nt * C * P)), rf.col_threads, rf.cols_smem, s>>>(
-                grid, p->dt.twiddle);
+            // slices of whole intervals, or of at least four frames; the same for every chunk of the call,
+            // whose partial sums add up over the chunks
+            const int S = std::max(1, std::min(p->plain_slices, p->sub > 0 ? nt / p->sub : std::min(p->time_chunk, T) / 4));
+            float* partial = nullptr;
+            if (S > 1 && p->sub == 0)
+                partial = reinterpret_cast<float*>(
+                    (uint8_t*)p->scratch + ((sizeof(float2) * (size_t)p->time_chunk * C * P * ny_max * N + 255) & ~(size_t)255));
+            ev_begin(p, "k_plain_cols", s);
+            rf.cols<<<dim3(N / rf.col_tile, C, S), rf.col_threads, cols_smem_for(p, rf), s>>>(
+                grid, nt, C, ny_max, p->dt.box, p->dt.twiddle, out, partial, partial ? t0 > 0 : acc, p->sub,
+                p->sub > 0 ? t0 / p->sub : 0);
             ev_end(p, s);
+            if (partial && t0 + nt == T) {
+                const size_t n4 = (size_t)C * p->nprod * N * N / 4;
+                ev_begin(p, "k_plain_sum", s);
+                k_plain_sum<<<(unsigned)std::min<size_t>((n4 + kThreads - 1) / kThreads, 8 * (size_t)p->sm_count), kThreads, 0, s>>>(
+                    reinterpret_cast<const float4*>(partial), n4, S, reinterpret_cast<float4*>(out), accumulate ? 1 : 0);
+                ev_end(p, s);
+            }
         } else {
+            ev_begin(p, "k_plain_grid", s);
+            if ((int)sg <= p->smem_optin)
+                k_plain_grid<<<dim3(nt, C), kThreads, sg, s>>>(volt, t0, C, A, P, N, bits, p->dt.box, p->dt.cell_off,
+                                                               p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, grid);
+            else
+                k_plain_grid_g<<<dim3(nt, C), kThreads, 0, s>>>(volt, t0, C, A, P, N, bits, p->dt.box, p->dt.cell_off,
+                                                                p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, grid);
+            ev_end(p, s);
+            const size_t n_rows = (size_t)nt * C * P * N;
             const int rpc = rows_per_cta_for(N);
             ev_begin(p, "k_plain_fft_rows_smem", s);
             k_plain_fft_rows_smem<<<(unsigned)((n_rows + rpc - 1) / rpc), kThreads, rows_smem(N), s>>>(
@@ -497,12 +851,11 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             k_plain_fft_cols_smem<<<dim3(N / col_tile_for(N), (unsigned)((size_t)nt * C * P)), kThreads,
                                     cols_smem(N), s>>>(grid, p->logN, col_tile_for(N), p->dt.twiddle);
             ev_end(p, s);
+            ev_begin(p, "k_plain_sqacc", s);
+            k_plain_sqacc<<<dim3((unsigned)(((size_t)N * N + kThreads - 1) / kThreads), C), kThreads, 0, s>>>(
+                grid, nt, C, P, N, out, acc, p->sub, p->sub > 0 ? t0 / p->sub : 0);
+            ev_end(p, s);
         }
-        ev_begin(p, "k_plain_sqacc", s);
-        k_plain_sqacc<<<dim3((unsigned)(((size_t)N * N + kThreads - 1) / kThreads), C), kThreads, 0, s>>>(
-            grid, nt, C, P, N, out, (accumulate || (t0 > 0 && p->sub == 0)) ? 1 : 0, p->sub,
-            p->sub > 0 ? t0 / p->sub : 0);
-        ev_end(p, s);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(p, e, "plain path launch");
     }
