@@ -133,7 +133,7 @@ struct MmaArgs {
     int iv0;                    // k_dftgemm_ws3: image set of the chunk's first sample
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
-    int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..4)
+    int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..6)
     const long long* wcum;      // k_dftgemm_ws3<true>: [C + 1] prefix sums of the channels' item costs per frame
     const int* item_order;      // k_dftgemm_ws3<false>: per channel group (from c0 ipc), items in the order dealt to blocks
 };
@@ -2133,7 +2133,7 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 // its last part is in.  Stage 2 and D2 come in two halves of 32 kx, so that the chain of one
 // half runs while epilogue 2 reads the other.  Sub-frames u = t H + h are counted through all
 // the items of a block: no barrier separates items, only the operand tables wait (A1 for the
-// last S1 of the item before, A2 for its last S2).  NB (2..4) tile-part buffers:
+// last S1 of the item before, A2 for its last S2).  NB (2..6) tile-part buffers:
 //   copy thread (warp 2, lane 0), per sub-frame u:
 //     wait tile_free(u-NB) -> copy tile part u -> tile_full
 //   stage-1 issuer (warp 1, lane 0), per sub-frame u:
@@ -2150,10 +2150,10 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 // epilogue-2 x 192: an epilogue-2 thread holds 32 pixels (128 sums) and 48 registers of
 // TMEM loads in flight.
 constexpr int kWs3Threads = 512;
-constexpr int kWs3CtlRegs = 72, kWs3E1Regs = 88, kWs3E2Regs = 176;
+constexpr int kWs3CtlRegs = 64, kWs3E1Regs = 96, kWs3E2Regs = 176;
 static_assert(kWs3CtlRegs + kWs3E1Regs + 2 * kWs3E2Regs == 4 * 128, "setmaxnreg shares are the launch's registers");
 constexpr int kWs3MaxBlocks = 256;  // blocks per launch (one per SM) the split bookkeeping holds
-constexpr int kWs3MaxTileBufs = 4;  // tile-part buffers of k_dftgemm_ws3 (short row parts need more in flight)
+constexpr int kWs3MaxTileBufs = 6;  // tile-part buffers of k_dftgemm_ws3 (short row parts need more in flight)
 
 // x of lane 0: the same for the warp (a value every lane holds alike, but read from memory)
 __device__ __forceinline__ int ws3_uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
@@ -2178,21 +2178,20 @@ __device__ __forceinline__ bool ws3_wait(uint64_t* bar, uint32_t& ph, int slot)
 }
 
 // One warp's share of epilogue 1: lanes = 32 kx of one (half, re | im) quarter of D1, NYC chunks
-// of 8 columns per pol -> the 16-byte chunks of B2 rows row (real part of E) and row + 32
-// (imaginary part).  B2's K order interleaves the parts: chunk 2 j holds rows 8 j .. 8 j + 7 of
-// the first part of [Hr | -Hi] or [Hi | Hr], chunk 2 j + 1 those of the second, so that the four
-// chunks of a batch sit at fixed offsets of one 64-wide K panel.  With one warp per SM
-// sub-partition the step is bound by its instructions, and a taken branch costs about 20 cycles
-// against 1.5 for straight-line code, so it is unrolled for each NYC.  The next batch is loaded
-// while the last one is stored; d1_free is signalled as soon as the last load is in registers.
-template <int NYC>
-__device__ __forceinline__ void ws3_epilogue1(uint32_t taddr, int P, bool imw, int lane, uint32_t b2, int row, int R2,
-                                              uint64_t* d1_free)
+// of 8 columns per pol -> 16-byte chunks of B2 rows row + 64 p (real part of E) and 32 below
+// (imaginary part).  B2's K order interleaves the parts: chunk 2 j holds rows 8 j .. 8 j + 7 of the
+// first part of [Hr | -Hi] or [Hi | Hr], chunk 2 j + 1 those of the second; it lies chunk by chunk,
+// 16 bytes a row (no swizzle, no padding: a warp's store is 512 contiguous bytes, and an LWA
+// station's buffer is 48 KB where 64-wide swizzled panels took 64, room for a third tile buffer).
+// With one warp per SM sub-partition the step is bound by its instructions, and a taken branch
+// costs about 20 cycles against 1.5 for straight-line code, so it is unrolled for each NYC and part.
+// The next batch is loaded while the last one is stored; d1_free is signalled as soon as the last
+// load is in registers.
+template <int NYC, int IM>
+__device__ __forceinline__ void ws3_epilogue1(uint32_t taddr, int P, int lane, uint32_t b2, int row, uint64_t* d1_free)
 {
-    constexpr int NB = (NYC + 3) / 4;  // batches of up to 4 chunks (one K panel) per pol
-    const uint32_t panel = (uint32_t)R2 * 128, sg = imw ? 0x80008000u : 0u;
-    const uint32_t x7 = (uint32_t)(lane & 7) << 4;
-    const uint32_t d0 = b2 + (uint32_t)(row + lane) * 128, e0 = imw ? 16u : 0u;
+    constexpr int NB = (NYC + 3) / 4;        // batches of up to 4 chunks per pol
+    const uint32_t cb = (uint32_t)(128 * P) * 16;  // bytes of a chunk
     uint32_t r[32];
     auto load = [&](uint32_t ta, int n) {
         if (n == 4) tc::tmem_ld32(ta, r);
@@ -2205,8 +2204,10 @@ __device__ __forceinline__ void ws3_epilogue1(uint32_t taddr, int P, bool imw, i
     };
     constexpr int first = NYC < 4 ? NYC : 4;
     load(taddr, first);
+    uint32_t q = b2 + (uint32_t)(row + lane) * 16;
 #pragma unroll 1
-    for (int p = 0; p < P; ++p) {
+    for (int p = 0; p < P; ++p, q += 64 * 16) {
+        uint32_t q0 = IM ? q + cb : q, q1 = (IM ? q : q + cb) + 32 * 16;
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
             const int n = NYC - 4 * j < 4 ? NYC - 4 * j : 4;
@@ -2223,12 +2224,11 @@ __device__ __forceinline__ void ws3_epilogue1(uint32_t taddr, int P, bool imw, i
                 __syncwarp();
                 if (lane == 0) mbar_arrive(d1_free);
             }
-            const uint32_t q = d0 + p * (64 * 128) + j * panel;
 #pragma unroll
-            for (int i = 0; i < n; ++i) {
-                const uint32_t lo = q + ((uint32_t)(32 * i) ^ x7 ^ e0), hi = q + ((uint32_t)(32 * i + 16) ^ x7 ^ e0);
-                tc::st_shared_v4(lo, h[4 * i] ^ sg, h[4 * i + 1] ^ sg, h[4 * i + 2] ^ sg, h[4 * i + 3] ^ sg);
-                tc::st_shared_v4(hi + 32 * 128, h[4 * i], h[4 * i + 1], h[4 * i + 2], h[4 * i + 3]);
+            for (int i = 0; i < n; ++i, q0 += 2 * cb, q1 += 2 * cb) {
+                constexpr uint32_t sg = IM ? 0x80008000u : 0u;  // Hr and -Hi in the real part's rows
+                tc::st_shared_v4(q0, h[4 * i] ^ sg, h[4 * i + 1] ^ sg, h[4 * i + 2] ^ sg, h[4 * i + 3] ^ sg);
+                tc::st_shared_v4(q1, h[4 * i], h[4 * i + 1], h[4 * i + 2], h[4 * i + 3]);
             }
         }
     }
@@ -2543,7 +2543,7 @@ __device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsign
                                        uint32_t& ph_e, uint32_t d2, uint32_t a2, int P, uint32_t b2, uint32_t b2_bytes,
                                        uint32_t lead)
 {
-    const uint32_t id2 = tc::idesc_f16_f32(128, 64 * P), pb = (uint32_t)(128 * P) * 8;
+    const uint32_t id2 = tc::idesc_f16_f32(128, 64 * P), pb = (uint32_t)(128 * P) * 2;  // a K step of B2, 16-byte units
 #pragma unroll 1
     for (int t = 0; t < nt; ++t) {
 #pragma unroll 1
@@ -2555,15 +2555,15 @@ __device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsign
             for (int f = 0; f < 2; ++f) {
                 if (h == 0 && any && !ws3_wait(&m.d2_empty[f], ph_e, f)) return false;
                 tc::fence_after_sync();
-                const uint32_t db = tc::desc_sw128_lo(b2 + sl * b2_bytes + 64 * P * 128 * f);
+                const uint32_t db = tc::desc_step_lo(b2 + sl * b2_bytes + 64 * P * 16 * f, 128 * P * 16);
                 const uint32_t d = d2 + 64 * P * f;
                 if (KS) {
 #pragma unroll
                     for (int k = 0; k < KS; ++k)
-                        tc::mma_f16_ta_lead(d, at + 8 * k, db + (k >> 2) * pb + (k & 3) * 2, id2, k > 0 || h > 0, lead);
+                        tc::mma_f16_ta_lead<tc::kDescStep128Hi>(d, at + 8 * k, db + k * pb, id2, k > 0 || h > 0, lead);
                 } else {
                     for (int k = 0; k < ks; ++k)
-                        tc::mma_f16_ta_lead(d, at + 8 * k, db + (k >> 2) * pb + (k & 3) * 2, id2, k > 0 || h > 0, lead);
+                        tc::mma_f16_ta_lead<tc::kDescStep128Hi>(d, at + 8 * k, db + k * pb, id2, k > 0 || h > 0, lead);
                 }
                 if (h == H - 1) tc::mma_commit_lead(&m.d2_full[f], lead);
             }
@@ -2575,10 +2575,10 @@ __device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsign
 }
 
 // Epilogue 1 of NU sub-frames.  held: B2 slots whose S2 was not waited for yet.
-template <int NYC>
+template <int NYC, int IM>
 __device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t& ph_d1, uint32_t& ph_bf, uint32_t& held,
-                                       uint32_t taddr, uint32_t d1_cols, int P, bool imw, int lane, uint32_t b2,
-                                       uint32_t b2_bytes, int row)
+                                       uint32_t taddr, uint32_t d1_cols, int P, int lane, uint32_t b2, uint32_t b2_bytes,
+                                       int row)
 {
 #pragma unroll 1
     for (const unsigned end = u + NU; u != end; ++u) {
@@ -2587,7 +2587,7 @@ __device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t
         if (((held >> sl) & 1u) && !ws3_wait(&m.b2_free[sl], ph_bf, sl)) return false;
         held |= 1u << sl;
         tc::fence_after_sync();
-        ws3_epilogue1<NYC>(taddr + sl * d1_cols, P, imw, lane, b2 + sl * b2_bytes, row, 128 * P, &m.d1_free[sl]);
+        ws3_epilogue1<NYC, IM>(taddr + sl * d1_cols, P, lane, b2 + sl * b2_bytes, row, &m.d1_free[sl]);
         tc::fence_proxy_async();
         tc::fence_before_sync();
         __syncwarp();
@@ -2819,7 +2819,13 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 if (lane == 0) mbar_arrive(&m.a2_full);
             }
             switch (nyc) {  // P nyh <= 256 columns and two slots of D1 beside A2: nyc <= 15
-#define EPIC_E1(n)                                                                                                    case n:                                                                                                               good = ws3_e1<n>(m, NU, u, ph_d1, ph_bf, held, tmem + lane_base, a.d1_cols, P, (q4 >> 1) != 0, lane, b2a,                          a.b2_bytes, 64 * P * (q4 & 1));                                                                  break;
+#define EPIC_E1(n)                                                                                                  \
+    case n:                                                                                                         \
+        good = q4 >> 1 ? ws3_e1<n, 1>(m, NU, u, ph_d1, ph_bf, held, tmem + lane_base, a.d1_cols, P, lane, b2a,       \
+                                      a.b2_bytes, 64 * P * (q4 & 1))                                                \
+                       : ws3_e1<n, 0>(m, NU, u, ph_d1, ph_bf, held, tmem + lane_base, a.d1_cols, P, lane, b2a,       \
+                                      a.b2_bytes, 64 * P * (q4 & 1));                                               \
+        break;
                 EPIC_KS_CASES(EPIC_E1)
 #undef EPIC_E1
                 default: good = false;
@@ -2846,7 +2852,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
 // chunk) take at most `budget` bytes, and the tile buffer for them.
 epic_status dftgemm_set_kernel(epic_plan_s* p, int variant)
 {
-    if (variant < 1 || variant > 3 || !p->tc.ws || ((p->sub > 0 || p->tc.parts) && variant != 3) ||
+    if (variant < 1 || variant > 3 || !p->tc.ws || ((p->sub > 0 || !p->tc.ws_old) && variant != 3) ||
         (variant == 3 && p->sm_count > kWs3MaxBlocks))
         return EPIC_ERR_UNSUPPORTED;
     p->tc.ws_variant = variant;
@@ -3341,25 +3347,30 @@ epic_status dftgemm_setup(epic_plan_s* p)
         }
         if (!ok || 2 * dmax + a2max > 256) continue;
         const size_t b1p = align_up(2ull * dmax * K1max, 1024);
-        const size_t b2w = align_up(2ull * 2 * 64 * P * pad64(2 * nyh_max), 1024);
-        // as many tile-part buffers (2..4) as fit: row parts are short steps, so more copies
-        // must be in flight to cover their latency
-        int nbt = 4;
-        auto need_for = [&](int nb) { return align_up(256ull * K1max, 1024) + nb * b1p + 2 * b2w; };
-        while (nbt > 2 && need_for(nbt) > limit) --nbt;
-        const size_t need_ws = need_for(nbt);
+        const size_t a1p = align_up(256ull * K1max, 1024);
+        const size_t b2w = align_up(2ull * 128 * P * 2 * nyh_max, 1024);
+        // as many tile-part buffers (2..6) as fit: a part's copy takes longer than its step
+        int nbt = kWs3MaxTileBufs;
+        while (nbt > 2 && a1p + nbt * b1p + 2 * b2w > limit) --nbt;
+        const size_t need_ws = a1p + nbt * b1p + 2 * b2w;
         if (need_ws > limit) continue;
         p->tc.ws = true;
         p->tc.parts = split;
         p->tc.tbox_h = tb;
         p->tc.nbt = nbt;
         p->tc.sA1 = 0;
-        p->tc.sB1 = (unsigned)align_up(256ull * K1max, 1024);
-        p->tc.sB2 = (unsigned)(p->tc.sB1 + nbt * b1p);
+        p->tc.sB1 = (unsigned)a1p;
         p->tc.b1_bytes = (unsigned)b1p;
-        p->tc.b2_bytes = (unsigned)b2w;
         p->tc.d1_cols = dmax;
-        p->tc.smem = (int)(need_ws + 1024);
+        p->tc.ws3_sB2 = (unsigned)(a1p + nbt * b1p);
+        p->tc.ws3_b2 = (unsigned)b2w;
+        p->tc.ws3_smem = (int)(need_ws + 1024);
+        // the older variants: two tile buffers, B2 with both parts' rows, one part per channel
+        const size_t b2o = align_up(2ull * 2 * 64 * P * pad64(2 * nyh_max), 1024), need_old = a1p + 2 * b1p + 2 * b2o;
+        p->tc.ws_old = !split && need_old <= limit;
+        p->tc.sB2 = (unsigned)(a1p + 2 * b1p);
+        p->tc.b2_bytes = (unsigned)b2o;
+        p->tc.smem = (int)std::max<size_t>(need_old + 1024, 120 * 1024);  // alone on its SM: it takes all of TMEM
     }
     if (!p->tc.ws)  // one part per channel for the other kernels' tile layout
         for (int c = 0; c < C; ++c) p->tc.tbox_h[c] = make_int4(p->box[c].ny, 1, p->box[c].ny, 0);
@@ -3650,7 +3661,7 @@ epic_status dftgemm_setup(epic_plan_s* p)
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<true>, p->smem_optin);
     p->tc.ws_variant = p->tc.ws ? 3 : 0;
     if (p->tc.ws && p->sm_count > kWs3MaxBlocks) p->tc.ws_variant = 1;
-    if (p->tc.parts && p->tc.ws_variant != 3) {
+    if (p->tc.ws && !p->tc.ws_old && p->tc.ws_variant != 3) {
         p->last_error = "tensor path: an occupied grid this tall needs the control-warp kernel";
         return EPIC_ERR_UNSUPPORTED;
     }
@@ -3858,11 +3869,13 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                 if (p->tc.ws_variant == 3) {
                     a.partial = p->tc.partial;
                     a.counters = p->tc.counters;
+                    a.sB2 = p->tc.ws3_sB2;
+                    a.b2_bytes = p->tc.ws3_b2;
                     if (p->sub == 0 && (p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
-                        k_dftgemm_ws3<true><<<p->sm_count, kWs3Threads, p->tc.smem, s>>>(a);
+                        k_dftgemm_ws3<true><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
                     else
-                        k_dftgemm_ws3<false><<<grid, kWs3Threads, p->tc.smem, s>>>(a);
+                        k_dftgemm_ws3<false><<<grid, kWs3Threads, p->tc.ws3_smem, s>>>(a);
                 }
                 else if (p->tc.ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);
                 else k_dftgemm_ws<0><<<grid, kWsThreads, p->tc.smem, s>>>(a);

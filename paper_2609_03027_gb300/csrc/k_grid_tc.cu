@@ -227,8 +227,8 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
                         if (!good) break;
                         ph_v ^= 1u << vs;
                         tc::fence_after_sync();
-                        const uint32_t wa = tc::desc_step128_lo(sW + ws * kGtWBytes);
-                        const uint32_t va = tc::desc_step128_lo(sV + vs * VB);
+                        const uint32_t wa = tc::desc_step_lo(sW + ws * kGtWBytes, 2048);
+                        const uint32_t va = tc::desc_step_lo(sV + vs * VB, 2048);
                         tc::mma_f16_lead<tc::kDescStep128Hi>(d, wa, va, id, s > 0, lead);
                         tc::mma_f16_lead<tc::kDescStep128Hi>(d + 128, wa + (4096 >> 4), va, id, s > 0, lead);
                         tc::mma_f16_lead<tc::kDescStep128Hi>(d, wa + (8192 >> 4), va, id, 1, lead);

@@ -189,9 +189,9 @@ __device__ __forceinline__ uint32_t elect_one()
 // Operand descriptors by their low words: the high word of smem_desc_sw128 is a constant.
 __device__ __forceinline__ uint32_t desc_sw128_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
 constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-// The same for an operand of 128 rows x 16 halves without swizzle: two K-major columns of 16-byte
-// row chunks, 2048 bytes apart (8 rows x 16 bytes a core matrix, 128 bytes to the next 8 rows).
-__device__ __forceinline__ uint32_t desc_step128_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | ((2048u >> 4) << 16); }
+// The same for a K step (16 halves) of an operand without swizzle: two columns of 16-byte row
+// chunks, `col` bytes apart (8 rows x 16 bytes a core matrix, 128 bytes to the next 8 rows).
+__device__ __forceinline__ uint32_t desc_step_lo(uint32_t saddr, uint32_t col) { return ((saddr >> 4) & 0x3FFFu) | ((col >> 4) << 16); }
 constexpr uint32_t kDescStep128Hi = (128u >> 4) | (1u << 14);
 template <uint32_t HI = kDescSw128Hi>
 __device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
@@ -207,6 +207,7 @@ __device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint
         "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(HI)
         : "memory");
 }
+template <uint32_t HI = kDescSw128Hi>
 __device__ __forceinline__ void mma_f16_ta_lead(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t idesc,
                                                 uint32_t accumulate, uint32_t lead)
 {
@@ -216,7 +217,7 @@ __device__ __forceinline__ void mma_f16_ta_lead(uint32_t d_tmem, uint32_t a_tmem
         "setp.ne.b32 q, %5, 0;\n\t"
         "mov.b64 y, {%2, %6};\n\t"
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], y, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(kDescSw128Hi)
+        "r"(a_tmem), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(HI)
         : "memory");
 }
 __device__ __forceinline__ void mma_commit_lead(uint64_t* bar, uint32_t lead)
