@@ -133,6 +133,7 @@ struct MmaArgs {
     int iv0;                    // k_dftgemm_ws3: image set of the chunk's first sample
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
+    int share;                  // k_dftgemm_ws3<true>: blocks that walk items of one channel side by side
     int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..6)
     const long long* wcum;      // k_dftgemm_ws3<true>: [C + 1] prefix sums of the channels' item costs per frame
     const int* item_order;      // k_dftgemm_ws3<false>: per channel group (from c0 ipc), items in the order dealt to blocks
@@ -2169,6 +2170,14 @@ __device__ __forceinline__ bool ws3_wait(uint64_t* bar, uint32_t parity)
     }
 }
 
+// Two barriers at once: both are polled before the one vote, which a step waits for anyway.
+__device__ __forceinline__ bool ws3_wait2(uint64_t* a, uint32_t pa, uint64_t* b, uint32_t pb)
+{
+    const uint32_t ra = tc::mbar_try_wait(a, pa), rb = tc::mbar_try_wait(b, pb);
+    if (__all_sync(0xffffffffu, ra & rb)) return true;
+    return ws3_wait(a, pa) && ws3_wait(b, pb);
+}
+
 // The same with the phase's parity in bit `slot` of ph, which flips when the phase is over.
 __device__ __forceinline__ bool ws3_wait(uint64_t* bar, uint32_t& ph, int slot)
 {
@@ -2332,18 +2341,19 @@ __device__ __forceinline__ void ws3_store_partial(float* slot, int pr, int tid2,
 
 // A split work item (equal shares) after this block stored its part to its slot: the block
 // that stores the item's last part -- counted on the item's counter -- adds all parts in block
-// order and writes (or adds) the images.  start: first unit of every block (shared memory,
+// order and writes (or adds) the images.  start: first unit of every block group (shared memory,
 // filled once per launch: searching the plan's weights here, on one thread, cost 40 us an
 // item).  Kept out of line so that the frame loop's register allocation does not carry it.
 __device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float* o, int nk, int tid2,
                                               const uint32_t* start, int* split_b)
 {
-    const uint32_t s0 = (uint32_t)item * (uint32_t)a.nt, s1 = s0 + (uint32_t)a.nt - 1;
+    const int Q = a.share, mine = item % Q;
+    const uint32_t s0 = (uint32_t)(item / Q) * (uint32_t)a.nt, s1 = s0 + (uint32_t)a.nt - 1;
     __threadfence();
     asm volatile("bar.sync 3, 256;" ::: "memory");
     if (tid2 == 0) {
-        const int G = gridDim.x;
-        auto owner = [&](uint32_t f) {  // the block whose range [start[b], start[b + 1]) holds f
+        const int G = gridDim.x / Q;
+        auto owner = [&](uint32_t f) {  // the block group whose range [start[b], start[b + 1]) holds f
             int lo = 0, hi = G;
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
@@ -2372,7 +2382,7 @@ __device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float*
             for (int b = b0; b <= b1; ++b) {
                 if (start[b] == start[b + 1]) continue;
                 const float4* q =
-                    reinterpret_cast<const float4*>(a.partial + (size_t)(2 * b + (s0 <= start[b] ? 0 : 1)) * 4 * 8192) +
+                    reinterpret_cast<const float4*>(a.partial + (size_t)(2 * (b * Q + mine) + (s0 <= start[b] ? 0 : 1)) * 4 * 8192) +
                     (size_t)8 * pr * 256 + tid2;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -2390,7 +2400,10 @@ __device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float*
 }
 
 // The segments (work item, first frame, frames) of a block: every role walks them alike.
-// SPLIT: the (item, frame) units [w, w1) in item-major order; else whole items.
+// SPLIT: the block group's (item group, frame) units [w, w1) in item-major order -- `share` blocks
+// walk `share` items of a channel side by side, so that a grid tile is read from HBM once and from
+// L2 by the others (apart, both items of an LWA channel read it from HBM: 6.3 GB a block at 5.7 TB/s,
+// the limit of the kernel) -- else whole items.
 struct Ws3Seg {
     int item, fs, nt;
 };
@@ -2400,7 +2413,7 @@ __device__ __forceinline__ bool ws3_next(const MmaArgs& a, int items, int it, lo
 {
     if (SPLIT) {
         if (w >= w1) return false;
-        s.item = (int)(w / a.nt);
+        s.item = (int)(w / a.nt) * a.share + blockIdx.x % a.share;
         s.fs = (int)(w % a.nt);
         s.nt = (int)min((long long)(a.nt - s.fs), w1 - w);
         w += s.nt;
@@ -2507,16 +2520,17 @@ struct Ws3Bars {
 
 // Stage 1: KS K steps of 16 from A1 and tile buffer b into D1[u & 1].
 template <int KS>
-__device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, int& b, int NB, uint32_t& ph_free,
-                                       uint32_t& ph_tile, uint32_t tmem, uint32_t d1_cols, uint32_t da, uint32_t b1,
+__device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, int& b, int NB, uint32_t& ph_tile,
+                                       uint32_t tmem, uint32_t d1_cols, uint32_t da, uint32_t b1,
                                        uint32_t b1_bytes, int N1, uint32_t lead)
 {
     const uint32_t id1 = tc::idesc_f16_f32(128, N1), pb = (uint32_t)N1 * 8;
 #pragma unroll 1
     for (const unsigned end = u + NU; u != end; ++u) {
         const int sl = u & 1;
-        if (u >= 2 && !ws3_wait(&m.d1_free[sl], ph_free, sl)) return false;  // E1(u-2) has read D1[sl]
-        if (!ws3_wait(&m.tile_full[b], ph_tile, b)) return false;
+        // E1(u-2) has read D1[sl] (a fresh barrier passes for the odd phase before its first)
+        if (!ws3_wait2(&m.tile_full[b], (ph_tile >> b) & 1u, &m.d1_free[sl], ((u >> 1) & 1u) ^ 1u)) return false;
+        ph_tile ^= 1u << b;
         tc::fence_after_sync();
         const uint32_t db = tc::desc_sw128_lo(b1 + b * b1_bytes);
         const uint32_t d = tmem + sl * d1_cols;
@@ -2539,8 +2553,7 @@ __device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, 
 
 // Stage 2: KS = nyh / 8 K steps from A2 (TMEM, part h at nyh words) and B2[u & 1] into both halves of D2.
 template <int KS>
-__device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsigned& u, bool& any, uint32_t& ph_b2,
-                                       uint32_t& ph_e, uint32_t d2, uint32_t a2, int P, uint32_t b2, uint32_t b2_bytes,
+__device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsigned& u, unsigned& fr, uint32_t d2, uint32_t a2, int P, uint32_t b2, uint32_t b2_bytes,
                                        uint32_t lead)
 {
     const uint32_t id2 = tc::idesc_f16_f32(128, 64 * P), pb = (uint32_t)(128 * P) * 2;  // a K step of B2, 16-byte units
@@ -2549,11 +2562,12 @@ __device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsign
 #pragma unroll 1
         for (int h = 0; h < H; ++h, ++u) {
             const int sl = u & 1;
-            if (!ws3_wait(&m.b2_full[sl], ph_b2, sl)) return false;
+            // E1(u) is done and, where a frame begins, E2 of the frame before has read half 0
+            if (!ws3_wait2(&m.b2_full[sl], (u >> 1) & 1u, &m.d2_empty[0], (fr & 1u) ^ 1u)) return false;
             const uint32_t at = a2 + h * 8 * ks;
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
-                if (h == 0 && any && !ws3_wait(&m.d2_empty[f], ph_e, f)) return false;
+                if (f == 1 && h == 0 && !ws3_wait(&m.d2_empty[1], (fr & 1u) ^ 1u)) return false;
                 tc::fence_after_sync();
                 const uint32_t db = tc::desc_step_lo(b2 + sl * b2_bytes + 64 * P * 16 * f, 128 * P * 16);
                 const uint32_t d = d2 + 64 * P * f;
@@ -2569,23 +2583,21 @@ __device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsign
             }
             tc::mma_commit_lead(&m.b2_free[sl], lead);  // S2(u) has read B2[sl]
         }
-        any = true;
+        ++fr;
     }
     return true;
 }
 
-// Epilogue 1 of NU sub-frames.  held: B2 slots whose S2 was not waited for yet.
+// Epilogue 1 of NU sub-frames.
 template <int NYC, int IM>
-__device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t& ph_d1, uint32_t& ph_bf, uint32_t& held,
-                                       uint32_t taddr, uint32_t d1_cols, int P, int lane, uint32_t b2, uint32_t b2_bytes,
+__device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t taddr, uint32_t d1_cols, int P, int lane, uint32_t b2, uint32_t b2_bytes,
                                        int row)
 {
 #pragma unroll 1
     for (const unsigned end = u + NU; u != end; ++u) {
         const int sl = u & 1;
-        if (!ws3_wait(&m.d1_full[sl], ph_d1, sl)) return false;
-        if (((held >> sl) & 1u) && !ws3_wait(&m.b2_free[sl], ph_bf, sl)) return false;
-        held |= 1u << sl;
+        // S1(u) is done and S2(u-2) has read B2[sl]
+        if (!ws3_wait2(&m.d1_full[sl], (u >> 1) & 1u, &m.b2_free[sl], ((u >> 1) & 1u) ^ 1u)) return false;
         tc::fence_after_sync();
         ws3_epilogue1<NYC, IM>(taddr + sl * d1_cols, P, lane, b2 + sl * b2_bytes, row, &m.d1_free[sl]);
         tc::fence_proxy_async();
@@ -2605,7 +2617,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     __shared__ Ws3Bars m;
     __shared__ uint32_t tmem_sh;
     __shared__ int err_sh;
-    __shared__ uint32_t start[SPLIT ? kWs3MaxBlocks + 1 : 1];  // first unit of every block
+    __shared__ uint32_t start[SPLIT ? kWs3MaxBlocks + 1 : 1];  // first unit of every block group
     __shared__ int split_b[2];  // blocks of a split item; the second is -1 unless this block completes it
     const int tid = threadIdx.x, warp = ws3_uni(tid >> 5), lane = tid & 31;
     if (warp == 0) {
@@ -2633,8 +2645,8 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     }
     const int ipc = a.n_kb * a.n_g, items = a.n_ch * ipc;  // items per channel, of the launch
     if (SPLIT)
-        for (int b = tid; b <= (int)gridDim.x; b += kWs3Threads)
-            start[b] = (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc, a.nt, b, gridDim.x);
+        for (int b = tid; b <= (int)(gridDim.x / a.share); b += kWs3Threads)
+            start[b] = (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt, b, gridDim.x / a.share);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -2644,10 +2656,10 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     const int P = a.P;
     const uint32_t a2col = 2u * a.d1_cols;
     const uint32_t b2a = tc::smem_u32(sbase + a.sB2);
-    // this block's share of the launch.  SPLIT: the (item, frame) units [wb0, wb1) in item-major
-    // order (items cut at share boundaries are summed by the block that stores their last part);
+    // this block's part of the launch.  SPLIT: its group's (item group, frame) units [wb0, wb1) in
+    // item-major order (items cut at range boundaries are summed by the block that stores their last part);
     // else whole items blockIdx.x, + gridDim.x, ...
-    const long long wb0 = SPLIT ? start[blockIdx.x] : 0, wb1 = SPLIT ? start[blockIdx.x + 1] : 0;
+    const long long wb0 = SPLIT ? start[blockIdx.x / a.share] : 0, wb1 = SPLIT ? start[blockIdx.x / a.share + 1] : 0;
     Ws3Seg s;
     long long w = wb0;
     bool good = true;
@@ -2717,7 +2729,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
         } else if (warp == 1) {  // stage 1: the whole warp in step, its leader issues
             const uint32_t lead = tc::elect_one();
             const uint32_t da = tc::desc_sw128_lo(tc::smem_u32(sA1));
-            uint32_t ph_free = 0, ph_tile = 0, ph_a = 0;
+            uint32_t ph_tile = 0, ph_a = 0;
             int b = 0;
             unsigned u = 0;  // sub-frames of all segments
             for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
@@ -2727,11 +2739,11 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 good = ws3_wait(&m.bar_a, ph_a, 0);
                 if (!good) break;
                 switch (ks) {
-#define EPIC_S1(n)                                                                                                   case n:                                                                                                              good = ws3_s1<n>(m, n, NU, u, b, NB, ph_free, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1),                          a.b1_bytes, N1, lead);                                                                          break;
+#define EPIC_S1(n)                                                                                                   case n:                                                                                                              good = ws3_s1<n>(m, n, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1),                          a.b1_bytes, N1, lead);                                                                          break;
                     EPIC_KS_CASES(EPIC_S1)
 #undef EPIC_S1
                     default:
-                        good = ws3_s1<0>(m, ks, NU, u, b, NB, ph_free, ph_tile, tmem, a.d1_cols, da,
+                        good = ws3_s1<0>(m, ks, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da,
                                          tc::smem_u32(sbase + a.sB1), a.b1_bytes, N1, lead);
                 }
             }
@@ -2742,20 +2754,19 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
             }
         } else if (warp == 0) {  // stage 2, likewise
             const uint32_t lead = tc::elect_one();
-            uint32_t ph_b2 = 0, ph_e = 0, ph_a2 = 0;
-            unsigned u = 0;
-            bool any = false;  // a frame was issued before
+            uint32_t ph_a2 = 0;
+            unsigned u = 0, fr = 0;  // sub-frames and frames of all segments
             for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
                 const int4 tp = a.tbox[a.c0 + s.item / ipc];
                 const int ks = ws3_uni(tp.x / 8), H = ws3_uni(tp.y), nt = ws3_uni(s.nt);
                 good = ws3_wait(&m.a2_full, ph_a2, 0);
                 if (!good) break;
                 switch (ks) {
-#define EPIC_S2(n)                                                                                                      case n:                                                                                                                 good = ws3_s2<n>(m, n, nt, H, u, any, ph_b2, ph_e, tmem + 256, tmem + a2col, P, b2a, a.b2_bytes, lead);              break;
+#define EPIC_S2(n)                                                                                                      case n:                                                                                                                 good = ws3_s2<n>(m, n, nt, H, u, fr, tmem + 256, tmem + a2col, P, b2a, a.b2_bytes, lead);              break;
                     EPIC_KS_CASES(EPIC_S2)
 #undef EPIC_S2
                     default:
-                        good = ws3_s2<0>(m, ks, nt, H, u, any, ph_b2, ph_e, tmem + 256, tmem + a2col, P, b2a,
+                        good = ws3_s2<0>(m, ks, nt, H, u, fr, tmem + 256, tmem + a2col, P, b2a,
                                          a.b2_bytes, lead);
                 }
             }
@@ -2769,20 +2780,20 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     } else if (warp < 8) {
         // ------------------------------------------------------------ epilogue 1
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWs3E1Regs) : "memory");
-        uint32_t ph_d1 = 0, ph_bf = 0, held = 0;
         const int q4 = warp & 3;
         const uint32_t lane_base = (uint32_t)(32 * q4) << 16;
         unsigned u = 0;
-        auto free_b2 = [&](int sl) -> bool {
-            if (!((held >> sl) & 1u)) return true;
-            held &= ~(1u << sl);
-            return ws3_wait(&m.b2_free[sl], ph_bf, sl);
+        // every S2 so far has read B2 (and A2): the last use of slot sl is sub-frame v = u-1 or u-2, its
+        // release the phase of number v >> 1 (none yet: the phase before the first, over from the start)
+        auto s2_done = [&]() -> bool {
+            auto last = [&](unsigned sl) { return ((u + 1 - sl) >> 1) + 1; };  // uses of the slot, + 1
+            return ws3_wait2(&m.b2_free[0], last(0) & 1u, &m.b2_free[1], last(1) & 1u);
         };
         for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
             const int kb = (s.item / a.n_g) % a.n_kb, c = a.c0 + s.item / ipc;
             const int4 tp = a.tbox[c];
             const int nyt = tp.z, nyc = ws3_uni(tp.x >> 3), H = tp.y, NU = ws3_uni(s.nt * H);
-            good = free_b2(0) && free_b2(1);  // every S2 of the item before has read A2
+            good = s2_done();  // every S2 of the item before has read A2
             if (!good) break;
             tc::fence_after_sync();
             {   // stage-2 DFT operand (every row part) -> TMEM (lane = ky row).  A row's part is
@@ -2821,9 +2832,9 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
             switch (nyc) {  // P nyh <= 256 columns and two slots of D1 beside A2: nyc <= 15
 #define EPIC_E1(n)                                                                                                  \
     case n:                                                                                                         \
-        good = q4 >> 1 ? ws3_e1<n, 1>(m, NU, u, ph_d1, ph_bf, held, tmem + lane_base, a.d1_cols, P, lane, b2a,       \
+        good = q4 >> 1 ? ws3_e1<n, 1>(m, NU, u, tmem + lane_base, a.d1_cols, P, lane, b2a,       \
                                       a.b2_bytes, 64 * P * (q4 & 1))                                                \
-                       : ws3_e1<n, 0>(m, NU, u, ph_d1, ph_bf, held, tmem + lane_base, a.d1_cols, P, lane, b2a,       \
+                       : ws3_e1<n, 0>(m, NU, u, tmem + lane_base, a.d1_cols, P, lane, b2a,       \
                                       a.b2_bytes, 64 * P * (q4 & 1));                                               \
         break;
                 EPIC_KS_CASES(EPIC_E1)
@@ -2831,7 +2842,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 default: good = false;
             }
         }
-        if (good) good = free_b2(0) && free_b2(1);
+        if (good) good = s2_done();
         if (!good) err_sh = 1;
     } else {
         // ------------------------------------------------------------ epilogue 2
@@ -3873,9 +3884,16 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.b2_bytes = p->tc.ws3_b2;
                     if (p->sub == 0 && (p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
+                    {
+                        // as many as divide a channel's items and the blocks (two for N = 128, eight for N = 256)
+                        const int ipc = a.n_kb * a.n_g;
+                        a.share = 8;
+                        while (ipc % a.share || p->sm_count % a.share) a.share >>= 1;
                         k_dftgemm_ws3<true><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
-                    else
+                    } else {
+                        a.share = 1;
                         k_dftgemm_ws3<false><<<grid, kWs3Threads, p->tc.ws3_smem, s>>>(a);
+                    }
                 }
                 else if (p->tc.ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);
                 else k_dftgemm_ws<0><<<grid, kWsThreads, p->tc.smem, s>>>(a);
