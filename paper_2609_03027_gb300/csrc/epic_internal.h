@@ -104,6 +104,7 @@ struct TcState {
     bool parts = false;            // some channel has H > 1 (only k_dftgemm_ws3 takes it)
     int nbt = 2;                   // k_dftgemm_ws3: tile-part buffers in shared memory (2..6),
     unsigned ws3_sB2 = 0, ws3_b2 = 0;  //   where B2 starts, bytes of a B2 buffer
+    unsigned ws3_stage = 0;        //   where the interval stores' staging starts (0: none)
     int ws3_smem = 0;
     bool ws_old = false;           // the older warp-specialised kernels take the plan too
     size_t n_counters = 0;         // entries of `counters`

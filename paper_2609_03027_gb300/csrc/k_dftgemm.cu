@@ -133,6 +133,7 @@ struct MmaArgs {
     int iv0;                    // k_dftgemm_ws3: image set of the chunk's first sample
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
+    unsigned sStage;            // k_dftgemm_ws3: 2 KB per epilogue-2 warp for interval stores, 0 = none
     int share;                  // k_dftgemm_ws3<true>: blocks that walk items of one channel side by side
     int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..6)
     const long long* wcum;      // k_dftgemm_ws3<true>: [C + 1] prefix sums of the channels' item costs per frame
@@ -2153,6 +2154,7 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 constexpr int kWs3Threads = 512;
 constexpr int kWs3CtlRegs = 64, kWs3E1Regs = 96, kWs3E2Regs = 176;
 static_assert(kWs3CtlRegs + kWs3E1Regs + 2 * kWs3E2Regs == 4 * 128, "setmaxnreg shares are the launch's registers");
+constexpr size_t kWs3Stage = 8 * 2048;  // interval stores: 2 KB for each epilogue-2 warp
 constexpr int kWs3MaxBlocks = 256;  // blocks per launch (one per SM) the split bookkeeping holds
 constexpr int kWs3MaxTileBufs = 6;  // tile-part buffers of k_dftgemm_ws3 (short row parts need more in flight)
 
@@ -2329,6 +2331,38 @@ __device__ __forceinline__ void ws3_store32(float* o, int nk, int accumulate, co
     }
 }
 
+// The same for a whole warp (rows ky0 + lane, 32 columns from kx0) through 2 KB of shared memory, so
+// that a store covers 8 rows x 64 bytes: the sub-integration schedule stores every few frames, and
+// a 16-byte store of each lane to a row of its own took 32 L1 wavefronts (LWA block of 128 samples with
+// an image set every 4: 0.62 ms of k_dftgemm_ws3).  o: pixel (ky0, kx0).
+__device__ __forceinline__ void ws3_store_rows(float* o, int N, int rows, int nk, int accumulate, int lane, float* stage,
+                                               const float (&v)[32])
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            *reinterpret_cast<float4*>(stage + lane * 16 + ((k ^ ((lane >> 1) & 3)) << 2)) =
+                make_float4(v[16 * h + 4 * k], v[16 * h + 4 * k + 1], v[16 * h + 4 * k + 2], v[16 * h + 4 * k + 3]);
+        __syncwarp();
+        const int c = lane & 3;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = 8 * i + (lane >> 2);
+            float4 w = *reinterpret_cast<const float4*>(stage + r * 16 + ((c ^ ((r >> 1) & 3)) << 2));
+            if (r < rows && 16 * h + 4 * c < nk) {
+                float4* q = reinterpret_cast<float4*>(o + (size_t)r * N + 16 * h + 4 * c);
+                if (accumulate) {
+                    const float4 u = *q;
+                    w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
+                }
+                *q = w;
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // Partial sums of a split item, as epilogue-2 thread `tid2` of 256 holds them: float4 k of
 // product pr at ((8 pr + k) 256 + tid2) 4 (consecutive threads, consecutive 16 bytes).
 __device__ __forceinline__ void ws3_store_partial(float* slot, int pr, int tid2, const float (&v)[32])
@@ -2446,7 +2480,7 @@ __device__ __forceinline__ bool ws3_e2_any(bool mine)
 template <bool SPLIT, int P>
 __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int items, long long w0, long long w1,
                                             int warp, int lane, uint64_t* d2_full, uint64_t* d2_empty,
-                                            const uint32_t* start, int* split_b)
+                                            const uint32_t* start, int* split_b, uint8_t* stage)
 {
     const int q4 = warp & 3, hf = (warp >> 2) & 1, tid2 = 32 * (warp - 8) + lane;
     const uint32_t taddr = tmem + ((uint32_t)(32 * q4) << 16) + 256 + 64 * P * hf;
@@ -2483,7 +2517,20 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
             tc::fence_after_sync();
             ws3_epilogue2<P>(taddr, xx, yy, rx, ix, lane, &d2_empty[hf]);
             if (!SPLIT && --left == 0) {  // write (or add) this interval's sums (without sub-integrations: never)
-                store(a.out + (size_t)iv * a.C * a.nprod * NN + px);
+                float* o = a.out + (size_t)iv * a.C * a.nprod * NN + px;
+                if (stage) {
+                    float* st = reinterpret_cast<float*>(stage) + (warp - 8) * 512;
+                    const int rows = min(32, a.N - (ky - lane)), nkw = min(32, a.N - kx0);
+                    o -= (size_t)lane * a.N;
+                    ws3_store_rows(o, a.N, rows, nkw, a.accumulate, lane, st, xx);
+                    if (P == 2) {
+                        ws3_store_rows(o + NN, a.N, rows, nkw, a.accumulate, lane, st, yy);
+                        ws3_store_rows(o + 2 * NN, a.N, rows, nkw, a.accumulate, lane, st, rx);
+                        ws3_store_rows(o + 3 * NN, a.N, rows, nkw, a.accumulate, lane, st, ix);
+                    }
+                } else {
+                    store(o);
+                }
                 clear();
                 ++iv;
                 left = a.sub;
@@ -2847,8 +2894,11 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     } else {
         // ------------------------------------------------------------ epilogue 2
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWs3E2Regs) : "memory");
-        good = P == 2 ? ws3_role_e2<SPLIT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b)
-                      : ws3_role_e2<SPLIT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b);
+        uint8_t* stage = !SPLIT && a.sStage ? sbase + a.sStage : nullptr;
+        good = P == 2 ? ws3_role_e2<SPLIT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
+                                              stage)
+                      : ws3_role_e2<SPLIT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
+                                              stage);
         if (!good) err_sh = 1;
     }
     tc::fence_before_sync();
@@ -3362,8 +3412,11 @@ epic_status dftgemm_setup(epic_plan_s* p)
         const size_t b2w = align_up(2ull * 128 * P * 2 * nyh_max, 1024);
         // as many tile-part buffers (2..6) as fit: a part's copy takes longer than its step
         int nbt = kWs3MaxTileBufs;
-        while (nbt > 2 && a1p + nbt * b1p + 2 * b2w > limit) --nbt;
-        const size_t need_ws = a1p + nbt * b1p + 2 * b2w;
+        const size_t fixed = a1p + 2 * b2w;
+        // sub-integrations: staging of the interval stores where it fits
+        const size_t stage = p->sub > 0 && fixed + 2 * b1p + kWs3Stage <= limit ? kWs3Stage : 0;
+        while (nbt > 2 && fixed + nbt * b1p + stage > limit) --nbt;
+        const size_t need_ws = fixed + nbt * b1p + stage;
         if (need_ws > limit) continue;
         p->tc.ws = true;
         p->tc.parts = split;
@@ -3375,6 +3428,7 @@ epic_status dftgemm_setup(epic_plan_s* p)
         p->tc.d1_cols = dmax;
         p->tc.ws3_sB2 = (unsigned)(a1p + nbt * b1p);
         p->tc.ws3_b2 = (unsigned)b2w;
+        p->tc.ws3_stage = stage ? (unsigned)(a1p + nbt * b1p + 2 * b2w) : 0u;
         p->tc.ws3_smem = (int)(need_ws + 1024);
         // the older variants: two tile buffers, B2 with both parts' rows, one part per channel
         const size_t b2o = align_up(2ull * 2 * 64 * P * pad64(2 * nyh_max), 1024), need_old = a1p + 2 * b1p + 2 * b2o;
@@ -3882,6 +3936,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.counters = p->tc.counters;
                     a.sB2 = p->tc.ws3_sB2;
                     a.b2_bytes = p->tc.ws3_b2;
+                    a.sStage = p->tc.ws3_stage;
                     if (p->sub == 0 && (p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
                     {
