@@ -134,10 +134,10 @@ struct MmaArgs {
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
     unsigned sStage;            // k_dftgemm_ws3: 2 KB per epilogue-2 warp for interval stores, 0 = none
-    int share;                  // k_dftgemm_ws3<true>: blocks that walk items of one channel side by side
+    int share;                  // k_dftgemm_ws3<1 or 2>: blocks that walk items of one channel side by side
     int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..6)
-    const long long* wcum;      // k_dftgemm_ws3<true>: [C + 1] prefix sums of the channels' item costs per frame
-    const int* item_order;      // k_dftgemm_ws3<false>: per channel group (from c0 ipc), items in the order dealt to blocks
+    const long long* wcum;      // k_dftgemm_ws3<1 or 2>: [C + 1] prefix sums of the channels' item costs per frame
+    const int* item_order;      // k_dftgemm_ws3<0>: per channel group (from c0 ipc), items in the order dealt to blocks
 };
 
 // byte offset of 16-byte chunk c (8 halves of K) of row r in an R-row operand in the
@@ -2434,7 +2434,7 @@ __device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float*
 }
 
 // The segments (work item, first frame, frames) of a block: every role walks them alike.
-// SPLIT: the block group's (item group, frame) units [w, w1) in item-major order -- `share` blocks
+// CUT > 0: the block group's (item group, frame) units [w, w1) in item-major order -- `share` blocks
 // walk `share` items of a channel side by side, so that a grid tile is read from HBM once and from
 // L2 by the others (apart, both items of an LWA channel read it from HBM: 6.3 GB a block at 5.7 TB/s,
 // the limit of the kernel) -- else whole items.
@@ -2442,10 +2442,10 @@ struct Ws3Seg {
     int item, fs, nt;
 };
 
-template <bool SPLIT>
+template <int CUT>
 __device__ __forceinline__ bool ws3_next(const MmaArgs& a, int items, int it, long long& w, long long w1, Ws3Seg& s)
 {
-    if (SPLIT) {
+    if (CUT) {
         if (w >= w1) return false;
         s.item = (int)(w / a.nt) * a.share + blockIdx.x % a.share;
         s.fs = (int)(w % a.nt);
@@ -2477,7 +2477,7 @@ __device__ __forceinline__ bool ws3_e2_any(bool mine)
 }
 
 // The epilogue-2 warps' walk through the block's segments.  Returns false when a wait ran out.
-template <bool SPLIT, int P>
+template <int CUT, int P>
 __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int items, long long w0, long long w1,
                                             int warp, int lane, uint64_t* d2_full, uint64_t* d2_empty,
                                             const uint32_t* start, int* split_b, uint8_t* stage)
@@ -2488,7 +2488,7 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
     uint32_t ph = 0;
     long long w = w0;
     Ws3Seg s;
-    for (int it = 0; ws3_next<SPLIT>(a, items, it, w, w1, s); ++it) {
+    for (int it = 0; ws3_next<CUT>(a, items, it, w, w1, s); ++it) {
         const int g = s.item % a.n_g, kb = (s.item / a.n_g) % a.n_kb, c = a.c0 + s.item / (a.n_g * a.n_kb);
         // this thread's pixels: row ky, kx0 .. kx0 + nk - 1 (none outside the image)
         const int ky = 128 * kb + 32 * q4 + lane, kx0 = 64 * g + 32 * hf;
@@ -2508,7 +2508,8 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
             }
         };
         clear();
-        int iv = a.iv0, left = a.sub;  // sub-integrations: image set of this frame and frames left in it
+        // sub-integrations: image set of this frame and frames left in it
+        int iv = a.iv0 + (CUT == 2 ? s.fs / a.sub : 0), left = a.sub;
         bool good = true;
         for (int t = 0; t < s.nt; ++t) {
             good = ws3_wait(&d2_full[hf], ph);
@@ -2516,7 +2517,7 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
             ph ^= 1u;
             tc::fence_after_sync();
             ws3_epilogue2<P>(taddr, xx, yy, rx, ix, lane, &d2_empty[hf]);
-            if (!SPLIT && --left == 0) {  // write (or add) this interval's sums (without sub-integrations: never)
+            if (CUT != 1 && --left == 0) {  // write (or add) this interval's sums (without sub-integrations: never)
                 float* o = a.out + (size_t)iv * a.C * a.nprod * NN + px;
                 if (stage) {
                     float* st = reinterpret_cast<float*>(stage) + (warp - 8) * 512;
@@ -2537,9 +2538,9 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
             }
         }
         // the epilogue-2 warps leave together when one of them gave up (ws3_split_finish has barriers)
-        if (SPLIT) good = !ws3_e2_any(!good);
+        if (CUT == 1) good = !ws3_e2_any(!good);
         if (!good) return false;
-        if (SPLIT && s.nt != a.nt) {  // part of an item: to this block's slot
+        if (CUT == 1 && s.nt != a.nt) {  // part of an item: to this block's slot
             float* slot = a.partial + (2 * (size_t)blockIdx.x + (it == 0 ? 0 : 1)) * 4 * 8192;
             ws3_store_partial(slot, 0, tid2, xx);
             if (P == 2) {
@@ -2548,7 +2549,7 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
                 ws3_store_partial(slot, 3, tid2, ix);
             }
             ws3_split_finish(a, s.item, a.out + px, nk, tid2, start, split_b);
-        } else if (a.sub == 0) {
+        } else if (CUT != 2 && a.sub == 0) {
             store(a.out + px);
         }
     }
@@ -2655,16 +2656,18 @@ __device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t
     return true;
 }
 
-// SPLIT: equal shares of the launch's (item, frame) units (items may be split between blocks),
-// else whole items, with sub-integrations when a.sub > 0.
-template <bool SPLIT>
+// How a launch's work is cut.  0: whole items per block, with sub-integrations when a.sub > 0.  1: equal
+// shares of its (item, frame) units, without sub-integrations; the parts of an item are summed through
+// a.partial.  2: sub-integrations, equal shares cut between them, so that no sums are shared (LWA block of 128
+// samples, an image set every 4: 264 whole items are two rounds of 152 blocks, the second mostly idle).
+template <int CUT>
 __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ Ws3Bars m;
     __shared__ uint32_t tmem_sh;
     __shared__ int err_sh;
-    __shared__ uint32_t start[SPLIT ? kWs3MaxBlocks + 1 : 1];  // first unit of every block group
+    __shared__ uint32_t start[CUT ? kWs3MaxBlocks + 1 : 1];  // first unit of every block group
     __shared__ int split_b[2];  // blocks of a split item; the second is -1 unless this block completes it
     const int tid = threadIdx.x, warp = ws3_uni(tid >> 5), lane = tid & 31;
     if (warp == 0) {
@@ -2691,9 +2694,12 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int ipc = a.n_kb * a.n_g, items = a.n_ch * ipc;  // items per channel, of the launch
-    if (SPLIT)
+    if (CUT) {
+        const int unit = CUT == 2 ? a.sub : 1;  // frames that stay together
         for (int b = tid; b <= (int)(gridDim.x / a.share); b += kWs3Threads)
-            start[b] = (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt, b, gridDim.x / a.share);
+            start[b] = (uint32_t)unit *
+                       (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt / unit, b, gridDim.x / a.share);
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -2703,10 +2709,10 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     const int P = a.P;
     const uint32_t a2col = 2u * a.d1_cols;
     const uint32_t b2a = tc::smem_u32(sbase + a.sB2);
-    // this block's part of the launch.  SPLIT: its group's (item group, frame) units [wb0, wb1) in
-    // item-major order (items cut at range boundaries are summed by the block that stores their last part);
+    // this block's part of the launch.  CUT: its group's (item group, frame) units [wb0, wb1) in
+    // item-major order (CUT 1: items cut at range boundaries are summed by the block that stores their last part);
     // else whole items blockIdx.x, + gridDim.x, ...
-    const long long wb0 = SPLIT ? start[blockIdx.x / a.share] : 0, wb1 = SPLIT ? start[blockIdx.x / a.share + 1] : 0;
+    const long long wb0 = CUT ? start[blockIdx.x / a.share] : 0, wb1 = CUT ? start[blockIdx.x / a.share + 1] : 0;
     Ws3Seg s;
     long long w = wb0;
     bool good = true;
@@ -2728,7 +2734,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 used &= ~(1u << j);
                 return true;
             };
-            for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+            for (int it = 0; good && ws3_next<CUT>(a, items, it, w, wb1, s); ++it) {
                 const int g = s.item % a.n_g, cl = s.item / ipc, c = a.c0 + cl;
                 const int4 tp = a.tbox[c];
                 const int H = tp.y, NU = s.nt * H;
@@ -2779,7 +2785,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
             uint32_t ph_tile = 0, ph_a = 0;
             int b = 0;
             unsigned u = 0;  // sub-frames of all segments
-            for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+            for (int it = 0; good && ws3_next<CUT>(a, items, it, w, wb1, s); ++it) {
                 const int c = a.c0 + s.item / ipc;
                 const int4 tp = a.tbox[c];
                 const int ks = ws3_uni(a.box[c].z / 8), N1 = ws3_uni(P * tp.x), NU = ws3_uni(s.nt * tp.y);
@@ -2803,7 +2809,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
             const uint32_t lead = tc::elect_one();
             uint32_t ph_a2 = 0;
             unsigned u = 0, fr = 0;  // sub-frames and frames of all segments
-            for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+            for (int it = 0; good && ws3_next<CUT>(a, items, it, w, wb1, s); ++it) {
                 const int4 tp = a.tbox[a.c0 + s.item / ipc];
                 const int ks = ws3_uni(tp.x / 8), H = ws3_uni(tp.y), nt = ws3_uni(s.nt);
                 good = ws3_wait(&m.a2_full, ph_a2, 0);
@@ -2836,7 +2842,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
             auto last = [&](unsigned sl) { return ((u + 1 - sl) >> 1) + 1; };  // uses of the slot, + 1
             return ws3_wait2(&m.b2_free[0], last(0) & 1u, &m.b2_free[1], last(1) & 1u);
         };
-        for (int it = 0; good && ws3_next<SPLIT>(a, items, it, w, wb1, s); ++it) {
+        for (int it = 0; good && ws3_next<CUT>(a, items, it, w, wb1, s); ++it) {
             const int kb = (s.item / a.n_g) % a.n_kb, c = a.c0 + s.item / ipc;
             const int4 tp = a.tbox[c];
             const int nyt = tp.z, nyc = ws3_uni(tp.x >> 3), H = tp.y, NU = ws3_uni(s.nt * H);
@@ -2894,10 +2900,10 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     } else {
         // ------------------------------------------------------------ epilogue 2
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWs3E2Regs) : "memory");
-        uint8_t* stage = !SPLIT && a.sStage ? sbase + a.sStage : nullptr;
-        good = P == 2 ? ws3_role_e2<SPLIT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
+        uint8_t* stage = CUT != 1 && a.sStage ? sbase + a.sStage : nullptr;
+        good = P == 2 ? ws3_role_e2<CUT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
                                               stage)
-                      : ws3_role_e2<SPLIT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
+                      : ws3_role_e2<CUT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
                                               stage);
         if (!good) err_sh = 1;
     }
@@ -3722,8 +3728,9 @@ epic_status dftgemm_setup(epic_plan_s* p)
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_dftgemm_grid)");
     e = allow_max_smem((const void*)k_dftgemm_ws<0>, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws2<0>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<false>, p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<true>, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<0>, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<1>, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<2>, p->smem_optin);
     p->tc.ws_variant = p->tc.ws ? 3 : 0;
     if (p->tc.ws && p->sm_count > kWs3MaxBlocks) p->tc.ws_variant = 1;
     if (p->tc.ws && !p->tc.ws_old && p->tc.ws_variant != 3) {
@@ -3937,17 +3944,18 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.sB2 = p->tc.ws3_sB2;
                     a.b2_bytes = p->tc.ws3_b2;
                     a.sStage = p->tc.ws3_stage;
-                    if (p->sub == 0 && (p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
+                    if ((p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
                     {
                         // as many as divide a channel's items and the blocks (two for N = 128, eight for N = 256)
                         const int ipc = a.n_kb * a.n_g;
                         a.share = 8;
                         while (ipc % a.share || p->sm_count % a.share) a.share >>= 1;
-                        k_dftgemm_ws3<true><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
+                        if (a.sub > 0) k_dftgemm_ws3<2><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
+                        else k_dftgemm_ws3<1><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
                     } else {
                         a.share = 1;
-                        k_dftgemm_ws3<false><<<grid, kWs3Threads, p->tc.ws3_smem, s>>>(a);
+                        k_dftgemm_ws3<0><<<grid, kWs3Threads, p->tc.ws3_smem, s>>>(a);
                     }
                 }
                 else if (p->tc.ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);
