@@ -68,6 +68,29 @@ __host__ __device__ __forceinline__ uint32_t tile_part_off(int y, int k, int nyh
     return (uint32_t)h * part_bytes + tile_half_off(y - h * nyh, k, P * nyh);
 }
 
+// The same without padding of K, for k_dftgemm_grid_tc and k_dftgemm_ws3: whole panels of 64 K indices as
+// above, then one of 32 (64-byte swizzle) and one of 16 (32-byte swizzle) as K1 = 2 nx needs them.  Padded,
+// a 48-wide box's rows ended in half a 128-byte line, and such tiles took 1.5 times as long a byte
+// to write as those of 64 or 96 columns.  tile_dense_row: bytes from a row to the next at K index k.
+__host__ __device__ __forceinline__ uint32_t tile_dense_row(int k, int K1)
+{
+    if ((k >> 6) < (K1 >> 6)) return 128;
+    return (K1 & 32) && (k & 63) < 32 ? 64 : 32;
+}
+
+__host__ __device__ __forceinline__ uint32_t tile_dense_off(int y, int k, int nyh, int P, int K1)
+{
+    const int h = y / nyh, R = y - h * nyh, N1 = P * nyh;
+    const uint32_t part = (uint32_t)h * (uint32_t)(N1 * K1 * 2);
+    if ((k >> 6) < (K1 >> 6)) return part + tile_half_off(R, k, N1);
+    uint32_t base = part + (uint32_t)((K1 >> 6) * N1 * 128);
+    if (K1 & 32) {
+        if ((k & 63) < 32) return base + (uint32_t)(R * 64 + ((((k >> 3) ^ (R >> 1)) & 3) << 4) + ((k & 7) << 1));
+        base += (uint32_t)N1 * 64;
+    }
+    return base + (uint32_t)(R * 32 + ((((k >> 3) ^ (R >> 2)) & 1) << 4) + ((k & 7) << 1));
+}
+
 // 8 consecutive 32-bit TMEM columns of this thread's lane
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r)
 {

@@ -133,6 +133,7 @@ struct MmaArgs {
     int iv0;                    // k_dftgemm_ws3: image set of the chunk's first sample
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
+    int dense;                  // k_dftgemm_ws3: the tiles' K is not padded (tile_dense_off)
     unsigned sStage;            // k_dftgemm_ws3: 2 KB per epilogue-2 warp for interval stores, 0 = none
     int share;                  // k_dftgemm_ws3<1 or 2>: blocks that walk items of one channel side by side
     int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..6)
@@ -2570,9 +2571,18 @@ struct Ws3Bars {
 template <int KS>
 __device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, int& b, int NB, uint32_t& ph_tile,
                                        uint32_t tmem, uint32_t d1_cols, uint32_t da, uint32_t b1,
-                                       uint32_t b1_bytes, int N1, uint32_t lead)
+                                       uint32_t b1_bytes, int N1, int dense, uint32_t lead)
 {
     const uint32_t id1 = tc::idesc_f16_f32(128, N1), pb = (uint32_t)N1 * 8;
+    // the up to three steps after the last whole panel: of that padded panel, or of narrower ones
+    const int full = (KS ? KS : ks) >> 2, rem = (KS ? KS : ks) & 3;
+    uint32_t tail[3], hi[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const bool wide = i < (rem & 2);
+        tail[i] = full * pb + (!dense ? i * 2 : wide ? i * 2 : (rem & 2) * (pb >> 2));
+        hi[i] = !dense ? tc::kDescSw128Hi : wide ? tc::kDescSw64Hi : tc::kDescSw32Hi;
+    }
 #pragma unroll 1
     for (const unsigned end = u + NU; u != end; ++u) {
         const int sl = u & 1;
@@ -2584,14 +2594,18 @@ __device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, 
         const uint32_t d = tmem + sl * d1_cols;
         if (KS) {
 #pragma unroll
-            for (int k = 0; k < KS; ++k)
+            for (int k = 0; k < (KS & ~3); ++k)
                 tc::mma_f16_lead(d, da + (k >> 2) * (128 * 8) + (k & 3) * 2, db + (k >> 2) * pb + (k & 3) * 2, id1, k > 0,
                                  lead);
         } else {
-            for (int k = 0; k < ks; ++k)
+            for (int k = 0; k < (ks & ~3); ++k)
                 tc::mma_f16_lead(d, da + (k >> 2) * (128 * 8) + (k & 3) * 2, db + (k >> 2) * pb + (k & 3) * 2, id1, k > 0,
                                  lead);
         }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            if (i < rem)
+                tc::mma_f16_lead_b(d, da + full * (128 * 8) + i * 2, db + tail[i], hi[i], id1, full > 0 || i > 0, lead);
         tc::mma_commit_lead(&m.d1_full[sl], lead);
         tc::mma_commit_lead(&m.tile_free[b], lead);
         if (++b == NB) b = 0;
@@ -2739,7 +2753,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 const int4 tp = a.tbox[c];
                 const int H = tp.y, NU = s.nt * H;
                 const int K1p = pad64(2 * a.box[c].z);
-                const uint32_t part_bytes = (uint32_t)(P * tp.x) * K1p * 2;
+                const uint32_t part_bytes = (uint32_t)(P * tp.x) * (a.dense ? 2 * a.box[c].z : K1p) * 2;
                 // next part to copy, advanced without division
                 const uint8_t* nxt = a.tiles + (size_t)cl * a.tile_stride + (size_t)s.fs * frame_step;
                 const uint32_t a1_bytes = 256u * K1p;
@@ -2792,12 +2806,12 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 good = ws3_wait(&m.bar_a, ph_a, 0);
                 if (!good) break;
                 switch (ks) {
-#define EPIC_S1(n)                                                                                                   case n:                                                                                                              good = ws3_s1<n>(m, n, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1),                          a.b1_bytes, N1, lead);                                                                          break;
+#define EPIC_S1(n)                                                                                                   case n:                                                                                                              good = ws3_s1<n>(m, n, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1),                          a.b1_bytes, N1, a.dense, lead);                                                                          break;
                     EPIC_KS_CASES(EPIC_S1)
 #undef EPIC_S1
                     default:
                         good = ws3_s1<0>(m, ks, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da,
-                                         tc::smem_u32(sbase + a.sB1), a.b1_bytes, N1, lead);
+                                         tc::smem_u32(sbase + a.sB1), a.b1_bytes, N1, a.dense, lead);
                 }
             }
             if (!good) {  // a wait ran out: let this warp's MMAs finish (bounded)
@@ -2917,6 +2931,8 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
 
 // Time samples per chunk so that the grid tiles of one (channel group, time
 // chunk) take at most `budget` bytes, and the tile buffer for them.
+int dftgemm_dense(const epic_plan_s* p) { return p->tc.ws && p->tc.ws_variant == 3 && p->tc.grid_variant == 4; }
+
 epic_status dftgemm_set_kernel(epic_plan_s* p, int variant)
 {
     if (variant < 1 || variant > 3 || !p->tc.ws || ((p->sub > 0 || !p->tc.ws_old) && variant != 3) ||
@@ -3944,6 +3960,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.sB2 = p->tc.ws3_sB2;
                     a.b2_bytes = p->tc.ws3_b2;
                     a.sStage = p->tc.ws3_stage;
+                    a.dense = dftgemm_dense(p);
                     if ((p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
                     {

@@ -11,17 +11,18 @@
 // w_hi v_hi + w_lo v_hi + w_hi v_lo is summed.  The gather kernels compute the same sums with FP32 FMAs and are
 // bound by shared-memory gathers and list walks (7.5 k SM cycles a frame of a 96 x 96 box); here
 // a frame takes its MMAs (64 cycles each, 4 a K step) and its tile stores.
-// Roles of the 512-thread block (one per SM), all walking the block's share of (channel, tile
+// Roles of the 640-thread block (one per SM), all walking the block's share of (channel, tile
 // slice, frame group) units alike; all hand-offs are mbarriers with bounded waits:
 //   warp 0      issues the MMAs of a K step: (even, odd) x (hi, lo), then frees its operands
 //   warps 1-3   build weight steps in a shared-memory ring: zeros, then the step's non-zero
 //               weights scattered (about 150 of 4096) -- far fewer bytes than reading the dense
 //               operands from L2 (80 KB a tile).  A tile of at most RW steps is built once for all
 //               the groups of a staged chunk, a denser one once per group.
-//   warps 4-7   stage the raw voltages of up to 4 groups (row stride odd in words, so that lanes
-//               = frames read without bank conflicts) and expand them, a K step at a time, into
-//               FP16 operands: lanes are frames, so a 16-byte chunk store of a warp is contiguous
-//   warps 8-15  read D (a lane is a cell pair, a column a frame) and store a pair's real and
+//   warps 4-11  stage the raw voltages of up to 4 groups (row stride odd in words, so that lanes
+//               = frames read without bank conflicts; 4-byte asynchronous copies, so that a whole
+//               chunk is in flight) and expand them, a K step at a time, into FP16 operands: lanes
+//               are frames, so a 16-byte chunk store of a warp is contiguous
+//   warps 12-19 read D (a lane is a cell pair, a column a frame) and store a pair's real and
 //               imaginary FP16 pairs as 8 bytes: 32 lanes fill whole sectors of the tile, no staging
 // D is double buffered (2 x 256 TMEM columns), the operand rings hold 6 weight and 8 voltage steps.
 #include <math.h>
@@ -39,11 +40,11 @@ namespace epic {
 
 namespace {
 
-constexpr int kGtThreads = 512;
+constexpr int kGtThreads = 640;
 constexpr int kGtRW = 6;               // weight steps in the ring (a multiple of the builder warps: a slot is one warp's)
 constexpr int kGtRV = 8;               // voltage steps in the ring (a multiple of the expander warps)
 constexpr int kGtEnt = 10;             // weights a lane loads ahead (320 a step: more than a 7 x 7 GCF's tile of 256 elements has)
-constexpr int kGtBuilders = 3, kGtExpanders = 4;
+constexpr int kGtBuilders = 3, kGtExpanders = 8;
 constexpr unsigned kGtWBytes = 16384;  // one weight step: (hi, lo) x (even, odd) x 128 pairs x 16 halves
 constexpr unsigned kGtVBytes = 4096;   // one voltage step: 128 columns x 16 halves (mixed: hi, then lo)
 
@@ -64,11 +65,12 @@ struct GridTcArgs {
     const int2* ent;        // weights: byte offset in the step's hi half, value (scaled)
     const int* el;          // 16 (complex weights: 8) elements of each K step
     const long long* wcum;  // [C + 1] prefix sums of the channels' costs per group
+    int dense;              // the tiles' K is not padded (k_dftgemm_ws3 reads them)
     int slices;             // tile slices of a channel (more units than groups when those are few)
     int ngr;                // frame groups of the launch
     int gc;                 // groups per staged chunk
     int raw_stride;         // bytes of a staged frame row (4 x odd)
-    int vec;                // voltage rows are 16-byte aligned and whole 16-byte chunks
+    int shift;              // rows are staged shifted to a word boundary (samples at no multiple of their size)
     uint32_t vscale, vbias; // half2: 2^-s, and what the decode's offset becomes
     const float4* jones;    // MIX: [C][A][2] polarisation-mixing rows (conj J)
     float unscale;          // MIX: 2^-s of the results (the weights are scaled, the voltages are not)
@@ -141,6 +143,11 @@ __device__ __forceinline__ float4 gt_mix(uint32_t raw, const float4* jm)
     return make_float4(mx.x, mx.y, my.x, my.y);
 }
 
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
 __device__ __forceinline__ float gt_lo(float v) { return v - __half2float(__float2half_rn(v)); }
 
 template <int P, int BITS, bool CPLX, bool MIX>
@@ -187,7 +194,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
     const long long u1 = split_start(a.wcum, a.c0, a.n_ch, S, ngr, blockIdx.x + 1, gridDim.x);
 
     // Every role's walk through the block's units: f(channel, local channel, tiles [T0, T1), first
-    // group, groups) per staged chunk.
+    // group, groups, end of the segment's groups) per staged chunk.
     auto walk = [&](auto&& f) {
         for (long long u = u0; u < u1;) {
             const int cl = gt_uni((int)(u / ((long long)S * ngr))), r = gt_uni((int)(u % ((long long)S * ngr)));
@@ -195,7 +202,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
             const int g1 = gt_uni((int)min((long long)ngr, g0 + (u1 - u)));
             const int ta = a.tile0[c], tn = a.tile0[c + 1] - ta;
             const int T0 = gt_uni(ta + tn * sl / S), T1 = gt_uni(ta + tn * (sl + 1) / S);
-            for (int gb = g0; gb < g1; gb += a.gc) f(c, cl, T0, T1, gb, min(a.gc, g1 - gb));
+            for (int gb = g0; gb < g1; gb += a.gc) f(c, cl, T0, T1, gb, min(a.gc, g1 - gb), g1);
             u += g1 - g0;
         }
     };
@@ -208,7 +215,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
         int ws = 0, vs = 0;                 // ring slots
         uint32_t ph_w = 0, ph_v = 0;        // parities, one bit a slot
         unsigned nd = 0;                    // D buffers filled so far
-        walk([&](int, int, int T0, int T1, int, int ng) {
+        walk([&](int, int, int T0, int T1, int, int ng, int) {
             for (int t = T0; t < T1 && good; ++t) {
                 const int steps = gt_uni(a.unit0[t + 1] - a.unit0[t]);
                 const bool keep = steps <= kGtRW;  // the tile's weights stay for every group
@@ -252,7 +259,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
     } else if (warp < 4) {
         // ------------------------------------------------------------ weight steps
         unsigned q = 0;  // steps built so far by all builders
-        walk([&](int, int, int T0, int T1, int, int ng) {
+        walk([&](int, int, int T0, int T1, int, int ng, int) {
             for (int t = T0; t < T1; ++t) {
                 const int ub = a.unit0[t], steps = gt_uni(a.unit0[t + 1] - ub);
                 const int n = steps <= kGtRW ? steps : steps * ng;
@@ -288,44 +295,40 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
             }
         });
         if (!good) err_sh = 1;
-    } else if (warp < 8) {
+    } else if (warp < 4 + kGtExpanders) {
         // ------------------------------------------------------------ voltages
         const int FB = a.A * P * (BITS / 4);
         unsigned q = 0;  // steps expanded so far by all expanders
-        walk([&](int c, int, int T0, int T1, int gb, int ng) {
+        walk([&](int c, int, int T0, int T1, int gb, int ng, int gend) {
             const int f0 = gb * FG, nf = min(a.nt - f0, ng * FG);
-            asm volatile("bar.sync 1, 128;" ::: "memory");  // the last chunk's rows are read
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kGtExpanders) : "memory");  // the last chunk's rows are read
             const uint8_t* src = a.volt + ((size_t)(a.t0 + f0) * a.C + c) * (size_t)FB;
             const size_t step = (size_t)a.C * FB;
-            // a warp takes rows w, w + 4, ..., four of them in flight
             const int xw = warp - 4;
-            if (a.vec) {
-                const int nv = FB >> 4;
-                for (int f = xw; f < nf; f += 16)
-                    for (int j = lane; j < nv; j += 32) {
-                        uint4 v[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (f + 4 * k < nf) v[k] = __ldg(reinterpret_cast<const uint4*>(src + (f + 4 * k) * step) + j);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (f + 4 * k < nf) {
-                                uint32_t* d = reinterpret_cast<uint32_t*>(raw + (size_t)(f + 4 * k) * a.raw_stride) + 4 * j;
-                                d[0] = v[k].x;
-                                d[1] = v[k].y;
-                                d[2] = v[k].z;
-                                d[3] = v[k].w;
-                            }
-                    }
-            } else {  // rows at any byte address: aligned words (each holds a byte of the row), shifted
+            if (!a.shift) {
+                // the aligned words that hold a byte of the row: its samples keep their offset in the first
+                for (int f = xw; f < nf; f += kGtExpanders) {
+                    const uint8_t* r = src + f * step;
+                    const int o = (int)((uintptr_t)r & 3), nw = (o + FB + 3) >> 2;
+                    const uint32_t d = tc::smem_u32(raw) + f * a.raw_stride;
+                    for (int j = lane; j < nw; j += 32) cp_async4(d + 4 * j, r - o + 4 * j);
+                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                // the next chunk's rows into L2
+                const int more = min(a.nt - f0, (gend - gb) * FG), lines = (FB + 127) >> 7;
+                for (int i = tid - 128; i < (more - nf) * lines && i < a.gc * FG * lines; i += 32 * kGtExpanders) {
+                    const int f = i / lines;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (nf + f) * step + 128 * (i - f * lines)));
+                }
+            } else {  // rows at any byte address: those words, shifted
                 const int nw = (FB + 3) >> 2;
-                for (int f = xw; f < nf; f += 16)
+                for (int f = xw; f < nf; f += 4 * kGtExpanders)
                     for (int j = lane; j < nw; j += 32) {
                         uint32_t v[4];
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            if (f + 4 * k < nf) {
-                                const uint8_t* r = src + (f + 4 * k) * step;
+                            if (f + kGtExpanders * k < nf) {
+                                const uint8_t* r = src + (f + kGtExpanders * k) * step;
                                 const int o = (int)((uintptr_t)r & 3);
                                 const uint32_t* p32 = reinterpret_cast<const uint32_t*>(r - o) + j;
                                 const uint32_t lo = __ldg(p32), hi = 4 * j + 4 < o + FB ? __ldg(p32 + 1) : 0u;
@@ -333,11 +336,11 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
                             }
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            if (f + 4 * k < nf)
-                                reinterpret_cast<uint32_t*>(raw + (size_t)(f + 4 * k) * a.raw_stride)[j] = v[k];
+                            if (f + kGtExpanders * k < nf)
+                                reinterpret_cast<uint32_t*>(raw + (size_t)(f + kGtExpanders * k) * a.raw_stride)[j] = v[k];
                     }
             }
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kGtExpanders) : "memory");
             for (int t = T0; t < T1; ++t) {
                 const int ub = a.unit0[t], steps = gt_uni(a.unit0[t + 1] - ub);
                 for (int g = 0; g < ng; ++g)
@@ -353,7 +356,9 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
                         const uint32_t dst = sV + slot * VB + lane * 16;
                         const float4* jm = MIX ? a.jones + (size_t)c * a.A * 2 : nullptr;
                         for (int h = 0; h < 2 / P; ++h) {  // one pol: two sets of 32 frames
-                            const uint8_t* row = raw + (size_t)(g * FG + 32 * h + lane) * a.raw_stride;
+                            const int f = g * FG + 32 * h + lane;
+                            const uint8_t* row = raw + (size_t)f * a.raw_stride;
+                            if (!a.shift) row += ((uint32_t)(uintptr_t)src + (uint32_t)f * (uint32_t)step) & 3u;
 #pragma unroll
                             for (int o = 0; o < 2; ++o) {  // 16-byte chunks (8 K positions)
                                 constexpr int NE = EL / 2;
@@ -437,15 +442,20 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
         const uint32_t lanes = tmem + ((uint32_t)(32 * q4) << 16) + (P == 2 ? 64 : 32) * j;
         const size_t frame_step = (size_t)a.n_ch * a.tile_stride;
         unsigned nd = 0;
-        walk([&](int c, int cl, int T0, int T1, int gb, int ng) {
+        walk([&](int c, int cl, int T0, int T1, int gb, int ng, int) {
             if (!good) return;
             const int4 bx = a.box[c], tp = a.tbox[c];
             const int half = bx.z >> 1, pairs = tp.z * half;
-            const uint32_t part_bytes = (uint32_t)(P * tp.x) * pad64(2 * bx.z) * 2;
+            const int K1 = 2 * bx.z;
+            const uint32_t part_bytes = (uint32_t)(P * tp.x) * pad64(K1) * 2;
             for (int t = T0; t < T1; ++t) {
                 const int pr = (t - a.tile0[c]) * 128 + 32 * q4 + lane, y = pr / half, x = 2 * (pr - y * half);
                 const bool live = pr < pairs;
-                const uint32_t off = live ? tile_part_off(y, 2 * x, tp.x, P, part_bytes) + (P == 2 ? j * tp.x * 128 : 0) : 0;
+                uint32_t off = 0;
+                if (live) {
+                    off = a.dense ? tile_dense_off(y, 2 * x, tp.x, P, K1) : tile_part_off(y, 2 * x, tp.x, P, part_bytes);
+                    if (P == 2) off += j * tp.x * (a.dense ? tile_dense_row(2 * x, K1) : 128);
+                }
                 for (int g = 0; g < ng; ++g, ++nd) {
                     const int b = nd & 1, f0 = (gb + g) * FG + (P == 2 ? 0 : 32 * j), nf = min(32, a.nt - f0);
                     good = gt_wait(&d_full[b], (nd >> 1) & 1u);
@@ -528,10 +538,11 @@ cudaError_t put(T** dst, const std::vector<T>& v, size_t* bytes)
     return e;
 }
 
-// bytes of a staged frame row: whole words, an odd number of them
+// bytes of a staged frame row: the words that hold a byte of it, wherever it begins (rows of whole
+// words: at a word), an odd number of them
 int raw_stride(const epic_plan_s* p)
 {
-    const int words = (p->A * p->P * (p->bits / 4) + 3) / 4;
+    const int fb = p->A * p->P * (p->bits / 4), words = fb % 4 ? (fb + 6) / 4 : fb / 4;
     return 4 * (words | 1);
 }
 
@@ -639,7 +650,7 @@ epic_status grid_tc_setup(epic_plan_s* p)
                 ent0.push_back((int)ent.size());
             }
             unit0.push_back((int)u + steps);
-            cost += 400 + 260LL * steps;
+            cost += std::max(2500LL, 260LL * steps);
         }
         tile0[c + 1] = tile0[c] + tiles;
         wcum[c + 1] = wcum[c] + cost;
@@ -672,6 +683,7 @@ void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0,
     a.tbox = p->tc.tbox;
     a.tiles = (uint8_t*)p->scratch;
     a.tile_stride = p->tc.stride;
+    a.dense = dftgemm_dense(p);
     a.status = p->tc.status;
     a.tile0 = p->tc.gt_tile0;
     a.unit0 = p->tc.gt_unit0;
@@ -683,7 +695,9 @@ void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0,
     a.ngr = (nt + FG - 1) / FG;
     a.gc = p->tc.grid_frames;
     a.raw_stride = raw_stride(p);
-    a.vec = (fb % 16 == 0 && ((uintptr_t)volt & 15) == 0) ? 1 : 0;
+    // a sample (all pols) of 4, 2 or 1 bytes is read from shared memory at its offset in the words, and
+    // rows of whole words have no word to spare for an offset
+    a.shift = (uintptr_t)volt % (p->P * p->bits / 4) != 0 || (fb % 4 == 0 && (uintptr_t)volt % 4 != 0) ? 1 : 0;
     // about four units a block, in slices of a channel's tiles where there are too few groups
     const long long groups = (long long)n_ch * a.ngr;
     a.slices = (int)std::max<long long>(1, std::min<long long>(8, 4LL * p->sm_count / groups));

@@ -207,6 +207,22 @@ __device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint
         "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(HI)
         : "memory");
 }
+// Operand B's upper half in a register: panels of 64-byte (8 rows x 64 bytes) and 32-byte swizzle.
+constexpr uint32_t kDescSw64Hi = (512u >> 4) | (1u << 14) | (4u << 29);
+constexpr uint32_t kDescSw32Hi = (256u >> 4) | (1u << 14) | (6u << 29);
+__device__ __forceinline__ void mma_f16_lead_b(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t bhi, uint32_t idesc,
+                                               uint32_t accumulate, uint32_t lead)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 x, y;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "mov.b64 x, {%1, %6};\n\t"
+        "mov.b64 y, {%2, %7};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(kDescSw128Hi), "r"(bhi)
+        : "memory");
+}
 template <uint32_t HI = kDescSw128Hi>
 __device__ __forceinline__ void mma_f16_ta_lead(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t idesc,
                                                 uint32_t accumulate, uint32_t lead)
