@@ -95,7 +95,7 @@ void free_path_state(epic_plan_s* p)
     cudaFree(p->tc.gt_ent0);
     cudaFree(p->tc.gt_ent);
     cudaFree(p->tc.gt_el);
-    cudaFree(p->tc.gt_wcum);
+    cudaFree(p->tc.gt_tcum);
     cudaFree(p->scratch);
     int* status = p->tc.status;
     p->tc = epic::TcState{};

@@ -70,9 +70,10 @@ struct TcState {
     int* gt_tile0 = nullptr;       // tensor-core gridding (k_grid_tc.cu): first cell-pair tile of each channel,
     int* gt_unit0 = nullptr;       //   first K step of each tile, first weight and the elements
     int* gt_ent0 = nullptr;        //   of each step, the weights (offset in the operand, value),
-    int2* gt_ent = nullptr;        //   prefix sums of the channels' costs and the power of two
+    int2* gt_ent = nullptr;        //   prefix sums of the tiles' costs and the power of two
     int* gt_el = nullptr;          //   the weights are scaled by
-    long long* gt_wcum = nullptr;
+    long long* gt_tcum = nullptr;
+    std::vector<int> gt_tiles_h;   //   gt_tile0 on the host
     int gt_scale = 0;
     int4* gtask = nullptr;         // balanced gridding: per-channel task lists (device)
     int* gtask_off = nullptr;      // [C + 1]

@@ -2736,7 +2736,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWs3CtlRegs) : "memory");
         const int NB = a.nbt;
         if (warp == 2 && lane == 0) {  // A1 and tile-part copies
-            const size_t frame_step = (size_t)a.n_ch * a.tile_stride;
+            const size_t frame_step = a.dense ? a.tile_stride : (size_t)a.n_ch * a.tile_stride;
             uint32_t used = 0, ph_free = 0, cph = 0, aph = 0;  // used: copied, its S1 not yet waited for
             int b = 0;
             auto free_buf = [&](int j) -> bool {
@@ -2755,7 +2755,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 const int K1p = pad64(2 * a.box[c].z);
                 const uint32_t part_bytes = (uint32_t)(P * tp.x) * (a.dense ? 2 * a.box[c].z : K1p) * 2;
                 // next part to copy, advanced without division
-                const uint8_t* nxt = a.tiles + (size_t)cl * a.tile_stride + (size_t)s.fs * frame_step;
+                const uint8_t* nxt = a.tiles + (size_t)cl * (a.dense ? a.nt : 1) * a.tile_stride + (size_t)s.fs * frame_step;
                 const uint32_t a1_bytes = 256u * K1p;
                 const uint16_t* a1src = a.a1p + a.a1p_off[(size_t)c * a.n_g + g];
                 if (it > 0) tc::bulk_prefetch_l2(a1src, a1_bytes);

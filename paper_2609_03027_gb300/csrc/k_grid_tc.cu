@@ -11,8 +11,12 @@
 // w_hi v_hi + w_lo v_hi + w_hi v_lo is summed.  The gather kernels compute the same sums with FP32 FMAs and are
 // bound by shared-memory gathers and list walks (7.5 k SM cycles a frame of a 96 x 96 box); here
 // a frame takes its MMAs (64 cycles each, 4 a K step) and its tile stores.
-// Roles of the 640-thread block (one per SM), all walking the block's share of (channel, tile
-// slice, frame group) units alike; all hand-offs are mbarriers with bounded waits:
+// Work: units of one M-tile and one chunk of up to 4 (8) groups, channel by channel and chunk by chunk, cut
+// into one range of equal modelled cost a block.  What bounds a unit is its tile stores (2.7 k
+// cycles a group at the memory's write rate), so a finer cut matters more than the weights' reuse: ranges of whole
+// channels' groups (SKA-Low: 4 or 5 of 33 tiles) left a fifth of the time to the longest.
+// Roles of the 640-thread block (one per SM), all walking the block's range alike; all hand-offs are
+// mbarriers with bounded waits:
 //   warp 0      issues the MMAs of a K step: (even, odd) x (hi, lo), then frees its operands
 //   warps 1-3   build weight steps in a shared-memory ring: zeros, then the step's non-zero
 //               weights scattered (about 150 of 4096) -- far fewer bytes than reading the dense
@@ -64,11 +68,10 @@ struct GridTcArgs {
     const int* ent0;        // [steps + 1] first weight of each K step
     const int2* ent;        // weights: byte offset in the step's hi half, value (scaled)
     const int* el;          // 16 (complex weights: 8) elements of each K step
-    const long long* wcum;  // [C + 1] prefix sums of the channels' costs per group
+    const long long* tcum;  // [tiles + 1] prefix sums of the tiles' costs per group
     int dense;              // the tiles' K is not padded (k_dftgemm_ws3 reads them)
-    int slices;             // tile slices of a channel (more units than groups when those are few)
     int ngr;                // frame groups of the launch
-    int gc;                 // groups per staged chunk
+    int gc, nch;            // groups per staged chunk, chunks
     int raw_stride;         // bytes of a staged frame row (4 x odd)
     int shift;              // rows are staged shifted to a word boundary (samples at no multiple of their size)
     uint32_t vscale, vbias; // half2: 2^-s, and what the decode's offset becomes
@@ -150,6 +153,34 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
 
 __device__ __forceinline__ float gt_lo(float v) { return v - __half2float(__float2half_rn(v)); }
 
+// Largest i of [lo, hi) with f(i) <= s, by a whole warp (f increasing, f(lo) <= s).
+template <class F>
+__device__ __forceinline__ int gt_find(int lo, int hi, int lane, long long s, F&& f)
+{
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 31) / 32, i = lo + lane * step;
+        const int k = 31 - __clz(__ballot_sync(0xffffffffu, i < hi && f(i) <= s) | 1);
+        lo += k * step;
+        hi = min(hi, lo + step);
+    }
+    return lo;
+}
+
+// First unit (local channel, chunk, tile) of block b: the one at its share of the launch's cost.
+__device__ __forceinline__ int4 gt_start(const GridTcArgs& a, int b, int lane)
+{
+    const int* t0 = a.tile0 + a.c0;
+    const long long base = __ldg(a.tcum + __ldg(t0)), all = __ldg(a.tcum + __ldg(t0 + a.n_ch)) - base;
+    if (b == (int)gridDim.x) return make_int4(a.n_ch, 0, __ldg(t0 + a.n_ch), 0);
+    const long long s = all * a.nch * b / gridDim.x;
+    const int cl = gt_find(0, a.n_ch, lane, s, [&](int c) { return (__ldg(a.tcum + __ldg(t0 + c)) - base) * a.nch; });
+    const int ta = __ldg(t0 + cl), tb = __ldg(t0 + cl + 1);
+    const long long cb = __ldg(a.tcum + ta), w = __ldg(a.tcum + tb) - cb, r = s - (cb - base) * a.nch;
+    const int ch = (int)min((long long)(a.nch - 1), r / w);
+    const int t = gt_find(ta, tb, lane, r - ch * w, [&](int i) { return __ldg(a.tcum + i) - cb; });
+    return make_int4(cl, ch, t, 0);
+}
+
 template <int P, int BITS, bool CPLX, bool MIX>
 __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
 {
@@ -160,6 +191,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
     __shared__ uint64_t w_full[kGtRW], w_free[kGtRW], v_full[kGtRV], v_free[kGtRV], d_full[2], d_empty[2], drain;
     __shared__ uint32_t tmem_sh;
     __shared__ int err_sh;
+    __shared__ int4 range[2];  // first unit and the next block's
     const int tid = threadIdx.x, warp = gt_uni(tid >> 5), lane = tid & 31;
     if (warp == 0) {
         tc::tmem_alloc(&tmem_sh, 512);
@@ -182,6 +214,10 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
         err_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == 2 || warp == 3) {
+        const int4 r = gt_start(a, blockIdx.x + warp - 2, lane);
+        if (lane == 0) range[warp - 2] = r;
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -189,21 +225,25 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
     uint8_t* sbase = smem + ((1024u - (tc::smem_u32(smem) & 1023u)) & 1023u);
     const uint32_t sW = tc::smem_u32(sbase), sV = sW + kGtRW * kGtWBytes;
     uint8_t* raw = sbase + gt_raw_at(MIX);
-    const int S = a.slices, ngr = a.ngr;
-    const long long u0 = split_start(a.wcum, a.c0, a.n_ch, S, ngr, blockIdx.x, gridDim.x);
-    const long long u1 = split_start(a.wcum, a.c0, a.n_ch, S, ngr, blockIdx.x + 1, gridDim.x);
+    const int4 first = range[0], last = range[1];
 
     // Every role's walk through the block's units: f(channel, local channel, tiles [T0, T1), first
-    // group, groups, end of the segment's groups) per staged chunk.
+    // group, groups, end of the groups that follow for the same tiles' channel) per staged chunk.
     auto walk = [&](auto&& f) {
-        for (long long u = u0; u < u1;) {
-            const int cl = gt_uni((int)(u / ((long long)S * ngr))), r = gt_uni((int)(u % ((long long)S * ngr)));
-            const int sl = r / ngr, g0 = r - sl * ngr, c = a.c0 + cl;
-            const int g1 = gt_uni((int)min((long long)ngr, g0 + (u1 - u)));
-            const int ta = a.tile0[c], tn = a.tile0[c + 1] - ta;
-            const int T0 = gt_uni(ta + tn * sl / S), T1 = gt_uni(ta + tn * (sl + 1) / S);
-            for (int gb = g0; gb < g1; gb += a.gc) f(c, cl, T0, T1, gb, min(a.gc, g1 - gb), g1);
-            u += g1 - g0;
+        int cl = gt_uni(first.x), ch = gt_uni(first.y), T0 = gt_uni(first.z);
+        const int ecl = gt_uni(last.x), ech = gt_uni(last.y), eT = gt_uni(last.z);
+        while (cl < ecl || (cl == ecl && (ch < ech || (ch == ech && T0 < eT)))) {
+            const int c = a.c0 + cl, Tn = gt_uni(a.tile0[c + 1]);
+            const int T1 = cl == ecl && ch == ech ? eT : Tn, gb = ch * a.gc, g1 = min(a.ngr, gb + a.gc);
+            const bool more = ch + 1 < a.nch && (cl < ecl || ch < ech);
+            if (T1 > T0) f(c, cl, T0, T1, gb, g1 - gb, more ? min(a.ngr, g1 + a.gc) : g1);
+            if (++ch == a.nch) {
+                ch = 0;
+                ++cl;
+                T0 = Tn;
+            } else {
+                T0 = gt_uni(a.tile0[c]);
+            }
         }
     };
     bool good = true;  // a role whose wait ran out walks on without waiting or working
@@ -440,7 +480,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
         const int q4 = warp & 3, j = (warp >> 2) & 1;  // cell pairs; pol j, or half j of the one pol's frames
         constexpr int IM = P == 2 ? 32 : 64;            // columns from a frame's real part to its imaginary part
         const uint32_t lanes = tmem + ((uint32_t)(32 * q4) << 16) + (P == 2 ? 64 : 32) * j;
-        const size_t frame_step = (size_t)a.n_ch * a.tile_stride;
+        const size_t frame_step = a.dense ? a.tile_stride : (size_t)a.n_ch * a.tile_stride;
         unsigned nd = 0;
         walk([&](int c, int cl, int T0, int T1, int gb, int ng, int) {
             if (!good) return;
@@ -461,7 +501,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
                     good = gt_wait(&d_full[b], (nd >> 1) & 1u);
                     if (!good) return;
                     tc::fence_after_sync();
-                    uint8_t* q = a.tiles + ((size_t)f0 * a.n_ch + cl) * a.tile_stride + off;
+                    uint8_t* q = a.tiles + (a.dense ? (size_t)cl * a.nt + f0 : (size_t)f0 * a.n_ch + cl) * a.tile_stride + off;
                     uint32_t d[4][8];  // real and imaginary parts of the even and the odd cell, 8 frames
                     auto load = [&](int k) {
                         const uint32_t at = lanes + 256 * b + 8 * k;
@@ -596,7 +636,7 @@ epic_status grid_tc_setup(epic_plan_s* p)
     const int EL = cplx ? 8 : 16;
     std::vector<int> tile0(C + 1, 0), unit0(1, 0), ent0(1, 0), el;
     std::vector<int2> ent;
-    std::vector<long long> wcum(C + 1, 0);
+    std::vector<long long> tcum(1, 0);
     ent.reserve(p->n_contrib * (cplx ? 2 : 1));
     struct En {
         int e, off;
@@ -617,7 +657,6 @@ epic_status grid_tc_setup(epic_plan_s* p)
                     lists[pr >> 7].push_back(En{e, (x & 1) * 4096 + (pr & 127) * 16, (float)p->w_re[o], (float)p->w_im[o]});
                 }
         }
-        long long cost = 0;
         for (const std::vector<En>& L : lists) {
             int n = 0;  // distinct elements
             for (size_t i = 0; i < L.size(); ++i) n += i == 0 || L[i].e != L[i - 1].e;
@@ -650,10 +689,10 @@ epic_status grid_tc_setup(epic_plan_s* p)
                 ent0.push_back((int)ent.size());
             }
             unit0.push_back((int)u + steps);
-            cost += std::max(2500LL, 260LL * steps);
+            // SM cycles of a group, as measured: the tile's stores, or its weight steps when they do not stay
+            tcum.push_back(tcum.back() + (steps <= kGtRW ? 2700LL : 800LL * steps));
         }
         tile0[c + 1] = tile0[c] + tiles;
-        wcum[c + 1] = wcum[c] + cost;
         if (ent.size() > (1u << 30) || el.size() > (1u << 30)) return EPIC_ERR_UNSUPPORTED;
     }
     size_t bytes = 0;
@@ -662,8 +701,9 @@ epic_status grid_tc_setup(epic_plan_s* p)
     if (e == cudaSuccess) e = put(&p->tc.gt_ent0, ent0, &bytes);
     if (e == cudaSuccess) e = put(&p->tc.gt_ent, ent, &bytes);
     if (e == cudaSuccess) e = put(&p->tc.gt_el, el, &bytes);
-    if (e == cudaSuccess) e = put(&p->tc.gt_wcum, wcum, &bytes);
+    if (e == cudaSuccess) e = put(&p->tc.gt_tcum, tcum, &bytes);
     p->tc.gt_scale = s;
+    p->tc.gt_tiles_h = tile0;
     p->dt.dft_bytes += bytes;
     if (e != cudaSuccess) return cuda_fail(p, e, "tensor-core gridding tables");
     return EPIC_OK;
@@ -690,17 +730,18 @@ void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0,
     a.ent0 = p->tc.gt_ent0;
     a.ent = p->tc.gt_ent;
     a.el = p->tc.gt_el;
-    a.wcum = p->tc.gt_wcum;
+    a.tcum = p->tc.gt_tcum;
     const int fb = p->A * p->P * (p->bits / 4), FG = 64 / p->P;
     a.ngr = (nt + FG - 1) / FG;
-    a.gc = p->tc.grid_frames;
     a.raw_stride = raw_stride(p);
     // a sample (all pols) of 4, 2 or 1 bytes is read from shared memory at its offset in the words, and
     // rows of whole words have no word to spare for an offset
     a.shift = (uintptr_t)volt % (p->P * p->bits / 4) != 0 || (fb % 4 == 0 && (uintptr_t)volt % 4 != 0) ? 1 : 0;
-    // about four units a block, in slices of a channel's tiles where there are too few groups
-    const long long groups = (long long)n_ch * a.ngr;
-    a.slices = (int)std::max<long long>(1, std::min<long long>(8, 4LL * p->sm_count / groups));
+    // chunks of equal numbers of groups, short enough for about 16 units a block
+    const int tiles = p->tc.gt_tiles_h[c0 + n_ch] - p->tc.gt_tiles_h[c0], full = (a.ngr + p->tc.grid_frames - 1) / p->tc.grid_frames;
+    const int want = std::max(full, std::min(a.ngr, (16 * p->sm_count + tiles - 1) / tiles));
+    a.gc = (a.ngr + want - 1) / want;
+    a.nch = (a.ngr + a.gc - 1) / a.gc;
     const int off = p->bits == 4 ? 1024 + 8 : 1024 + 128;
     const uint32_t sc = (uint32_t)(15 - p->tc.gt_scale) << 10;  // FP16 2^-s
     const __half hb = __float2half((float)-ldexp((double)off, -p->tc.gt_scale));
@@ -710,7 +751,7 @@ void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0,
     a.unscale = (float)ldexp(1.0, -p->tc.gt_scale);
     a.vscale = sc | (sc << 16);
     a.vbias = (uint32_t)bb | ((uint32_t)bb << 16);
-    grid_tc_fn(p)<<<(unsigned)std::min<long long>(p->sm_count, groups * a.slices), kGtThreads, p->tc.grid_smem, s>>>(a);
+    grid_tc_fn(p)<<<(unsigned)std::min<long long>(p->sm_count, (long long)tiles * a.nch), kGtThreads, p->tc.grid_smem, s>>>(a);
 }
 
 }  // namespace epic
