@@ -45,6 +45,31 @@ __device__ __forceinline__ long long split_start(const long long* wcum, int c0, 
     return (long long)lo * per + u;
 }
 
+// Largest i of [lo, hi) with f(i) <= s, by a whole warp (f increasing, f(lo) <= s): two rounds of loads where one
+// thread's search takes a chain of eight.
+template <class F>
+__device__ __forceinline__ int warp_find(int lo, int hi, int lane, long long s, F&& f)
+{
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 31) / 32, i = lo + lane * step;
+        const int k = 31 - __clz(__ballot_sync(0xffffffffu, i < hi && f(i) <= s) | 1);
+        lo += k * step;
+        hi = min(hi, lo + step);
+    }
+    return lo;
+}
+
+// split_start (with weights) by a whole warp
+__device__ __forceinline__ long long split_start_warp(const long long* wcum, int c0, int n_ch, int ipc, int nt, int b, int G,
+                                                      int lane)
+{
+    const long long per = (long long)ipc * nt, base = __ldg(wcum + c0);
+    const long long s = per * (__ldg(wcum + c0 + n_ch) - base) * b / G;
+    const int lo = warp_find(0, n_ch, lane, s, [&](int c) { return per * (__ldg(wcum + c0 + c) - base); });
+    const long long w = __ldg(wcum + c0 + lo + 1) - __ldg(wcum + c0 + lo);
+    return (long long)lo * per + min(per, (s - per * (__ldg(wcum + c0 + lo) - base)) / w);
+}
+
 // K order of a grid tile's rows: the cell pair (x, x + 1), x even, takes K indices 2 x .. 2 x + 3 as
 // (re x, re x+1, im x, im x+1), so that a thread with a pair's sums stores 8 bytes and the pairs of
 // a row fill whole 32-byte sectors whatever the box width (with all real parts before the imaginary

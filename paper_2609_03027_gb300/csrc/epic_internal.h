@@ -93,7 +93,7 @@ struct TcState {
     long long* a1p_off = nullptr;
     int n_gp = 0;                  // 64-column pairs per channel
     float* partial = nullptr;      // k_dftgemm_ws3: partial sums of items split between blocks
-    int* counters = nullptr;       // k_dftgemm_ws3: per item, parts stored so far
+    int* counters = nullptr;       // k_dftgemm_ws3: per item and per slot, parts stored so far
     int split = -1;                // k_dftgemm_ws3 work split: -1 auto, 0 whole items, 1 equal shares
     int group = 0;                 // channels per launch: 0 groups of about two work items per SM,
     int cg_items = 0;              //   1 every channel (cg_items: the size group 0 gives)
@@ -105,7 +105,6 @@ struct TcState {
     bool parts = false;            // some channel has H > 1 (only k_dftgemm_ws3 takes it)
     int nbt = 2;                   // k_dftgemm_ws3: tile-part buffers in shared memory (2..6),
     unsigned ws3_sB2 = 0, ws3_b2 = 0;  //   where B2 starts, bytes of a B2 buffer
-    unsigned ws3_stage = 0;        //   where the interval stores' staging starts (0: none)
     int ws3_smem = 0;
     bool ws_old = false;           // the older warp-specialised kernels take the plan too
     size_t n_counters = 0;         // entries of `counters`

@@ -129,12 +129,12 @@ struct MmaArgs {
     const long long* a1p_off;
     float* partial;             // k_dftgemm_ws3: 2 slots per block of 4 x 128 x 64 partial sums
     int* counters;              // k_dftgemm_ws3: per item, blocks that stored a part (reset by the last)
+    int* run_counters;          //   per slot of a run's first part, likewise
     int sub;                    // k_dftgemm_ws3: samples per image set
     int iv0;                    // k_dftgemm_ws3: image set of the chunk's first sample
     int C;                      // channels of the plan (image sets are [C][nprod][N][N])
     const int4* tbox;           // k_dftgemm_ws3: per channel row parts (nyh, H, H nyh, 0)
     int dense;                  // k_dftgemm_ws3: the tiles' K is not padded (tile_dense_off)
-    unsigned sStage;            // k_dftgemm_ws3: 2 KB per epilogue-2 warp for interval stores, 0 = none
     int share;                  // k_dftgemm_ws3<1 or 2>: blocks that walk items of one channel side by side
     int nbt;                    // k_dftgemm_ws3: tile-part buffers in shared memory (2..6)
     const long long* wcum;      // k_dftgemm_ws3<1 or 2>: [C + 1] prefix sums of the channels' item costs per frame
@@ -2155,7 +2155,6 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 constexpr int kWs3Threads = 512;
 constexpr int kWs3CtlRegs = 64, kWs3E1Regs = 96, kWs3E2Regs = 176;
 static_assert(kWs3CtlRegs + kWs3E1Regs + 2 * kWs3E2Regs == 4 * 128, "setmaxnreg shares are the launch's registers");
-constexpr size_t kWs3Stage = 8 * 2048;  // interval stores: 2 KB for each epilogue-2 warp
 constexpr int kWs3MaxBlocks = 256;  // blocks per launch (one per SM) the split bookkeeping holds
 constexpr int kWs3MaxTileBufs = 6;  // tile-part buffers of k_dftgemm_ws3 (short row parts need more in flight)
 
@@ -2315,7 +2314,7 @@ __device__ __forceinline__ void ws3_epilogue2(uint32_t taddr, float (&xx)[32], f
     }
 }
 
-// 32 consecutive image pixels of one product (nk of them inside the image, a multiple of 8):
+// 32 consecutive image pixels of one product (nk of them inside the image, a multiple of 4):
 // written, or added to what is there
 __device__ __forceinline__ void ws3_store32(float* o, int nk, int accumulate, const float (&v)[32])
 {
@@ -2332,27 +2331,38 @@ __device__ __forceinline__ void ws3_store32(float* o, int nk, int accumulate, co
     }
 }
 
-// The same for a whole warp (rows ky0 + lane, 32 columns from kx0) through 2 KB of shared memory, so
-// that a store covers 8 rows x 64 bytes: the sub-integration schedule stores every few frames, and
-// a 16-byte store of each lane to a row of its own took 32 L1 wavefronts (LWA block of 128 samples with
-// an image set every 4: 0.62 ms of k_dftgemm_ws3).  o: pixel (ky0, kx0).
-__device__ __forceinline__ void ws3_store_rows(float* o, int N, int rows, int nk, int accumulate, int lane, float* stage,
-                                               const float (&v)[32])
+// A warp's 32 x 32 pixels of one product, lane = row, v = 32 columns: rows and columns within the image
+// (`rows`, nk: multiples of 4) written to o (the first pixel), or added to what is there.  Four lanes
+// exchange 16-byte pieces first, so that a store covers 8 rows x 64 bytes instead of 32 rows x 16.
+// For sub-integrations, which store every few frames (LWA block of 128 samples with an image set
+// every 4: 0.62 ms without, 0.35 with it and equal shares); whole items keep ws3_store32, whose stores wait
+// for the memory in either form, while these exchanges cost their frame loop 1 % by its register allocation.
+__device__ __forceinline__ void ws3_store_rows(float* o, int N, int rows, int nk, int accumulate, int lane,
+                                               float (&v)[32])
 {
+    auto swap = [&](int a, int b, int m) {  // the upper lane of a pair keeps b and gets the other's b for its a
+        const bool up = lane & m;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+        for (int e = 0; e < 4; ++e) {
+            const float t = __shfl_xor_sync(0xffffffffu, up ? v[a + e] : v[b + e], m);
+            if (up) v[a + e] = t;
+            else v[b + e] = t;
+        }
+    };
+    o += (size_t)(lane & ~3) * N + 4 * (lane & 3);
+    rows -= lane & ~3;
+    nk -= 4 * (lane & 3);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            *reinterpret_cast<float4*>(stage + lane * 16 + ((k ^ ((lane >> 1) & 3)) << 2)) =
-                make_float4(v[16 * h + 4 * k], v[16 * h + 4 * k + 1], v[16 * h + 4 * k + 2], v[16 * h + 4 * k + 3]);
-        __syncwarp();
-        const int c = lane & 3;
+    for (int h = 0; h < 32; h += 16) {
+        swap(h, h + 4, 1);
+        swap(h + 8, h + 12, 1);
+        swap(h, h + 8, 2);
+        swap(h + 4, h + 12, 2);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = 8 * i + (lane >> 2);
-            float4 w = *reinterpret_cast<const float4*>(stage + r * 16 + ((c ^ ((r >> 1) & 3)) << 2));
-            if (r < rows && 16 * h + 4 * c < nk) {
-                float4* q = reinterpret_cast<float4*>(o + (size_t)r * N + 16 * h + 4 * c);
+        for (int k = 0; k < 4; ++k) {  // row k of the four, piece lane & 3 of the 16 columns from h
+            if (k < rows && h < nk) {
+                float4* q = reinterpret_cast<float4*>(o + (size_t)k * N + h);
+                float4 w = make_float4(v[h + 4 * k], v[h + 4 * k + 1], v[h + 4 * k + 2], v[h + 4 * k + 3]);
                 if (accumulate) {
                     const float4 u = *q;
                     w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
@@ -2360,9 +2370,13 @@ __device__ __forceinline__ void ws3_store_rows(float* o, int N, int rows, int nk
                 *q = w;
             }
         }
-        __syncwarp();
     }
 }
+
+// What ws3_split_finish adds: n slots (0: nothing, another block will), of the item's block groups b0..b1.
+struct Ws3Split {
+    int n, b0, b1, run, slot[16];
+};
 
 // Partial sums of a split item, as epilogue-2 thread `tid2` of 256 holds them: float4 k of
 // product pr at ((8 pr + k) 256 + tid2) 4 (consecutive threads, consecutive 16 bytes).
@@ -2376,14 +2390,18 @@ __device__ __forceinline__ void ws3_store_partial(float* slot, int pr, int tid2,
 
 // A split work item (equal shares) after this block stored its part to its slot: the block
 // that stores the item's last part -- counted on the item's counter -- adds all parts in block
-// order and writes (or adds) the images.  start: first unit of every block group (shared memory,
-// filled once per launch: searching the plan's weights here, on one thread, cost 40 us an
-// item).  Kept out of line so that the frame loop's register allocation does not carry it.
+// order and writes (or adds) the images.  Of more than 8 parts, runs of about the root of their number are added
+// first, each by the block that stores its last part, into the slot of the run's first (four items
+// on 152 blocks: 38 parts took the last block 18 us, 6 + 7 take 6).  Parts are read one ahead of the sums.
+// start: first unit of every block group (shared memory; searching the plan's weights here, on one
+// thread, cost 40 us an item).  Kept out of line so that the frame loop's register allocation does not carry it.
 __device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float* o, int nk, int tid2,
-                                              const uint32_t* start, int* split_b)
+                                              const uint32_t* start, Ws3Split& sp)
 {
     const int Q = a.share, mine = item % Q;
     const uint32_t s0 = (uint32_t)(item / Q) * (uint32_t)a.nt, s1 = s0 + (uint32_t)a.nt - 1;
+    const size_t NN = (size_t)a.N * a.N;
+    auto slot_of = [&](int b) { return 2 * (b * Q + mine) + (s0 <= start[b] ? 0 : 1); };
     __threadfence();
     asm volatile("bar.sync 3, 256;" ::: "memory");
     if (tid2 == 0) {
@@ -2397,41 +2415,78 @@ __device__ __noinline__ void ws3_split_finish(const MmaArgs& a, int item, float*
             }
             return lo;
         };
-        const int b0 = owner(s0), b1 = owner(s1);
-        int n = 0;  // parts: blocks with any frames
-        for (int b = b0; b <= b1; ++b) n += start[b] != start[b + 1];
-        const bool last = atomicAdd(&a.counters[item], 1) == n - 1;
-        if (last) a.counters[item] = 0;  // ready for the next launch
-        split_b[0] = b0;
-        split_b[1] = last ? b1 : -1;
+        const int b0 = owner(s0), b1 = owner(s1), nb = b1 - b0 + 1;
+        int run = nb;
+        if (nb > 8)
+            for (run = 3; run * run < nb; ++run) {}
+        const int lo = b0 + ((int)blockIdx.x / Q - b0) / run * run, hi = min(b1, lo + run - 1);
+        int n = 0;  // the run's parts: blocks with any frames
+        for (int b = lo; b <= hi; ++b)
+            if (start[b] != start[b + 1]) sp.slot[n++] = slot_of(b);
+        int* ctr = nb > 8 ? a.run_counters + slot_of(lo) : a.counters + item;
+        const bool last = atomicAdd(ctr, 1) == n - 1;
+        if (last) *ctr = 0;  // ready for the next launch
+        sp.n = last ? n : 0;
+        sp.b0 = b0;
+        sp.b1 = b1;
+        sp.run = run;
     }
     asm volatile("bar.sync 3, 256;" ::: "memory");
-    const int b0 = split_b[0], b1 = split_b[1];
-    if (b1 >= 0 && nk > 0) {
+    bool whole = sp.b1 - sp.b0 < 8;  // the parts to add are all of the item's
+    while (sp.n > 0) {
         __threadfence();
-        const size_t NN = (size_t)a.N * a.N;
+        const int n = sp.n;
+        auto part = [&](int pr, int k) {
+            return reinterpret_cast<const float4*>(a.partial + (size_t)sp.slot[k] * 4 * 8192) + (size_t)8 * pr * 256 + tid2;
+        };
+        float4 next[8];
+        auto load = [&](int pr, int k) {
+            const float4* q = part(pr, k);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) next[i] = __ldcg(q + (size_t)i * 256);
+        };
+        load(0, 0);
         for (int pr = 0; pr < a.nprod; ++pr) {  // one product at a time: 32 live sums
             float sum[32];
 #pragma unroll
             for (int i = 0; i < 32; ++i) sum[i] = 0.f;
-            for (int b = b0; b <= b1; ++b) {
-                if (start[b] == start[b + 1]) continue;
-                const float4* q =
-                    reinterpret_cast<const float4*>(a.partial + (size_t)(2 * (b * Q + mine) + (s0 <= start[b] ? 0 : 1)) * 4 * 8192) +
-                    (size_t)8 * pr * 256 + tid2;
+            for (int k = 0; k < n; ++k) {
+                float4 u[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) u[i] = next[i];
+                if (k + 1 < n) load(pr, k + 1);
+                else if (pr + 1 < a.nprod) load(pr + 1, 0);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const float4 u = __ldcg(q + (size_t)i * 256);
-                    sum[4 * i] += u.x;
-                    sum[4 * i + 1] += u.y;
-                    sum[4 * i + 2] += u.z;
-                    sum[4 * i + 3] += u.w;
+                    sum[4 * i] += u[i].x;
+                    sum[4 * i + 1] += u[i].y;
+                    sum[4 * i + 2] += u[i].z;
+                    sum[4 * i + 3] += u[i].w;
                 }
             }
-            ws3_store32(o + (size_t)pr * NN, nk, a.accumulate, sum);
+            if (whole) ws3_store32(o + (size_t)pr * NN, nk, a.accumulate, sum);
+            else ws3_store_partial(a.partial + (size_t)sp.slot[0] * 4 * 8192, pr, tid2, sum);
         }
+        if (whole) break;
+        // a run is added: the last of the item's runs adds them
+        __threadfence();
+        asm volatile("bar.sync 3, 256;" ::: "memory");
+        if (tid2 == 0) {
+            int n2 = 0;
+            for (int lo = sp.b0; lo <= sp.b1; lo += sp.run)
+                for (int b = lo; b <= min(sp.b1, lo + sp.run - 1); ++b)
+                    if (start[b] != start[b + 1]) {
+                        sp.slot[n2++] = slot_of(b);
+                        break;
+                    }
+            const bool last = atomicAdd(a.counters + item, 1) == n2 - 1;
+            if (last) a.counters[item] = 0;
+            sp.n = last ? n2 : 0;
+        }
+        asm volatile("bar.sync 3, 256;" ::: "memory");
+        whole = true;
     }
-    asm volatile("bar.sync 3, 256;" ::: "memory");  // split_b is free again
+    asm volatile("bar.sync 3, 256;" ::: "memory");  // sp is free again
 }
 
 // The segments (work item, first frame, frames) of a block: every role walks them alike.
@@ -2481,7 +2536,7 @@ __device__ __forceinline__ bool ws3_e2_any(bool mine)
 template <int CUT, int P>
 __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int items, long long w0, long long w1,
                                             int warp, int lane, uint64_t* d2_full, uint64_t* d2_empty,
-                                            const uint32_t* start, int* split_b, uint8_t* stage)
+                                            const uint32_t* start, Ws3Split& sp)
 {
     const int q4 = warp & 3, hf = (warp >> 2) & 1, tid2 = 32 * (warp - 8) + lane;
     const uint32_t taddr = tmem + ((uint32_t)(32 * q4) << 16) + 256 + 64 * P * hf;
@@ -2501,11 +2556,17 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
             for (int i = 0; i < 32; ++i) xx[i] = yy[i] = rx[i] = ix[i] = 0.f;
         };
         auto store = [&](float* o) {
-            ws3_store32(o, nk, a.accumulate, xx);
+            auto one = [&](float* q, float(&v)[32]) {
+                if (CUT == 2)
+                    ws3_store_rows(q - (size_t)lane * a.N, a.N, min(32, a.N - (ky - lane)), min(32, a.N - kx0), a.accumulate,
+                                   lane, v);
+                else ws3_store32(q, nk, a.accumulate, v);
+            };
+            one(o, xx);
             if (P == 2) {
-                ws3_store32(o + NN, nk, a.accumulate, yy);
-                ws3_store32(o + 2 * NN, nk, a.accumulate, rx);
-                ws3_store32(o + 3 * NN, nk, a.accumulate, ix);
+                one(o + NN, yy);
+                one(o + 2 * NN, rx);
+                one(o + 3 * NN, ix);
             }
         };
         clear();
@@ -2519,20 +2580,7 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
             tc::fence_after_sync();
             ws3_epilogue2<P>(taddr, xx, yy, rx, ix, lane, &d2_empty[hf]);
             if (CUT != 1 && --left == 0) {  // write (or add) this interval's sums (without sub-integrations: never)
-                float* o = a.out + (size_t)iv * a.C * a.nprod * NN + px;
-                if (stage) {
-                    float* st = reinterpret_cast<float*>(stage) + (warp - 8) * 512;
-                    const int rows = min(32, a.N - (ky - lane)), nkw = min(32, a.N - kx0);
-                    o -= (size_t)lane * a.N;
-                    ws3_store_rows(o, a.N, rows, nkw, a.accumulate, lane, st, xx);
-                    if (P == 2) {
-                        ws3_store_rows(o + NN, a.N, rows, nkw, a.accumulate, lane, st, yy);
-                        ws3_store_rows(o + 2 * NN, a.N, rows, nkw, a.accumulate, lane, st, rx);
-                        ws3_store_rows(o + 3 * NN, a.N, rows, nkw, a.accumulate, lane, st, ix);
-                    }
-                } else {
-                    store(o);
-                }
+                store(a.out + (size_t)iv * a.C * a.nprod * NN + px);
                 clear();
                 ++iv;
                 left = a.sub;
@@ -2549,7 +2597,7 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
                 ws3_store_partial(slot, 2, tid2, rx);
                 ws3_store_partial(slot, 3, tid2, ix);
             }
-            ws3_split_finish(a, s.item, a.out + px, nk, tid2, start, split_b);
+            ws3_split_finish(a, s.item, a.out + px, nk, tid2, start, sp);
         } else if (CUT != 2 && a.sub == 0) {
             store(a.out + px);
         }
@@ -2681,8 +2729,9 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     __shared__ Ws3Bars m;
     __shared__ uint32_t tmem_sh;
     __shared__ int err_sh;
-    __shared__ uint32_t start[CUT ? kWs3MaxBlocks + 1 : 1];  // first unit of every block group
-    __shared__ int split_b[2];  // blocks of a split item; the second is -1 unless this block completes it
+    __shared__ uint32_t start[CUT == 1 ? kWs3MaxBlocks + 1 : 1];  // first unit of every block group
+    __shared__ uint32_t wb[2];                                    // this one's and the next's
+    __shared__ Ws3Split split;
     const int tid = threadIdx.x, warp = ws3_uni(tid >> 5), lane = tid & 31;
     if (warp == 0) {
         tc::tmem_alloc(&tmem_sh, 512);
@@ -2708,11 +2757,11 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int ipc = a.n_kb * a.n_g, items = a.n_ch * ipc;  // items per channel, of the launch
-    if (CUT) {
-        const int unit = CUT == 2 ? a.sub : 1;  // frames that stay together
-        for (int b = tid; b <= (int)(gridDim.x / a.share); b += kWs3Threads)
-            start[b] = (uint32_t)unit *
-                       (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt / unit, b, gridDim.x / a.share);
+    const int unit = CUT == 2 ? a.sub : 1;  // frames that stay together
+    if (CUT && (warp == 2 || warp == 3)) {
+        const long long f = split_start_warp(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt / unit,
+                                             blockIdx.x / a.share + warp - 2, gridDim.x / a.share, lane);
+        if (lane == 0) wb[warp - 2] = (uint32_t)unit * (uint32_t)f;
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -2726,7 +2775,7 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     // this block's part of the launch.  CUT: its group's (item group, frame) units [wb0, wb1) in
     // item-major order (CUT 1: items cut at range boundaries are summed by the block that stores their last part);
     // else whole items blockIdx.x, + gridDim.x, ...
-    const long long wb0 = CUT ? start[blockIdx.x / a.share] : 0, wb1 = CUT ? start[blockIdx.x / a.share + 1] : 0;
+    const long long wb0 = CUT ? wb[0] : 0, wb1 = CUT ? wb[1] : 0;
     Ws3Seg s;
     long long w = wb0;
     bool good = true;
@@ -2914,11 +2963,13 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     } else {
         // ------------------------------------------------------------ epilogue 2
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWs3E2Regs) : "memory");
-        uint8_t* stage = CUT != 1 && a.sStage ? sbase + a.sStage : nullptr;
-        good = P == 2 ? ws3_role_e2<CUT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
-                                              stage)
-                      : ws3_role_e2<CUT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split_b,
-                                              stage);
+        if (CUT == 1) {  // while the first frame is on its way
+            for (int b = tid - 256; b <= (int)(gridDim.x / a.share); b += 256)
+                start[b] = (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt, b, gridDim.x / a.share);
+            asm volatile("bar.sync 3, 256;" ::: "memory");
+        }
+        good = P == 2 ? ws3_role_e2<CUT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split)
+                      : ws3_role_e2<CUT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split);
         if (!good) err_sh = 1;
     }
     tc::fence_before_sync();
@@ -3434,11 +3485,8 @@ epic_status dftgemm_setup(epic_plan_s* p)
         const size_t b2w = align_up(2ull * 128 * P * 2 * nyh_max, 1024);
         // as many tile-part buffers (2..6) as fit: a part's copy takes longer than its step
         int nbt = kWs3MaxTileBufs;
-        const size_t fixed = a1p + 2 * b2w;
-        // sub-integrations: staging of the interval stores where it fits
-        const size_t stage = p->sub > 0 && fixed + 2 * b1p + kWs3Stage <= limit ? kWs3Stage : 0;
-        while (nbt > 2 && fixed + nbt * b1p + stage > limit) --nbt;
-        const size_t need_ws = fixed + nbt * b1p + stage;
+        while (nbt > 2 && a1p + nbt * b1p + 2 * b2w > limit) --nbt;
+        const size_t need_ws = a1p + nbt * b1p + 2 * b2w;
         if (need_ws > limit) continue;
         p->tc.ws = true;
         p->tc.parts = split;
@@ -3450,7 +3498,6 @@ epic_status dftgemm_setup(epic_plan_s* p)
         p->tc.d1_cols = dmax;
         p->tc.ws3_sB2 = (unsigned)(a1p + nbt * b1p);
         p->tc.ws3_b2 = (unsigned)b2w;
-        p->tc.ws3_stage = stage ? (unsigned)(a1p + nbt * b1p + 2 * b2w) : 0u;
         p->tc.ws3_smem = (int)(need_ws + 1024);
         // the older variants: two tile buffers, B2 with both parts' rows, one part per channel
         const size_t b2o = align_up(2ull * 2 * 64 * P * pad64(2 * nyh_max), 1024), need_old = a1p + 2 * b1p + 2 * b2o;
@@ -3758,7 +3805,8 @@ epic_status dftgemm_setup(epic_plan_s* p)
         return EPIC_ERR_UNSUPPORTED;
     }
     if (p->tc.ws && e == cudaSuccess) {
-        const size_t n_items = (size_t)C * n_kb * n_gp;  // the largest channel group
+        // items of the largest channel group, and the slots
+        const size_t n_items = (size_t)C * n_kb * n_gp + 2 * (size_t)p->sm_count;
         e = cudaMalloc(&p->tc.partial, (size_t)p->sm_count * 2 * 4 * 8192 * sizeof(float));
         if (e == cudaSuccess) e = cudaMalloc(&p->tc.counters, n_items * sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(p->tc.counters, 0, n_items * sizeof(int));
@@ -3959,7 +4007,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.counters = p->tc.counters;
                     a.sB2 = p->tc.ws3_sB2;
                     a.b2_bytes = p->tc.ws3_b2;
-                    a.sStage = p->tc.ws3_stage;
+                    a.run_counters = p->tc.counters + (p->tc.n_counters - 2 * (size_t)p->sm_count);
                     a.dense = dftgemm_dense(p);
                     if ((p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel

@@ -153,19 +153,6 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
 
 __device__ __forceinline__ float gt_lo(float v) { return v - __half2float(__float2half_rn(v)); }
 
-// Largest i of [lo, hi) with f(i) <= s, by a whole warp (f increasing, f(lo) <= s).
-template <class F>
-__device__ __forceinline__ int gt_find(int lo, int hi, int lane, long long s, F&& f)
-{
-    while (hi - lo > 1) {
-        const int step = (hi - lo + 31) / 32, i = lo + lane * step;
-        const int k = 31 - __clz(__ballot_sync(0xffffffffu, i < hi && f(i) <= s) | 1);
-        lo += k * step;
-        hi = min(hi, lo + step);
-    }
-    return lo;
-}
-
 // First unit (local channel, chunk, tile) of block b: the one at its share of the launch's cost.
 __device__ __forceinline__ int4 gt_start(const GridTcArgs& a, int b, int lane)
 {
@@ -173,11 +160,11 @@ __device__ __forceinline__ int4 gt_start(const GridTcArgs& a, int b, int lane)
     const long long base = __ldg(a.tcum + __ldg(t0)), all = __ldg(a.tcum + __ldg(t0 + a.n_ch)) - base;
     if (b == (int)gridDim.x) return make_int4(a.n_ch, 0, __ldg(t0 + a.n_ch), 0);
     const long long s = all * a.nch * b / gridDim.x;
-    const int cl = gt_find(0, a.n_ch, lane, s, [&](int c) { return (__ldg(a.tcum + __ldg(t0 + c)) - base) * a.nch; });
+    const int cl = warp_find(0, a.n_ch, lane, s, [&](int c) { return (__ldg(a.tcum + __ldg(t0 + c)) - base) * a.nch; });
     const int ta = __ldg(t0 + cl), tb = __ldg(t0 + cl + 1);
     const long long cb = __ldg(a.tcum + ta), w = __ldg(a.tcum + tb) - cb, r = s - (cb - base) * a.nch;
     const int ch = (int)min((long long)(a.nch - 1), r / w);
-    const int t = gt_find(ta, tb, lane, r - ch * w, [&](int i) { return __ldg(a.tcum + i) - cb; });
+    const int t = warp_find(ta, tb, lane, r - ch * w, [&](int i) { return __ldg(a.tcum + i) - cb; });
     return make_int4(cl, ch, t, 0);
 }
 
