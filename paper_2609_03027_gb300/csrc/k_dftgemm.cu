@@ -2807,7 +2807,18 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 const uint8_t* nxt = a.tiles + (size_t)cl * (a.dense ? a.nt : 1) * a.tile_stride + (size_t)s.fs * frame_step;
                 const uint32_t a1_bytes = 256u * K1p;
                 const uint16_t* a1src = a.a1p + a.a1p_off[(size_t)c * a.n_g + g];
-                if (it > 0) tc::bulk_prefetch_l2(a1src, a1_bytes);
+                auto copy_a1 = [&]() {
+                    tc::mbar_expect_tx(&m.bar_a, a1_bytes);
+                    tc::bulk_g2s(sA1, a1src, a1_bytes, &m.bar_a);
+                    aph ^= 1u;
+                    cph |= 0x80u;
+                };
+                if (it > 0) {
+                    tc::bulk_prefetch_l2(a1src, a1_bytes);
+                } else {
+                    copy_a1();
+                    tc::grid_wait();  // the tiles, of the kernel before, are complete
+                }
                 int nh = 0;
                 for (int k = 0; k < NU && good; ++k) {
                     good = free_buf(b);
@@ -2823,18 +2834,16 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                     } else {
                         nxt += part_bytes;
                     }
-                    if (k == min(NB, NU) - 1) {
+                    if (it > 0 && k == min(NB, NU) - 1) {
                         // A1 once every S1 of the item before is done: its parts are in the buffers
                         // refilled above, or in those this short segment left alone
                         for (int j = 0; j < NB - NU && good; ++j) good = free_buf((b + j) % NB);
                         if (!good) break;
-                        tc::mbar_expect_tx(&m.bar_a, a1_bytes);
-                        tc::bulk_g2s(sA1, a1src, a1_bytes, &m.bar_a);
-                        aph ^= 1u;
-                        cph |= 0x80u;
+                        copy_a1();
                     }
                 }
             }
+            tc::grid_wait();  // blocks without work too: a launch never ends before the one that it waits for
             for (int j = 0; j < NB && good; ++j) good = free_buf(j);
             if (!good) {  // a wait ran out: no bulk copy may be in flight when the block releases its memory
                 err_sh = 1;
@@ -2976,6 +2985,24 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem, 512);
     if (err_sh && tid == 0) atomicExch(a.status, 1);
+}
+
+// early: behind a gridding kernel whose blocks let it start as they end, its tables, barriers and operands
+// load meanwhile, and its copy thread waits for the whole grid of tiles.  The first frame took 8 to 12 us of
+// every launch (cold operand tables, and reads that wait for the tiles on their way out of L2).
+void ws3_launch(void (*fn)(MmaArgs), int grid, int smem, cudaStream_t s, const MmaArgs& a, bool early)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kWs3Threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = early;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, fn, a);  // errors: as after any launch, by cudaGetLastError
 }
 
 }  // namespace
@@ -4009,18 +4036,32 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.b2_bytes = p->tc.ws3_b2;
                     a.run_counters = p->tc.counters + (p->tc.n_counters - 2 * (size_t)p->sm_count);
                     a.dense = dftgemm_dense(p);
-                    if ((p->tc.split == 1 || (p->tc.split < 0 && items % p->sm_count != 0)) &&
+                    // modelled SM cycles: the launch's per SM, and of whole items dealt in rounds
+                    const int ipc = a.n_kb * a.n_g, rounds = (items + p->sm_count - 1) / p->sm_count;
+                    long long sum = 0, most = 0;
+                    for (int c = c0; c < c0 + ng; ++c) {
+                        const long long w = ws3_item_cost(p->tc.tbox_h[c]);
+                        sum += w;
+                        most = std::max(most, w);
+                    }
+                    const long long equal = sum * ipc * nt / p->sm_count, whole = most * rounds * nt;
+                    // Sharing items costs 40 k cycles of partial sums and further segments (LWA bursts of 4, 16, 32
+                    // and 64 samples: 46, 63, 83, 121 us in equal shares, 24, 47, 72, 120 us as 264 whole items)
+                    const bool cut = items % p->sm_count != 0 && (p->sub > 0 || whole > equal + 40000);
+                    // Starting under the gridding kernel's last blocks saves 5 to 9 us of a launch but scatters blocks
+                    // that share tiles over the chip, 1 to 2 % of long ones (tiny station 33 -> 29 us, LWA burst of 32
+                    // samples 115 -> 108, LWA block of 1000 1781 -> 1799)
+                    const bool early = equal < 500000;
+                    if ((p->tc.split == 1 || (p->tc.split < 0 && cut)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
                     {
                         // as many as divide a channel's items and the blocks (two for N = 128, eight for N = 256)
-                        const int ipc = a.n_kb * a.n_g;
                         a.share = 8;
                         while (ipc % a.share || p->sm_count % a.share) a.share >>= 1;
-                        if (a.sub > 0) k_dftgemm_ws3<2><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
-                        else k_dftgemm_ws3<1><<<p->sm_count, kWs3Threads, p->tc.ws3_smem, s>>>(a);
+                        ws3_launch(a.sub > 0 ? k_dftgemm_ws3<2> : k_dftgemm_ws3<1>, p->sm_count, p->tc.ws3_smem, s, a, early);
                     } else {
                         a.share = 1;
-                        k_dftgemm_ws3<0><<<grid, kWs3Threads, p->tc.ws3_smem, s>>>(a);
+                        ws3_launch(k_dftgemm_ws3<0>, grid, p->tc.ws3_smem, s, a, early);
                     }
                 }
                 else if (p->tc.ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);

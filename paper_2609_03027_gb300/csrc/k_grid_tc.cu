@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
     uint8_t* sbase = smem + ((1024u - (tc::smem_u32(smem) & 1023u)) & 1023u);
     const uint32_t sW = tc::smem_u32(sbase), sV = sW + kGtRW * kGtWBytes;
     uint8_t* raw = sbase + gt_raw_at(MIX);
+    if (tid == 0) tc::grid_launch_dependents();  // k_dftgemm_ws3, which waits for the tiles
     const int4 first = range[0], last = range[1];
 
     // Every role's walk through the block's units: f(channel, local channel, tiles [T0, T1), first

@@ -207,6 +207,10 @@ __device__ __forceinline__ void mma_f16_lead(uint32_t d_tmem, uint32_t alo, uint
         "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "n"(HI)
         : "memory");
 }
+// Programmatic dependent launch: the next kernel of the stream may start where blocks of this one have
+// ended / wait for the kernel before and its memory (nothing to wait for after an ordinary launch)
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Operand B's upper half in a register: panels of 64-byte (8 rows x 64 bytes) and 32-byte swizzle.
 constexpr uint32_t kDescSw64Hi = (512u >> 4) | (1u << 14) | (4u << 29);
 constexpr uint32_t kDescSw32Hi = (256u >> 4) | (1u << 14) | (6u << 29);
