@@ -18,6 +18,7 @@
 
 #include "epic_internal.h"
 #include "kcommon.cuh"
+#include "tc_ptx.cuh"
 
 namespace epic {
 
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
     constexpr int L1 = ilog2(N1), L2 = ilog2(N2), YR = RPC / (F * P);
     static_assert(YR >= 1, "a batch holds a row of every frame and pol");
     extern __shared__ float2 sm[];
+    tc::grid_launch_dependents();  // k_plain_cols
     const int tid = threadIdx.x, c = blockIdx.y, f0 = F * blockIdx.x;
     const int4 b = box[c];
     const int nx = min(b.z, N - b.x), ny = min(b.w, N - b.y);  // box padding beyond the grid holds nothing
@@ -231,6 +233,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) z[n1] = yr[j * (N1 + 1) + n1];
         dft_reg<N1>(z);
+        if (yb == 0) tc::grid_wait();  // the chunk before is read
         if (f0 + rf < nt && yb + ry < ny) {
             float2* o = rows + ((((size_t)(f0 + rf) * C + c) * P + rp) * ny_max + yb + ry) * N + j;
 #pragma unroll
@@ -337,6 +340,8 @@ __global__ void __launch_bounds__(TX * N2) k_plain_cols(const float2* __restrict
     };
     clear();
     bool add = accumulate != 0;
+    tc::grid_launch_dependents();  // k_plain_rows of the next chunk
+    tc::grid_wait();               // this chunk's rows are complete
     if (ST) {
         fetch(ta);
         fetch(ta + 1);
@@ -795,6 +800,25 @@ epic_status plain_setup(epic_plan_s* p)
     return plain_set_chunk(p, kGridBudget);
 }
 
+// A launch that may start where blocks of the kernel before it on the stream have ended (early; that kernel
+// allows it, and this one waits for its end before it touches what the other reads or writes): a chunk's two
+// kernels of 0.2 ms each left the chip half empty at every end.
+template <class F, class... X>
+static void launch_early(bool early, F* fn, dim3 grid, int threads, size_t smem, cudaStream_t s, X... x)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = early;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, fn, x...);  // errors: as after any launch, by cudaGetLastError
+}
+
 epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s, float* out, bool accumulate)
 {
     const int C = p->C, P = p->P, N = p->N, A = p->A;
@@ -809,9 +833,9 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             const RegFft rf = reg_fft_for(p, form == kFrameStaged);
             const int ny_max = std::min(p->box_max_y, N);
             ev_begin(p, "k_plain_rows", s);
-            rf.rows<<<dim3((nt + kRowFrames - 1) / kRowFrames, C), kRowThreads, rows_base_smem(p, rf) + frame_smem(p, form), s>>>(
-                volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off, p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w,
-                p->dt.jones, form == kFrameBytes ? 1 : 0, rows_ld(std::min(p->box_max_x, N)), ny_max, p->dt.twiddle, grid);
+            launch_early(t0 > 0, rf.rows, dim3((nt + kRowFrames - 1) / kRowFrames, C), kRowThreads,
+                         rows_base_smem(p, rf) + frame_smem(p, form), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
+                         p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, rows_ld(std::min(p->box_max_x, N)), ny_max, p->dt.twiddle, grid);
             ev_end(p, s);
             // slices of whole intervals, or of at least four frames; the same for every chunk of the call,
             // whose partial sums add up over the chunks
@@ -821,9 +845,9 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
                 partial = reinterpret_cast<float*>(
                     (uint8_t*)p->scratch + ((sizeof(float2) * (size_t)p->time_chunk * C * P * ny_max * N + 255) & ~(size_t)255));
             ev_begin(p, "k_plain_cols", s);
-            rf.cols<<<dim3(N / rf.col_tile, C, S), rf.col_threads, cols_smem_for(p, rf), s>>>(
-                grid, nt, C, ny_max, p->dt.box, p->dt.twiddle, out, partial, partial ? t0 > 0 : acc, p->sub,
-                p->sub > 0 ? t0 / p->sub : 0);
+            launch_early(true, rf.cols, dim3(N / rf.col_tile, C, S), rf.col_threads, cols_smem_for(p, rf), s,
+                         (const float2*)grid, nt, C, ny_max, p->dt.box, p->dt.twiddle, out, partial, partial ? t0 > 0 : acc,
+                         p->sub, p->sub > 0 ? t0 / p->sub : 0);
             ev_end(p, s);
             if (partial && t0 + nt == T) {
                 const size_t n4 = (size_t)C * p->nprod * N * N / 4;
