@@ -130,7 +130,8 @@ __host__ __device__ constexpr size_t rows_fft_smem()
 }
 
 // Gridded and row-transformed frames (LWA station: 5.5 ms a block, 2.9 ms of it the 12.9 GB of row
-// stores, the rest the gather's dependent list and voltage reads): block = frames 2 blockIdx.x, + 1 of channel blockIdx.y.
+// stores, the rest the gather's dependent list and voltage reads): block = frames 2 blockIdx.x, + 1 of
+// channel blockIdx.y, slice blockIdx.z of the box rows.
 // Rows go in batches of 256 / N2 (both frames, all pols, a few y): the batch's cells are gathered
 // one per thread and step, both frames and pols at once, then N2 threads a row run the two FFT
 // passes (thread j takes n1 = j, j + N2 in pass 1 and k2 = j in pass 2; Y is stored [k2][n1] with
@@ -153,7 +154,9 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
     tc::grid_launch_dependents();  // k_plain_cols
     const int tid = threadIdx.x, c = blockIdx.y, f0 = F * blockIdx.x;
     const int4 b = box[c];
-    const int nx = min(b.z, N - b.x), ny = min(b.w, N - b.y);  // box padding beyond the grid holds nothing
+    // box padding beyond the grid holds nothing; the rows end with this block's slice of the batches
+    const int nx = min(b.z, N - b.x), nb = (min(b.w, N - b.y) + YR - 1) / YR;
+    const int ny = min(min(b.w, N - b.y), nb * ((int)blockIdx.z + 1) / (int)gridDim.z * YR);
     float2* tw = sm;               // [N2][N1]
     float2* y = tw + N;            // [RPC][N2][N1 + 1]
     float2* g = y + RPC * S;       // [F][P][YR][ld]
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
     const int* ptr = cell_ptr + cell_off[c];
     const int rl = tid / N2, j = tid % N2;             // this thread's row of a batch and its place in it
     const int rf = rl / (P * YR), rp = rl / YR % P, ry = rl % YR;
-    for (int yb = 0; yb < ny; yb += YR) {
+    for (int yb = nb * (int)blockIdx.z / (int)gridDim.z * YR; yb < ny; yb += YR) {
         __syncthreads();  // frames staged; the last batch's rows are read
         for (int i = tid; i < YR * nx; i += kRowThreads) {
             const int r = i / nx, x = i - r * nx;
@@ -233,7 +236,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) z[n1] = yr[j * (N1 + 1) + n1];
         dft_reg<N1>(z);
-        if (yb == 0) tc::grid_wait();  // the chunk before is read
+        tc::grid_wait();  // the chunk before is read (later batches: at once)
         if (f0 + rf < nt && yb + ry < ny) {
             float2* o = rows + ((((size_t)(f0 + rf) * C + c) * P + rp) * ny_max + yb + ry) * N + j;
 #pragma unroll
@@ -437,6 +440,7 @@ struct RegFft {
                  const float4*, int, int, int, const float2*, float2*);
     void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int);
     int col_tile, col_threads;
+    int rows_batch;               // box rows a block transforms at once
     size_t rows_fft, rows_cells;  // rows_cells: per box column, what a block gathers per batch
     size_t cols_smem, cols_row;   // cols_row: per box row, the staged frames
 };
@@ -453,6 +457,7 @@ RegFft reg_fft_p(bool staged, bool cplx)
     f.cols = k_plain_cols<N1, N2, TX, P>;
     f.col_tile = TX;
     f.col_threads = TX * N2;
+    f.rows_batch = kRowThreads / N2 / (kRowFrames * P);
     f.rows_fft = rows_fft_smem<N1, N2>();
     f.rows_cells = sizeof(float2) * (kRowThreads / N2);  // F P YR rows
     f.cols_smem = sizeof(float2) * ((size_t)N + (size_t)P * N * TX);
@@ -833,7 +838,11 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             const RegFft rf = reg_fft_for(p, form == kFrameStaged);
             const int ny_max = std::min(p->box_max_y, N);
             ev_begin(p, "k_plain_rows", s);
-            launch_early(t0 > 0, rf.rows, dim3((nt + kRowFrames - 1) / kRowFrames, C), kRowThreads,
+            // slices of the rows where frames and channels alone leave fewer than eight blocks an SM (one channel
+            // of a 512-pixel grid: 2.45 ms a block of 1024 samples with 128 blocks a chunk, 1.97 with slices)
+            const int fb = (nt + kRowFrames - 1) / kRowFrames, batches = (ny_max + rf.rows_batch - 1) / rf.rows_batch;
+            const int Z = std::max(1, std::min(batches, (int)(8LL * p->sm_count / ((long long)fb * C))));
+            launch_early(t0 > 0, rf.rows, dim3(fb, C, Z), kRowThreads,
                          rows_base_smem(p, rf) + frame_smem(p, form), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
                          p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, rows_ld(std::min(p->box_max_x, N)), ny_max, p->dt.twiddle, grid);
             ev_end(p, s);
