@@ -233,8 +233,8 @@ epic_status epic_plan_get_info(epic_plan_t plan, epic_plan_info* info);
  *                 mma_kernel   1: epilogue warps issue the tensor-core work, 2: a
  *                              control warp does, 3: a control warpgroup with its own
  *                              register budget does (when the occupied box allows each);
- *                 split        work of the control-warp kernel: -1 automatic (equal shares unless
- *                              the items divide evenly), 0 whole work items per SM, 1 equal
+ *                 split        work of the control-warp kernel: -1 automatic (equal shares where
+ *                              whole items would idle SMs for longer), 0 whole work items, 1 equal
  *                              (item, time sample) shares per SM;
  *                 grid_kernel  gridding kernel: 1 row-major cell walk, 2 cells in lists sorted
  *                              by length (Gaussian GCF, when its tiles fit in shared memory),

@@ -2128,7 +2128,8 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 // pipe is busy) hold up none of them.  What bounds it is the tensor pipe with its
 // shared-memory operand reads: a frame of an LWA-station item (48 x 48 box, two pols) is
 // 1056 cycles of MMAs at the math rate.  With both epilogues on the same 16 warps, one
-// after the other (the form before this one), a frame took about 2.9 k cycles.
+// after the other (the form before this one), a frame took about 2.9 k cycles, now 1.78 k (LWA block
+// of 1000 samples 2.47 -> 1.24 ms, SKA-Low block 6.42 -> 3.19, dense lattice 2.67 -> 1.33).
 // Work item, operands and TMEM layout as k_dftgemm_ws2, except that a channel's box rows
 // may come in H row parts (tall boxes): stage 2 sums over the box rows, so part h of frame t
 // is a step of its own -- its tile part through stage 1 (D1 of P nyh columns), epilogue 1 and
@@ -2149,9 +2150,9 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
 //     -> at h = H-1 d2_full[f]; after both halves b2_free[u&1]
 //   epilogue-2 warps 8-11 (half 0) and 12-15 (half 1), per frame t:
 //     wait d2_full[f](t) -> D2 to registers -> arrive d2_empty[f] -> products
-// Registers: 512 threads x 128 at launch = 128 control x 40 + 128 epilogue-1 x 88 + 256
-// epilogue-2 x 192: an epilogue-2 thread holds 32 pixels (128 sums) and 48 registers of
-// TMEM loads in flight.
+// Registers: 512 threads x 128 at launch = 128 control x 64 + 128 epilogue-1 x 96 + 256
+// epilogue-2 x 176: an epilogue-2 thread holds 32 pixels (128 sums) and 32 registers of
+// TMEM loads in flight (more for it and fewer for the others spilled in their loops).
 constexpr int kWs3Threads = 512;
 constexpr int kWs3CtlRegs = 64, kWs3E1Regs = 96, kWs3E2Regs = 176;
 static_assert(kWs3CtlRegs + kWs3E1Regs + 2 * kWs3E2Regs == 4 * 128, "setmaxnreg shares are the launch's registers");
@@ -3022,9 +3023,10 @@ epic_status dftgemm_set_kernel(epic_plan_s* p, int variant)
 
 static epic_status upload_item_order(epic_plan_s* p);
 
-// SM cycles of one frame of a work item with row parts r = (nyh, H, H nyh), as measured with 152
-// channels of one frequency: 24 x 24 box 1444, 48 x 48 1882, 64 x 64 (H = 2) 2851, 72 x 72
-// (H = 3) 3607, 96 x 96 (H = 3) 4264.
+// SM cycles of one frame of a work item with row parts r = (nyh, H, H nyh).  Measured with 152
+// channels of one frequency: 24 x 24 box 1432, 40 x 40 1625, 48 x 48 1776, 64 x 64 (H = 2) 2525,
+// 72 x 72 (H = 2) 2982, 88 x 80 (H = 2) 3206, 96 x 96 (H = 3) 3965; the model gives 1432, 1720, 1864,
+// 2852, 2996, 3140 and 4128 (a plan's channels are near one another in size).
 static long long ws3_item_cost(int4 r) { return 300 + 700LL * r.y + 18LL * r.z; }
 
 // Channels per launch of the warp-specialised kernels: 0 = groups of about two work items
