@@ -2722,7 +2722,7 @@ __device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t
 // How a launch's work is cut.  0: whole items per block, with sub-integrations when a.sub > 0.  1: equal
 // shares of its (item, frame) units, without sub-integrations; the parts of an item are summed through
 // a.partial.  2: sub-integrations, equal shares cut between them, so that no sums are shared (LWA block of 128
-// samples, an image set every 4: 264 whole items are two rounds of 152 blocks, the second mostly idle).
+// samples, an image set every 4: 256 whole items are two rounds of 152 blocks, the second with 48 idle).
 template <int CUT>
 __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
 {
@@ -4048,7 +4048,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     }
                     const long long equal = sum * ipc * nt / p->sm_count, whole = most * rounds * nt;
                     // Sharing items costs 40 k cycles of partial sums and further segments (LWA bursts of 4, 16, 32
-                    // and 64 samples: 46, 63, 83, 121 us in equal shares, 24, 47, 72, 120 us as 264 whole items)
+                    // and 64 samples: 46, 63, 83, 121 us in equal shares, 24, 47, 72, 120 us as 256 whole items)
                     const bool cut = items % p->sm_count != 0 && (p->sub > 0 || whole > equal + 40000);
                     // Starting under the gridding kernel's last blocks saves 5 to 9 us of a launch but scatters blocks
                     // that share tiles over the chip, 1 to 2 % of long ones (tiny station 33 -> 29 us, LWA burst of 32

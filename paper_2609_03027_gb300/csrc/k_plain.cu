@@ -121,16 +121,16 @@ __device__ __forceinline__ void frame_sample(const float2* sv, const uint8_t* fr
 constexpr int kRowThreads = 256;
 constexpr int kRowFrames = 2;  // frames of a block: each list entry read from L1 serves both
 
-// bytes of k_plain_rows's shared memory: twiddles, Y, the rows' box columns, the frames
-inline int rows_ld(int nx) { return (nx & 15) == 8 ? nx : nx + 8; }  // row stride = 8 mod 16
+// bytes of k_plain_rows's shared memory beside the frames: twiddles, Y (whose rows the box columns share)
 template <int N1, int N2>
 __host__ __device__ constexpr size_t rows_fft_smem()
 {
     return sizeof(float2) * ((size_t)N1 * N2 + (size_t)(kRowThreads / N2) * N2 * (N1 + 1));
 }
 
-// Gridded and row-transformed frames (LWA station: 5.5 ms a block, 2.9 ms of it the 12.9 GB of row
-// stores, the rest the gather's dependent list and voltage reads): block = frames 2 blockIdx.x, + 1 of
+// Gridded and row-transformed frames (LWA station: 5.1 ms a block, 2.9 ms of it the 12.9 GB of row
+// stores, the rest the gather's dependent list and voltage reads; 5.6 ms with three blocks an SM instead of
+// four, before a row's cells shared Y's memory): block = frames 2 blockIdx.x, + 1 of
 // channel blockIdx.y, slice blockIdx.z of the box rows.
 // Rows go in batches of 256 / N2 (both frames, all pols, a few y): the batch's cells are gathered
 // one per thread and step, both frames and pols at once, then N2 threads a row run the two FFT
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
                                                             const int* __restrict__ cell_ptr,
                                                             const int* __restrict__ ce, const float2* __restrict__ cw,
                                                             const float4* __restrict__ jones, int frame_in_smem,
-                                                            int ld, int ny_max, const float2* __restrict__ twg,
+                                                            int ny_max, const float2* __restrict__ twg,
                                                             float2* __restrict__ rows)
 {
     constexpr int N = N1 * N2, RPC = kRowThreads / N2, S = N2 * (N1 + 1), T = N1 / N2, F = kRowFrames;
@@ -159,8 +159,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
     const int ny = min(min(b.w, N - b.y), nb * ((int)blockIdx.z + 1) / (int)gridDim.z * YR);
     float2* tw = sm;               // [N2][N1]
     float2* y = tw + N;            // [RPC][N2][N1 + 1]
-    float2* g = y + RPC * S;       // [F][P][YR][ld]
-    uint8_t* fr_s = reinterpret_cast<uint8_t*>(g + F * P * YR * ld);
+    uint8_t* fr_s = reinterpret_cast<uint8_t*>(y + RPC * S);
     float2* sv = reinterpret_cast<float2*>(fr_s);  // [F][A][P]
     const int FB = A * P * (bits / 4);
     const float4* jm = jones ? jones + (size_t)c * A * 2 : nullptr;
@@ -213,19 +212,21 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
 #pragma unroll
             for (int f = 0; f < F; ++f)
 #pragma unroll
-                for (int p = 0; p < P; ++p) g[((f * P + p) * YR + r) * ld + x] = acc[f][p];
+                for (int p = 0; p < P; ++p) y[((f * P + p) * YR + r) * S + x] = acc[f][p];
         }
         __syncthreads();
-        const float2* gr = g + (size_t)rl * ld;
         float2 u[T][N2];
-        float2* yr = y + rl * S;
+        float2* yr = y + rl * S;  // the row's cells (nx <= N of them), then its Y
 #pragma unroll
-        for (int t = 0; t < T; ++t) {
+        for (int t = 0; t < T; ++t)
 #pragma unroll
             for (int n2 = 0; n2 < N2; ++n2) {
                 const int x = j + N2 * t + N1 * n2 - b.x;
-                u[t][n2] = x >= 0 && x < nx ? gr[x] : make_float2(0.f, 0.f);
+                u[t][n2] = x >= 0 && x < nx ? yr[x] : make_float2(0.f, 0.f);
             }
+        __syncwarp();  // a row's N2 threads are of one warp: its cells are read
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
             dft_reg<N2>(u[t]);
             const int n1 = j + N2 * t;
 #pragma unroll
@@ -437,11 +438,11 @@ __global__ void __launch_bounds__(kThreads) k_plain_sum(const float4* __restrict
 // the register-FFT kernels of one N, number of pols and form of the frames and weights
 struct RegFft {
     void (*rows)(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
-                 const float4*, int, int, int, const float2*, float2*);
+                 const float4*, int, int, const float2*, float2*);
     void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int);
     int col_tile, col_threads;
     int rows_batch;               // box rows a block transforms at once
-    size_t rows_fft, rows_cells;  // rows_cells: per box column, what a block gathers per batch
+    size_t rows_fft;
     size_t cols_smem, cols_row;   // cols_row: per box row, the staged frames
 };
 
@@ -459,7 +460,6 @@ RegFft reg_fft_p(bool staged, bool cplx)
     f.col_threads = TX * N2;
     f.rows_batch = kRowThreads / N2 / (kRowFrames * P);
     f.rows_fft = rows_fft_smem<N1, N2>();
-    f.rows_cells = sizeof(float2) * (kRowThreads / N2);  // F P YR rows
     f.cols_smem = sizeof(float2) * ((size_t)N + (size_t)P * N * TX);
     f.cols_row = sizeof(float2) * (size_t)col_stages(N) * P * TX;
     return f;
@@ -490,11 +490,6 @@ RegFft reg_fft_for(const epic_plan_s* p, bool staged)
     }
 }
 
-size_t rows_base_smem(const epic_plan_s* p, const RegFft& f)
-{
-    return f.rows_fft + f.rows_cells * rows_ld(std::min(p->box_max_x, p->N));
-}
-
 size_t cols_smem_for(const epic_plan_s* p, const RegFft& f)
 {
     return f.cols_smem + f.cols_row * std::min(p->box_max_y, p->N);
@@ -509,9 +504,11 @@ size_t frame_smem(const epic_plan_s* p, FrameForm form)
 
 FrameForm frame_form(const epic_plan_s* p)
 {
-    const size_t base = rows_base_smem(p, reg_fft_for(p, true)), lim = (size_t)p->smem_optin;
-    if (base + frame_smem(p, kFrameStaged) <= lim) return kFrameStaged;
-    return base + frame_smem(p, kFrameBytes) <= lim ? kFrameBytes : kFrameGlobal;
+    const size_t base = reg_fft_for(p, true).rows_fft, lim = (size_t)p->smem_optin;
+    // in a third of an SM: three blocks hide the gather's latency (20 000 elements as bytes in one block an SM
+    // 1.97 ms, through L1 1.45); mixed samples stay staged while they fit at all, or every tap would mix again
+    if (base + frame_smem(p, kFrameStaged) <= (p->jones.empty() ? lim / 3 : lim)) return kFrameStaged;
+    return base + frame_smem(p, kFrameBytes) <= lim / 3 ? kFrameBytes : kFrameGlobal;
 }
 
 // Slices of a chunk's frames for k_plain_cols: the number that loses least to the last wave -- of
@@ -794,7 +791,7 @@ epic_status plain_setup(epic_plan_s* p)
     e = allow_max_smem((const void*)k_plain_fft_cols_smem, p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_fft_cols_smem)");
     const RegFft rf = reg_fft_for(p, frame_form(p) == kFrameStaged);
-    if (rows_base_smem(p, rf) > (size_t)p->smem_optin || cols_smem_for(p, rf) > (size_t)p->smem_optin) {
+    if (rf.rows_fft > (size_t)p->smem_optin || cols_smem_for(p, rf) > (size_t)p->smem_optin) {
         p->last_error = "plain path: FFT shared memory exceeds the device limit";
         return EPIC_ERR_UNSUPPORTED;
     }
@@ -843,8 +840,8 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             const int fb = (nt + kRowFrames - 1) / kRowFrames, batches = (ny_max + rf.rows_batch - 1) / rf.rows_batch;
             const int Z = std::max(1, std::min(batches, (int)(8LL * p->sm_count / ((long long)fb * C))));
             launch_early(t0 > 0, rf.rows, dim3(fb, C, Z), kRowThreads,
-                         rows_base_smem(p, rf) + frame_smem(p, form), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
-                         p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, rows_ld(std::min(p->box_max_x, N)), ny_max, p->dt.twiddle, grid);
+                         rf.rows_fft + frame_smem(p, form), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
+                         p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, ny_max, p->dt.twiddle, grid);
             ev_end(p, s);
             // slices of whole intervals, or of at least four frames; the same for every chunk of the call,
             // whose partial sums add up over the chunks
