@@ -20,8 +20,11 @@ CASES = [
     (30, 1, 1, 128, 3, 45, 34.0, 4, 0, False, 1),   # ... and several chunks of them
     (30, 2, 2, 128, 7, 12, 136.0, 8, 3, True, 1),   # a box wider than the grid's padding, intervals
     (25, 1, 2, 256, 3, 18, 60.0, 4, 6, False, 1),   # intervals in slices
-    (15000, 1, 2, 512, 2, 4, 190.0, 4, 0, False, 64),   # frames as bytes in shared memory
-    (15000, 1, 2, 64, 2, 3, 20.0, 8, 0, True, 64),      # mixed from bytes
+    (15000, 1, 2, 512, 2, 4, 190.0, 4, 0, False, 64),   # frames read through L1, rows in slices
+    (15000, 1, 2, 64, 2, 3, 20.0, 8, 0, True, 64),      # mixed from there
+    (3000, 2, 2, 64, 2, 5, 20.0, 4, 0, False, 64),      # frames as bytes in shared memory
+    (3001, 1, 1, 128, 2, 5, 20.0, 8, 0, False, 64),
+    (3000, 1, 2, 64, 2, 3, 20.0, 4, 0, True, 64),       # mixed samples in more than a third of an SM
     (70000, 1, 1, 32, 2, 3, 8.0, 8, 0, False, 64),      # frames read through L1
 ]
 
