@@ -102,7 +102,6 @@ struct TcState {
     // (P * nyh rows) and a stage-1 / stage-2 step of its own, so tall boxes fit in TMEM.
     std::vector<int4> tbox_h;      // [C] (nyh, H, H * nyh, 0) on the host
     int4* tbox = nullptr;          // same, on the device (every tensor-path plan)
-    bool parts = false;            // some channel has H > 1 (only k_dftgemm_ws3 takes it)
     int nbt = 2;                   // k_dftgemm_ws3: tile-part buffers in shared memory (2..6),
     unsigned ws3_sB2 = 0, ws3_b2 = 0;  //   where B2 starts, bytes of a B2 buffer
     int ws3_smem = 0;

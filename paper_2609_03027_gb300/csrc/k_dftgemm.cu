@@ -2336,7 +2336,7 @@ __device__ __forceinline__ void ws3_store32(float* o, int nk, int accumulate, co
 // (`rows`, nk: multiples of 4) written to o (the first pixel), or added to what is there.  Four lanes
 // exchange 16-byte pieces first, so that a store covers 8 rows x 64 bytes instead of 32 rows x 16.
 // For sub-integrations, which store every few frames (LWA block of 128 samples with an image set
-// every 4: 0.62 ms without, 0.35 with it and equal shares); whole items keep ws3_store32, whose stores wait
+// every 4: 0.62 ms without, 0.32 with it and equal shares); whole items keep ws3_store32, whose stores wait
 // for the memory in either form, while these exchanges cost their frame loop 1 % by its register allocation.
 __device__ __forceinline__ void ws3_store_rows(float* o, int N, int rows, int nk, int accumulate, int lane,
                                                float (&v)[32])
@@ -3493,7 +3493,6 @@ epic_status dftgemm_setup(epic_plan_s* p)
     // memory; 2 D1 slots + A2 + D2 in TMEM.  Each channel's box rows go in H_c parts of nyh_c
     // rows (row_parts), chosen for the largest D1 slot width D that fits both memories.
     p->tc.tbox_h.assign(C, make_int4(0, 0, 0, 0));
-    p->tc.parts = false;
     p->tc.ws = false;
     for (int D = 256; D >= 16 && !p->tc.ws; D -= 16) {
         int dmax = 0, a2max = 0, nyh_max = 0;
@@ -3518,7 +3517,6 @@ epic_status dftgemm_setup(epic_plan_s* p)
         const size_t need_ws = a1p + nbt * b1p + 2 * b2w;
         if (need_ws > limit) continue;
         p->tc.ws = true;
-        p->tc.parts = split;
         p->tc.tbox_h = tb;
         p->tc.nbt = nbt;
         p->tc.sA1 = 0;
