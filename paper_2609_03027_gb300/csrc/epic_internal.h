@@ -253,6 +253,7 @@ epic_status dftgemm_set_group(epic_plan_s* p, int v);
 // k_grid_tc.cu
 epic_status grid_tc_setup(epic_plan_s* p);
 epic_status grid_tc_config(epic_plan_s* p, int gc);
+bool grid_tc_configured(const epic_plan_s* p);
 int dftgemm_dense(const epic_plan_s* p);  // tiles without K padding: gridded and read by the tensor-core kernels
 void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0, int n_ch, cudaStream_t s);
 

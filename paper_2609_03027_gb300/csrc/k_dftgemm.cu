@@ -3217,32 +3217,49 @@ static epic_status grid_bal_config(epic_plan_s* p, int F)
 
 static epic_status grid_lists_setup(epic_plan_s* p);
 
+// The chosen gridding kernel and what its launches take
+struct GridLaunch {
+    int variant, frames, smem, blocks;
+    bool pl_stage;
+};
+
+static GridLaunch grid_launch_of(const epic_plan_s* p)
+{
+    return GridLaunch{p->tc.grid_variant, p->tc.grid_frames, p->tc.grid_smem, p->tc.grid_blocks, p->tc.pl_stage};
+}
+
+static void grid_launch_set(epic_plan_s* p, const GridLaunch& g)
+{
+    p->tc.grid_variant = g.variant;
+    p->tc.grid_frames = g.frames;
+    p->tc.grid_smem = g.smem;
+    p->tc.grid_blocks = g.blocks;
+    p->tc.pl_stage = g.pl_stage;
+}
+
 // Gridding kernel variant: 1 = persistent row-major gather, 2 = balanced task lists,
 // 3 = row-major pair lists, 4 = tensor cores.  Keeps the frames per pass if the variant
 // allows them, else the largest it allows.  The lists of 2 and 3 are built when first asked for.
+// Every refusal leaves the kernel and its launch as they were: building the lists configures
+// the kernels that it tries.
 epic_status dftgemm_set_grid_kernel(epic_plan_s* p, int variant)
 {
     if (variant < 1 || variant > 4) return EPIC_ERR_UNSUPPORTED;
-    const int old_variant = p->tc.grid_variant, old_f = p->tc.grid_frames;
-    if ((variant == 2 || variant == 3) && !p->tc.lists_built) {
-        const epic_status ls = grid_lists_setup(p);
-        p->tc.grid_variant = old_variant;
-        if (ls != EPIC_OK) {
-            dftgemm_grid_config(p, old_f);
-            return ls;
-        }
-    }
-    if (variant == 4 && !p->tc.gt_tile0) return EPIC_ERR_UNSUPPORTED;
-    if (variant == 2 && !p->tc.gtask) return EPIC_ERR_UNSUPPORTED;
-    if (variant == 3 && !p->tc.pl_ptr) return EPIC_ERR_UNSUPPORTED;
-    if (variant == 1 && !p->tc.grid_ps) return EPIC_ERR_UNSUPPORTED;
-    p->tc.grid_variant = variant;
+    const GridLaunch old = grid_launch_of(p);
     epic_status st = EPIC_ERR_UNSUPPORTED;
-    for (int F = old_f; F >= 1 && st == EPIC_ERR_UNSUPPORTED; F >>= 1) st = dftgemm_grid_config(p, F);
-    if (st != EPIC_OK) {
-        p->tc.grid_variant = old_variant;
-        dftgemm_grid_config(p, old_f);
+    if ((variant == 2 || variant == 3) && !p->tc.lists_built) {
+        st = grid_lists_setup(p);
+        grid_launch_set(p, old);
+        if (st != EPIC_OK) return st;
     }
+    const bool have = variant == 4 ? p->tc.gt_tile0 != nullptr
+                    : variant == 3 ? p->tc.pl_ptr != nullptr
+                    : variant == 2 ? p->tc.gtask != nullptr : p->tc.grid_ps;
+    if (!have) return EPIC_ERR_UNSUPPORTED;
+    p->tc.grid_variant = variant;
+    st = EPIC_ERR_UNSUPPORTED;
+    for (int F = old.frames; F >= 1 && st == EPIC_ERR_UNSUPPORTED; F >>= 1) st = dftgemm_grid_config(p, F);
+    if (st != EPIC_OK) grid_launch_set(p, old);
     return st;
 }
 
@@ -3895,6 +3912,10 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
             const int nt = std::min(p->tc.tc, T - t0);
             const dim3 gg((nt + fpc - 1) / fpc, ng);
             if (p->tc.grid_variant == 4) {
+                if (!grid_tc_configured(p)) {
+                    p->last_error = "tensor path: gridding kernel configuration out of step (internal)";
+                    return EPIC_ERR_CUDA;
+                }
                 ev_begin(p, "k_dftgemm_grid", s);
                 grid_tc_launch(p, volt, t0, nt, c0, ng, s);
                 ev_end(p, s);

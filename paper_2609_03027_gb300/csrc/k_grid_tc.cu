@@ -698,6 +698,12 @@ epic_status grid_tc_setup(epic_plan_s* p)
     return EPIC_OK;
 }
 
+// Whether the plan's launch configuration is this kernel's for its frames
+bool grid_tc_configured(const epic_plan_s* p)
+{
+    return p->tc.gt_tile0 && (size_t)p->tc.grid_smem == grid_tc_smem(p, p->tc.grid_frames);
+}
+
 void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0, int n_ch, cudaStream_t s)
 {
     GridTcArgs a{};

@@ -1,0 +1,36 @@
+"""A refused tuning parameter leaves the plan as it was: the same parameters and bit-equal images."""
+import pytest
+
+import epic_synth as synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2609_03027_gb300 as E  # noqa: E402
+
+GRID = ("grid_kernel", "grid_frames")
+
+
+def test_refused_gridding_kernel_leaves_the_tensor_core_one_as_it_was():
+    # the tallest SKA-Low channel: the balanced kernel's tiles, tasks and entries do not fit, and trying
+    # them configures the pair-list kernel on the way
+    cfg = synth.config(3).subset([383], n_time=20)
+    v = torch.from_numpy(synth.make_voltages(cfg)).cuda()
+    with E.Plan.from_config(cfg, path="dftgemm") as plan:
+        before = {k: plan.get_param(k) for k in GRID}
+        assert before["grid_kernel"] == 4
+        for bad in (2, 0, 5):
+            with pytest.raises(E.EpicError) as ex:
+                plan.set_param("grid_kernel", bad)
+            assert ex.value.status == 7
+            assert {k: plan.get_param(k) for k in GRID} == before, bad
+        got = plan.image(v)       # a launch out of step with its configuration is an error, not a kernel
+        plan.sync()
+        with E.Plan.from_config(cfg, path="dftgemm") as fresh:
+            assert torch.equal(got, fresh.image(v))
+            fresh.sync()
+        plan.set_param("grid_kernel", 3)
+        plan.set_param("grid_kernel", 4)
+        assert plan.get_param("grid_kernel") == 4
+        assert torch.equal(got, plan.image(v))
+        plan.sync()
