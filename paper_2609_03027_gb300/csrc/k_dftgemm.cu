@@ -3135,7 +3135,6 @@ static epic_status grid_pl_config(epic_plan_s* p, int F)
        : (S ? (const void*)k_dftgemm_grid_pl<FF, false, true> : (const void*)k_dftgemm_grid_pl<FF, false, false>))
     const void* fn = F == 8 ? EPIC_PL_FN(8) : F == 4 ? EPIC_PL_FN(4) : F == 2 ? EPIC_PL_FN(2) : EPIC_PL_FN(1);
 #undef EPIC_PL_FN
-    p->tc.pl_stage = S;
     cudaFuncAttributes fa{};
     cudaError_t e = cudaFuncGetAttributes(&fa, fn);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncGetAttributes(k_dftgemm_grid_pl)");
@@ -3146,6 +3145,7 @@ static epic_status grid_pl_config(epic_plan_s* p, int F)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kGridPlThreads, bytes);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(k_dftgemm_grid_pl)");
     if (occ < 1) return EPIC_ERR_UNSUPPORTED;
+    p->tc.pl_stage = S;
     p->tc.grid_frames = F;
     p->tc.grid_smem = (int)bytes;
     p->tc.grid_blocks = p->sm_count * occ;

@@ -34,3 +34,20 @@ def test_refused_gridding_kernel_leaves_the_tensor_core_one_as_it_was():
         assert plan.get_param("grid_kernel") == 4
         assert torch.equal(got, plan.image(v))
         plan.sync()
+
+
+def test_refused_frames_of_the_pair_list_kernel_leave_its_staging_as_it_was():
+    # 2430 dual-pol elements: the lists fit beside four frames of voltages, eight frames do not fit at all
+    cfg = synth.small_config(n_ant=2430, n_chan=2, n_pol=2, grid_n=128, gcf_k=2, n_time=5, seed=8, diameter_m=60.0,
+                             sigma=0.7)
+    v = torch.from_numpy(synth.make_voltages(cfg)).cuda()
+    with E.Plan.from_config(cfg, path="dftgemm", max_time=5) as plan:
+        plan.set_param("grid_kernel", 3)
+        plan.set_param("grid_frames", 4)
+        before = plan.image(v)
+        with pytest.raises(E.EpicError) as ex:
+            plan.set_param("grid_frames", 8)
+        assert ex.value.status == 7
+        assert plan.get_param("grid_frames") == 4
+        assert torch.equal(plan.image(v), before)
+        plan.sync()
