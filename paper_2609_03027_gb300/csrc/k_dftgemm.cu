@@ -3293,7 +3293,7 @@ static epic_status grid_lists_setup(epic_plan_s* p)
     std::vector<TaskW> pl_w;
     bool fits = true;
     int tmax = 0, emax = 0;
-    for (int c = 0; c < C && fits; ++c) {
+    for (int c = 0; c < C; ++c) {
         toff[c] = (int)tasks.size();
         eoff[c] = (int)ell_e.size();
         const int* ptr = &cptr[coff[c]];
@@ -3330,6 +3330,7 @@ static epic_status grid_lists_setup(epic_plan_s* p)
             }
         }
         pl_ptr.push_back((int)pl_e.size());
+        if (!fits) continue;  // an earlier channel's lists are too long for a task: pair lists only
         std::vector<int> idx;
         for (int q = 0; q < hp * bx.ny; ++q)
             if (!plist[q].empty()) idx.push_back(q);
