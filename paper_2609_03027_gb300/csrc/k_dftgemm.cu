@@ -34,11 +34,13 @@
 
 #include <algorithm>
 #include <cstring>
+#include <new>
 #include <type_traits>
 
 #include "dftgemm_common.cuh"
 #include "epic_internal.h"
 #include "kcommon.cuh"
+#include "table_upload.h"
 #include "tc_ptx.cuh"
 
 namespace epic {
@@ -3248,7 +3250,12 @@ epic_status dftgemm_set_grid_kernel(epic_plan_s* p, int variant)
     const GridLaunch old = grid_launch_of(p);
     epic_status st = EPIC_ERR_UNSUPPORTED;
     if ((variant == 2 || variant == 3) && !p->tc.lists_built) {
-        st = grid_lists_setup(p);
+        try {
+            st = grid_lists_setup(p);
+        } catch (const std::bad_alloc&) {  // nothing was uploaded yet
+            p->last_error = "gridding lists: no host memory";
+            st = EPIC_ERR_OOM;
+        }
         grid_launch_set(p, old);
         if (st != EPIC_OK) return st;
     }
@@ -3269,9 +3276,10 @@ epic_status dftgemm_set_grid_kernel(epic_plan_s* p, int variant)
 static epic_status grid_lists_setup(epic_plan_s* p)
 {
     const int C = p->C;
-    p->tc.lists_built = true;
-    if (p->tc.grid_cplx) return EPIC_OK;
-    cudaError_t e = cudaSuccess;
+    if (p->tc.grid_cplx) {
+        p->tc.lists_built = true;
+        return EPIC_OK;
+    }
     std::vector<int> coff, cptr, ce;
     std::vector<float2> cw;
     build_csr(p, coff, cptr, ce, cw);
@@ -3399,44 +3407,34 @@ static epic_status grid_lists_setup(epic_plan_s* p)
     }
     toff[C] = (int)tasks.size();
     eoff[C] = (int)ell_e.size();
+    // Every table is up before the plan holds any of them: a build that fails leaves the plan without lists,
+    // and a later request builds them again.
+    const bool pairs = kTaskCells == 2 && !pl_e.empty() && pl_e.size() < (1u << 31), balanced = fits && !tasks.empty();
+    TableUpload up;
+    if (pairs) {  // for k_dftgemm_grid_pl
+        up.add(&p->tc.pl_ptr, pl_ptr);
+        up.add(&p->tc.pl_off, pl_off);
+        up.add(&p->tc.pl_e, pl_e);
+        up.add(&p->tc.pl_w, pl_w);
+    }
+    const size_t pair_bytes = up.bytes();
+    if (balanced) {
+        up.add(&p->tc.gtask, tasks);
+        up.add(&p->tc.gtask_off, toff);
+        up.add(&p->tc.gell_e, ell_e);
+        up.add(&p->tc.gell_w, ell_w);
+        up.add(&p->tc.gell_off, eoff);
+    }
+    const cudaError_t e = up.upload();
+    if (e != cudaSuccess) return cuda_fail(p, e, "gridding lists upload");
+    p->tc.lists_built = true;
+    p->dt.dft_bytes += pair_bytes;
     for (int c = 0; c < C; ++c) {  // largest offsets / entries of a channel (staged lists)
         const int np = p->box[c].ny * (p->box[c].nx / kTaskCells) + 1;
         p->tc.pl_max_ptr = std::max(p->tc.pl_max_ptr, np);
         p->tc.pl_max_ent = std::max(p->tc.pl_max_ent, pl_ptr[pl_off[c] + np - 1] - pl_ptr[pl_off[c]]);
     }
-    if (kTaskCells == 2 && !pl_e.empty() && pl_e.size() < (1u << 31)) {  // pair lists for k_dftgemm_grid_pl
-        e = cudaMalloc(&p->tc.pl_ptr, pl_ptr.size() * sizeof(int));
-        if (e == cudaSuccess)
-            e = cudaMemcpy(p->tc.pl_ptr, pl_ptr.data(), pl_ptr.size() * sizeof(int), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_off, pl_off.size() * sizeof(int));
-        if (e == cudaSuccess)
-            e = cudaMemcpy(p->tc.pl_off, pl_off.data(), pl_off.size() * sizeof(int), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_e, pl_e.size() * sizeof(int));
-        if (e == cudaSuccess)
-            e = cudaMemcpy(p->tc.pl_e, pl_e.data(), pl_e.size() * sizeof(int), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.pl_w, pl_w.size() * sizeof(float2));
-        if (e == cudaSuccess)
-            e = cudaMemcpy(p->tc.pl_w, pl_w.data(), pl_w.size() * sizeof(float2), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(p, e, "pair-list upload");
-        p->dt.dft_bytes += (pl_ptr.size() + pl_off.size() + pl_e.size()) * sizeof(int) + pl_w.size() * sizeof(float2);
-    }
-    if (fits && !tasks.empty()) {
-        e = cudaMalloc(&p->tc.gtask, tasks.size() * sizeof(int4));
-        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gtask, tasks.data(), tasks.size() * sizeof(int4),
-                                             cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gtask_off, toff.size() * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gtask_off, toff.data(), toff.size() * sizeof(int),
-                                             cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_e, ell_e.size() * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_e, ell_e.data(), ell_e.size() * sizeof(int),
-                                             cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_w, ell_w.size() * sizeof(TaskW));
-        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_w, ell_w.data(), ell_w.size() * sizeof(TaskW),
-                                             cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&p->tc.gell_off, eoff.size() * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemcpy(p->tc.gell_off, eoff.data(), eoff.size() * sizeof(int),
-                                             cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(p, e, "gridding task lists upload");
+    if (balanced) {
         p->tc.gtask_max = tmax;
         p->tc.gell_max = emax;
         const int keep_f = p->tc.grid_frames;
@@ -3475,8 +3473,7 @@ static epic_status grid_lists_setup(epic_plan_s* p)
                 }
             }
         } else {
-            p->dt.dft_bytes += tasks.size() * sizeof(int4) + ell_e.size() * (sizeof(int) + sizeof(TaskW)) +
-                               (toff.size() + eoff.size()) * sizeof(int);
+            p->dt.dft_bytes += up.bytes() - pair_bytes;
         }
     }
     return EPIC_OK;
