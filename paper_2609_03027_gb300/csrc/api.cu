@@ -157,6 +157,39 @@ epic_status cuda_fail(epic_plan_s* p, cudaError_t e, const char* what)
     return e == cudaErrorMemoryAllocation ? EPIC_ERR_OOM : EPIC_ERR_CUDA;
 }
 
+epic_status no_scratch(epic_plan_s* p)
+{
+    p->last_error = "the plan has no scratch: neither a new size nor the one before could be allocated";
+    return EPIC_ERR_OOM;
+}
+
+// A failed allocation leaves the plan with its scratch of before (or with none: no_scratch), and does not show up
+// again at the next launch's check.
+epic_status scratch_resize(epic_plan_s* p, size_t bytes, bool zero, const char* what)
+{
+    if (p->scratch && bytes == p->scratch_bytes) return EPIC_OK;
+    const size_t had = p->scratch_bytes;
+    auto take = [&](size_t n) {
+        cudaError_t e = cudaMalloc(&p->scratch, n);
+        if (e != cudaSuccess) {
+            p->scratch = nullptr;
+            cudaGetLastError();
+            return e;
+        }
+        p->scratch_bytes = n;
+        if (zero) e = cudaMemset(p->scratch, 0, n);
+        if (zero && e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // a later call's stream may not wait for the default one
+        return e;
+    };
+    cudaFree(p->scratch);  // first: both sizes need not fit together
+    p->scratch = nullptr;
+    p->scratch_bytes = 0;
+    const cudaError_t e = take(bytes);
+    if (e == cudaSuccess) return EPIC_OK;
+    if (!p->scratch && had) take(had);
+    return cuda_fail(p, e, what);
+}
+
 cudaError_t allow_max_smem(const void* fn, int optin)
 {
     cudaFuncAttributes fa{};

@@ -208,6 +208,9 @@ cudaError_t allow_max_smem(const void* fn, int optin);
 void ev_begin(epic_plan_s* p, const char* name, cudaStream_t s);
 void ev_end(epic_plan_s* p, cudaStream_t s);
 epic_status cuda_fail(epic_plan_s* p, cudaError_t e, const char* what);
+// The plan's scratch at `bytes` (zeroed on request).  On failure the plan keeps a scratch of the size before.
+epic_status scratch_resize(epic_plan_s* p, size_t bytes, bool zero, const char* what);
+epic_status no_scratch(epic_plan_s* p);  // the error of a call on a plan that could not get its scratch back
 // Switch the plan to another path (frees the current path's tables and scratch, sets up the
 // new one; on failure the plan is back on its previous path and the status is returned).
 epic_status set_path(epic_plan_s* p, int path);

@@ -3100,22 +3100,13 @@ epic_status dftgemm_set_chunk(epic_plan_s* p, size_t budget)
     const size_t per_t = (size_t)p->tc.cg * p->tc.stride;
     int tcn = (int)std::max<size_t>(1, std::min<size_t>((size_t)p->max_time, budget / per_t));
     if (p->sub > 0) tcn = std::max(p->sub, tcn - tcn % p->sub);  // whole sub-integrations per chunk
-    const size_t bytes = per_t * tcn;
+    // zeroed: tile bytes no gridding kernel writes (K padding past 2 nx) then hold zeros or
+    // FP16 values of other tiles, never stale non-finite bits, and meet zero DFT operands
+    const epic_status st = scratch_resize(p, per_t * tcn, true, "tensor path tile buffer");
+    if (st != EPIC_OK) return st;
     p->chunk_budget = budget;
     p->tc.tc = tcn;
     p->time_chunk = tcn;
-    if (p->scratch && bytes == p->scratch_bytes) return EPIC_OK;
-    cudaFree(p->scratch);
-    p->scratch = nullptr;
-    p->scratch_bytes = 0;
-    cudaError_t e = cudaMalloc(&p->scratch, bytes);
-    if (e != cudaSuccess) return cuda_fail(p, e, "cudaMalloc(tensor path tile buffer)");
-    // zero once: tile bytes no gridding kernel writes (K padding past 2 nx) then hold zeros or
-    // FP16 values of other tiles, never stale non-finite bits, and meet zero DFT operands
-    e = cudaMemset(p->scratch, 0, bytes);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // a later call's stream may not wait for the default one
-    if (e != cudaSuccess) return cuda_fail(p, e, "cudaMemset(tensor path tile buffer)");
-    p->scratch_bytes = bytes;
     return EPIC_OK;
 }
 
@@ -3867,6 +3858,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                         const GroupHooks* hooks)
 {
     const int C = p->C, P = p->P, A = p->A;
+    if (!p->scratch) return no_scratch(p);
     MmaArgs a{};
     a.tiles = (const uint8_t*)p->scratch;
     a.tile_stride = p->tc.stride;

@@ -750,16 +750,11 @@ epic_status plain_set_chunk(epic_plan_s* p, size_t budget)
         slices = col_slices(p, f, tcn, std::max(1, occ) * p->sm_count);
         if (p->sub == 0 && slices > 1) bytes += sizeof(float) * (size_t)slices * p->C * p->nprod * p->N * p->N;
     }
+    const epic_status st = scratch_resize(p, bytes, false, "plain grid buffer");
+    if (st != EPIC_OK) return st;
     p->chunk_budget = budget;
     p->plain_slices = slices;
     p->time_chunk = tcn;
-    if (p->scratch && bytes == p->scratch_bytes) return EPIC_OK;
-    cudaFree(p->scratch);
-    p->scratch = nullptr;
-    p->scratch_bytes = 0;
-    cudaError_t e = cudaMalloc(&p->scratch, bytes);
-    if (e != cudaSuccess) return cuda_fail(p, e, "cudaMalloc(plain grid buffer)");
-    p->scratch_bytes = bytes;
     return EPIC_OK;
 }
 
@@ -829,6 +824,7 @@ static void launch_early(bool early, F* fn, dim3 grid, int threads, size_t smem,
 epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s, float* out, bool accumulate)
 {
     const int C = p->C, P = p->P, N = p->N, A = p->A;
+    if (!p->scratch) return no_scratch(p);
     float2* grid = (float2*)p->scratch;
     const size_t sg = sizeof(float2) * (size_t)A * P;
     const int bits = p->bits;

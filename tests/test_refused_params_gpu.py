@@ -51,3 +51,19 @@ def test_refused_frames_of_the_pair_list_kernel_leave_its_staging_as_it_was():
         assert plan.get_param("grid_frames") == 4
         assert torch.equal(plan.image(v), before)
         plan.sync()
+
+
+def test_scratch_that_cannot_be_had_leaves_the_plan_working():
+    # 100,000 samples of 64 channels as tiles are more than the device's memory
+    cfg = synth.small_config(n_ant=40, n_chan=64, n_pol=2, grid_n=128, gcf_k=3, n_time=20, seed=31, diameter_m=85.0)
+    v = torch.from_numpy(synth.make_voltages(cfg)).cuda()
+    with E.Plan.from_config(cfg, path="dftgemm", max_time=100_000) as plan:
+        before = plan.image(v)
+        info, budget = plan.info(), plan.get_param("chunk_mb")
+        with pytest.raises(E.EpicError) as ex:
+            plan.set_param("chunk_mb", 2_000_000)
+        assert ex.value.status == 3               # EPIC_ERR_OOM
+        assert plan.info() == info and plan.get_param("chunk_mb") == budget
+        for _ in range(2):                        # no error left over for the next calls
+            assert torch.equal(plan.image(v), before)
+            plan.sync()
