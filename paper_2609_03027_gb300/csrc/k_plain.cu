@@ -422,22 +422,29 @@ __global__ void __launch_bounds__(TX * N2) k_plain_cols(const float2* __restrict
     if (sub == 0 && ta >= tb) store(image(ta), add);  // no frames: zeros
 }
 
-// out (+)= the slices' partial sums, in slice order
-__global__ void __launch_bounds__(kThreads) k_plain_sum(const float4* __restrict__ partial, size_t n4, int S,
-                                                        float4* __restrict__ out, int accumulate)
+__device__ __forceinline__ float add(float a, float b) { return a + b; }
+__device__ __forceinline__ float4 add(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+// out (+)= the slices' partial sums, in slice order, a V at a time (float4 where `out` begins at 16 bytes,
+// else float)
+template <class V>
+__global__ void __launch_bounds__(kThreads) k_plain_sum(const V* __restrict__ partial, size_t n, int S, V* __restrict__ out,
+                                                        int accumulate)
 {
-    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n4; i += (size_t)gridDim.x * kThreads) {
-        float4 a = partial[i];
-        for (int k = 1; k < S; ++k) {
-            const float4 v = partial[k * n4 + i];
-            a = make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w);
-        }
-        if (accumulate) {
-            const float4 o = out[i];
-            a = make_float4(a.x + o.x, a.y + o.y, a.z + o.z, a.w + o.w);
-        }
-        out[i] = a;
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kThreads) {
+        V a = partial[i];
+        for (int k = 1; k < S; ++k) a = add(a, partial[k * n + i]);
+        out[i] = accumulate ? add(a, out[i]) : a;
     }
+}
+
+template <class V>
+void sum_slices(const epic_plan_s* p, const float* partial, size_t n, int S, float* out, bool accumulate, cudaStream_t s)
+{
+    n /= sizeof(V) / sizeof(float);
+    const unsigned blocks = (unsigned)std::min<size_t>((n + kThreads - 1) / kThreads, 8 * (size_t)p->sm_count);
+    k_plain_sum<V><<<blocks, kThreads, 0, s>>>(reinterpret_cast<const V*>(partial), n, S, reinterpret_cast<V*>(out),
+                                               accumulate ? 1 : 0);
 }
 
 // the register-FFT kernels of one N, number of pols and form of the frames and weights
@@ -857,10 +864,10 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
                          p->sub, p->sub > 0 ? t0 / p->sub : 0);
             ev_end(p, s);
             if (partial && t0 + nt == T) {
-                const size_t n4 = (size_t)C * p->nprod * N * N / 4;
+                const size_t n = (size_t)C * p->nprod * N * N;
                 ev_begin(p, "k_plain_sum", s);
-                k_plain_sum<<<(unsigned)std::min<size_t>((n4 + kThreads - 1) / kThreads, 8 * (size_t)p->sm_count), kThreads, 0, s>>>(
-                    reinterpret_cast<const float4*>(partial), n4, S, reinterpret_cast<float4*>(out), accumulate ? 1 : 0);
+                if (((uintptr_t)out & 15) == 0) sum_slices<float4>(p, partial, n, S, out, accumulate, s);
+                else sum_slices<float>(p, partial, n, S, out, accumulate, s);
                 ev_end(p, s);
             }
         } else {
