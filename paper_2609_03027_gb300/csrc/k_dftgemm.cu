@@ -150,22 +150,33 @@ __device__ __forceinline__ size_t sw_chunk(int r, int c, int R)
     return (size_t)(c >> 3) * ((size_t)R * 128) + (size_t)r * 128 + (((c & 7) ^ (r & 7)) << 4);
 }
 
+// 4 consecutive image pixels of one product: written, or added to what is there.  ANY: they begin at any float
+// of an allocation, else at 16 bytes.
+template <bool ANY>
+__device__ __forceinline__ void store_pixels4(float* q, int accumulate, float4 w)
+{
+    if (ANY && (reinterpret_cast<uintptr_t>(q) & 15) != 0) {
+        q[0] = (accumulate ? q[0] : 0.f) + w.x;
+        q[1] = (accumulate ? q[1] : 0.f) + w.y;
+        q[2] = (accumulate ? q[2] : 0.f) + w.z;
+        q[3] = (accumulate ? q[3] : 0.f) + w.w;
+        return;
+    }
+    if (accumulate) {
+        const float4 u = *reinterpret_cast<const float4*>(q);
+        w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
+    }
+    *reinterpret_cast<float4*>(q) = w;
+}
+
 // 16 consecutive image pixels of one product: written, or added to what is there.
+template <bool ANY>
 __device__ __forceinline__ void store_pixels16(float* op, int nk, int accumulate, const float (&v)[16])
 {
     if (nk == 16) {
 #pragma unroll
-        for (int i = 0; i < 16; i += 4) {
-            float4 w = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            if (accumulate) {
-                const float4 u = *reinterpret_cast<const float4*>(op + i);
-                w.x += u.x;
-                w.y += u.y;
-                w.z += u.z;
-                w.w += u.w;
-            }
-            *reinterpret_cast<float4*>(op + i) = w;
-        }
+        for (int i = 0; i < 16; i += 4)
+            store_pixels4<ANY>(op + i, accumulate, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i)
@@ -1309,11 +1320,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_dftgemm_mma(MmaArgs a)
             const size_t NN = (size_t)a.N * a.N;
             float* o = a.out + (size_t)c * a.nprod * NN + (size_t)ky * a.N + kx0;
             const int nk = min(16, a.N - kx0);
-            store_pixels16(o, nk, a.accumulate, axx);
+            store_pixels16<true>(o, nk, a.accumulate, axx);
             if (a.nprod == 4) {
-                store_pixels16(o + NN, nk, a.accumulate, ayy);
-                store_pixels16(o + 2 * NN, nk, a.accumulate, arx);
-                store_pixels16(o + 3 * NN, nk, a.accumulate, aix);
+                store_pixels16<true>(o + NN, nk, a.accumulate, ayy);
+                store_pixels16<true>(o + 2 * NN, nk, a.accumulate, arx);
+                store_pixels16<true>(o + 3 * NN, nk, a.accumulate, aix);
             }
         }
     }
@@ -1507,11 +1518,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_dftgemm_mma_fast(MmaArgs a)
             const size_t NN = (size_t)a.N * a.N;
             float* o = a.out + (size_t)c * a.nprod * NN + (size_t)ky * a.N + kx0;
             const int nk = min(16, a.N - kx0);
-            store_pixels16(o, nk, a.accumulate, axx);
+            store_pixels16<true>(o, nk, a.accumulate, axx);
             if (a.nprod == 4) {
-                store_pixels16(o + NN, nk, a.accumulate, ayy);
-                store_pixels16(o + 2 * NN, nk, a.accumulate, arx);
-                store_pixels16(o + 3 * NN, nk, a.accumulate, aix);
+                store_pixels16<true>(o + NN, nk, a.accumulate, ayy);
+                store_pixels16<true>(o + 2 * NN, nk, a.accumulate, arx);
+                store_pixels16<true>(o + 3 * NN, nk, a.accumulate, aix);
             }
         }
     }
@@ -1851,11 +1862,11 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dftgemm_ws(MmaArgs a)
             const size_t NN = (size_t)a.N * a.N;
             float* o = a.out + (size_t)c * a.nprod * NN + (size_t)ky * a.N + kx0;
             const int nk = min(16, a.N - kx0);
-            store_pixels16(o, nk, a.accumulate, axx);
+            store_pixels16<false>(o, nk, a.accumulate, axx);
             if (a.nprod == 4) {
-                store_pixels16(o + NN, nk, a.accumulate, ayy);
-                store_pixels16(o + 2 * NN, nk, a.accumulate, arx);
-                store_pixels16(o + 3 * NN, nk, a.accumulate, aix);
+                store_pixels16<false>(o + NN, nk, a.accumulate, ayy);
+                store_pixels16<false>(o + 2 * NN, nk, a.accumulate, arx);
+                store_pixels16<false>(o + 3 * NN, nk, a.accumulate, aix);
             }
         }
     }
@@ -2109,11 +2120,11 @@ __global__ void __launch_bounds__(kWs2Threads, 1) k_dftgemm_ws2(MmaArgs a)
             const size_t NN = (size_t)a.N * a.N;
             float* o = a.out + (size_t)c * a.nprod * NN + (size_t)ky * a.N + kx0;
             const int nk = min(16, a.N - kx0);
-            store_pixels16(o, nk, a.accumulate, axx);
+            store_pixels16<false>(o, nk, a.accumulate, axx);
             if (a.nprod == 4) {
-                store_pixels16(o + NN, nk, a.accumulate, ayy);
-                store_pixels16(o + 2 * NN, nk, a.accumulate, arx);
-                store_pixels16(o + 3 * NN, nk, a.accumulate, aix);
+                store_pixels16<false>(o + NN, nk, a.accumulate, ayy);
+                store_pixels16<false>(o + 2 * NN, nk, a.accumulate, arx);
+                store_pixels16<false>(o + 3 * NN, nk, a.accumulate, aix);
             }
         }
     }
@@ -2319,19 +2330,12 @@ __device__ __forceinline__ void ws3_epilogue2(uint32_t taddr, float (&xx)[32], f
 
 // 32 consecutive image pixels of one product (nk of them inside the image, a multiple of 4):
 // written, or added to what is there
+template <bool ANY = false>
 __device__ __forceinline__ void ws3_store32(float* o, int nk, int accumulate, const float (&v)[32])
 {
 #pragma unroll
-    for (int i = 0; i < 32; i += 4) {
-        if (i < nk) {
-            float4 w = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            if (accumulate) {
-                const float4 u = *reinterpret_cast<const float4*>(o + i);
-                w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
-            }
-            *reinterpret_cast<float4*>(o + i) = w;
-        }
-    }
+    for (int i = 0; i < 32; i += 4)
+        if (i < nk) store_pixels4<ANY>(o + i, accumulate, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
 }
 
 // A warp's 32 x 32 pixels of one product, lane = row, v = 32 columns: rows and columns within the image
@@ -2363,15 +2367,9 @@ __device__ __forceinline__ void ws3_store_rows(float* o, int N, int rows, int nk
         swap(h + 4, h + 12, 2);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {  // row k of the four, piece lane & 3 of the 16 columns from h
-            if (k < rows && h < nk) {
-                float4* q = reinterpret_cast<float4*>(o + (size_t)k * N + h);
-                float4 w = make_float4(v[h + 4 * k], v[h + 4 * k + 1], v[h + 4 * k + 2], v[h + 4 * k + 3]);
-                if (accumulate) {
-                    const float4 u = *q;
-                    w = make_float4(w.x + u.x, w.y + u.y, w.z + u.z, w.w + u.w);
-                }
-                *q = w;
-            }
+            if (k < rows && h < nk)
+                store_pixels4<false>(o + (size_t)k * N + h, accumulate,
+                                     make_float4(v[h + 4 * k], v[h + 4 * k + 1], v[h + 4 * k + 2], v[h + 4 * k + 3]));
         }
     }
 }
@@ -2536,7 +2534,7 @@ __device__ __forceinline__ bool ws3_e2_any(bool mine)
 }
 
 // The epilogue-2 warps' walk through the block's segments.  Returns false when a wait ran out.
-template <int CUT, int P>
+template <int CUT, int P, bool ANY>
 __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int items, long long w0, long long w1,
                                             int warp, int lane, uint64_t* d2_full, uint64_t* d2_empty,
                                             const uint32_t* start, Ws3Split& sp)
@@ -2563,7 +2561,7 @@ __device__ __forceinline__ bool ws3_role_e2(const MmaArgs& a, uint32_t tmem, int
                 if (CUT == 2)
                     ws3_store_rows(q - (size_t)lane * a.N, a.N, min(32, a.N - (ky - lane)), min(32, a.N - kx0), a.accumulate,
                                    lane, v);
-                else ws3_store32(q, nk, a.accumulate, v);
+                else ws3_store32<ANY>(q, nk, a.accumulate, v);
             };
             one(o, xx);
             if (P == 2) {
@@ -2725,7 +2723,9 @@ __device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t
 // shares of its (item, frame) units, without sub-integrations; the parts of an item are summed through
 // a.partial.  2: sub-integrations, equal shares cut between them, so that no sums are shared (LWA block of 128
 // samples, an image set every 4: 256 whole items are two rounds of 152 blocks, the second with 48 idle).
-template <int CUT>
+// ANY (with 0): images that do not begin at 16 bytes.  A form of its own: the test at each store took
+// registers of the frame loop (that block of 128 samples 384 -> 505 us, a burst of 32 samples 97 -> 100).
+template <int CUT, bool ANY = false>
 __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -2980,8 +2980,8 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 start[b] = (uint32_t)split_start(a.wcum, a.c0, a.n_ch, ipc / a.share, a.nt, b, gridDim.x / a.share);
             asm volatile("bar.sync 3, 256;" ::: "memory");
         }
-        good = P == 2 ? ws3_role_e2<CUT, 2>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split)
-                      : ws3_role_e2<CUT, 1>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split);
+        good = P == 2 ? ws3_role_e2<CUT, 2, ANY>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split)
+                      : ws3_role_e2<CUT, 1, ANY>(a, tmem, items, wb0, wb1, warp, lane, m.d2_full, m.d2_empty, start, split);
         if (!good) err_sh = 1;
     }
     tc::fence_before_sync();
@@ -3825,6 +3825,7 @@ epic_status dftgemm_setup(epic_plan_s* p)
     e = allow_max_smem((const void*)k_dftgemm_ws<0>, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws2<0>, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<0>, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<0, true>, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<1>, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_ws3<2>, p->smem_optin);
     p->tc.ws_variant = p->tc.ws ? 3 : 0;
@@ -3890,6 +3891,9 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
     a.nbt = p->tc.nbt;
     a.wcum = p->tc.wcum;
     a.item_order = p->tc.item_order;
+    // Images that do not begin at 16 bytes: k_dftgemm_ws3 has a form for them, its two predecessors have not
+    const bool aligned = ((uintptr_t)out & 15) == 0;
+    const int ws_variant = aligned ? p->tc.ws_variant : 3;
     const int fpc = kGridFramesPerBlock;
     const int F = p->tc.grid_frames;
     for (int c0 = 0; c0 < C; c0 += p->tc.cg) {
@@ -4036,11 +4040,11 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
             a.C = C;
             const int items = ng * a.n_kb * (p->tc.ws ? p->tc.n_gp : a.n_s);
             const int grid = std::min(items, p->sm_count);
-            ev_begin(p, p->tc.ws ? (p->tc.ws_variant == 3 ? "k_dftgemm_ws3" : p->tc.ws_variant == 2 ? "k_dftgemm_ws2" : "k_dftgemm_ws")
+            ev_begin(p, p->tc.ws ? (ws_variant == 3 ? "k_dftgemm_ws3" : ws_variant == 2 ? "k_dftgemm_ws2" : "k_dftgemm_ws")
                                  : p->tc.fast ? "k_dftgemm_mma_fast" : "k_dftgemm_mma", s);
             if (p->tc.ws) {
                 a.n_g = p->tc.n_gp;
-                if (p->tc.ws_variant == 3) {
+                if (ws_variant == 3) {
                     a.partial = p->tc.partial;
                     a.counters = p->tc.counters;
                     a.sB2 = p->tc.ws3_sB2;
@@ -4063,7 +4067,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     // that share tiles over the chip, 1 to 2 % of long ones (tiny station 33 -> 29 us, LWA burst of 32
                     // samples 115 -> 108, LWA block of 1000 1781 -> 1799)
                     const bool early = equal < 500000;
-                    if ((p->tc.split == 1 || (p->tc.split < 0 && cut)) &&
+                    if (aligned && (p->tc.split == 1 || (p->tc.split < 0 && cut)) &&
                         (long long)items * nt < (1LL << 32))  // (item, frame) units are 32-bit in the kernel
                     {
                         // as many as divide a channel's items and the blocks (two for N = 128, eight for N = 256)
@@ -4072,10 +4076,10 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                         ws3_launch(a.sub > 0 ? k_dftgemm_ws3<2> : k_dftgemm_ws3<1>, p->sm_count, p->tc.ws3_smem, s, a, early);
                     } else {
                         a.share = 1;
-                        ws3_launch(k_dftgemm_ws3<0>, grid, p->tc.ws3_smem, s, a, early);
+                        ws3_launch(aligned ? k_dftgemm_ws3<0> : k_dftgemm_ws3<0, true>, grid, p->tc.ws3_smem, s, a, early);
                     }
                 }
-                else if (p->tc.ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);
+                else if (ws_variant == 2) k_dftgemm_ws2<0><<<grid, kWs2Threads, p->tc.smem, s>>>(a);
                 else k_dftgemm_ws<0><<<grid, kWsThreads, p->tc.smem, s>>>(a);
             } else if (p->tc.fast) k_dftgemm_mma_fast<0><<<grid, kMmaThreads, p->tc.smem, s>>>(a);
             else if (p->tc.nb == 2) k_dftgemm_mma<2><<<grid, kMmaThreads, p->tc.smem, s>>>(a);
