@@ -9,6 +9,7 @@
 #include <string>
 
 #include "epic_internal.h"
+#include "wait_flag.h"
 
 namespace {
 std::mutex g_err_mu;
@@ -557,13 +558,10 @@ extern "C" {
 // EPIC_ERR_TIMEOUT when a kernel's wait ran out since the flag was last cleared.
 static epic_status take_timeout(epic_plan_t p)
 {
-    if (!p->tc.status) return EPIC_OK;
     int flag = 0;
-    cudaError_t e = cudaMemcpy(&flag, p->tc.status, sizeof(int), cudaMemcpyDeviceToHost);
+    const cudaError_t e = epic::take_wait_flag(epic::CudaRt{}, p->tc.status, p->tc.counters, p->tc.n_counters, &flag);
     if (e != cudaSuccess) return epic::cuda_fail(p, e, "bounded-wait flag");
     if (!flag) return EPIC_OK;
-    e = cudaMemset(p->tc.status, 0, sizeof(int));
-    if (e != cudaSuccess) return epic::cuda_fail(p, e, "bounded-wait flag");
     p->last_error = "a device-side bounded wait ran out; the images of that call are incomplete";
     return EPIC_ERR_TIMEOUT;
 }

@@ -184,6 +184,9 @@ void worker_loop(epic_server_s* s)
         epic_status status = epic::call_scratch_fit(j->plan, mem);
         cudaError_t e = cudaSuccess;
         if (status == EPIC_OK) e = cudaMemsetAsync(mem.status, 0, sizeof(int), st);
+        // a wait of the slot's last block ran out: counts of split work items may be left standing (wait_flag.h)
+        if (status == EPIC_OK && e == cudaSuccess && s->slot_flag[slot] && mem.counters)
+            e = cudaMemsetAsync(mem.counters, 0, mem.n_counters * sizeof(int), st);
         if (e == cudaSuccess && j->bytes) e = cudaMemcpyAsync(dev, j->host, j->bytes, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) status = EPIC_ERR_CUDA;
         if (status == EPIC_OK) {
