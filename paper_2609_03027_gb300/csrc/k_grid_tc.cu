@@ -40,6 +40,7 @@
 #include "epic_internal.h"
 #include "kcommon.cuh"
 #include "tc_ptx.cuh"
+#include "voltage_words.h"
 
 namespace epic {
 
@@ -75,6 +76,7 @@ struct GridTcArgs {
     int gc, nch;            // groups per staged chunk, chunks
     int raw_stride;         // bytes of a staged frame row (4 x odd)
     int shift;              // rows are staged shifted to a word boundary (samples at no multiple of their size)
+    int edges;              // rows that do not begin and end at a word
     uint32_t vscale, vbias; // half2: 2^-s, and what the decode's offset becomes
     const float4* jones;    // MIX: [C][A][2] polarisation-mixing rows (conj J)
     float unscale;          // MIX: 2^-s of the results (the weights are scaled, the voltages are not)
@@ -150,6 +152,52 @@ __device__ __forceinline__ float4 gt_mix(uint32_t raw, const float4* jm)
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Stages rows that do not begin and end at a word: the aligned words that hold a byte of the row, whose samples keep
+// their offset in the first, or (shift) those words shifted to a word boundary.  Words that reach outside the
+// launch's voltages (of its first row and its last) are read by bytes.
+__device__ __forceinline__ void gt_stage_edges(const uint8_t* lo, const uint8_t* hi, const uint8_t* src, size_t step, int FB, int nf,
+                                            uint8_t* raw, int raw_stride, int shift, int xw, int lane)
+{
+    auto byte = [](const uint8_t* q) { return __ldg(q); };
+    auto word = [&](const uint8_t* q) {
+        return in_block(q, 4, lo, hi) ? __ldg(reinterpret_cast<const uint32_t*>(q)) : edge_word(q, lo, hi, byte);
+    };
+    if (!shift) {
+        for (int f = xw; f < nf; f += kGtExpanders) {
+            const uint8_t* r = src + f * step;
+            const int o = (int)((uintptr_t)r & 3), nw = row_words(o, FB);
+            const uint8_t* w = r - o;
+            const uint32_t d = tc::smem_u32(raw) + f * raw_stride;
+            if (in_block(w, 4 * nw, lo, hi)) {
+                for (int j = lane; j < nw; j += 32) cp_async4(d + 4 * j, w + 4 * j);
+            } else {
+                for (int j = lane; j < nw; j += 32)
+                    if (in_block(w + 4 * j, 4, lo, hi)) cp_async4(d + 4 * j, w + 4 * j);
+                    else reinterpret_cast<uint32_t*>(raw + (size_t)f * raw_stride)[j] = edge_word(w + 4 * j, lo, hi, byte);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return;
+    }
+    const int nw = (FB + 3) >> 2;
+    for (int f = xw; f < nf; f += 4 * kGtExpanders)
+        for (int j = lane; j < nw; j += 32) {
+            uint32_t v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (f + kGtExpanders * k < nf) {
+                    const uint8_t* r = src + (f + kGtExpanders * k) * step;
+                    const int o = (int)((uintptr_t)r & 3);
+                    const uint8_t* w = r - o + 4 * j;
+                    v[k] = __funnelshift_r(word(w), 4 * j + 4 < o + FB ? word(w + 4) : 0u, 8 * o);
+                }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (f + kGtExpanders * k < nf)
+                    reinterpret_cast<uint32_t*>(raw + (size_t)(f + kGtExpanders * k) * raw_stride)[j] = v[k];
+        }
 }
 
 __device__ __forceinline__ float gt_lo(float v) { return v - __half2float(__float2half_rn(v)); }
@@ -334,40 +382,23 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
             const uint8_t* src = a.volt + ((size_t)(a.t0 + f0) * a.C + c) * (size_t)FB;
             const size_t step = (size_t)a.C * FB;
             const int xw = warp - 4;
-            if (!a.shift) {
-                // the aligned words that hold a byte of the row: its samples keep their offset in the first
+            if (!a.edges) {  // rows of whole words
                 for (int f = xw; f < nf; f += kGtExpanders) {
                     const uint8_t* r = src + f * step;
-                    const int o = (int)((uintptr_t)r & 3), nw = (o + FB + 3) >> 2;
                     const uint32_t d = tc::smem_u32(raw) + f * a.raw_stride;
-                    for (int j = lane; j < nw; j += 32) cp_async4(d + 4 * j, r - o + 4 * j);
+                    for (int j = lane; j < FB >> 2; j += 32) cp_async4(d + 4 * j, r + 4 * j);
                 }
                 asm volatile("cp.async.wait_all;" ::: "memory");
+            } else {
+                gt_stage_edges(a.volt, a.volt + (size_t)(a.t0 + a.nt) * step, src, step, FB, nf, raw, a.raw_stride, a.shift, xw, lane);
+            }
+            if (!a.shift) {
                 // the next chunk's rows into L2
                 const int more = min(a.nt - f0, (gend - gb) * FG), lines = (FB + 127) >> 7;
                 for (int i = tid - 128; i < (more - nf) * lines && i < a.gc * FG * lines; i += 32 * kGtExpanders) {
                     const int f = i / lines;
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (nf + f) * step + 128 * (i - f * lines)));
                 }
-            } else {  // rows at any byte address: those words, shifted
-                const int nw = (FB + 3) >> 2;
-                for (int f = xw; f < nf; f += 4 * kGtExpanders)
-                    for (int j = lane; j < nw; j += 32) {
-                        uint32_t v[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (f + kGtExpanders * k < nf) {
-                                const uint8_t* r = src + (f + kGtExpanders * k) * step;
-                                const int o = (int)((uintptr_t)r & 3);
-                                const uint32_t* p32 = reinterpret_cast<const uint32_t*>(r - o) + j;
-                                const uint32_t lo = __ldg(p32), hi = 4 * j + 4 < o + FB ? __ldg(p32 + 1) : 0u;
-                                v[k] = __funnelshift_r(lo, hi, 8 * o);
-                            }
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (f + kGtExpanders * k < nf)
-                                reinterpret_cast<uint32_t*>(raw + (size_t)(f + kGtExpanders * k) * a.raw_stride)[j] = v[k];
-                    }
             }
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kGtExpanders) : "memory");
             for (int t = T0; t < T1; ++t) {
@@ -732,6 +763,7 @@ void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0,
     // a sample (all pols) of 4, 2 or 1 bytes is read from shared memory at its offset in the words, and
     // rows of whole words have no word to spare for an offset
     a.shift = (uintptr_t)volt % (p->P * p->bits / 4) != 0 || (fb % 4 == 0 && (uintptr_t)volt % 4 != 0) ? 1 : 0;
+    a.edges = fb % 4 != 0 || (uintptr_t)volt % 4 != 0 ? 1 : 0;
     // chunks of equal numbers of groups, short enough for about 16 units a block
     const int tiles = p->tc.gt_tiles_h[c0 + n_ch] - p->tc.gt_tiles_h[c0], full = (a.ngr + p->tc.grid_frames - 1) / p->tc.grid_frames;
     const int want = std::max(full, std::min(a.ngr, (16 * p->sm_count + tiles - 1) / tiles));
