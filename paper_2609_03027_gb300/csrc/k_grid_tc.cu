@@ -639,10 +639,12 @@ epic_status grid_tc_setup(epic_plan_s* p)
     const int A = p->A, C = p->C, K = p->K, P = p->P;
     const bool cplx = p->gcf.kind != EPIC_GCF_GAUSSIAN;
     if (grid_tc_smem(p, 1) + 2048 > (size_t)p->smem_optin) return EPIC_ERR_UNSUPPORTED;
-    if (!p->jones.empty()) {  // mixed samples: at most 2 sqrt(2) 128 |J|, split without scaling
+    // Mixed samples are split without scaling: at most 4 |J| of the largest sample, J's largest part, in FP16's range
+    if (!p->jones.empty()) {
         float jmax = 0.f;
         for (float j : p->jones) jmax = std::max(jmax, fabsf(j));
-        if (!(jmax >= 0.25f && jmax <= 128.f)) return EPIC_ERR_UNSUPPORTED;
+        const float vmax = p->bits == 8 ? 128.f : 8.f;
+        if (!(jmax >= 0.25f && jmax <= 128.f && 4.f * vmax * jmax <= 65504.f)) return EPIC_ERR_UNSUPPORTED;
     }
     double wmax = 0.0;
     for (double w : p->w_re) wmax = std::max(wmax, fabs(w));
