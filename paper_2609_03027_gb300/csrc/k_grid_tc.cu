@@ -6,9 +6,10 @@
 //   D_even[pair][n] = W_even[pair][e] . V[n][e]      n = (pol, re | im, frame): 128 columns
 //   D_odd [pair][n] = W_odd [pair][e] . V[n][e]
 // with the voltages exact in FP16 (4- and 8-bit samples times a power of two) and each weight
-// split into FP16 w_hi + w_lo (the remainder: 2^-23 of the weight, as FP32's own rounding), both
+// split into FP16 w_hi + w_lo (what is left: up to 2^-23 of the weight, where FP32 rounds to 2^-24), both
 // accumulated in FP32 in TMEM.  Polarisation-mixed voltages (FP32) are split the same way, and
-// w_hi v_hi + w_lo v_hi + w_hi v_lo is summed.  The gather kernels compute the same sums with FP32 FMAs and are
+// w_hi v_hi + w_lo v_hi + w_hi v_lo is summed (w_lo v_lo, up to 2^-22 of a product, is left out).  The
+// tiles round to 2^-12: errors against 64 bits are those of the FP32 gather kernels to three digits.  The gather kernels compute the same sums with FP32 FMAs and are
 // bound by shared-memory gathers and list walks (7.5 k SM cycles a frame of a 96 x 96 box); here
 // a frame takes its MMAs (64 cycles each, 4 a K step, 32 frames) and its tile stores, which bound it (LWA
 // block of 1000 samples: 0.46 ms for 2.4 GB, 0.28 with the stores of a group to one frame; 0.97 by gather).
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(kGtThreads, 1) k_dftgemm_grid_tc(GridTcArgs a)
                         tc::mma_f16_lead<tc::kDescStep128Hi>(d + 128, wa + (4096 >> 4), va, id, s > 0, lead);
                         tc::mma_f16_lead<tc::kDescStep128Hi>(d, wa + (8192 >> 4), va, id, 1, lead);
                         tc::mma_f16_lead<tc::kDescStep128Hi>(d + 128, wa + (12288 >> 4), va, id, 1, lead);
-                        if (MIX) {  // w_hi v_lo (w_lo v_lo is below FP32's rounding)
+                        if (MIX) {  // w_hi v_lo (w_lo v_lo is far below the tiles' rounding)
                             tc::mma_f16_lead<tc::kDescStep128Hi>(d, wa, va + (kGtVBytes >> 4), id, 1, lead);
                             tc::mma_f16_lead<tc::kDescStep128Hi>(d + 128, wa + (4096 >> 4), va + (kGtVBytes >> 4), id, 1, lead);
                         }
@@ -639,10 +640,18 @@ epic_status grid_tc_setup(epic_plan_s* p)
     const int A = p->A, C = p->C, K = p->K, P = p->P;
     const bool cplx = p->gcf.kind != EPIC_GCF_GAUSSIAN;
     if (grid_tc_smem(p, 1) + 2048 > (size_t)p->smem_optin) return EPIC_ERR_UNSUPPORTED;
-    // Mixed samples are split without scaling: at most 4 |J| of the largest sample, J's largest part, in FP16's range
+    // Mixed samples are split without scaling: at most 4 |J| of the largest sample, J's largest part, in FP16's
+    // range, and the parts' absolute floor (2^-25) below the rounding of the tiles in every channel: with gains of
+    // 1/64 it adds 1e-4 to the tiles' error squared (with 1e-5, images were off by 4.0e-4 of their norm; 2.6e-4
+    // by the gather kernels).  A channel of zeros is exact.
     if (!p->jones.empty()) {
         float jmax = 0.f;
-        for (float j : p->jones) jmax = std::max(jmax, fabsf(j));
+        for (int c = 0; c < C; ++c) {
+            float m = 0.f;
+            for (size_t i = (size_t)c * A * 8; i < (size_t)(c + 1) * A * 8; ++i) m = std::max(m, fabsf(p->jones[i]));
+            if (m > 0.f && m < 0.015625f) return EPIC_ERR_UNSUPPORTED;
+            jmax = std::max(jmax, m);
+        }
         const float vmax = p->bits == 8 ? 128.f : 8.f;
         if (!(jmax >= 0.25f && jmax <= 128.f && 4.f * vmax * jmax <= 65504.f)) return EPIC_ERR_UNSUPPORTED;
     }

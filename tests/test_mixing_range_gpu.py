@@ -27,3 +27,22 @@ def test_largest_matrices_with_the_largest_samples_stay_finite():
         got = plan.image(torch.from_numpy(v).cuda()).cpu().numpy()
         plan.sync()
     assert_parity(got, ref, "dftgemm", "largest mixing matrices")
+
+
+def test_channels_of_small_gains_are_as_accurate_as_with_single_precision_gridding():
+    # gains of one in one channel and of 1e-5 in another: the split's absolute floor of 2^-25 is 1e-3 of a sample there
+    cfg = synth.small_config(n_ant=60, n_chan=2, n_pol=2, grid_n=64, gcf_k=4, n_time=24, seed=7, diameter_m=18.0, sigma=0.8)
+    cfg.jones = synth.make_jones(cfg, seed=3, gain_rms=0.2, leak_rms=0.2)
+    cfg.jones[1] *= 1e-5
+    v = synth.make_voltages(cfg)
+    ref = oracle.image_cfg(cfg, v)
+    err = {}
+    with E.Plan.from_config(cfg, path="dftgemm") as plan:
+        for kernel in (None, 1):                  # the plan's choice, then sums in FP32
+            if kernel:
+                plan.set_param("grid_kernel", kernel)
+            got = plan.image(torch.from_numpy(v).cuda()).cpu().numpy()
+            plan.sync()
+            err[kernel] = [np.linalg.norm(got[c] - ref[c]) / np.linalg.norm(ref[c]) for c in range(2)]
+    for c in range(2):
+        assert err[None][c] <= 1.05 * err[1][c], (c, err)
