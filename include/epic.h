@@ -241,7 +241,7 @@ epic_status epic_plan_get_info(epic_plan_t plan, epic_plan_info* info);
  *                              3 row-major lists of cell pairs (Gaussian GCF), 4 tensor cores
  *                              (max_time >= 16);
  *                 grid_frames  frames per pass of the gridding kernel (4: groups of 64 / n_pol
- *                              frames staged at once);
+ *                              frames staged at once, as many of them as fit);
  *                 chunk_mb     tile-buffer budget of one (channel group, time chunk), 96 MiB to
  *                              24 GiB (the block's samples at most)
  * Images after tuning equal those before up to FP32 rounding order.  reps calls

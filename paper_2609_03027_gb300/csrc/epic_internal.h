@@ -75,6 +75,7 @@ struct TcState {
     long long* gt_tcum = nullptr;
     std::vector<int> gt_tiles_h;   //   gt_tile0 on the host
     int gt_scale = 0;
+    int gt_groups = 0;             //   groups of frames staged at once (grid_frames, or fewer that fit)
     int4* gtask = nullptr;         // balanced gridding: per-channel task lists (device)
     int* gtask_off = nullptr;      // [C + 1]
     int gtask_max = 0;             // largest task list

@@ -3212,13 +3212,14 @@ static epic_status grid_lists_setup(epic_plan_s* p);
 
 // The chosen gridding kernel and what its launches take
 struct GridLaunch {
-    int variant, frames, smem, blocks;
+    int variant, frames, smem, blocks, gt_groups;
     bool pl_stage;
 };
 
 static GridLaunch grid_launch_of(const epic_plan_s* p)
 {
-    return GridLaunch{p->tc.grid_variant, p->tc.grid_frames, p->tc.grid_smem, p->tc.grid_blocks, p->tc.pl_stage};
+    return GridLaunch{p->tc.grid_variant, p->tc.grid_frames, p->tc.grid_smem, p->tc.grid_blocks, p->tc.gt_groups,
+                      p->tc.pl_stage};
 }
 
 static void grid_launch_set(epic_plan_s* p, const GridLaunch& g)
@@ -3227,6 +3228,7 @@ static void grid_launch_set(epic_plan_s* p, const GridLaunch& g)
     p->tc.grid_frames = g.frames;
     p->tc.grid_smem = g.smem;
     p->tc.grid_blocks = g.blocks;
+    p->tc.gt_groups = g.gt_groups;
     p->tc.pl_stage = g.pl_stage;
 }
 
@@ -3782,9 +3784,10 @@ epic_status dftgemm_setup(epic_plan_s* p)
     if (gst == EPIC_OK) {
         const int keep_v = p->tc.grid_variant, keep_f = p->tc.grid_frames;
         p->tc.grid_variant = 4;
-        gst = EPIC_ERR_UNSUPPORTED;
-        for (int gc = 4; gc >= 1 && gst == EPIC_ERR_UNSUPPORTED; gc >>= 1) gst = grid_tc_config(p, gc);
-        if (gst != EPIC_OK) {
+        gst = grid_tc_config(p, 4);
+        if (gst == EPIC_OK) {
+            p->tc.grid_frames = p->tc.gt_groups;
+        } else {
             p->tc.grid_variant = keep_v;
             p->tc.grid_frames = keep_f;
         }

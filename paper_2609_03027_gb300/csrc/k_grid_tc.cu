@@ -9,8 +9,8 @@
 // split into FP16 w_hi + w_lo (what is left: up to 2^-23 of the weight, where FP32 rounds to 2^-24), both
 // accumulated in FP32 in TMEM.  Polarisation-mixed voltages (FP32) are split the same way, and
 // w_hi v_hi + w_lo v_hi + w_hi v_lo is summed (w_lo v_lo, up to 2^-22 of a product, is left out).  The
-// tiles round to 2^-12: errors against 64 bits are those of the FP32 gather kernels to three digits.  The gather kernels compute the same sums with FP32 FMAs and are
-// bound by shared-memory gathers and list walks (7.5 k SM cycles a frame of a 96 x 96 box); here
+// tiles round to 2^-12: errors against 64 bits are those of the FP32 gather kernels to three digits.
+// The gather kernels compute the same sums with FP32 FMAs and are bound by shared-memory gathers and list walks (7.5 k SM cycles a frame of a 96 x 96 box); here
 // a frame takes its MMAs (64 cycles each, 4 a K step, 32 frames) and its tile stores, which bound it (LWA
 // block of 1000 samples: 0.46 ms for 2.4 GB, 0.28 with the stores of a group to one frame; 0.97 by gather).
 // Work: units of one M-tile and one chunk of up to 4 (8) groups, channel by channel and chunk by chunk, cut
@@ -614,20 +614,23 @@ size_t grid_tc_smem(const epic_plan_s* p, int gc)
 
 }  // namespace
 
-// Groups of frames per staged chunk (parameter grid_frames: 1, 2, 4 or 8 groups of 64 / pols frames).
+// Groups of frames per staged chunk (parameter grid_frames: 1, 2, 4 or 8 groups of 64 / pols frames, of which as
+// many are staged as fit: values that the gather kernels take stay valid).
 epic_status grid_tc_config(epic_plan_s* p, int gc)
 {
     if (!p->tc.gt_tile0 || (gc != 1 && gc != 2 && gc != 4 && gc != 8)) return EPIC_ERR_UNSUPPORTED;
-    const size_t bytes = grid_tc_smem(p, gc);
     const void* fn = (const void*)grid_tc_fn(p);
     cudaFuncAttributes fa{};
     cudaError_t e = cudaFuncGetAttributes(&fa, fn);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncGetAttributes(k_dftgemm_grid_tc)");
-    if (bytes + fa.sharedSizeBytes > (size_t)p->smem_optin) return EPIC_ERR_UNSUPPORTED;
+    int fit = gc;
+    while (fit > 1 && grid_tc_smem(p, fit) + fa.sharedSizeBytes > (size_t)p->smem_optin) fit >>= 1;
+    if (grid_tc_smem(p, fit) + fa.sharedSizeBytes > (size_t)p->smem_optin) return EPIC_ERR_UNSUPPORTED;
     e = allow_max_smem(fn, p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_dftgemm_grid_tc)");
     p->tc.grid_frames = gc;
-    p->tc.grid_smem = (int)bytes;
+    p->tc.gt_groups = fit;
+    p->tc.grid_smem = (int)grid_tc_smem(p, fit);
     p->tc.grid_blocks = p->sm_count;
     return EPIC_OK;
 }
@@ -743,7 +746,7 @@ epic_status grid_tc_setup(epic_plan_s* p)
 // Whether the plan's launch configuration is this kernel's for its frames
 bool grid_tc_configured(const epic_plan_s* p)
 {
-    return p->tc.gt_tile0 && (size_t)p->tc.grid_smem == grid_tc_smem(p, p->tc.grid_frames);
+    return p->tc.gt_tile0 && (size_t)p->tc.grid_smem == grid_tc_smem(p, p->tc.gt_groups);
 }
 
 void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0, int n_ch, cudaStream_t s)
@@ -776,7 +779,7 @@ void grid_tc_launch(epic_plan_s* p, const uint8_t* volt, int t0, int nt, int c0,
     a.shift = (uintptr_t)volt % (p->P * p->bits / 4) != 0 || (fb % 4 == 0 && (uintptr_t)volt % 4 != 0) ? 1 : 0;
     a.edges = fb % 4 != 0 || (uintptr_t)volt % 4 != 0 ? 1 : 0;
     // chunks of equal numbers of groups, short enough for about 16 units a block
-    const int tiles = p->tc.gt_tiles_h[c0 + n_ch] - p->tc.gt_tiles_h[c0], full = (a.ngr + p->tc.grid_frames - 1) / p->tc.grid_frames;
+    const int tiles = p->tc.gt_tiles_h[c0 + n_ch] - p->tc.gt_tiles_h[c0], full = (a.ngr + p->tc.gt_groups - 1) / p->tc.gt_groups;
     const int want = std::max(full, std::min(a.ngr, (16 * p->sm_count + tiles - 1) / tiles));
     a.gc = (a.ngr + want - 1) / want;
     a.nch = (a.ngr + a.gc - 1) / a.gc;

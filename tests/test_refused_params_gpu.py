@@ -67,3 +67,17 @@ def test_scratch_that_cannot_be_had_leaves_the_plan_working():
         for _ in range(2):                        # no error left over for the next calls
             assert torch.equal(plan.image(v), before)
             plan.sync()
+
+
+def test_frames_that_the_gather_kernels_take_stay_valid():
+    # 600 dual-pol elements: the tensor-core kernel stages two groups at most
+    cfg = synth.small_config(n_ant=600, n_chan=2, n_pol=2, grid_n=64, gcf_k=3, n_time=70, seed=9, diameter_m=25.0)
+    v = torch.from_numpy(synth.make_voltages(cfg)).cuda()
+    with E.Plan.from_config(cfg, path="dftgemm") as plan:
+        assert plan.get_param("grid_kernel") == 4 and plan.get_param("grid_frames") == 2
+        want = plan.image(v)
+        for F in (4, 8, 1):
+            plan.set_param("grid_frames", F)
+            assert plan.get_param("grid_frames") == F
+            assert torch.equal(plan.image(v), want)
+            plan.sync()
