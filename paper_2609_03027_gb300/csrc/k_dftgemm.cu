@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __rest
                 for (int f = 0; f < F; ++f) g[j][f] = make_float4(0.f, 0.f, 0.f, 0.f);
                 const int r = y * nxp + x + j;
                 const int q1 = y < nyp ? ptr[r + 1] : 0;
+#pragma unroll 4
                 for (int q = y < nyp ? ptr[r] : 0; q < q1; ++q) {
                     int e;
                     float2 w;
@@ -432,30 +433,35 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid_ps(GridArgs a)
         __syncthreads();
         const int half = nxp >> 1;
         const int tasks = tp.z * half;
-        for (int task = tid; task < tasks; task += blockDim.x) {
-            const int y = task / half, x = 2 * (task - y * half);
-            float4 g[2][F];
+        // frames fi0 .. fi0 + M - 1 of the pass: no test of the pass's length in the list walk, so that a
+        // step's loads do not wait for the step before (lists of some 340 entries, 672 elements on an 8 x 8 grid,
+        // one frame of 6 channels: 37 us; 64 to 103 with the test, as the compiler laid the loop out)
+        auto grid_frames = [&](auto width, int fi0) {
+            constexpr int M = decltype(width)::value;
+            for (int task = tid; task < tasks; task += blockDim.x) {
+                const int y = task / half, x = 2 * (task - y * half);
+                float4 g[2][M];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+                for (int j = 0; j < 2; ++j) {
 #pragma unroll
-                for (int fi = 0; fi < F; ++fi) g[j][fi] = make_float4(0.f, 0.f, 0.f, 0.f);
-                const int r = y * nxp + x + j;
-                const int q1 = y < nyp ? sptr[r + 1] : 0;
-                for (int q = y < nyp ? sptr[r] : 0; q < q1; ++q) {
-                    int e;
-                    float2 wv;
-                    if (CPLX) {
-                        e = cone[q];
-                        wv = conw[q];
-                    } else {
-                        const int2 cr = con[q];
-                        e = cr.x;
-                        wv = make_float2(__int_as_float(cr.y), 0.f);
-                    }
+                    for (int fi = 0; fi < M; ++fi) g[j][fi] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const int r = y * nxp + x + j;
+                    const int q1 = y < nyp ? sptr[r + 1] : 0;
+#pragma unroll 4
+                    for (int q = y < nyp ? sptr[r] : 0; q < q1; ++q) {
+                        int e;
+                        float2 wv;
+                        if (CPLX) {
+                            e = cone[q];
+                            wv = conw[q];
+                        } else {
+                            const int2 cr = con[q];
+                            e = cr.x;
+                            wv = make_float2(__int_as_float(cr.y), 0.f);
+                        }
 #pragma unroll
-                    for (int fi = 0; fi < F; ++fi) {
-                        if (fi < nf) {
-                            const float4 v = sv[fi * A + e];
+                        for (int fi = 0; fi < M; ++fi) {
+                            const float4 v = sv[(fi0 + fi) * A + e];
                             if (!CPLX) {
                                 g[j][fi].x = fmaf(wv.x, v.x, g[j][fi].x);
                                 g[j][fi].y = fmaf(wv.x, v.y, g[j][fi].y);
@@ -469,22 +475,28 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid_ps(GridArgs a)
                         }
                     }
                 }
-            }
-            const int kc = x >> 2, within = (x & 2) * 4;  // K index 2 x (re pair) and 2 x + 2 (im pair)
-            const int hpart = y / nyh, R0 = y - hpart * nyh;
+                const int kc = x >> 2, within = (x & 2) * 4;  // K index 2 x (re pair) and 2 x + 2 (im pair)
+                const int hpart = y / nyh, R0 = y - hpart * nyh;
 #pragma unroll
-            for (int fi = 0; fi < F; ++fi) {
-                if (fi >= nf) break;
-                uint8_t* tile =
-                    a.tiles + ((size_t)(f + fi) * a.n_ch + cl) * a.tile_stride + (size_t)hpart * part_bytes;
-                *reinterpret_cast<uint2*>(tile + sw_chunk(R0, kc, N1h) + within) =
-                    make_uint2(pack_h2(g[0][fi].x, g[1][fi].x), pack_h2(g[0][fi].y, g[1][fi].y));
-                if (P == 2) {
-                    const int R1 = nyh + R0;
-                    *reinterpret_cast<uint2*>(tile + sw_chunk(R1, kc, N1h) + within) =
-                        make_uint2(pack_h2(g[0][fi].z, g[1][fi].z), pack_h2(g[0][fi].w, g[1][fi].w));
+                for (int fi = 0; fi < M; ++fi) {
+                    uint8_t* tile = a.tiles + ((size_t)(f + fi0 + fi) * a.n_ch + cl) * a.tile_stride + (size_t)hpart * part_bytes;
+                    *reinterpret_cast<uint2*>(tile + sw_chunk(R0, kc, N1h) + within) =
+                        make_uint2(pack_h2(g[0][fi].x, g[1][fi].x), pack_h2(g[0][fi].y, g[1][fi].y));
+                    if (P == 2) {
+                        const int R1 = nyh + R0;
+                        *reinterpret_cast<uint2*>(tile + sw_chunk(R1, kc, N1h) + within) =
+                            make_uint2(pack_h2(g[0][fi].z, g[1][fi].z), pack_h2(g[0][fi].w, g[1][fi].w));
+                    }
                 }
             }
+        };
+        if (nf == F) {
+            grid_frames(std::integral_constant<int, F>{}, 0);
+        } else {  // a short pass: its frames by powers of two
+            int done = 0;
+            if (F > 4 && nf & 4) grid_frames(std::integral_constant<int, F < 4 ? F : 4>{}, done), done += 4;
+            if (F > 2 && nf & 2) grid_frames(std::integral_constant<int, F < 2 ? F : 2>{}, done), done += 2;
+            if (nf & 1) grid_frames(std::integral_constant<int, 1>{}, done);
         }
         __syncthreads();  // sv and the cell lists are reused by the next pass
         w = wn;

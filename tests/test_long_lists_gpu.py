@@ -28,3 +28,33 @@ def test_pair_lists_of_every_channel_where_task_lists_are_too_long(T):
         plan.sync()
     assert np.all(np.isfinite(got))
     assert_parity(got, ref, "dftgemm", f"T={T}")
+
+
+@pytest.mark.parametrize("tab", [0, 4])
+@pytest.mark.parametrize("T", list(range(1, 12)))
+def test_short_passes_of_the_row_major_kernel(T, tab):
+    # a pass of fewer frames than the kernel's goes by powers of two of them: the same sums in the same order
+    cfg = synth.small_config(n_ant=70, n_chan=2, n_pol=2, grid_n=32, gcf_k=3, n_time=T, seed=14, diameter_m=8.0, sigma=0.7)
+    kw = {}
+    if tab:
+        d = np.arange(3 * tab + 1) / tab - 1.5
+        x, y = np.meshgrid(d, d)
+        kw = {"gcf_table": (np.exp(-(x * x + y * y)) * np.exp(1j * (0.3 * x - 0.2 * y))).astype(np.complex64).view(np.float32),
+              "oversample": tab}
+    v = torch.from_numpy(synth.make_voltages(cfg)).cuda()
+    with E.Plan(cfg.pos_m, cfg.freq_hz, 2, 32, 3, cfg.sigma_cells, cfg.f_ref_hz, False, None, "dftgemm", 15, **kw) as plan:
+        if not tab:
+            plan.set_param("grid_kernel", 1)
+        got = []
+        for F in (1, 2, 4, 8):
+            plan.set_param("grid_frames", F)
+            got.append(plan.image(v))
+            plan.sync()
+        assert all(torch.equal(g, got[0]) for g in got)
+        ref = plan.image(v[:1].contiguous())
+        for t in range(1, T):
+            plan.image(v[t:t + 1].contiguous(), out=ref, accumulate=True)
+        plan.sync()
+    # the frames' products in FP32 sums of another order
+    tol = max(T, 8) * 2.0 ** -24
+    assert (got[0] - ref).norm() <= tol * ref.norm()
