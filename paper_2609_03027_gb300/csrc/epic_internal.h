@@ -74,6 +74,7 @@ struct TcState {
     int* gt_el = nullptr;          //   the weights are scaled by
     long long* gt_tcum = nullptr;
     std::vector<int> gt_tiles_h;   //   gt_tile0 on the host
+    std::vector<long long> gt_cost_h;  //   [C + 1] gt_tcum at each channel's first tile, on the host
     int gt_scale = 0;
     int gt_groups = 0;             //   groups of frames staged at once (grid_frames, or fewer that fit)
     int4* gtask = nullptr;         // balanced gridding: per-channel task lists (device)

@@ -191,7 +191,8 @@ __device__ __forceinline__ void store_pixels16(float* op, int nk, int accumulate
 // then writes the cells as FP16 pairs: consecutive threads cover consecutive
 // cell pairs of a row, so a warp fills whole 128-byte rows of the swizzled tile.
 // With CSR_SMEM the channel's cell lists sit in shared memory as (element, real
-// weight) pairs (Gaussian GCF), otherwise they are read through L1.
+// weight) pairs (Gaussian GCF), otherwise they are read through L1.  The blocks of gridDim.z share the
+// cell pairs.
 template <bool CSR_SMEM, int F>
 __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __restrict__ volt, int t0, int c0,
                                                            int n_ch, int nt, int fpc, int C, int A, int P,
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __rest
             sv[f * A + e] = load_quad(fr, e, P, bits, jm);
         }
         __syncthreads();
-        for (int task = threadIdx.x; task < tasks; task += blockDim.x) {
+        for (int task = threadIdx.x + blockIdx.z * blockDim.x; task < tasks; task += blockDim.x * gridDim.z) {
             const int y = task / half, x = 2 * (task - y * half);
             float4 g[2][F];
 #pragma unroll
@@ -3920,7 +3921,23 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
         for (int t0 = 0; t0 < T; t0 += p->tc.tc) {
             const int nt = std::min(p->tc.tc, T - t0);
             const dim3 gg((nt + fpc - 1) / fpc, ng);
-            if (p->tc.grid_variant == 4) {
+            // One frame fills a 32nd (64th) of the columns of the tensor-core gridding kernel, which builds every
+            // weight operand for it all the same: where that takes more than about 10 us (modelled SM cycles), it is
+            // gathered from the cell lists that every plan has.  Calls of one sample, us: LWA station 40 (tensor
+            // cores) and 30 (gather), SKA-Low 186 and 154, with mixing 204 and 156, 600 elements 47 and 35, 1500
+            // elements with an 8 x 8 GCF 141 and 97.  Two frames: the tensor cores (48 against 71 for 600 elements).
+            // Below that the kernels are a few us apart, and a block's frames called one by one equal the block.
+            const bool one = p->tc.grid_variant == 4 && nt == 1 &&
+                             p->tc.gt_cost_h[c0 + ng] - p->tc.gt_cost_h[c0] > 20000LL * p->sm_count;
+            if (one) {
+                const int pairs = p->tc.grid_max_cells / 2;
+                const unsigned z = std::max(1, std::min((pairs + kThreads - 1) / kThreads, 8 * p->sm_count / ng));
+                ev_begin(p, "k_dftgemm_grid", s);
+                k_dftgemm_grid<false, 1><<<dim3(1, ng, z), kThreads, sizeof(float4) * (size_t)A, s>>>(
+                    volt, t0, c0, ng, nt, 1, C, A, P, p->bits, p->dt.box, p->dt.cell_off, p->dt.cell_ptr, p->dt.contrib_e,
+                    p->dt.contrib_w, p->dt.jones, p->tc.tbox, (uint8_t*)p->scratch, p->tc.stride);
+                ev_end(p, s);
+            } else if (p->tc.grid_variant == 4) {
                 if (!grid_tc_configured(p)) {
                     p->last_error = "tensor path: gridding kernel configuration out of step (internal)";
                     return EPIC_ERR_CUDA;
@@ -4065,7 +4082,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                     a.sB2 = p->tc.ws3_sB2;
                     a.b2_bytes = p->tc.ws3_b2;
                     a.run_counters = p->tc.counters + (p->tc.n_counters - 2 * (size_t)p->sm_count);
-                    a.dense = dftgemm_dense(p);
+                    a.dense = one ? 0 : dftgemm_dense(p);
                     // modelled SM cycles: the launch's per SM, and of whole items dealt in rounds
                     const int ipc = a.n_kb * a.n_g, rounds = (items + p->sm_count - 1) / p->sm_count;
                     long long sum = 0, most = 0;

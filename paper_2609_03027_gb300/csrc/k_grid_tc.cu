@@ -738,6 +738,8 @@ epic_status grid_tc_setup(epic_plan_s* p)
     if (e == cudaSuccess) e = put(&p->tc.gt_tcum, tcum, &bytes);
     p->tc.gt_scale = s;
     p->tc.gt_tiles_h = tile0;
+    p->tc.gt_cost_h.resize(C + 1);
+    for (int c = 0; c <= C; ++c) p->tc.gt_cost_h[c] = tcum[tile0[c]];
     p->dt.dft_bytes += bytes;
     if (e != cudaSuccess) return cuda_fail(p, e, "tensor-core gridding tables");
     return EPIC_OK;
