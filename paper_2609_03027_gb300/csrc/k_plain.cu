@@ -119,7 +119,7 @@ __device__ __forceinline__ void frame_sample(const float2* sv, const uint8_t* fr
 }
 
 constexpr int kRowThreads = 256;
-constexpr int kRowFrames = 2;  // frames of a block: each list entry read from L1 serves both
+constexpr int kRowFrames = 2;  // frames of a block: each list entry read from L1 serves both (one in short launches)
 
 // bytes of k_plain_rows's shared memory beside the frames: twiddles, Y (whose rows the box columns share)
 template <int N1, int N2>
@@ -130,14 +130,14 @@ __host__ __device__ constexpr size_t rows_fft_smem()
 
 // Gridded and row-transformed frames (LWA station: 5.1 ms a block, 2.9 ms of it the 12.9 GB of row
 // stores, the rest the gather's dependent list and voltage reads; 5.6 ms with three blocks an SM instead of
-// four, before a row's cells shared Y's memory): block = frames 2 blockIdx.x, + 1 of
+// four, before a row's cells shared Y's memory): block = frames F blockIdx.x ... of
 // channel blockIdx.y, slice blockIdx.z of the box rows.
 // Rows go in batches of 256 / N2 (both frames, all pols, a few y): the batch's cells are gathered
 // one per thread and step, both frames and pols at once, then N2 threads a row run the two FFT
 // passes (thread j takes n1 = j, j + N2 in pass 1 and k2 = j in pass 2; Y is stored [k2][n1] with
 // stride N1 + 1, which no pass-1 store or pass-2 load of a warp meets twice in one bank) and
 // store rows[(t C + c) P + p][y - y0][N].
-template <int N1, int N2, int P, bool STAGED, bool CPLX>
+template <int N1, int N2, int P, bool STAGED, bool CPLX, int F>
 __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __restrict__ volt, int t0, int nt, int C, int A,
                                                             int bits, const int4* __restrict__ box,
                                                             const int* __restrict__ cell_off,
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
                                                             int ny_max, const float2* __restrict__ twg,
                                                             float2* __restrict__ rows)
 {
-    constexpr int N = N1 * N2, RPC = kRowThreads / N2, S = N2 * (N1 + 1), T = N1 / N2, F = kRowFrames;
+    constexpr int N = N1 * N2, RPC = kRowThreads / N2, S = N2 * (N1 + 1), T = N1 / N2;
     constexpr int L1 = ilog2(N1), L2 = ilog2(N2), YR = RPC / (F * P);
     static_assert(YR >= 1, "a batch holds a row of every frame and pol");
     extern __shared__ float2 sm[];
@@ -194,17 +194,29 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
                 for (int p = 0; p < P; ++p) acc[f][p] = make_float2(0.f, 0.f);
             if (yb + r < ny) {
                 const int cell = (yb + r) * b.z + x, q1 = __ldg(ptr + cell + 1);
-                for (int q = __ldg(ptr + cell); q < q1; ++q) {
-                    const int e = __ldg(ce + q);
-                    const float2 w = CPLX ? __ldg(cw + q) : make_float2(__ldg(&cw[q].x), 0.f);
-#pragma unroll
-                    for (int f = 0; f < F; ++f) {
+                if constexpr (F == 1) {  // short launches: four entries' loads at once (lists of 81 entries: 227 -> 162 us)
+                    auto entry = [&](int i) {
+                        const float2 w = CPLX ? __ldg(cw + i) : make_float2(__ldg(&cw[i].x), 0.f);
                         float2 v[P];
-                        frame_sample<P, STAGED>(sv + (size_t)f * A * P, fr[f], e, bits, jm, v);
+                        frame_sample<P, STAGED>(sv, fr[0], __ldg(ce + i), bits, jm, v);
 #pragma unroll
-                        for (int p = 0; p < P; ++p) {
-                            if (CPLX) acc[f][p] = cfma(w, v[p], acc[f][p]);
-                            else acc[f][p] = make_float2(fmaf(w.x, v[p].x, acc[f][p].x), fmaf(w.x, v[p].y, acc[f][p].y));
+                        for (int p = 0; p < P; ++p) acc[0][p] = cfma(w, v[p], acc[0][p]);
+                    };
+#pragma unroll 4
+                    for (int q = __ldg(ptr + cell); q < q1; ++q) entry(q);
+                } else {
+                    for (int q = __ldg(ptr + cell); q < q1; ++q) {
+                        const int e = __ldg(ce + q);
+                        const float2 w = CPLX ? __ldg(cw + q) : make_float2(__ldg(&cw[q].x), 0.f);
+#pragma unroll
+                        for (int f = 0; f < F; ++f) {
+                            float2 v[P];
+                            frame_sample<P, STAGED>(sv + (size_t)f * A * P, fr[f], e, bits, jm, v);
+#pragma unroll
+                            for (int p = 0; p < P; ++p) {
+                                if (CPLX) acc[f][p] = cfma(w, v[p], acc[f][p]);
+                                else acc[f][p] = make_float2(fmaf(w.x, v[p].x, acc[f][p].x), fmaf(w.x, v[p].y, acc[f][p].y));
+                            }
                         }
                     }
                 }
@@ -449,11 +461,12 @@ void sum_slices(const epic_plan_s* p, const float* partial, size_t n, int S, flo
 
 // the register-FFT kernels of one N, number of pols and form of the frames and weights
 struct RegFft {
-    void (*rows)(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
-                 const float4*, int, int, const float2*, float2*);
+    // of one frame a block, of kRowFrames
+    void (*rows[2])(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
+                    const float4*, int, int, const float2*, float2*);
     void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int);
     int col_tile, col_threads;
-    int rows_batch;               // box rows a block transforms at once
+    int rows_batch[2];            // box rows a block transforms at once
     size_t rows_fft;
     size_t cols_smem, cols_row;   // cols_row: per box row, the staged frames
 };
@@ -465,12 +478,15 @@ RegFft reg_fft_p(bool staged, bool cplx)
     // 128 threads a block (fewer for the smallest grids): four to eight blocks an SM hide the barriers
     constexpr int TX = 128 / N2 < N ? 128 / N2 : N;
     RegFft f{};
-    f.rows = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true> : k_plain_rows<N1, N2, P, true, false>)
-                    : (cplx ? k_plain_rows<N1, N2, P, false, true> : k_plain_rows<N1, N2, P, false, false>);
+    f.rows[0] = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true, 1> : k_plain_rows<N1, N2, P, true, false, 1>)
+                       : (cplx ? k_plain_rows<N1, N2, P, false, true, 1> : k_plain_rows<N1, N2, P, false, false, 1>);
+    f.rows[1] = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true, kRowFrames> : k_plain_rows<N1, N2, P, true, false, kRowFrames>)
+                       : (cplx ? k_plain_rows<N1, N2, P, false, true, kRowFrames> : k_plain_rows<N1, N2, P, false, false, kRowFrames>);
     f.cols = k_plain_cols<N1, N2, TX, P>;
     f.col_tile = TX;
     f.col_threads = TX * N2;
-    f.rows_batch = kRowThreads / N2 / (kRowFrames * P);
+    f.rows_batch[0] = kRowThreads / N2 / P;
+    f.rows_batch[1] = kRowThreads / N2 / (kRowFrames * P);
     f.rows_fft = rows_fft_smem<N1, N2>();
     f.cols_smem = sizeof(float2) * ((size_t)N + (size_t)P * N * TX);
     f.cols_row = sizeof(float2) * (size_t)col_stages(N) * P * TX;
@@ -507,11 +523,11 @@ size_t cols_smem_for(const epic_plan_s* p, const RegFft& f)
     return f.cols_smem + f.cols_row * std::min(p->box_max_y, p->N);
 }
 
-size_t frame_smem(const epic_plan_s* p, FrameForm form)
+size_t frame_smem(const epic_plan_s* p, FrameForm form, int frames = kRowFrames)
 {
     const size_t fb = (size_t)p->A * p->P * (p->bits / 4);
-    if (form == kFrameStaged) return kRowFrames * sizeof(float2) * (size_t)p->A * p->P;
-    return form == kFrameBytes ? kRowFrames * ((fb + 15) & ~(size_t)15) : 0;
+    if (form == kFrameStaged) return frames * sizeof(float2) * (size_t)p->A * p->P;
+    return form == kFrameBytes ? frames * ((fb + 15) & ~(size_t)15) : 0;
 }
 
 FrameForm frame_form(const epic_plan_s* p)
@@ -803,7 +819,8 @@ epic_status plain_setup(epic_plan_s* p)
         p->last_error = "plain path: FFT shared memory exceeds the device limit";
         return EPIC_ERR_UNSUPPORTED;
     }
-    e = allow_max_smem((const void*)rf.rows, p->smem_optin);
+    e = allow_max_smem((const void*)rf.rows[0], p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)rf.rows[1], p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_rows)");
     e = allow_max_smem((const void*)rf.cols, p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_cols)");
@@ -846,10 +863,21 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             ev_begin(p, "k_plain_rows", s);
             // slices of the rows where frames and channels alone leave fewer than eight blocks an SM (one channel
             // of a 512-pixel grid: 2.45 ms a block of 1024 samples with 128 blocks a chunk, 1.97 with slices)
-            const int fb = (nt + kRowFrames - 1) / kRowFrames, batches = (ny_max + rf.rows_batch - 1) / rf.rows_batch;
-            const int Z = std::max(1, std::min(batches, (int)(8LL * p->sm_count / ((long long)fb * C))));
-            launch_early(t0 > 0, rf.rows, dim3(fb, C, Z), kRowThreads,
-                         rf.rows_fft + frame_smem(p, form), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
+            auto grid_of = [&](int frames) {
+                const int batch = rf.rows_batch[frames > 1], fb = (nt + frames - 1) / frames;
+                return dim3(fb, C, std::max(1, std::min((ny_max + batch - 1) / batch, (int)(8LL * p->sm_count / ((long long)fb * C)))));
+            };
+            // One frame a block while two would leave SMs with fewer than two blocks, unless a thread then walks more
+            // lists: a walk takes 1.4 times as long for two frames, but a batch of one has up to twice the rows.  Us of
+            // rows with two frames a block and with one: 41 channels of 16 x 16 cells of 53 entries, 2 samples 66 and 45;
+            // 113 of 32 x 32 cells of 81 entries, one sample 227 and 113; 4 of 32 x 32 cells of 96 entries, one 77
+            // and 130.
+            auto walks = [&](int i) { return (std::min(rf.rows_batch[i], ny_max) * p->box_max_x + kRowThreads - 1) / kRowThreads; };
+            dim3 g = grid_of(kRowFrames);
+            const int frames = (long long)g.x * g.y * g.z < 2LL * p->sm_count && 5 * walks(0) <= 7 * walks(1) ? 1 : kRowFrames;
+            if (frames == 1) g = grid_of(1);
+            launch_early(t0 > 0, rf.rows[frames > 1], g, kRowThreads,
+                         rf.rows_fft + frame_smem(p, form, frames), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
                          p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, ny_max, p->dt.twiddle, grid);
             ev_end(p, s);
             // slices of whole intervals, or of at least four frames; the same for every chunk of the call,

@@ -52,3 +52,19 @@ def test_box_rows_and_columns(case):
     assert np.allclose(twice, 2 * a, rtol=1e-6, atol=1e-6 * np.abs(a).max())
     for k, (g, r) in enumerate(zip(a, ref) if sub else [(a, ref)]):
         assert_parity(g, r, "plain", f"{case} set {k}")
+
+
+@pytest.mark.parametrize("case", [
+    # A, C, P, N, K, T, diameter, bits: one frame a block where two would leave the chip empty, both forms of the gather
+    (300, 41, 2, 32, 4, 3, 7.0, 4), (300, 41, 1, 32, 4, 3, 7.0, 8), (9000, 3, 2, 32, 2, 1, 7.0, 4),
+    (400, 4, 2, 64, 7, 1, 24.0, 4),     # two all the same: a batch of one frame has twice the rows
+], ids=lambda c: "-".join(str(x) for x in c))
+def test_short_launches(case):
+    A, C, P, N, K, T, diam, bits = case
+    cfg = synth.small_config(n_ant=A, n_chan=C, n_pol=P, grid_n=N, gcf_k=K, n_time=T, seed=A + T, diameter_m=diam, sigma=0.7)
+    cfg = dataclasses.replace(cfg, input_bits=bits)
+    v = synth.random_bytes((T, C, A, P) + ((2,) if bits == 8 else ()), seed=A)
+    with E.Plan.from_config(cfg, path="plain", max_time=T) as plan:
+        got = plan.image(torch.from_numpy(v).cuda()).cpu().numpy()
+        plan.sync()
+    assert_parity(got, oracle_image(cfg, v), "plain", str(case))
