@@ -172,6 +172,7 @@ struct epic_plan_s {
     int plain_fft = 0;                    // plain path: 0 register two-pass FFTs, 1 shared-memory Stockham
     int plain_slices = 1;                 // plain path: slices of a chunk's frames in k_plain_cols
     int plain_slots = 1;                  //   blocks of it that are resident at once
+    int plain_cuts = 1;                   //   slices of each interval (with sub-integrations)
 
     size_t chunk_budget = 0;              // scratch budget of one time chunk (chunked paths)
 

@@ -291,18 +291,20 @@ constexpr int kColRun = 64;
 constexpr int col_stages(int N) { return N <= 256 ? 3 : 0; }
 
 // Column transforms and products: block = TX adjacent columns of channel blockIdx.y and slice
-// blockIdx.z of the chunk's frames (of its intervals, with sub-integrations); N2 threads a column,
+// blockIdx.z of the chunk's frames (with sub-integrations: of its intervals, or slice blockIdx.z % cuts of
+// interval blockIdx.z / cuts); N2 threads a column,
 // lanes on adjacent columns (every global access of a warp one contiguous run per row, Y
 // [n1][k2][column] without bank conflicts).  The box rows of the next two frames are on their way
 // into shared memory while a frame is transformed (loaded when needed, the HBM latency of each
 // pol showed: 4.4 k cycles a tile and frame).  A thread ends up with the pixels ky = j + N2 k1 of
 // its column and keeps their sums in registers; at N1 = 32 X's pixels wait in the thread's own
 // slots of the exchange buffer while Y is transformed.  out: the images, or the slice's partial sums.
-template <int N1, int N2, int TX, int P>
+// CUT: that last form (a form of its own: the LWA station's columns took 2 % longer with the choice inside).
+template <int N1, int N2, int TX, int P, bool CUT>
 __global__ void __launch_bounds__(TX * N2) k_plain_cols(const float2* __restrict__ rows, int nt, int C, int ny_max,
                                                         const int4* __restrict__ box, const float2* __restrict__ twg,
                                                         float* __restrict__ out, float* __restrict__ partial,
-                                                        int accumulate, int sub, int out_iv0)
+                                                        int accumulate, int sub, int out_iv0, int cuts)
 {
     constexpr int N = N1 * N2, T = N1 / N2, L1 = ilog2(N1), L2 = ilog2(N2), NP = P == 2 ? 4 : 1, ST = col_stages(N);
     constexpr size_t NN = (size_t)N * N;
@@ -316,7 +318,9 @@ __global__ void __launch_bounds__(TX * N2) k_plain_cols(const float2* __restrict
     const int y0 = b.y, ny = min(b.w, N - b.y);
     load_step_twiddles<N1, N2>(tw, twg);
     const int unit = sub > 0 ? sub : 1, units = nt / unit, S = gridDim.z;
-    const int ta = (int)((long long)units * blockIdx.z / S) * unit, tb = (int)((long long)units * (blockIdx.z + 1) / S) * unit;
+    const int z = CUT ? blockIdx.z % cuts : 0, i0 = CUT ? blockIdx.z / cuts * sub : 0;
+    const int ta = CUT ? i0 + (int)((long long)sub * z / cuts) : (int)((long long)units * blockIdx.z / S) * unit;
+    const int tb = CUT ? i0 + (int)((long long)sub * (z + 1) / cuts) : (int)((long long)units * (blockIdx.z + 1) / S) * unit;
     float xx[N1], yy[P == 2 ? N1 : 1], rxy[P == 2 ? N1 : 1], ixy[P == 2 ? N1 : 1];
     auto clear = [&]() {
 #pragma unroll
@@ -351,6 +355,7 @@ __global__ void __launch_bounds__(TX * N2) k_plain_cols(const float2* __restrict
         cp_async_commit();
     };
     auto image = [&](int t) {  // where frame t's sums go
+        if (CUT) return partial + (((size_t)z * units + t / sub) * C + c) * NP * NN;  // this slice's sums of every interval
         return sub > 0 ? out + ((size_t)(out_iv0 + t / sub) * C + c) * NP * NN
                        : (partial ? partial + (size_t)blockIdx.z * C * NP * NN : out) + (size_t)c * NP * NN;
     };
@@ -464,7 +469,8 @@ struct RegFft {
     // of one frame a block, of kRowFrames
     void (*rows[2])(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
                     const float4*, int, int, const float2*, float2*);
-    void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int);
+    void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int, int);
+    void (*cut)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int, int);
     int col_tile, col_threads;
     int rows_batch[2];            // box rows a block transforms at once
     size_t rows_fft;
@@ -482,7 +488,8 @@ RegFft reg_fft_p(bool staged, bool cplx)
                        : (cplx ? k_plain_rows<N1, N2, P, false, true, 1> : k_plain_rows<N1, N2, P, false, false, 1>);
     f.rows[1] = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true, kRowFrames> : k_plain_rows<N1, N2, P, true, false, kRowFrames>)
                        : (cplx ? k_plain_rows<N1, N2, P, false, true, kRowFrames> : k_plain_rows<N1, N2, P, false, false, kRowFrames>);
-    f.cols = k_plain_cols<N1, N2, TX, P>;
+    f.cols = k_plain_cols<N1, N2, TX, P, false>;
+    f.cut = k_plain_cols<N1, N2, TX, P, true>;
     f.col_tile = TX;
     f.col_threads = TX * N2;
     f.rows_batch[0] = kRowThreads / N2 / P;
@@ -544,21 +551,29 @@ FrameForm frame_form(const epic_plan_s* p)
 // each -- and to the partial sums' traffic beside the rows'.  One for the LWA station's 1024 tiles
 // (6.1 ms a block; 6.8 in three slices), nine for the 64 tiles of the one-channel 512 x 512 station
 // (1.65 ms; 1.84 in four, 3.4 in two).
-int col_slices(const epic_plan_s* p, const RegFft& f, int nt, int slots)
+// With sub-integrations a slice is of whole intervals, or each interval is cut (`cuts` slices, whose partial
+// sums k_plain_sum adds up): two 250-sample intervals of 8 channels of 64 x 64 pixels 188 us whole, 57 and
+// 8 for the sums cut.
+int col_slices(const epic_plan_s* p, const RegFft& f, int nt, int slots, int* cuts)
 {
     const double B = (double)(p->N / f.col_tile) * p->C;
+    const int iv = p->sub > 0 ? std::max(1, nt / p->sub) : 1;
     const double img = sizeof(float) * (double)p->C * p->nprod * p->N * p->N;
     const double rows = sizeof(float2) * (double)nt * p->C * p->P * p->box_max_y * p->N;
     int best = 1;
     double cost = 1e30;
-    for (int S = 1; S <= 16 && S <= std::max(1, nt / 4); ++S) {
+    auto take = [&](int S, double sums) {  // sums: the partial sums' images
         const double w = B * S / slots, m = B * S / p->sm_count;
-        const double k = 0.5 * std::ceil(w) / w + 0.5 * std::ceil(m) / m + (S > 1 && p->sub == 0 ? 2.0 * S * img / rows : 0.0);
-        if (k < cost - 1e-9) {
-            cost = k;
-            best = S;
-        }
-    }
+        const double k = 0.5 * std::ceil(w) / w + 0.5 * std::ceil(m) / m + 2.0 * sums * img / rows;
+        if (k >= cost - 1e-9) return false;
+        cost = k;
+        best = S;
+        return true;
+    };
+    *cuts = 1;
+    for (int S = 1; S <= 16 && S <= std::max(1, p->sub > 0 ? std::min(nt / 4, iv) : nt / 4); ++S) take(S, S > 1 && p->sub == 0 ? S : 0);
+    for (int q = 2; p->sub > 0 && q <= 16 && q <= p->sub / 4; ++q)
+        if (take(iv * q, (double)iv * q)) *cuts = q;
     return best;
 }
 
@@ -764,20 +779,22 @@ epic_status plain_set_chunk(epic_plan_s* p, size_t budget)
         return EPIC_ERR_UNSUPPORTED;
     }
     size_t bytes = (per_t * tcn + 255) & ~(size_t)255;
-    int slices = 1;
+    int slices = 1, cuts = 1;
     if (p->plain_fft == 0) {
         const RegFft f = reg_fft_for(p, frame_form(p) == kFrameStaged);
         int occ = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)f.cols, f.col_threads, cols_smem_for(p, f));
         if (e != cudaSuccess) return cuda_fail(p, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(k_plain_cols)");
         p->plain_slots = std::max(1, occ) * p->sm_count;
-        slices = col_slices(p, f, tcn, p->plain_slots);
-        if (p->sub == 0 && slices > 1) bytes += sizeof(float) * (size_t)slices * p->C * p->nprod * p->N * p->N;
+        slices = col_slices(p, f, tcn, p->plain_slots, &cuts);
+        const int sums = p->sub == 0 ? (slices > 1 ? slices : 0) : cuts > 1 ? tcn / p->sub * cuts : 0;
+        bytes += sizeof(float) * (size_t)sums * p->C * p->nprod * p->N * p->N;
     }
     const epic_status st = scratch_resize(p, bytes, false, "plain grid buffer");
     if (st != EPIC_OK) return st;
     p->chunk_budget = budget;
     p->plain_slices = slices;
+    p->plain_cuts = cuts;
     p->time_chunk = tcn;
     return EPIC_OK;
 }
@@ -823,6 +840,7 @@ epic_status plain_setup(epic_plan_s* p)
     if (e == cudaSuccess) e = allow_max_smem((const void*)rf.rows[1], p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_rows)");
     e = allow_max_smem((const void*)rf.cols, p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)rf.cut, p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_cols)");
     return plain_set_chunk(p, kGridBudget);
 }
@@ -882,24 +900,27 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             ev_end(p, s);
             // slices of whole intervals, or of at least four frames; the same for every chunk of the call,
             // whose partial sums add up over the chunks
-            const int S = std::max(1, std::min(p->plain_slices, p->sub > 0 ? nt / p->sub : std::min(p->time_chunk, T) / 4));
+            const int iv = p->sub > 0 ? nt / p->sub : 0, cuts = p->plain_cuts;
+            const int S = cuts > 1 ? iv * cuts
+                                   : std::max(1, std::min(p->plain_slices, p->sub > 0 ? iv : std::min(p->time_chunk, T) / 4));
             float* partial = nullptr;
-            if (S > 1 && p->sub == 0)
+            if (cuts > 1 || (S > 1 && p->sub == 0))
                 partial = reinterpret_cast<float*>(
                     (uint8_t*)p->scratch + ((sizeof(float2) * (size_t)p->time_chunk * C * P * ny_max * N + 255) & ~(size_t)255));
             ev_begin(p, "k_plain_cols", s);
             // Early where its blocks fill the chip: fewer of them would crowd onto the SMs that come free first (21
             // blocks of 100 frames, one 32 x 32 image set: 158 us a call, 62 in turn)
             const bool full = (long long)(N / rf.col_tile) * C * S >= p->plain_slots;
-            launch_early(full, rf.cols, dim3(N / rf.col_tile, C, S), rf.col_threads, cols_smem_for(p, rf), s,
-                         (const float2*)grid, nt, C, ny_max, p->dt.box, p->dt.twiddle, out, partial, partial ? t0 > 0 : acc,
-                         p->sub, p->sub > 0 ? t0 / p->sub : 0);
+            launch_early(full, cuts > 1 ? rf.cut : rf.cols, dim3(N / rf.col_tile, C, S), rf.col_threads, cols_smem_for(p, rf), s,
+                         (const float2*)grid, nt, C, ny_max, p->dt.box, p->dt.twiddle, out, partial,
+                         cuts > 1 ? 0 : partial ? t0 > 0 : acc, p->sub, p->sub > 0 ? t0 / p->sub : 0, cuts);
             ev_end(p, s);
-            if (partial && t0 + nt == T) {
-                const size_t n = (size_t)C * p->nprod * N * N;
+            if (partial && (cuts > 1 || t0 + nt == T)) {
+                const size_t set = (size_t)C * p->nprod * N * N, n = cuts > 1 ? iv * set : set;
+                float* o = out + (cuts > 1 ? t0 / p->sub * set : 0);
                 ev_begin(p, "k_plain_sum", s);
-                if (((uintptr_t)out & 15) == 0) sum_slices<float4>(p, partial, n, S, out, accumulate, s);
-                else sum_slices<float>(p, partial, n, S, out, accumulate, s);
+                if (((uintptr_t)o & 15) == 0) sum_slices<float4>(p, partial, n, cuts > 1 ? cuts : S, o, accumulate, s);
+                else sum_slices<float>(p, partial, n, cuts > 1 ? cuts : S, o, accumulate, s);
                 ev_end(p, s);
             }
         } else {

@@ -68,3 +68,30 @@ def test_short_launches(case):
         got = plan.image(torch.from_numpy(v).cuda()).cpu().numpy()
         plan.sync()
     assert_parity(got, oracle_image(cfg, v), "plain", str(case))
+
+
+@pytest.mark.parametrize("case", [
+    # A, C, P, N, K, T, diameter, sub, chunk: intervals cut into slices
+    (20, 3, 2, 8, 2, 8, 3.0, 8, 64), (20, 2, 1, 32, 3, 66, 7.0, 33, 64), (30, 1, 2, 64, 3, 300, 17.0, 100, 1),
+    (25, 1, 2, 256, 3, 26, 60.0, 13, 64), (25, 1, 1, 512, 2, 18, 120.0, 9, 16),
+], ids=lambda c: "-".join(str(x) for x in c))
+def test_cut_intervals(case):
+    A, C, P, N, K, T, diam, sub, mb = case
+    cfg = synth.small_config(n_ant=A, n_chan=C, n_pol=P, grid_n=N, gcf_k=K, n_time=T, seed=A + T, diameter_m=diam, sigma=0.7)
+    cfg = dataclasses.replace(cfg, sub_int=sub)
+    v = synth.random_bytes((T, C, A, P), seed=A)
+    ref = oracle_image(cfg, v)
+    with E.Plan.from_config(cfg, path="plain", max_time=T) as plan:
+        d = torch.from_numpy(v).cuda()
+        assert plan.info()["n_kernels"] == 3
+        got = plan.image(d)
+        a = got.cpu().numpy()
+        plan.set_param("chunk_mb", mb)
+        b = plan.image(d).cpu().numpy()
+        assert np.linalg.norm(b - a) <= 1e-6 * np.linalg.norm(a)
+        plan.image(d, out=got)
+        twice = plan.image(d, out=got, accumulate=True).cpu().numpy()
+        plan.sync()
+    assert np.allclose(twice, 2 * b, rtol=1e-6, atol=1e-6 * np.abs(a).max())
+    for k, (g, r) in enumerate(zip(a, ref)):
+        assert_parity(g, r, "plain", f"{case} set {k}")
