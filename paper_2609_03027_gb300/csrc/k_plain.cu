@@ -836,8 +836,8 @@ epic_status plain_setup(epic_plan_s* p)
         p->last_error = "plain path: FFT shared memory exceeds the device limit";
         return EPIC_ERR_UNSUPPORTED;
     }
-    e = allow_max_smem((const void*)rf.rows[0], p->smem_optin);
-    if (e == cudaSuccess) e = allow_max_smem((const void*)rf.rows[1], p->smem_optin);
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i)  // short launches stage their frames
+        e = allow_max_smem((const void*)(i < 2 ? rf : reg_fft_for(p, true)).rows[i & 1], p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_rows)");
     e = allow_max_smem((const void*)rf.cols, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)rf.cut, p->smem_optin);
@@ -875,8 +875,8 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
         const int nt = std::min(p->time_chunk, T - t0);
         const int acc = (accumulate || (t0 > 0 && p->sub == 0)) ? 1 : 0;
         if (p->plain_fft == 0) {
-            const FrameForm form = frame_form(p);
-            const RegFft rf = reg_fft_for(p, form == kFrameStaged);
+            FrameForm form = frame_form(p);
+            RegFft rf = reg_fft_for(p, form == kFrameStaged);
             const int ny_max = std::min(p->box_max_y, N);
             ev_begin(p, "k_plain_rows", s);
             // slices of the rows where frames and channels alone leave fewer than eight blocks an SM (one channel
@@ -885,15 +885,26 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
                 const int batch = rf.rows_batch[frames > 1], fb = (nt + frames - 1) / frames;
                 return dim3(fb, C, std::max(1, std::min((ny_max + batch - 1) / batch, (int)(8LL * p->sm_count / ((long long)fb * C)))));
             };
-            // One frame a block while two would leave SMs with fewer than two blocks, unless a thread then walks more
-            // lists: a walk takes 1.4 times as long for two frames, but a batch of one has up to twice the rows.  Us of
-            // rows with two frames a block and with one: 41 channels of 16 x 16 cells of 53 entries, 2 samples 66 and 45;
-            // 113 of 32 x 32 cells of 81 entries, one sample 227 and 113; 4 of 32 x 32 cells of 96 entries, one 77
-            // and 130.
+            auto blocks = [](dim3 g) { return (long long)g.x * g.y * g.z; };
+            // Short launches.  Frames are staged as FP32 samples wherever all blocks are resident with them (1861 elements,
+            // 54 channels of 16 x 16 cells, one sample: 138 us, 337 as bytes).  One frame a block while two would
+            // leave SMs with fewer than four blocks, unless a thread then walks more lists: a walk takes 1.4 times as
+            // long for two frames, but a batch of one has up to twice the rows.  Us of rows with two frames a block and
+            // with one: 41 channels of 16 x 16 cells of 53 entries, 2 samples 66 and 45; 113 of 32 x 32 cells of 81
+            // entries, one sample 227 and 113; 4 of 32 x 32 cells of 96 entries, one 77 and 130.
+            auto fits = [&](int frames, dim3 g) {
+                const size_t per_sm = (size_t)((blocks(g) + p->sm_count - 1) / p->sm_count);
+                return form == kFrameStaged || rf.rows_fft + frame_smem(p, kFrameStaged, frames) <= (size_t)p->smem_optin / per_sm;
+            };
             auto walks = [&](int i) { return (std::min(rf.rows_batch[i], ny_max) * p->box_max_x + kRowThreads - 1) / kRowThreads; };
             dim3 g = grid_of(kRowFrames);
-            const int frames = (long long)g.x * g.y * g.z < 2LL * p->sm_count && 5 * walks(0) <= 7 * walks(1) ? 1 : kRowFrames;
+            const int frames =
+                blocks(g) < 4LL * p->sm_count && 5 * walks(0) <= 7 * walks(1) && fits(1, grid_of(1)) ? 1 : kRowFrames;
             if (frames == 1) g = grid_of(1);
+            if (form != kFrameStaged && fits(frames, g)) {
+                form = kFrameStaged;
+                rf = reg_fft_for(p, true);
+            }
             launch_early(t0 > 0, rf.rows[frames > 1], g, kRowThreads,
                          rf.rows_fft + frame_smem(p, form, frames), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
                          p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, ny_max, p->dt.twiddle, grid);

@@ -95,3 +95,11 @@ def test_cut_intervals(case):
     assert np.allclose(twice, 2 * b, rtol=1e-6, atol=1e-6 * np.abs(a).max())
     for k, (g, r) in enumerate(zip(a, ref)):
         assert_parity(g, r, "plain", f"{case} set {k}")
+
+
+@pytest.mark.parametrize("case", [
+    # A, C, P, N, K, T, diameter, bits: more elements than the staged form takes in long launches, staged in these
+    (1900, 30, 2, 32, 3, 5, 7.0, 4), (2000, 2, 2, 64, 7, 5, 24.0, 8), (1900, 60, 2, 32, 3, 16, 7.0, 4),
+], ids=lambda c: "-".join(str(x) for x in c))
+def test_short_launches_of_many_elements(case):
+    test_short_launches(case)
