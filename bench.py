@@ -85,7 +85,7 @@ def kernel_model(name, cfg, T, info):
         return "hbm", row_bytes + 2 * C * nprod * N * N * 4, "B"
     if name == "k_plain_grid":
         return "hbm", nt * C * A * P + grid_bytes, "B"
-    if name in ("k_plain_fft_rows", "k_plain_fft_cols"):
+    if name in ("k_plain_fft_rows_smem", "k_plain_fft_cols_smem"):
         return "hbm", 2 * grid_bytes, "B"
     if name == "k_plain_sqacc":
         return "hbm", grid_bytes + 2 * C * nprod * N * N * 4, "B"

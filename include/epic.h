@@ -170,7 +170,8 @@ epic_status epic_plan_destroy(epic_plan_t plan);
 /* Image one voltage block (Eq. 1-2) on `stream` (a cudaStream_t; NULL = legacy
  * default stream).  volt: device uint8[T][C][A][P] (uint8[T][C][A][P][2] for 8+8-bit
  * input); out: device float32 [C][n_prod][N][N] ([T/S][C][n_prod][N][N] with
- * sub-integrations of S samples), written (EPIC_RESET) or added to (EPIC_ACCUMULATE).
+ * sub-integrations of S samples), written (EPIC_RESET) or added to (EPIC_ACCUMULATE).  volt may begin at any
+ * byte, out at any float (16-byte aligned images take the faster stores); nothing outside them is read.
  * 0 <= T <= max_time; T = 0 with EPIC_RESET zeroes out.  Asynchronous: returns
  * after launching.  The plan's scratch is reused by every call, so calls on one
  * plan must not overlap on different streams.
@@ -199,7 +200,8 @@ epic_status epic_image_host(epic_plan_t plan, const uint8_t* volt_host, int T, v
 /* Wait for the plan's last stream and report any asynchronous CUDA error, or
  * EPIC_ERR_TIMEOUT when a bounded device-side wait of one of the plan's kernels
  * ran out since the last report (the images of that call are incomplete; the
- * plan stays usable).  The flag is read and cleared here and by epic_image_host. */
+ * plan stays usable: the counts of split work items are cleared with the flag).  The flag is read and
+ * cleared here and by epic_image_host. */
 epic_status epic_sync(epic_plan_t plan);
 
 /* Failure-detection self-test: on `stream`, one block that holds tensor memory

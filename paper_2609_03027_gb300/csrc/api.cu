@@ -457,7 +457,8 @@ epic_status epic_plan_get_info(epic_plan_t p, epic_plan_info* info)
     info->device_bytes = p->table_bytes + p->scratch_bytes + p->dt.dft_bytes + p->stage_bytes;
     int nk = 0;
     const int chunks = p->time_chunk > 0 ? (p->max_time + p->time_chunk - 1) / p->time_chunk : 1;
-    if (p->path == EPIC_PATH_PLAIN_FP32) nk = p->plain_fft ? 4 * chunks : (p->plain_cuts > 1 ? 3 : 2) * chunks + (p->sub == 0 && p->plain_slices > 1 ? 1 : 0);
+    if (p->path == EPIC_PATH_PLAIN_FP32)
+        nk = p->plain_fft ? 4 * chunks : (p->plain_cuts > 1 ? 3 : 2) * chunks + (p->sub == 0 && p->plain_slices > 1 ? 1 : 0);
     else if (p->path == EPIC_PATH_DFTGEMM_FP16) nk = 2 * chunks * ((p->C + p->tc.cg - 1) / std::max(1, p->tc.cg));
     else nk = p->scratch ? 2 : 1;
     info->n_kernels = nk;

@@ -2678,8 +2678,8 @@ __device__ __forceinline__ bool ws3_s1(Ws3Bars& m, int ks, int NU, unsigned& u, 
 
 // Stage 2: KS = nyh / 8 K steps from A2 (TMEM, part h at nyh words) and B2[u & 1] into both halves of D2.
 template <int KS>
-__device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsigned& u, unsigned& fr, uint32_t d2, uint32_t a2, int P, uint32_t b2, uint32_t b2_bytes,
-                                       uint32_t lead)
+__device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsigned& u, unsigned& fr, uint32_t d2,
+                                       uint32_t a2, int P, uint32_t b2, uint32_t b2_bytes, uint32_t lead)
 {
     const uint32_t id2 = tc::idesc_f16_f32(128, 64 * P), pb = (uint32_t)(128 * P) * 2;  // a K step of B2, 16-byte units
 #pragma unroll 1
@@ -2715,8 +2715,8 @@ __device__ __forceinline__ bool ws3_s2(Ws3Bars& m, int ks, int nt, int H, unsign
 
 // Epilogue 1 of NU sub-frames.
 template <int NYC, int IM>
-__device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t taddr, uint32_t d1_cols, int P, int lane, uint32_t b2, uint32_t b2_bytes,
-                                       int row)
+__device__ __forceinline__ bool ws3_e1(Ws3Bars& m, int NU, unsigned& u, uint32_t taddr, uint32_t d1_cols, int P, int lane,
+                                       uint32_t b2, uint32_t b2_bytes, int row)
 {
 #pragma unroll 1
     for (const unsigned end = u + NU; u != end; ++u) {
@@ -2881,7 +2881,11 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 good = ws3_wait(&m.bar_a, ph_a, 0);
                 if (!good) break;
                 switch (ks) {
-#define EPIC_S1(n)                                                                                                   case n:                                                                                                              good = ws3_s1<n>(m, n, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1),                          a.b1_bytes, N1, a.dense, lead);                                                                          break;
+#define EPIC_S1(n)                                                                                                  \
+    case n:                                                                                                         \
+        good = ws3_s1<n>(m, n, NU, u, b, NB, ph_tile, tmem, a.d1_cols, da, tc::smem_u32(sbase + a.sB1), a.b1_bytes, \
+                         N1, a.dense, lead);                                                                        \
+        break;
                     EPIC_KS_CASES(EPIC_S1)
 #undef EPIC_S1
                     default:
@@ -2904,7 +2908,10 @@ __global__ void __launch_bounds__(kWs3Threads, 1) k_dftgemm_ws3(MmaArgs a)
                 good = ws3_wait(&m.a2_full, ph_a2, 0);
                 if (!good) break;
                 switch (ks) {
-#define EPIC_S2(n)                                                                                                      case n:                                                                                                                 good = ws3_s2<n>(m, n, nt, H, u, fr, tmem + 256, tmem + a2col, P, b2a, a.b2_bytes, lead);              break;
+#define EPIC_S2(n)                                                                                                  \
+    case n:                                                                                                         \
+        good = ws3_s2<n>(m, n, nt, H, u, fr, tmem + 256, tmem + a2col, P, b2a, a.b2_bytes, lead);                   \
+        break;
                     EPIC_KS_CASES(EPIC_S2)
 #undef EPIC_S2
                     default:
@@ -3065,8 +3072,8 @@ epic_status dftgemm_set_group(epic_plan_s* p, int v)
     return st != EPIC_OK ? st : so;
 }
 
-// Work split of k_dftgemm_ws3: -1 = automatic (equal shares unless the launch's items are
-// a whole number per SM), 0 = whole items per block, 1 = equal (item, frame) shares.
+// Work split of k_dftgemm_ws3: -1 = automatic (equal shares where whole items would idle SMs for longer
+// than sharing costs), 0 = whole items per block, 1 = equal (item, frame) shares.
 epic_status dftgemm_set_split(epic_plan_s* p, int mode)
 {
     if (!p->tc.ws || mode < -1 || mode > 1 || (p->sub > 0 && mode == 1)) return EPIC_ERR_UNSUPPORTED;

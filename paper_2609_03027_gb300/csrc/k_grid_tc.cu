@@ -10,9 +10,9 @@
 // accumulated in FP32 in TMEM.  Polarisation-mixed voltages (FP32) are split the same way, and
 // w_hi v_hi + w_lo v_hi + w_hi v_lo is summed (w_lo v_lo, up to 2^-22 of a product, is left out).  The
 // tiles round to 2^-12: errors against 64 bits are those of the FP32 gather kernels to three digits.
-// The gather kernels compute the same sums with FP32 FMAs and are bound by shared-memory gathers and list walks (7.5 k SM cycles a frame of a 96 x 96 box); here
-// a frame takes its MMAs (64 cycles each, 4 a K step, 32 frames) and its tile stores, which bound it (LWA
-// block of 1000 samples: 0.46 ms for 2.4 GB, 0.28 with the stores of a group to one frame; 0.97 by gather).
+// The gather kernels compute the same sums with FP32 FMAs and are bound by shared-memory gathers and list walks
+// (7.5 k SM cycles a frame of a 96 x 96 box); here a frame takes its MMAs (64 cycles each, 4 a K step, 32
+// frames) and its tile stores, which bound it (LWA block of 1000 samples: 0.46 ms for 2.4 GB, 0.28 with the stores of a group to one frame; 0.97 by gather).
 // Work: units of one M-tile and one chunk of up to 4 (8) groups, channel by channel and chunk by chunk, cut
 // into one range of equal modelled cost a block.  What bounds a unit is its tile stores (2.7 k
 // cycles a group at the memory's write rate), so a finer cut matters more than the weights' reuse: ranges of whole

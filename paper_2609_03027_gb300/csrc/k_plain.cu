@@ -9,7 +9,7 @@
 //   k_plain_sum      adds the partial sums up where a chunk's frames were cut into slices
 // The transforms are register-resident two-pass FFTs.  With full N x N grids going through HBM
 // between four kernels (grid, rows, columns, products) the LWA-station block took 34.0 ms, six
-// passes over 33.5 GB at 0.97 of the copy rate; the box rows are 48 of 128 there and go through
+// passes over 33.5 GB at 0.87 of the copy rate; the box rows are 48 of 128 there and go through
 // once each way.  The tuner's second form (fft = 1) keeps the four kernels with radix-4/2 Stockham
 // transforms in shared memory:
 //   k_plain_grid, k_plain_fft_rows_smem, k_plain_fft_cols_smem, k_plain_sqacc
@@ -128,7 +128,7 @@ __host__ __device__ constexpr size_t rows_fft_smem()
     return sizeof(float2) * ((size_t)N1 * N2 + (size_t)(kRowThreads / N2) * N2 * (N1 + 1));
 }
 
-// Gridded and row-transformed frames (LWA station: 5.1 ms a block, 2.9 ms of it the 12.9 GB of row
+// Gridded and row-transformed frames (LWA station: 5.1 ms a block, 2.9 ms of it the 12.6 GB of row
 // stores, the rest the gather's dependent list and voltage reads; 5.6 ms with three blocks an SM instead of
 // four, before a row's cells shared Y's memory): block = frames F blockIdx.x ... of
 // channel blockIdx.y, slice blockIdx.z of the box rows.
@@ -883,7 +883,8 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             // of a 512-pixel grid: 2.45 ms a block of 1024 samples with 128 blocks a chunk, 1.97 with slices)
             auto grid_of = [&](int frames) {
                 const int batch = rf.rows_batch[frames > 1], fb = (nt + frames - 1) / frames;
-                return dim3(fb, C, std::max(1, std::min((ny_max + batch - 1) / batch, (int)(8LL * p->sm_count / ((long long)fb * C)))));
+                const int fill = (int)(8LL * p->sm_count / ((long long)fb * C));
+                return dim3(fb, C, std::max(1, std::min((ny_max + batch - 1) / batch, fill)));
             };
             auto blocks = [](dim3 g) { return (long long)g.x * g.y * g.z; };
             // Short launches.  Frames are staged as FP32 samples wherever all blocks are resident with them (1861 elements,

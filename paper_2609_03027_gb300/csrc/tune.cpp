@@ -42,7 +42,7 @@ std::vector<Knob> knobs_for(const epic_plan_s* p)
         knobs.push_back({"slab", {8, 16, 32}, p->slab, set_fused_slab});
     } else if (p->path == EPIC_PATH_DFTGEMM_FP16) {
         if (p->tc.ws) knobs.push_back({"group", {0, 1}, p->tc.group, set_dft_group});
-        if (p->tc.ws && p->sub == 0) {  // sub-integrations use the control-warp kernel on whole items
+        if (p->tc.ws && p->sub == 0) {  // sub-integrations use the control-warp kernel, cut between intervals
             knobs.push_back({"mma_kernel", {1, 2, 3}, p->tc.ws_variant, set_dft_kernel});
             knobs.push_back({"split", {-1, 0, 1}, p->tc.split, set_dft_split});
         }
