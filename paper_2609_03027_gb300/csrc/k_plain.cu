@@ -888,19 +888,22 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             };
             auto blocks = [](dim3 g) { return (long long)g.x * g.y * g.z; };
             // Short launches.  Frames are staged as FP32 samples wherever all blocks are resident with them (1861 elements,
-            // 54 channels of 16 x 16 cells, one sample: 138 us, 337 as bytes).  One frame a block while two would
-            // leave SMs with fewer than four blocks, unless a thread then walks more lists: a walk takes 1.4 times as
+            // 54 channels of 16 x 16 cells, one sample: 138 us, 337 as bytes).  Long lists: one frame a block while two
+            // would leave SMs with fewer than four blocks, unless a thread then walks more of them: a walk takes 1.4 times as
             // long for two frames, but a batch of one has up to twice the rows.  Us of rows with two frames a block and
             // with one: 41 channels of 16 x 16 cells of 53 entries, 2 samples 66 and 45; 113 of 32 x 32 cells of 81
-            // entries, one sample 227 and 113; 4 of 32 x 32 cells of 96 entries, one 77 and 130.
+            // entries, one sample 227 and 113; 4 of 32 x 32 cells of 96 entries, one 77 and 130.  Short lists gain nothing
+            // (44 channels of 16 x 16 cells of 2 entries, 24 samples: 21 us a call with two, 24 with one).
             auto fits = [&](int frames, dim3 g) {
                 const size_t per_sm = (size_t)((blocks(g) + p->sm_count - 1) / p->sm_count);
                 return form == kFrameStaged || rf.rows_fft + frame_smem(p, kFrameStaged, frames) <= (size_t)p->smem_optin / per_sm;
             };
             auto walks = [&](int i) { return (std::min(rf.rows_batch[i], ny_max) * p->box_max_x + kRowThreads - 1) / kRowThreads; };
             dim3 g = grid_of(kRowFrames);
-            const int frames =
-                blocks(g) < 4LL * p->sm_count && 5 * walks(0) <= 7 * walks(1) && fits(1, grid_of(1)) ? 1 : kRowFrames;
+            const bool longer = (double)A * p->K * p->K >= 8.0 * p->box_max_x * ny_max;  // eight entries a cell
+            const int frames = longer && blocks(g) < 4LL * p->sm_count && 5 * walks(0) <= 7 * walks(1) && fits(1, grid_of(1))
+                                   ? 1
+                                   : kRowFrames;
             if (frames == 1) g = grid_of(1);
             if (form != kFrameStaged && fits(frames, g)) {
                 form = kFrameStaged;
@@ -920,10 +923,14 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
                 partial = reinterpret_cast<float*>(
                     (uint8_t*)p->scratch + ((sizeof(float2) * (size_t)p->time_chunk * C * P * ny_max * N + 255) & ~(size_t)255));
             ev_begin(p, "k_plain_cols", s);
-            // Early where its blocks fill the chip: fewer of them would crowd onto the SMs that come free first (21
-            // blocks of 100 frames, one 32 x 32 image set: 158 us a call, 62 in turn)
-            const bool full = (long long)(N / rf.col_tile) * C * S >= p->plain_slots;
-            launch_early(full, cuts > 1 ? rf.cut : rf.cols, dim3(N / rf.col_tile, C, S), rf.col_threads, cols_smem_for(p, rf), s,
+            // Started early, few blocks would crowd onto the SMs that come free first (21 blocks of 100 frames: 158 us a call,
+            // 62 in turn): they ask for as much shared memory as spreads them evenly (8 channels of 32 x 32 pixels, 243
+            // samples in 16 slices: 35 us in turn, 49 early, 32 early and spread).
+            const int per_sm = (int)(((long long)(N / rf.col_tile) * C * S + p->sm_count - 1) / p->sm_count);
+            size_t smem = cols_smem_for(p, rf);
+            if (per_sm < p->plain_slots / p->sm_count)  // an SM has 1 KB more than a block may take, and keeps 1 KB of each
+                smem = std::max(smem, ((size_t)p->smem_optin + 1024) / per_sm - 1024);
+            launch_early(true, cuts > 1 ? rf.cut : rf.cols, dim3(N / rf.col_tile, C, S), rf.col_threads, smem, s,
                          (const float2*)grid, nt, C, ny_max, p->dt.box, p->dt.twiddle, out, partial,
                          cuts > 1 ? 0 : partial ? t0 > 0 : acc, p->sub, p->sub > 0 ? t0 / p->sub : 0, cuts);
             ev_end(p, s);

@@ -19,12 +19,8 @@ __device__ __forceinline__ float2 unpack44(uint32_t b)
 // real byte followed by an imaginary byte (bits 8, paper Sec. 4), two's complement.
 __device__ __forceinline__ float2 load_sample(const uint8_t* frame, size_t idx, int bits)
 {
-    if (bits == 8) {  // frames begin at any byte
-        const uint8_t* q = frame + 2 * idx;
-        const char2 v = (reinterpret_cast<uintptr_t>(q) & 1) == 0 ? *reinterpret_cast<const char2*>(q)
-                                                                  : make_char2((signed char)q[0], (signed char)q[1]);
-        return make_float2((float)v.x, (float)v.y);
-    }
+    if (bits == 8)  // by bytes: frames begin at any
+        return make_float2((float)(int8_t)frame[2 * idx], (float)(int8_t)frame[2 * idx + 1]);
     return unpack44(frame[idx]);
 }
 
