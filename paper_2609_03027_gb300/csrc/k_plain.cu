@@ -96,12 +96,16 @@ __device__ __forceinline__ void load_step_twiddles(float2* tw, const float2* __r
     }
 }
 
-// Samples of element e (0 .. P-1 pols) of a frame: staged FP32 pairs, or decoded from its bytes.
-template <int P, bool STAGED>
+// How k_plain_rows reads a frame's samples: decoded from the frame (which begins at an even byte where samples have
+// 8 bits), staged FP32 pairs, or decoded by bytes.
+enum RowForm { kRowDecode, kRowStaged, kRowBytes };
+
+// Samples of element e (0 .. P-1 pols) of a frame.
+template <int P, int FORM>
 __device__ __forceinline__ void frame_sample(const float2* sv, const uint8_t* fr, int e, int bits, const float4* jm,
                                              float2 (&v)[P])
 {
-    if (STAGED) {
+    if (FORM == kRowStaged) {
         if (P == 2) {
             const float4 q = *reinterpret_cast<const float4*>(sv + 2 * e);
             v[0] = make_float2(q.x, q.y);
@@ -110,11 +114,11 @@ __device__ __forceinline__ void frame_sample(const float2* sv, const uint8_t* fr
             v[0] = sv[e];
         }
     } else if (P == 2) {
-        const float4 q = load_pair(fr, e, bits, jm);
+        const float4 q = load_pair<FORM == kRowDecode>(fr, e, bits, jm);
         v[0] = make_float2(q.x, q.y);
         v[P - 1] = make_float2(q.z, q.w);
     } else {
-        v[0] = load_sample(fr, e, bits);
+        v[0] = load_sample<FORM == kRowDecode>(fr, e, bits);
     }
 }
 
@@ -137,7 +141,7 @@ __host__ __device__ constexpr size_t rows_fft_smem()
 // passes (thread j takes n1 = j, j + N2 in pass 1 and k2 = j in pass 2; Y is stored [k2][n1] with
 // stride N1 + 1, which no pass-1 store or pass-2 load of a warp meets twice in one bank) and
 // store rows[(t C + c) P + p][y - y0][N].
-template <int N1, int N2, int P, bool STAGED, bool CPLX, int F>
+template <int N1, int N2, int P, int FORM, bool CPLX, int F>
 __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __restrict__ volt, int t0, int nt, int C, int A,
                                                             int bits, const int4* __restrict__ box,
                                                             const int* __restrict__ cell_off,
@@ -167,7 +171,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
 #pragma unroll
     for (int f = 0; f < F; ++f) {
         fr[f] = volt + ((size_t)(t0 + min(f0 + f, nt - 1)) * C + c) * (size_t)FB;  // an odd last frame twice
-        if (STAGED) {
+        if (FORM == kRowStaged) {
             stage_frame(sv + (size_t)f * A * P, fr[f], A, P, bits, jm);
         } else if (frame_in_smem) {
             uint8_t* d = fr_s + (size_t)f * ((FB + 15) & ~15);
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
                     auto entry = [&](int i) {
                         const float2 w = CPLX ? __ldg(cw + i) : make_float2(__ldg(&cw[i].x), 0.f);
                         float2 v[P];
-                        frame_sample<P, STAGED>(sv, fr[0], __ldg(ce + i), bits, jm, v);
+                        frame_sample<P, FORM>(sv, fr[0], __ldg(ce + i), bits, jm, v);
 #pragma unroll
                         for (int p = 0; p < P; ++p) acc[0][p] = cfma(w, v[p], acc[0][p]);
                     };
@@ -211,7 +215,7 @@ __global__ void __launch_bounds__(kRowThreads) k_plain_rows(const uint8_t* __res
 #pragma unroll
                         for (int f = 0; f < F; ++f) {
                             float2 v[P];
-                            frame_sample<P, STAGED>(sv + (size_t)f * A * P, fr[f], e, bits, jm, v);
+                            frame_sample<P, FORM>(sv + (size_t)f * A * P, fr[f], e, bits, jm, v);
 #pragma unroll
                             for (int p = 0; p < P; ++p) {
                                 if (CPLX) acc[f][p] = cfma(w, v[p], acc[f][p]);
@@ -469,6 +473,9 @@ struct RegFft {
     // of one frame a block, of kRowFrames
     void (*rows[2])(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
                     const float4*, int, int, const float2*, float2*);
+    // of one frame, read by bytes: 8-bit samples at an odd address in frames that are not staged at all
+    void (*rows_bytes)(const uint8_t*, int, int, int, int, int, const int4*, const int*, const int*, const int*, const float2*,
+                       const float4*, int, int, const float2*, float2*);
     void (*cols)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int, int);
     void (*cut)(const float2*, int, int, int, const int4*, const float2*, float*, float*, int, int, int, int);
     int col_tile, col_threads;
@@ -484,10 +491,11 @@ RegFft reg_fft_p(bool staged, bool cplx)
     // 128 threads a block (fewer for the smallest grids): four to eight blocks an SM hide the barriers
     constexpr int TX = 128 / N2 < N ? 128 / N2 : N;
     RegFft f{};
-    f.rows[0] = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true, 1> : k_plain_rows<N1, N2, P, true, false, 1>)
-                       : (cplx ? k_plain_rows<N1, N2, P, false, true, 1> : k_plain_rows<N1, N2, P, false, false, 1>);
-    f.rows[1] = staged ? (cplx ? k_plain_rows<N1, N2, P, true, true, kRowFrames> : k_plain_rows<N1, N2, P, true, false, kRowFrames>)
-                       : (cplx ? k_plain_rows<N1, N2, P, false, true, kRowFrames> : k_plain_rows<N1, N2, P, false, false, kRowFrames>);
+#define EPIC_ROWS(form, F) (cplx ? k_plain_rows<N1, N2, P, form, true, F> : k_plain_rows<N1, N2, P, form, false, F>)
+    f.rows[0] = staged ? EPIC_ROWS(kRowStaged, 1) : EPIC_ROWS(kRowDecode, 1);
+    f.rows[1] = staged ? EPIC_ROWS(kRowStaged, kRowFrames) : EPIC_ROWS(kRowDecode, kRowFrames);
+    f.rows_bytes = EPIC_ROWS(kRowBytes, 1);
+#undef EPIC_ROWS
     f.cols = k_plain_cols<N1, N2, TX, P, false>;
     f.cut = k_plain_cols<N1, N2, TX, P, true>;
     f.col_tile = TX;
@@ -838,6 +846,7 @@ epic_status plain_setup(epic_plan_s* p)
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)  // short launches stage their frames
         e = allow_max_smem((const void*)(i < 2 ? rf : reg_fft_for(p, true)).rows[i & 1], p->smem_optin);
+    if (e == cudaSuccess) e = allow_max_smem((const void*)rf.rows_bytes, p->smem_optin);
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_plain_rows)");
     e = allow_max_smem((const void*)rf.cols, p->smem_optin);
     if (e == cudaSuccess) e = allow_max_smem((const void*)rf.cut, p->smem_optin);
@@ -904,12 +913,13 @@ epic_status plain_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t s
             const int frames = longer && blocks(g) < 4LL * p->sm_count && 5 * walks(0) <= 7 * walks(1) && fits(1, grid_of(1))
                                    ? 1
                                    : kRowFrames;
-            if (frames == 1) g = grid_of(1);
-            if (form != kFrameStaged && fits(frames, g)) {
+            const bool odd = bits == 8 && ((uintptr_t)volt & 1) != 0 && form == kFrameGlobal;
+            if (frames == 1 || odd) g = grid_of(1);
+            if (form != kFrameStaged && !odd && fits(frames, g)) {
                 form = kFrameStaged;
                 rf = reg_fft_for(p, true);
             }
-            launch_early(t0 > 0, rf.rows[frames > 1], g, kRowThreads,
+            launch_early(t0 > 0, odd ? rf.rows_bytes : rf.rows[frames > 1], g, kRowThreads,
                          rf.rows_fft + frame_smem(p, form, frames), s, volt, t0, nt, C, A, bits, p->dt.box, p->dt.cell_off,
                          p->dt.cell_ptr, p->dt.contrib_e, p->dt.contrib_w, p->dt.jones, form == kFrameBytes ? 1 : 0, ny_max, p->dt.twiddle, grid);
             ev_end(p, s);

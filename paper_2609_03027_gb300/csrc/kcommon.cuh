@@ -17,8 +17,14 @@ __device__ __forceinline__ float2 unpack44(uint32_t b)
 
 // Complex sample idx (= element * P + pol) of one frame: a 4+4-bit byte (bits 4) or a
 // real byte followed by an imaginary byte (bits 8, paper Sec. 4), two's complement.
+// WORDS: 8-bit samples of frames that begin at an even byte, read whole.
+template <bool WORDS = false>
 __device__ __forceinline__ float2 load_sample(const uint8_t* frame, size_t idx, int bits)
 {
+    if (WORDS && bits == 8) {
+        const char2 v = *reinterpret_cast<const char2*>(frame + 2 * idx);
+        return make_float2((float)v.x, (float)v.y);
+    }
     if (bits == 8)  // by bytes: frames begin at any
         return make_float2((float)(int8_t)frame[2 * idx], (float)(int8_t)frame[2 * idx + 1]);
     return unpack44(frame[idx]);
@@ -32,10 +38,11 @@ __device__ __forceinline__ float2 cfma(float2 w, float2 v, float2 acc);
 // complex 2x2 J per element and channel) the sample of output polarisation a is
 // sum_p conj(J_e^{ap}) E_e^p, which is what gridding with W^{ap*} gives once W*
 // is factored out; jm[2 e + a] = (conj J^{a0}, conj J^{a1}).  jm == nullptr: no mixing.
+template <bool WORDS = false>
 __device__ __forceinline__ float4 load_pair(const uint8_t* frame, int e, int bits, const float4* jm)
 {
-    const float2 x = load_sample(frame, (size_t)e * 2, bits);
-    const float2 y = load_sample(frame, (size_t)e * 2 + 1, bits);
+    const float2 x = load_sample<WORDS>(frame, (size_t)e * 2, bits);
+    const float2 y = load_sample<WORDS>(frame, (size_t)e * 2 + 1, bits);
     if (!jm) return make_float4(x.x, x.y, y.x, y.y);
     const float4 r0 = jm[2 * e], r1 = jm[2 * e + 1];
     const float2 mx = cfma(make_float2(r0.z, r0.w), y, cmul(make_float2(r0.x, r0.y), x));
