@@ -191,9 +191,9 @@ __device__ __forceinline__ void store_pixels16(float* op, int nk, int accumulate
 // then writes the cells as FP16 pairs: consecutive threads cover consecutive
 // cell pairs of a row, so a warp fills whole 128-byte rows of the swizzled tile.
 // With CSR_SMEM the channel's cell lists sit in shared memory as (element, real
-// weight) pairs (Gaussian GCF), otherwise they are read through L1.  The blocks of gridDim.z share the
-// cell pairs.
-template <bool CSR_SMEM, int F>
+// weight) pairs (Gaussian GCF), otherwise they are read through L1.  With ONE (launches of one
+// frame, lists through L1) the blocks of gridDim.z share the cell pairs.
+template <bool CSR_SMEM, int F, bool ONE = false>
 __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __restrict__ volt, int t0, int c0,
                                                            int n_ch, int nt, int fpc, int C, int A, int P,
                                                            int bits, const int4* __restrict__ box,
@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __rest
             sv[f * A + e] = load_quad(fr, e, P, bits, jm);
         }
         __syncthreads();
-        for (int task = threadIdx.x + blockIdx.z * blockDim.x; task < tasks; task += blockDim.x * gridDim.z) {
+        for (int task = threadIdx.x + (ONE ? blockIdx.z * blockDim.x : 0); task < tasks;
+             task += ONE ? blockDim.x * gridDim.z : blockDim.x) {
             const int y = task / half, x = 2 * (task - y * half);
             float4 g[2][F];
 #pragma unroll
@@ -249,30 +250,43 @@ __global__ void __launch_bounds__(kThreads) k_dftgemm_grid(const uint8_t* __rest
                 for (int f = 0; f < F; ++f) g[j][f] = make_float4(0.f, 0.f, 0.f, 0.f);
                 const int r = y * nxp + x + j;
                 const int q1 = y < nyp ? ptr[r + 1] : 0;
-#pragma unroll (F == 1 ? 4 : 2)
-                for (int q = y < nyp ? ptr[r] : 0; q < q1; ++q) {
-                    int e;
-                    float2 w;
-                    if (CSR_SMEM) {
-                        const int2 cr = con[q];
-                        e = cr.x;
-                        w = make_float2(__int_as_float(cr.y), 0.f);
-                    } else {
-                        e = ce[q];
-                        w = cw[q];
-                    }
-#pragma unroll
-                    for (int f = 0; f < F; ++f) {
-                        const float4 v = sv[f * A + e];
+                if constexpr (ONE) {  // four entries' loads at once (1500 elements with an 8 x 8 GCF: 136 -> 75 us); the
+                                      // other forms keep the compiler's own layout, with which 4000 elements on 32 x 32
+                                      // cells take 281 us and not 305
+                    auto entry = [&](int q) {
+                        const float4 v = sv[ce[q]];
+                        const float2 w = cw[q];
+                        const float2 gx = cfma(w, make_float2(v.x, v.y), make_float2(g[j][0].x, g[j][0].y));
+                        const float2 gy = cfma(w, make_float2(v.z, v.w), make_float2(g[j][0].z, g[j][0].w));
+                        g[j][0] = make_float4(gx.x, gx.y, gy.x, gy.y);
+                    };
+#pragma unroll 4
+                    for (int q = y < nyp ? ptr[r] : 0; q < q1; ++q) entry(q);
+                } else {
+                    for (int q = y < nyp ? ptr[r] : 0; q < q1; ++q) {
+                        int e;
+                        float2 w;
                         if (CSR_SMEM) {
-                            g[j][f].x = fmaf(w.x, v.x, g[j][f].x);
-                            g[j][f].y = fmaf(w.x, v.y, g[j][f].y);
-                            g[j][f].z = fmaf(w.x, v.z, g[j][f].z);
-                            g[j][f].w = fmaf(w.x, v.w, g[j][f].w);
+                            const int2 cr = con[q];
+                            e = cr.x;
+                            w = make_float2(__int_as_float(cr.y), 0.f);
                         } else {
-                            const float2 gx = cfma(w, make_float2(v.x, v.y), make_float2(g[j][f].x, g[j][f].y));
-                            const float2 gy = cfma(w, make_float2(v.z, v.w), make_float2(g[j][f].z, g[j][f].w));
-                            g[j][f] = make_float4(gx.x, gx.y, gy.x, gy.y);
+                            e = ce[q];
+                            w = cw[q];
+                        }
+#pragma unroll
+                        for (int f = 0; f < F; ++f) {
+                            const float4 v = sv[f * A + e];
+                            if (CSR_SMEM) {
+                                g[j][f].x = fmaf(w.x, v.x, g[j][f].x);
+                                g[j][f].y = fmaf(w.x, v.y, g[j][f].y);
+                                g[j][f].z = fmaf(w.x, v.z, g[j][f].z);
+                                g[j][f].w = fmaf(w.x, v.w, g[j][f].w);
+                            } else {
+                                const float2 gx = cfma(w, make_float2(v.x, v.y), make_float2(g[j][f].x, g[j][f].y));
+                                const float2 gy = cfma(w, make_float2(v.z, v.w), make_float2(g[j][f].z, g[j][f].w));
+                                g[j][f] = make_float4(gx.x, gx.y, gy.x, gy.y);
+                            }
                         }
                     }
                 }
@@ -3844,6 +3858,7 @@ epic_status dftgemm_setup(epic_plan_s* p)
     EPIC_GRID_ATTR(false, 4)
     EPIC_GRID_ATTR(false, 2)
     EPIC_GRID_ATTR(false, 1)
+    if (e == cudaSuccess) e = allow_max_smem((const void*)k_dftgemm_grid<false, 1, true>, p->smem_optin);
 #undef EPIC_GRID_ATTR
     if (e != cudaSuccess) return cuda_fail(p, e, "cudaFuncSetAttribute(k_dftgemm_grid)");
     e = allow_max_smem((const void*)k_dftgemm_ws<0>, p->smem_optin);
@@ -3941,7 +3956,7 @@ epic_status dftgemm_run(epic_plan_s* p, const uint8_t* volt, int T, cudaStream_t
                 const int pairs = p->tc.grid_max_cells / 2;
                 const unsigned z = std::max(1, std::min((pairs + kThreads - 1) / kThreads, 8 * p->sm_count / ng));
                 ev_begin(p, "k_dftgemm_grid", s);
-                k_dftgemm_grid<false, 1><<<dim3(1, ng, z), kThreads, sizeof(float4) * (size_t)A, s>>>(
+                k_dftgemm_grid<false, 1, true><<<dim3(1, ng, z), kThreads, sizeof(float4) * (size_t)A, s>>>(
                     volt, t0, c0, ng, nt, 1, C, A, P, p->bits, p->dt.box, p->dt.cell_off, p->dt.cell_ptr, p->dt.contrib_e,
                     p->dt.contrib_w, p->dt.jones, p->tc.tbox, (uint8_t*)p->scratch, p->tc.stride);
                 ev_end(p, s);
